@@ -1326,7 +1326,7 @@ int emc_sparse_update(emc_ctx* ctx, const float* P, float* Num, float* den, emc_
   const Layout& y = ctx->lay;
   const bool csr = (ctx->cfg.flags & EMC_FLAG_SPARSE_K) != 0;  // frames' non-zero lists
   CU(launch_sparse_update(ctx->Kb, ctx->cfg.precision == EMC_PREC_FP16_SPLIT, y.ld_pix,
-                          ctx->cfg.n_pix, (const int64_t*)(ctx->ws + y.coff),
+                          (const int64_t*)(ctx->ws + y.coff),
                           (const int2*)(ctx->ws + y.cent), ctx->cfg.n_cand, P, y.rows,
                           csr ? (const int64_t*)(ctx->ws + y.skoff) : nullptr,
                           csr ? (const uint32_t*)(ctx->ws + y.skent) : nullptr, Num, den,

@@ -343,7 +343,7 @@ cudaError_t launch_sparse_lse(const double* Sc, int64_t n_data, int64_t ld_data,
                               const double* shift = nullptr);
 // Bsum, invn (non-NULL): Poisson-fluence model, Num_j = sum P_jk K_k B_j / N_k
 // and den_j = sum P_jk
-cudaError_t launch_sparse_update(const uint16_t* Kb, int kf16, int64_t ld_pix, int64_t n_pix,
+cudaError_t launch_sparse_update(const uint16_t* Kb, int kf16, int64_t ld_pix,
                                  const int64_t* off, const int2* ent, int M, const float* Pc,
                                  int64_t rows, const int64_t* koff, const uint32_t* kent,
                                  float* Num, float* den, cudaStream_t s,
