@@ -38,7 +38,316 @@ __device__ __forceinline__ int block_prefix(int flag, int* warp_tot, int* total)
   return before + in_warp;
 }
 
-// One CTA (256 threads) per row: radix selection of the M-th largest key over
+// Top M in one read of the row (M <= kTopHold), one CTA of 512 threads per row.
+//  * A sample of 512 groups of 8 values spread over the row gives a threshold
+//    that about 1.2 to 3 M of the row's values exceed (topm_rank). Each warp then reads a
+//    contiguous sixteenth of the row, several loads in flight and no barrier, and
+//    packs the values above the threshold into a list of its own, in index order.
+//  * The M-th largest key T of the lists is built bit by bit from block-wide
+//    counts of the keys in registers, which does not depend on how the keys are
+//    spread (a histogram's atomics pile up on the few exponents logits share).
+//  * A row that the sample misjudges (fewer than M values above the threshold, or a
+//    full list; ordered or tied rows), a short row or a long list is streamed
+//    instead: values enter a buffer of 8192 in order; when it is full, T of its entries
+//    is found, the M that count stay, and from then on a value must exceed T to enter (an
+//    equal one comes later in the order, so it loses every tie).
+// Index order is kept throughout, so the last selection writes the result out.
+// Bound by the one read: 2048 x 50100 logits, M = 512 took 701 us with five
+// reads and histograms, 337 us streamed, 198 us so (61 us at the copy rate).
+constexpr int kTopThreads = 512;
+constexpr int kTopHold = 4096;   // longest list
+constexpr int kTopCap = 8192;    // buffer entries: 16 per thread
+constexpr int kTopChunk = 8 * kTopThreads;
+constexpr int kTopPad = kTopCap + kTopCap / 16;  // entry e at e + e / 16: fewer bank conflicts
+constexpr int kTopWarp = 256;    // entries of a warp's list
+constexpr int kTopLists = 16 * kTopWarp;
+static_assert(kTopHold + kTopChunk <= kTopCap, "a chunk fits after a selection");
+constexpr size_t kTopSmem = 2 * sizeof(uint32_t) * kTopPad;
+__device__ __forceinline__ int top_at(int e) { return e + (e >> 4); }
+
+// Rank in the sample of 8 * 512 that leaves at least M of n values above it
+// but for a chance of about 1e-4, or 0 where the lists would be too full (or
+// the row too short to gain): four standard deviations of the sample's count more.
+int topm_rank(int64_t n, int M) {
+  const double mean = (double)M * kTopChunk / (double)n;
+  const int r = (int)(mean + 4.0 * sqrt(mean) + 4.0);
+  return n >= 4 * kTopChunk && (double)r * n <= 2048.0 * kTopChunk ? r : 0;
+}
+
+// block-wide sum; wt: one of two 16-entry buffers used in turn
+__device__ __forceinline__ int top_sum(int v, int* wt) {
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  v = __reduce_add_sync(0xffffffffu, v);
+  if (lane == 0) wt[wid] = v;
+  __syncthreads();
+  return __reduce_add_sync(0xffffffffu, lane < 16 ? wt[lane] : 0);
+}
+
+// block-wide exclusive prefix of v; *total: the sum
+__device__ __forceinline__ int top_prefix(int v, int* wt, int* total) {
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  int inc = v;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int u = __shfl_up_sync(0xffffffffu, inc, o);
+    if (lane >= o) inc += u;
+  }
+  if (lane == 31) wt[wid] = inc;
+  __syncthreads();
+  const int w = lane < 16 ? wt[lane] : 0;
+  *total = __reduce_add_sync(0xffffffffu, w);
+  return inc - v + __reduce_add_sync(0xffffffffu, lane < wid ? w : 0);
+}
+
+// The M-th largest of the keys in the threads' registers (per of them each;
+// unused ones are 0 and there are at least M others), down to bit `low`
+// (bits below it 0: a lower bound). par: the buffer of wt that is next.
+template <int MAXPER>
+__device__ __forceinline__ uint32_t top_key(const uint32_t (&k)[MAXPER], int per, int M, int low,
+                                            int* wt, int& par) {
+  uint32_t T = 0;
+  for (int bit = 31; bit >= low; bit--) {
+    const uint32_t c = T | (1u << bit);  // > 0: unused keys do not count
+    int g = 0;
+#pragma unroll
+    for (int i = 0; i < MAXPER; i++) {
+      if (i >= per) break;
+      g += k[i] >= c;
+    }
+    g = top_sum(g, wt + 16 * par);
+    par ^= 1;
+    if (g >= M) T = c;
+    if (g == M) break;  // exactly the keys >= T
+  }
+  return T;
+}
+
+// T, the M-th largest of the buffer's cnt >= M keys (returned); the M entries
+// that count stay, in index order: in the buffer, or (FINAL) in out, the larger
+// ones first and then the first equal ones. s_min: a word of shared memory.
+template <bool FINAL>
+__device__ __forceinline__ uint32_t top_select(uint32_t* keys, int* idx, int cnt, int M, int* wt,
+                                               int& par, uint32_t* s_min, int32_t* out) {
+  const int per = (cnt + kTopThreads - 1) / kTopThreads;  // <= 16
+  const int e0 = threadIdx.x * per, mine = min(max(cnt - e0, 0), per);
+  if (threadIdx.x == 0) *s_min = 0xffffffffu;
+  uint32_t k[16];
+#pragma unroll
+  for (int i = 0; i < 16; i++) k[i] = i < mine ? keys[top_at(e0 + i)] : 0u;
+  uint32_t T = top_key(k, per, M, 0, wt, par);
+  // where the bits ended early (exactly M keys >= T): the smallest of those
+  uint32_t lo = 0xffffffffu;
+#pragma unroll
+  for (int i = 0; i < 16; i++)
+    if (i < mine && k[i] >= T) lo = min(lo, k[i]);
+  lo = __reduce_min_sync(0xffffffffu, lo);
+  if ((threadIdx.x & 31) == 0) atomicMin(s_min, lo);
+  __syncthreads();
+  T = *s_min;
+  int gt = 0, eq = 0;
+#pragma unroll
+  for (int i = 0; i < 16; i++) {
+    gt += i < mine && k[i] > T;
+    eq += i < mine && k[i] == T;
+  }
+  int total;
+  const int before = top_prefix(gt | (eq << 16), wt + 16 * par, &total);
+  par ^= 1;
+  const int need = M - (total & 0xffff);
+  int ng = before & 0xffff, ne = before >> 16;
+  if (FINAL) {
+#pragma unroll
+    for (int i = 0; i < 16; i++) {
+      if (i >= mine) break;
+      if (k[i] > T) {
+        out[ng++] = idx[top_at(e0 + i)];
+      } else if (k[i] == T) {
+        if (ne < need) out[M - need + ne] = idx[top_at(e0 + i)];
+        ne++;
+      }
+    }
+  } else {
+    int id[16];
+#pragma unroll
+    for (int i = 0; i < 16; i++) id[i] = i < mine ? idx[top_at(e0 + i)] : 0;
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < 16; i++) {
+      if (i >= mine) break;
+      const bool g = k[i] > T, q = k[i] == T;
+      if (g || (q && ne < need)) {
+        const int at = top_at(ng + min(ne, need));
+        keys[at] = k[i];
+        idx[at] = id[i];
+      }
+      ng += g;
+      ne += q;
+    }
+    __syncthreads();
+  }
+  return T;
+}
+
+// VEC: rows start on 16-byte boundaries
+template <bool VEC>
+__device__ __forceinline__ void top_load8(const float* z, int64_t e, int n, float (&v)[8]) {
+  if (VEC && e + 8 <= n) {
+    const float4 a = *reinterpret_cast<const float4*>(z + e);
+    const float4 b = *reinterpret_cast<const float4*>(z + e + 4);
+    v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
+    v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
+  } else {
+#pragma unroll
+    for (int i = 0; i < 8; i++) v[i] = e + i < n ? z[e + i] : 0.f;
+  }
+}
+
+// the streamed form; returns the entries left in the buffer
+template <bool VEC>
+__device__ __noinline__ int top_stream(const float* z, int n, int M, uint32_t* keys, int* idx,
+                                       int* wt, uint32_t* s_min) {
+  int par = 0, cnt = 0;
+  bool has = false;   // T bounds what may enter
+  uint32_t T = 0;
+  float v[8];
+  top_load8<VEC>(z, 8 * threadIdx.x, n, v);
+  for (int64_t base = 0; base < n; base += kTopChunk) {
+    const int64_t e = base + 8 * threadIdx.x;
+    uint32_t k[8];
+#pragma unroll
+    for (int i = 0; i < 8; i++) k[i] = order_key(v[i]);
+    if (base + kTopChunk < n) top_load8<VEC>(z, e + kTopChunk, n, v);
+    int at, total;
+    unsigned enter;
+    while (true) {
+      enter = 0;
+#pragma unroll
+      for (int i = 0; i < 8; i++) enter |= (e + i < n && (!has || k[i] > T)) ? 1u << i : 0u;
+      at = top_prefix(__popc(enter), wt + 16 * par, &total);
+      par ^= 1;
+      if (cnt + total <= kTopCap) break;
+      T = top_select<false>(keys, idx, cnt, M, wt, par, s_min, nullptr);
+      has = true;
+      cnt = M;
+    }
+    at += cnt;
+#pragma unroll
+    for (int i = 0; i < 8; i++)
+      if (enter & (1u << i)) {
+        const int p = top_at(at++);
+        keys[p] = k[i];
+        idx[p] = (int)(e + i);
+      }
+    cnt += total;
+  }
+  __syncthreads();
+  return cnt;
+}
+
+template <bool VEC>
+__global__ void __launch_bounds__(kTopThreads, 2)
+    topm_stream_kernel(const float* __restrict__ logits, int64_t ld, int n, int M, int rank,
+                       int32_t* __restrict__ cand) {
+  const float* z = logits + (int64_t)blockIdx.x * ld;
+  extern __shared__ uint32_t top_smem[];
+  uint32_t* keys = top_smem;
+  int* idx = reinterpret_cast<int*>(top_smem + kTopPad);
+  __shared__ int wt[32];
+  __shared__ int lists[17];
+  __shared__ uint32_t s_min;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  int par = 0, cnt = 0;
+  bool ok = false;
+  if (rank > 0) {
+    // the sample: 8 values every n / 512, the start rounded to a multiple of 8
+    const int64_t at = ((int64_t)threadIdx.x * (n - 8) / (kTopThreads - 1)) & ~(int64_t)7;
+    float v[8];
+    top_load8<VEC>(z, at, n, v);
+    uint32_t k[8];
+#pragma unroll
+    for (int i = 0; i < 8; i++) k[i] = order_key(v[i]);
+    const uint32_t T0 = top_key(k, 8, rank, 16, wt, par);
+    // the warp's sixteenth, 512 values a step (4 x 4 consecutive ones per lane)
+    const int64_t seg = ((int64_t)(n + 15) / 16 + 3) & ~(int64_t)3;
+    const int64_t b = wid * seg, end = min((int64_t)n, b + seg);
+    uint32_t* lk = keys + wid * kTopWarp;
+    int* li = idx + wid * kTopWarp;
+    int len = 0;
+    const unsigned below = (1u << lane) - 1u;
+    for (int64_t e0 = b; e0 < end; e0 += 512) {
+      float4 w[4];
+#pragma unroll
+      for (int u = 0; u < 4; u++) {
+        const int64_t e = e0 + u * 128 + 4 * lane;
+        if (VEC && e + 4 <= end) {
+          w[u] = __ldcs(reinterpret_cast<const float4*>(z + e));
+        } else {
+          w[u].x = e < end ? z[e] : 0.f;
+          w[u].y = e + 1 < end ? z[e + 1] : 0.f;
+          w[u].z = e + 2 < end ? z[e + 2] : 0.f;
+          w[u].w = e + 3 < end ? z[e + 3] : 0.f;
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < 4; u++) {
+        const int64_t e = e0 + u * 128 + 4 * lane;
+        const uint32_t kk[4] = {order_key(w[u].x), order_key(w[u].y), order_key(w[u].z),
+                                order_key(w[u].w)};
+        unsigned m = 0;
+#pragma unroll
+        for (int i = 0; i < 4; i++) m |= (e + i < end && kk[i] >= T0) ? 1u << i : 0u;
+        if (!__any_sync(0xffffffffu, m)) continue;
+        int p = len, tot = 0;
+#pragma unroll
+        for (int i = 0; i < 4; i++) {
+          const unsigned bal = __ballot_sync(0xffffffffu, m & (1u << i));
+          p += __popc(bal & below);
+          tot += __popc(bal);
+        }
+#pragma unroll
+        for (int i = 0; i < 4; i++)
+          if (m & (1u << i)) {
+            if (p < kTopWarp) {
+              lk[p] = kk[i];
+              li[p] = (int)(e + i);
+            }
+            p++;
+          }
+        len += tot;  // beyond kTopWarp: the row is streamed
+      }
+    }
+    if (lane == 0) lists[wid] = len;
+    __syncthreads();
+    int start = 0, most = 0;
+#pragma unroll
+    for (int w = 0; w < 16; w++) {
+      if (w < wid) start += lists[w];
+      cnt += lists[w];
+      most = max(most, lists[w]);
+    }
+    ok = most <= kTopWarp && cnt >= M;
+    if (ok) {
+      // the lists behind one another, above them in the same arrays
+      uint32_t* ck = keys + kTopLists;
+      int* ci = idx + kTopLists;
+      __syncwarp();
+      for (int t = lane; t < len; t += 32) {
+        ck[top_at(start + t)] = lk[t];
+        ci[top_at(start + t)] = li[t];
+      }
+      keys = ck;
+      idx = ci;
+    }
+    __syncthreads();
+  }
+  if (!ok) {
+    cnt = top_stream<VEC>(z, n, M, keys, idx, wt, &s_min);
+    par = 0;
+  }
+  top_select<true>(keys, idx, cnt, M, wt, par, &s_min, cand + (int64_t)blockIdx.x * M);
+}
+
+// Longer lists. One CTA (256 threads) per row: radix selection of the M-th largest key over
 // four 8-bit digits, then the keys above it in index order followed by the
 // first equal keys in index order (ties towards the lower index).
 __global__ void __launch_bounds__(256)
@@ -98,6 +407,15 @@ __global__ void __launch_bounds__(256)
 cudaError_t launch_topm(const float* logits, int64_t B, int64_t n, int64_t ld, int M,
                         int32_t* cand, cudaStream_t s) {
   if (B <= 0) return cudaSuccess;
+  if (M <= kTopHold) {
+    const bool vec = ld % 4 == 0 && ((uintptr_t)logits & 15) == 0;
+    auto kern = vec ? topm_stream_kernel<true> : topm_stream_kernel<false>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)kTopSmem);
+    if (e != cudaSuccess) return e;
+    kern<<<(unsigned)B, kTopThreads, kTopSmem, s>>>(logits, ld, (int)n, M, topm_rank(n, M), cand);
+    return cudaGetLastError();
+  }
   topm_kernel<<<(unsigned)B, 256, 0, s>>>(logits, ld, (int)n, M, cand);
   return cudaGetLastError();
 }
