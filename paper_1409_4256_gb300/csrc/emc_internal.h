@@ -275,6 +275,10 @@ int64_t tc_pass1_tiles(int64_t rows);
 cudaError_t launch_tc_store(const Planes& A, int64_t rows, const uint16_t* Kb, int64_t ld_data,
                             int64_t ld_pix, float* C, int f16, int32_t* status, cudaStream_t s,
                             TcCtl ctl = TcCtl{});
+// C[M][N] (FP32) = A[M][K] B[N][K]^T, both BF16 with K contiguous; M a multiple of
+// 128, N of 32, K of 64: narrow tiles, for few rows and columns and a long sum.
+cudaError_t launch_tc_nt(const uint16_t* A, const uint16_t* B, int64_t M, int64_t N, int64_t K,
+                         float* C, int32_t* status, cudaStream_t s);
 // Bound pass of the pruned pass 1: per 128-row tile and frame, the maximum of
 // S^hi = (first plane of L) K^T + bias into part_m[rows / 128][ld_data]
 // (pairs of row tiles per CTA tile sharing the frame operand).

@@ -9,14 +9,17 @@
 //
 // Matrix products use BF16-rounded operands with FP32 accumulation ("BF16
 // matmuls, FP32 master weights"). The output layer (512 x n_out, nearly all
-// of the work) runs on the tensor cores through the update form of the
-// tcgen05 kernel (K-major A, MN-major B, FP32 rows out): Z = H3 W4,
-// dH3 = dZ (W4^T) and dW4 = (H3^T) dZ, from BF16 copies (W4, its transpose,
-// H3^T, dZ) made by the kernels below, whenever the batch is a multiple of
+// of the work) runs on the tensor cores: Z = H3 W4 and dW4 = (H3^T) dZ
+// through the update form of the tcgen05 kernel (K-major A, MN-major B, FP32
+// rows out), dH3 = dZ W4^T through its store form (both K-major), from BF16
+// copies made by the kernels below, whenever the batch is a multiple of
 // 128. The 512 x 512 layers and other batches use a tiled SIMT kernel that
 // serves the three layouts (X W, dY W^T, X^T dY). Parameters live in one FP32
 // array: W1[512][512] b1[512] W2 b2 W3 b3 W4[512][ld_out] b4[ld_out],
 // ld_out = round_up(n_out, 64).
+#include <algorithm>
+#include <utility>
+
 #include "emc_common.cuh"
 #include "emc_internal.h"
 
@@ -54,10 +57,15 @@ cudaError_t launch_features(const uint16_t* Kb, int kf16, int64_t ld_pix, int64_
 }
 
 // -------------------------------------------------------------------- GEMM --
-// C[M][N] = op(A) op(B) (+ bias[N]); op(A)[m][k] = TA ? A[k*lda + m] : A[m*lda + k],
+// C[M][N] = op(A) op(B); op(A)[m][k] = TA ? A[k*lda + m] : A[m*lda + k],
 // op(B)[k][n] = TB ? B[n*ldb + k] : B[k*ldb + n]. EPI: 0 plain, 1 bias,
-// 2 bias + GELU (the pre-activation goes to `pre`, GELU of it to C).
-constexpr int G_BM = 64, G_BN = 64, G_BK = 16, G_THREADS = 256;
+// 2 bias + GELU (the pre-activation goes to `pre`, GELU of it to C, and where
+// given its BF16 copies to hb [M][ldc] and transposed to ht [N][M]),
+// 3 times GELU'(pre) (the backward pass through the activation).
+// A 512 x 512 x 512 layer is 32 x 64 tiles on 128 CTAs, one per SM, the next K
+// block's loads in flight while this one is summed: 38 -> 22 us (64 x 64 tiles on
+// 64 CTAs waited out every block's load latency). Every element still sums its products in order of k.
+constexpr int G_BM = 32, G_BN = 64, G_BK = 32, G_THREADS = 256;
 
 __device__ __forceinline__ float bf16_round(float x) { return bf16_val(bf16_bits(x)); }
 
@@ -69,67 +77,95 @@ __device__ __forceinline__ float gelu_grad_f(float x) {
          x * __expf(-0.5f * x * x) * 0.39894228040143268f;
 }
 
+struct GemmEpi {
+  const float* bias;
+  float* pre;
+  int64_t ldpre;
+  uint16_t* hb;
+  uint16_t* ht;
+  float* bsum;  // column sums of op(B) in order of k, unrounded (EPI 0; bias gradients)
+};
+
 template <bool TA, bool TB, int EPI>
 __global__ void __launch_bounds__(G_THREADS)
     mlp_gemm_kernel(int M, int N, int K, const float* __restrict__ A, int64_t lda,
                     const float* __restrict__ B, int64_t ldb, float* __restrict__ C, int64_t ldc,
-                    const float* __restrict__ bias, float* __restrict__ pre, int64_t ldpre) {
-  __shared__ float As[G_BK][G_BM + 4];
-  __shared__ float Bs[G_BK][G_BN + 4];
+                    const GemmEpi ep) {
+  __shared__ __align__(16) float As[G_BK][G_BM + 4];
+  __shared__ __align__(16) float Bs[G_BK][G_BN + 4];
+  constexpr int NA = G_BM * G_BK / G_THREADS, NB = G_BN * G_BK / G_THREADS;
+  __shared__ float Bw[EPI == 0 ? G_BK : 1][G_BN];
   const int t = threadIdx.x, tx = t & 15, ty = t >> 4;
   const int m0 = blockIdx.y * G_BM, n0 = blockIdx.x * G_BN;
-  float acc[4][4] = {};
-  for (int k0 = 0; k0 < K; k0 += G_BK) {
-    // 64 x 16 tiles of op(A) and 16 x 64 of op(B): 4 elements per thread each
+  const bool sums = EPI == 0 && ep.bsum && blockIdx.y == 0;
+  float bs = 0.f;
+  float ra[NA], rb[NB];
+  auto load = [&](int k0) {
 #pragma unroll
-    for (int u = 0; u < 4; u++) {
+    for (int u = 0; u < NA; u++) {
       const int e = t + u * G_THREADS;
-      {
-        int mm, kk;
-        if (TA) { kk = e / G_BM; mm = e % G_BM; } else { mm = e / G_BK; kk = e % G_BK; }
-        const int gm = m0 + mm, gk = k0 + kk;
-        float v = 0.f;
-        if (gm < M && gk < K) v = TA ? A[(int64_t)gk * lda + gm] : A[(int64_t)gm * lda + gk];
-        As[kk][mm] = bf16_round(v);
-      }
-      {
-        int nn, kk;
-        if (TB) { nn = e / G_BK; kk = e % G_BK; } else { kk = e / G_BN; nn = e % G_BN; }
-        const int gn = n0 + nn, gk = k0 + kk;
-        float v = 0.f;
-        if (gn < N && gk < K) v = TB ? B[(int64_t)gn * ldb + gk] : B[(int64_t)gk * ldb + gn];
-        Bs[kk][nn] = bf16_round(v);
-      }
+      const int gm = m0 + (TA ? e % G_BM : e / G_BK), gk = k0 + (TA ? e / G_BM : e % G_BK);
+      ra[u] = gm < M && gk < K ? (TA ? A[(int64_t)gk * lda + gm] : A[(int64_t)gm * lda + gk]) : 0.f;
+    }
+#pragma unroll
+    for (int u = 0; u < NB; u++) {
+      const int e = t + u * G_THREADS;
+      const int gn = n0 + (TB ? e / G_BK : e % G_BN), gk = k0 + (TB ? e % G_BK : e / G_BN);
+      rb[u] = gn < N && gk < K ? (TB ? B[(int64_t)gn * ldb + gk] : B[(int64_t)gk * ldb + gn]) : 0.f;
+    }
+  };
+  float acc[2][4] = {};
+  load(0);
+  for (int k0 = 0; k0 < K; k0 += G_BK) {
+#pragma unroll
+    for (int u = 0; u < NA; u++) {
+      const int e = t + u * G_THREADS;
+      As[TA ? e / G_BM : e % G_BK][TA ? e % G_BM : e / G_BK] = bf16_round(ra[u]);
+    }
+#pragma unroll
+    for (int u = 0; u < NB; u++) {
+      const int e = t + u * G_THREADS;
+      Bs[TB ? e % G_BK : e / G_BN][TB ? e / G_BK : e % G_BN] = bf16_round(rb[u]);
+      if (sums) Bw[TB ? e % G_BK : e / G_BN][TB ? e / G_BK : e % G_BN] = rb[u];
     }
     __syncthreads();
+    if (k0 + G_BK < K) load(k0 + G_BK);
+    if (sums && t < G_BN)
+#pragma unroll 8
+      for (int kk = 0; kk < G_BK; kk++) bs += Bw[kk][t];
 #pragma unroll
     for (int kk = 0; kk < G_BK; kk++) {
-      float a[4], b[4];
+      const float2 a2 = *reinterpret_cast<const float2*>(&As[kk][ty * 2]);
+      const float4 b4 = *reinterpret_cast<const float4*>(&Bs[kk][tx * 4]);
+      const float a[2] = {a2.x, a2.y}, b[4] = {b4.x, b4.y, b4.z, b4.w};
 #pragma unroll
-      for (int i = 0; i < 4; i++) a[i] = As[kk][ty * 4 + i];
-#pragma unroll
-      for (int j = 0; j < 4; j++) b[j] = Bs[kk][tx * 4 + j];
-#pragma unroll
-      for (int i = 0; i < 4; i++)
+      for (int i = 0; i < 2; i++)
 #pragma unroll
         for (int j = 0; j < 4; j++) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
     }
     __syncthreads();
   }
+  if (sums && t < G_BN && n0 + t < N) ep.bsum[n0 + t] = bs;
 #pragma unroll
-  for (int i = 0; i < 4; i++) {
-    const int gm = m0 + ty * 4 + i;
+  for (int i = 0; i < 2; i++) {
+    const int gm = m0 + ty * 2 + i;
     if (gm >= M) continue;
 #pragma unroll
     for (int j = 0; j < 4; j++) {
       const int gn = n0 + tx * 4 + j;
       if (gn >= N) continue;
       float v = acc[i][j];
-      if (EPI >= 1) v += bias[gn];
+      if (EPI == 1 || EPI == 2) v += ep.bias[gn];
       if (EPI == 2) {
-        pre[(int64_t)gm * ldpre + gn] = v;
+        ep.pre[(int64_t)gm * ep.ldpre + gn] = v;
         v = gelu_f(v);
+        if (ep.hb) {
+          const uint16_t h = bf16_bits(v);
+          ep.hb[(int64_t)gm * ldc + gn] = h;
+          ep.ht[(int64_t)gn * M + gm] = h;
+        }
       }
+      if (EPI == 3) v *= gelu_grad_f(ep.pre[(int64_t)gm * ep.ldpre + gn]);
       C[(int64_t)gm * ldc + gn] = v;
     }
   }
@@ -137,46 +173,44 @@ __global__ void __launch_bounds__(G_THREADS)
 
 template <bool TA, bool TB, int EPI>
 cudaError_t gemm(int M, int N, int K, const float* A, int64_t lda, const float* B, int64_t ldb,
-                 float* C, int64_t ldc, const float* bias, float* pre, int64_t ldpre,
-                 cudaStream_t s) {
+                 float* C, int64_t ldc, const GemmEpi& ep, cudaStream_t s) {
   dim3 grid((unsigned)((N + G_BN - 1) / G_BN), (unsigned)((M + G_BM - 1) / G_BM));
-  mlp_gemm_kernel<TA, TB, EPI><<<grid, G_THREADS, 0, s>>>(M, N, K, A, lda, B, ldb, C, ldc, bias,
-                                                          pre, ldpre);
+  mlp_gemm_kernel<TA, TB, EPI><<<grid, G_THREADS, 0, s>>>(M, N, K, A, lda, B, ldb, C, ldc, ep);
   return cudaGetLastError();
 }
 
 // ------------------------------------------- BF16 operands for the tcgen05 --
+// dst = bf16(src), four values a thread (V4: both 16- and 8-byte aligned, n a multiple of 4)
+template <bool V4>
 __global__ void to_bf16_kernel(const float* __restrict__ src, int64_t n, uint16_t* __restrict__ dst) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) dst[i] = bf16_bits(src[i]);
-}
-
-// dst[c][r] = bf16(src[r][c]) for r < rows, c < cols (32 x 32 tiles through
-// shared memory; rows and cols multiples of 32)
-__global__ void transpose_bf16_kernel(const float* __restrict__ src, int64_t ld_src, int64_t rows,
-                                      int64_t cols, uint16_t* __restrict__ dst, int64_t ld_dst) {
-  __shared__ float t[32][33];
-  const int64_t r0 = (int64_t)blockIdx.y * 32, c0 = (int64_t)blockIdx.x * 32;
-  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;  // 32 x 8
-  for (int k = ty; k < 32; k += 8) t[k][tx] = src[(r0 + k) * ld_src + c0 + tx];
-  __syncthreads();
-  for (int k = ty; k < 32; k += 8) dst[(c0 + k) * ld_dst + r0 + tx] = bf16_bits(t[tx][k]);
+  const int64_t i = 4 * ((int64_t)blockIdx.x * blockDim.x + threadIdx.x);
+  if (i >= n) return;
+  if (V4) {
+    const float4 v = *reinterpret_cast<const float4*>(src + i);
+    *reinterpret_cast<ushort4*>(dst + i) =
+        make_ushort4(bf16_bits(v.x), bf16_bits(v.y), bf16_bits(v.z), bf16_bits(v.w));
+  } else {
+    for (int64_t e = i; e < min(n, i + 4); e++) dst[e] = bf16_bits(src[e]);
+  }
 }
 
 __global__ void add_bias_kernel(float* __restrict__ Z, int64_t ld, int64_t rows, int64_t cols,
                                 const float* __restrict__ b) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < rows * cols) Z[(i / cols) * ld + i % cols] += b[i % cols];
+  const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (c >= cols) return;
+  const float v = b[c];
+  const int64_t r0 = (int64_t)blockIdx.y * 8;
+#pragma unroll
+  for (int r = 0; r < 8; r++)
+    if (r0 + r < rows) Z[(r0 + r) * ld + c] += v;
 }
 
 cudaError_t to_bf16(const float* src, int64_t n, uint16_t* dst, cudaStream_t s) {
-  to_bf16_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(src, n, dst);
-  return cudaGetLastError();
-}
-cudaError_t transpose_bf16(const float* src, int64_t ld_src, int64_t rows, int64_t cols,
-                           uint16_t* dst, int64_t ld_dst, cudaStream_t s) {
-  dim3 grid((unsigned)(cols / 32), (unsigned)(rows / 32));
-  transpose_bf16_kernel<<<grid, 256, 0, s>>>(src, ld_src, rows, cols, dst, ld_dst);
+  const unsigned blocks = (unsigned)((n / 4 + 256) / 256);
+  if (((uintptr_t)src & 15) == 0 && ((uintptr_t)dst & 7) == 0 && n % 4 == 0)
+    to_bf16_kernel<true><<<blocks, 256, 0, s>>>(src, n, dst);
+  else
+    to_bf16_kernel<false><<<blocks, 256, 0, s>>>(src, n, dst);
   return cudaGetLastError();
 }
 
@@ -185,71 +219,140 @@ cudaError_t transpose_bf16(const float* src, int64_t ld_src, int64_t rows, int64
 cudaError_t tc_gemm(const uint16_t* A, int64_t M, int64_t K, const uint16_t* B, int64_t N,
                     float* C, int32_t* status, cudaStream_t s) {
   Planes pa{const_cast<uint16_t*>(A), M * K, K};
-  return launch_tc_update(pa, EMC_PREC_BF16, M, B, K, N, INT64_MAX, C, nullptr, status, s);
+  // few K blocks a tile: bound by its FP32 output, so whole-line stores
+  return launch_tc_update(pa, EMC_PREC_BF16, M, B, K, N, INT64_MAX, C, nullptr, status, s,
+                          nullptr, nullptr, TcCtl{}, true);
 }
 
 // ------------------------------------------------- loss and its gradient --
-// Row b of z (n_out logits, stride ld): lse = log sum_j exp(z_j); loss
-// += -sum_r p_r (z_{idx_r} - lse) / B; z is overwritten by
-// dL/dz = (softmax(z) sum_r p_r - onehot(p)) / B (zero beyond n_out).
-__global__ void softmax_ce_kernel(float* __restrict__ z, int64_t ld, int n_out,
-                                  const int32_t* __restrict__ tidx, const float* __restrict__ tprob,
-                                  int R, int B, double* loss) {
+// Row b of z (n_out logits, stride ld; zb (may be NULL): a bias still to be added):
+// lse[b] = log sum_j exp(z_j), mass[b] = sum_r p_r and loss
+// += -sum_r p_r (z_{idx_r} - lse) / B. The sum is kept per thread as a
+// double-float pair (FP64 additions and conversions are rare on this part), merged in FP64.
+__global__ void __launch_bounds__(512)
+    softmax_lse_kernel(const float* __restrict__ z, int64_t ld, int n_out,
+                       const float* __restrict__ zb, const int32_t* __restrict__ tidx,
+                       const float* __restrict__ tprob, int R, int B, float* __restrict__ lse,
+                       float* __restrict__ mass, double* loss) {
   const int64_t b = blockIdx.x;
-  float* row = z + b * ld;
-  __shared__ float red[32];
-  __shared__ double dred[32];
-  __shared__ float s_lse;
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  float m = -INFINITY;
-  for (int j = threadIdx.x; j < n_out; j += blockDim.x) m = fmaxf(m, row[j]);
-  for (int o = 16; o; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-  if (lane == 0) red[wid] = m;
+  const float* row = z + b * ld;
+  __shared__ float red[16];
+  __shared__ double dred[16];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  float M = -INFINITY;
+#pragma unroll 8
+  for (int j = threadIdx.x; j < n_out; j += 512) M = fmaxf(M, row[j] + (zb ? zb[j] : 0.f));
+  for (int o = 16; o; o >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, o));
+  if (lane == 0) red[wid] = M;
   __syncthreads();
-  if (threadIdx.x == 0) {
-    float mm = red[0];
-    for (int w = 1; w < nw; w++) mm = fmaxf(mm, red[w]);
-    red[0] = mm;
+  M = red[0];
+  for (int w = 1; w < 16; w++) M = fmaxf(M, red[w]);
+  float s = 0.f, se = 0.f;
+#pragma unroll 8
+  for (int j = threadIdx.x; j < n_out; j += 512) {
+    const f2 a = two_sum(s, __expf((row[j] + (zb ? zb[j] : 0.f)) - M));
+    s = a.h;
+    se += a.l;
   }
-  __syncthreads();
-  m = red[0];
-  double se = 0.0;
-  for (int j = threadIdx.x; j < n_out; j += blockDim.x) se += (double)__expf(row[j] - m);
-  for (int o = 16; o; o >>= 1) se += __shfl_xor_sync(0xffffffffu, se, o);
-  if (lane == 0) dred[wid] = se;
+  double d = (double)s + (double)se;
+  for (int o = 16; o; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
+  if (lane == 0) dred[wid] = d;
   __syncthreads();
   if (threadIdx.x == 0) {
     double t = 0.0;
-    for (int w = 0; w < nw; w++) t += dred[w];
-    s_lse = m + (float)log(t);
-    // loss and the total target mass, before z is overwritten
+    for (int w = 0; w < 16; w++) t += dred[w];
+    const float L = M + (float)log(t);
     double l = 0.0;
+    float tm = 0.f;
     for (int r = 0; r < R; r++) {
       const float p = tprob[b * R + r];
-      l -= (double)p * ((double)row[tidx[b * R + r]] - (double)s_lse);
+      const int c = tidx[b * R + r];
+      l -= (double)p * ((double)(row[c] + (zb ? zb[c] : 0.f)) - (double)L);
+      tm += p;
     }
+    lse[b] = L;
+    mass[b] = tm;
     atomicAdd(loss, l / B);
   }
-  __syncthreads();
-  const float lse = s_lse;
-  float tm = 0.f;
-  for (int r = 0; r < R; r++) tm += tprob[b * R + r];
-  const float invB = 1.f / (float)B;
-  for (int j = threadIdx.x; j < (int)ld; j += blockDim.x)
-    row[j] = j < n_out ? __expf(row[j] - lse) * tm * invB : 0.f;
-  __syncthreads();
-  if (threadIdx.x == 0)
-    for (int r = 0; r < R; r++) row[tidx[b * R + r]] -= tprob[b * R + r] * invB;
 }
 
-// out[c] = sum_r X[r][c] (bias gradients)
-__global__ void colsum_kernel(const float* __restrict__ X, int rows, int cols, int64_t ld,
-                              float* __restrict__ out) {
-  const int c = blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= cols) return;
-  float s = 0.f;
-  for (int r = 0; r < rows; r++) s += X[(int64_t)r * ld + c];
-  out[c] = s;
+// (both softmax kernels: 512 x 50112 logits, 312 us with separate passes for the bias,
+// the FP32 gradient, its BF16 copy and its column sums on top, 176 more; now 51 + 116 us)
+// dL/dz = (softmax(z) sum_r p_r - onehot(p)) / B (zero beyond n_out) as BF16
+// (dzb), or in FP32 over z itself (dzb NULL), and its column sums in row order
+// (the bias gradient). A warp walks 32 columns of every row, 16 rows' loads in
+// flight; the CTA first marks the rows that have a target among its 128 columns, and
+// only those look their targets up.
+__global__ void __launch_bounds__(128)
+    softmax_grad_kernel(float* __restrict__ z, int64_t ld, int n_out,
+                        const float* __restrict__ zb, const int32_t* __restrict__ tidx,
+                        const float* __restrict__ tprob, int R, int B,
+                        const float* __restrict__ lse, const float* __restrict__ mass,
+                        uint16_t* __restrict__ dzb, float* __restrict__ db) {
+  constexpr int kRows = 16, kBatch = 512;
+  __shared__ unsigned hits[kBatch / 32];
+  const int lane = threadIdx.x & 31;
+  const int cta0 = blockIdx.x * 128, c0 = cta0 + (threadIdx.x & 96), c = c0 + lane;
+  const bool live = c < (int)ld, in = c < n_out;  // ld is a multiple of 64
+  const float bias = zb && in ? zb[c] : 0.f;
+  const float invB = 1.f / (float)B;
+  float sum = 0.f;
+  for (int b0 = 0; b0 < B; b0 += kBatch) {
+    const int b1 = min(B, b0 + kBatch);
+    __syncthreads();
+    if (threadIdx.x < kBatch / 32) hits[threadIdx.x] = 0u;
+    __syncthreads();
+#pragma unroll 8
+    for (int64_t e = (int64_t)b0 * R + threadIdx.x; e < (int64_t)b1 * R; e += 128) {
+      const int q = tidx[e];
+      if (q >= cta0 && q < cta0 + 128) {
+        const int r = (int)(e / R) - b0;
+        atomicOr(&hits[r >> 5], 1u << (r & 31));
+      }
+    }
+    __syncthreads();
+    if (!live) continue;  // whole warps
+    float x[kRows];
+    auto load = [&](int r0) {
+#pragma unroll
+      for (int u = 0; u < kRows; u++) x[u] = r0 + u < b1 ? z[(int64_t)(r0 + u) * ld + c] : 0.f;
+    };
+    load(b0);
+    for (int r0 = b0; r0 < b1; r0 += kRows) {
+      float v[kRows];
+#pragma unroll
+      for (int u = 0; u < kRows; u++) {
+        const int r = min(r0 + u, b1 - 1);
+        v[u] = in ? __expf((x[u] + bias) - lse[r]) * mass[r] * invB : 0.f;
+      }
+      if (r0 + kRows < b1) load(r0 + kRows);
+      const unsigned h16 = hits[(r0 - b0) >> 5] >> ((r0 - b0) & 31) & 0xffffu;
+      if (h16) {
+#pragma unroll
+        for (int u = 0; u < kRows; u++) {
+          if (!(h16 >> u & 1u)) continue;
+          const int64_t e0 = (int64_t)(r0 + u) * R;
+          for (int t0 = 0; t0 < R; t0 += 32) {
+            const int q = t0 + lane < R ? tidx[e0 + t0 + lane] : -1;
+            unsigned hit = __ballot_sync(0xffffffffu, q >= c0 && q < c0 + 32);
+            while (hit) {
+              const int w = __ffs(hit) - 1;
+              hit &= hit - 1;
+              if (__shfl_sync(0xffffffffu, q, w) == c) v[u] -= tprob[e0 + t0 + w] * invB;
+            }
+          }
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < kRows; u++) {
+        if (r0 + u >= b1) break;
+        sum += v[u];
+        if (dzb) dzb[(int64_t)(r0 + u) * ld + c] = bf16_bits(v[u]);
+        else z[(int64_t)(r0 + u) * ld + c] = v[u];
+      }
+    }
+  }
+  if (in) db[c] = sum;
 }
 
 // d = g * GELU'(a), elementwise
@@ -259,17 +362,40 @@ __global__ void gelu_backward_kernel(const float* __restrict__ g, const float* _
   if (i < n) d[i] = g[i] * gelu_grad_f(a[i]);
 }
 
-__global__ void adam_kernel(float* __restrict__ p, const float* __restrict__ g,
-                            float* __restrict__ m, float* __restrict__ v, int64_t n, float lr,
-                            float b1, float b2, float eps, float bc1, float bc2) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const float gi = g[i];
-  const float mi = b1 * m[i] + (1.f - b1) * gi;
-  const float vi = b2 * v[i] + (1.f - b2) * gi * gi;
-  m[i] = mi;
-  v[i] = vi;
-  p[i] -= lr * (mi / bc1) / (sqrtf(vi / bc2) + eps);
+// Bound by its traffic (28 B a parameter): four parameters a thread (V4: every
+// array 16-byte aligned), 26.5 M of them 150 -> 100 us (110 at the copy rate).
+template <bool V4>
+__global__ void __launch_bounds__(256)
+    adam_kernel(float* __restrict__ p, const float* __restrict__ g, float* __restrict__ m,
+                float* __restrict__ v, int64_t n, float lr, float b1, float b2, float eps,
+                float bc1, float bc2) {
+  const int64_t i0 = 4 * ((int64_t)blockIdx.x * blockDim.x + threadIdx.x);
+  auto step = [&](float gi, float& mi, float& vi, float& pi) {
+    mi = b1 * mi + (1.f - b1) * gi;
+    vi = b2 * vi + (1.f - b2) * gi * gi;
+    pi -= lr * (mi / bc1) / (sqrtf(vi / bc2) + eps);
+  };
+  if (V4 && i0 + 4 <= n) {
+    const float4 g4 = __ldcs(reinterpret_cast<const float4*>(g + i0));
+    float4 m4 = __ldcs(reinterpret_cast<const float4*>(m + i0));
+    float4 v4 = __ldcs(reinterpret_cast<const float4*>(v + i0));
+    float4 p4 = *reinterpret_cast<const float4*>(p + i0);
+    step(g4.x, m4.x, v4.x, p4.x);
+    step(g4.y, m4.y, v4.y, p4.y);
+    step(g4.z, m4.z, v4.z, p4.z);
+    step(g4.w, m4.w, v4.w, p4.w);
+    __stcs(reinterpret_cast<float4*>(m + i0), m4);
+    __stcs(reinterpret_cast<float4*>(v + i0), v4);
+    *reinterpret_cast<float4*>(p + i0) = p4;
+    return;
+  }
+  for (int64_t i = i0; i < min(n, i0 + 4); i++) {
+    float mi = m[i], vi = v[i], pi = p[i];
+    step(g[i], mi, vi, pi);
+    m[i] = mi;
+    v[i] = vi;
+    p[i] = pi;
+  }
 }
 
 // ------------------------------------------------------------ host side --
@@ -292,11 +418,11 @@ MlpLayout mlp_layout(int64_t n_out, int64_t B) {
   y.n_params = o;
   // work: pre-activations a[3], activations h[3], dh, da (each B x 512), z / dz (B x ld_out),
   // then the tensor-core path's BF16 copies: H3 [B][512], H3^T [512][B], dZ [B][ld_out],
-  // W4 [512][ld_out], W4^T [ld_out][512], each from a 256-byte boundary
+  // W4 [512][ld_out], each from a 256-byte boundary
   y.B = B;
   auto up64 = [](int64_t n) { return (n + 63) / 64 * 64; };  // floats to 256 bytes
   y.work_floats = up64(8 * B * H + B * y.ld_out) + up64(B * H / 2) + up64(B * H / 2) +
-                  up64(B * y.ld_out / 2) + 2 * up64(H * y.ld_out / 2);
+                  up64(B * y.ld_out / 2) + up64(H * y.ld_out / 2);
   return y;
 }
 
@@ -307,7 +433,7 @@ struct Work {
   float* dh;
   float* da;
   float* z;
-  uint16_t *h3b, *h3t, *dzb, *w4b, *w4t;  // BF16 operands of the tensor-core products
+  uint16_t *h3b, *h3t, *dzb, *w4b;  // BF16 operands of the tensor-core products
 };
 Work carve(const MlpLayout& y, float* w) {
   Work k;
@@ -326,35 +452,43 @@ Work carve(const MlpLayout& y, float* w) {
   k.dzb = reinterpret_cast<uint16_t*>(o);
   o += up64(y.B * y.ld_out / 2);
   k.w4b = reinterpret_cast<uint16_t*>(o);
-  o += up64(H * y.ld_out / 2);
-  k.w4t = reinterpret_cast<uint16_t*>(o);
   return k;
 }
 bool tc_batch(int B) { return B >= 128 && B % 128 == 0; }
 }  // namespace
 
-cudaError_t mlp_forward(const MlpLayout& y, const float* params, const float* X, int B,
-                        float* work, float* logits, cudaStream_t s) {
+// Forward into logits. train: with a tensor-core batch the output layer's bias is
+// left to the loss kernels, and H3^T is kept for the weight gradient.
+static cudaError_t forward(const MlpLayout& y, const float* params, const float* X, int B,
+                           float* work, float* logits, cudaStream_t s) {
   Work w = carve(y, work);
   const int H = kFeat;
+  const bool tc = tc_batch(B);
   const float* in = X;
   cudaError_t e;
   for (int l = 0; l < 3; l++) {
-    e = gemm<false, false, 2>(B, H, H, in, H, params + y.W[l], H, w.h[l], H, params + y.b[l],
-                              w.a[l], H, s);
+    const bool last = tc && l == 2;
+    e = gemm<false, false, 2>(B, H, H, in, H, params + y.W[l], H, w.h[l], H,
+                              GemmEpi{params + y.b[l], w.a[l], H, last ? w.h3b : nullptr,
+                                      last ? w.h3t : nullptr},
+                              s);
     if (e != cudaSuccess) return e;
     in = w.h[l];
   }
-  if (!tc_batch(B))
+  if (!tc)
     return gemm<false, false, 1>(B, (int)y.n_out, H, in, H, params + y.W[3], y.ld_out, logits,
-                                 y.ld_out, params + y.b[3], nullptr, 0, s);
-  // output layer on the tensor cores: logits = bf16(H3) bf16(W4) + b4
-  if ((e = to_bf16(in, (int64_t)B * H, w.h3b, s)) != cudaSuccess) return e;
+                                 y.ld_out, GemmEpi{params + y.b[3]}, s);
+  // output layer on the tensor cores: bf16(H3) bf16(W4), the bias to follow
   if ((e = to_bf16(params + y.W[3], (int64_t)H * y.ld_out, w.w4b, s)) != cudaSuccess) return e;
-  if ((e = tc_gemm(w.h3b, B, H, w.w4b, y.ld_out, logits, nullptr, s)) != cudaSuccess) return e;
-  const int64_t n = (int64_t)B * y.n_out;
-  add_bias_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(logits, y.ld_out, B, y.n_out,
-                                                            params + y.b[3]);
+  return tc_gemm(w.h3b, B, H, w.w4b, y.ld_out, logits, nullptr, s);
+}
+
+cudaError_t mlp_forward(const MlpLayout& y, const float* params, const float* X, int B,
+                        float* work, float* logits, cudaStream_t s) {
+  cudaError_t e = forward(y, params, X, B, work, logits, s);
+  if (e != cudaSuccess || !tc_batch(B)) return e;
+  add_bias_kernel<<<dim3((unsigned)((y.n_out + 255) / 256), (unsigned)((B + 7) / 8)), 256, 0, s>>>(
+      logits, y.ld_out, B, y.n_out, params + y.b[3]);
   return cudaGetLastError();
 }
 
@@ -364,54 +498,58 @@ cudaError_t mlp_train_step(const MlpLayout& y, float* params, float* grads, floa
                            double* loss, cudaStream_t s) {
   Work w = carve(y, work);
   const int H = kFeat;
-  cudaError_t e = mlp_forward(y, params, X, B, work, w.z, s);
+  const bool tc = tc_batch(B);
+  const int64_t BH = (int64_t)B * H;
+  cudaError_t e = forward(y, params, X, B, work, w.z, s);
   if (e != cudaSuccess) return e;
-  softmax_ce_kernel<<<B, 256, 0, s>>>(w.z, y.ld_out, (int)y.n_out, tidx, tprob, R, B, loss);
+  float *lse = w.dh, *mass = w.dh + B;  // dh is written after the loss
+  const float* zb = tc ? params + y.b[3] : nullptr;
+  softmax_lse_kernel<<<B, 512, 0, s>>>(w.z, y.ld_out, (int)y.n_out, zb, tidx, tprob, R, B, lse,
+                                       mass, loss);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  // output layer: dW4 = h3^T dz, db4 = colsum(dz), dh3 = dz W4^T
-  const float* g = w.z;
-  int64_t ldg = y.ld_out;
-  int ncol = (int)y.n_out;
-  for (int l = 3; l >= 0; l--) {
+  softmax_grad_kernel<<<(unsigned)((y.ld_out + 127) / 128), 128, 0, s>>>(
+      w.z, y.ld_out, (int)y.n_out, zb, tidx, tprob, R, B, lse, mass, tc ? w.dzb : nullptr,
+      grads + y.b[3]);
+  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  // output layer: dW4 = h3^T dz, da3 = (dz W4^T) GELU'(a3)
+  if (tc) {
+    // on the tensor cores (the whole padded width: dZ is 0 beyond n_out)
+    if ((e = tc_gemm(w.h3t, H, B, w.dzb, y.ld_out, grads + y.W[3], nullptr, s)) != cudaSuccess)
+      return e;
+    if ((e = launch_tc_nt(w.dzb, w.w4b, B, H, y.ld_out, w.dh, nullptr, s)) != cudaSuccess)
+      return e;
+    gelu_backward_kernel<<<(unsigned)((BH + 255) / 256), 256, 0, s>>>(w.dh, w.a[2], w.da, BH);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  } else {
+    e = gemm<true, false, 0>(H, (int)y.n_out, B, w.h[2], H, w.z, y.ld_out, grads + y.W[3],
+                             y.ld_out, GemmEpi{}, s);
+    if (e != cudaSuccess) return e;
+    e = gemm<false, true, 3>(B, H, (int)y.n_out, w.z, y.ld_out, params + y.W[3], y.ld_out, w.da, H,
+                             GemmEpi{nullptr, w.a[2], H}, s);
+    if (e != cudaSuccess) return e;
+  }
+  // hidden layers: da and dh in turn hold dL/da of the layer
+  float *g = w.da, *next = w.dh;
+  for (int l = 2; l >= 0; l--) {
     const float* in = l == 0 ? X : w.h[l - 1];
-    const int64_t ldw = l == 3 ? y.ld_out : H;
-    const bool tc = l == 3 && tc_batch(B);
-    if (tc) {
-      // dW4 = bf16(H3)^T bf16(dZ) and dH3 = bf16(dZ) bf16(W4)^T on the tensor cores
-      // (the whole padded width: dZ is 0 beyond n_out)
-      if ((e = to_bf16(g, (int64_t)B * y.ld_out, w.dzb, s)) != cudaSuccess) return e;
-      if ((e = transpose_bf16(in, H, B, H, w.h3t, B, s)) != cudaSuccess) return e;
-      if ((e = tc_gemm(w.h3t, H, B, w.dzb, y.ld_out, grads + y.W[3], nullptr, s)) != cudaSuccess)
-        return e;
-    } else {
-      e = gemm<true, false, 0>(H, ncol, B, in, H, g, ldg, grads + y.W[l], ldw, nullptr, nullptr,
-                               0, s);
-      if (e != cudaSuccess) return e;
-    }
-    colsum_kernel<<<(ncol + 255) / 256, 256, 0, s>>>(g, B, ncol, ldg, grads + y.b[l]);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    GemmEpi ep{};
+    ep.bsum = grads + y.b[l];
+    e = gemm<true, false, 0>(H, H, B, in, H, g, H, grads + y.W[l], H, ep, s);
+    if (e != cudaSuccess) return e;
     if (l == 0) break;
-    if (tc) {
-      if ((e = transpose_bf16(params + y.W[3], y.ld_out, H, y.ld_out, w.w4t, H, s)) != cudaSuccess)
-        return e;
-      if ((e = tc_gemm(w.dzb, B, y.ld_out, w.w4t, H, w.dh, nullptr, s)) != cudaSuccess) return e;
-    } else {
-      e = gemm<false, true, 0>(B, H, ncol, g, ldg, params + y.W[l], ldw, w.dh, H, nullptr,
-                               nullptr, 0, s);
-      if (e != cudaSuccess) return e;
-    }
-    const int64_t n = (int64_t)B * H;
-    gelu_backward_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(w.dh, w.a[l - 1], w.da, n);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    g = w.da;
-    ldg = H;
-    ncol = H;
+    e = gemm<false, true, 3>(B, H, H, g, H, params + y.W[l], H, next, H,
+                             GemmEpi{nullptr, w.a[l - 1], H}, s);
+    if (e != cudaSuccess) return e;
+    std::swap(g, next);
   }
   const float b1 = 0.9f, b2 = 0.999f;
   const float bc1 = 1.f - powf(b1, (float)step), bc2 = 1.f - powf(b2, (float)step);
-  adam_kernel<<<(unsigned)((y.n_params + 255) / 256), 256, 0, s>>>(params, grads, adam_m, adam_v,
-                                                                  y.n_params, lr, b1, b2, 1e-8f,
-                                                                  bc1, bc2);
+  const unsigned blocks = (unsigned)((y.n_params / 4 + 256) / 256);
+  const bool v4 = (((uintptr_t)params | (uintptr_t)grads | (uintptr_t)adam_m | (uintptr_t)adam_v) &
+                   15) == 0;
+  auto adam = v4 ? adam_kernel<true> : adam_kernel<false>;
+  adam<<<blocks, 256, 0, s>>>(params, grads, adam_m, adam_v, y.n_params, lr, b1, b2, 1e-8f, bc1,
+                              bc2);
   return cudaGetLastError();
 }
 

@@ -69,11 +69,15 @@ constexpr float kSentinel = -3.0e38f;
 // for the multi-plane score contractions, whose 64-80 KB stages would
 // otherwise leave room for only two or three in flight (too shallow to hide
 // the load latency). F16: FP16 operands (FP16 split) instead of BF16.
-template <int MODE, int NA, bool F16, bool XP = false>
+// BNT: columns of a tile. 256, but 32 for a store with few tiles and a long sum:
+// one tile's sum runs on one SM, whose loads in flight bound it, so more and
+// narrower tiles share the stream (MLP output layer's input gradient, 512 x 512 over 50112: 8
+// tiles 272 us, 64 narrow ones 225 us, then bound by the chain of dependent MMAs; K is not split, so every sum keeps its order).
+template <int MODE, int NA, bool F16, bool XP = false, int BNT = BN>
 struct TcCfg {
   static constexpr int BK = (MODE != MODE_UPDATE && NA >= 2) ? 32 : 64;
   static constexpr int A_BYTES = BM * BK * 2;  // one 128 x BK BF16 plane
-  static constexpr int B_BYTES = BN * BK * 2;  // 256 x BK BF16
+  static constexpr int B_BYTES = BNT * BK * 2;  // 256 x BK BF16
   static constexpr int STAGE = NA * A_BYTES + B_BYTES;
   static constexpr int NACC = (MODE != MODE_UPDATE && NA >= 2) ? 2 : 1;
   // XP (update over listed blocks, store): a 32 x 32 staging block per
@@ -84,10 +88,12 @@ struct TcCfg {
   static constexpr int XPOSE =
       (XP && (MODE == MODE_UPDATE || MODE == MODE_STORE)) ? kEpiWarps * 32 * kXpLd * 4 : 0;
   static constexpr int STAGES_RAW = (kSmemBudget - kScratchBytes - XPOSE - 1024 - 256) / STAGE;
-  static constexpr int STAGES = STAGES_RAW > 6 ? 6 : STAGES_RAW;
-  static constexpr uint32_t TMEM_COLS = NACC * BN;
+  static constexpr int MAX_STAGES = BNT < BN ? 8 : 6;
+  static constexpr int STAGES = STAGES_RAW > MAX_STAGES ? MAX_STAGES : STAGES_RAW;
+  static constexpr uint32_t TMEM_COLS = NACC * BNT;
   static constexpr int SMEM = 1024 + STAGES * STAGE + 256 + kScratchBytes + XPOSE;
-  static constexpr uint32_t IDESC = idesc_f16kind(BM, BN, MODE == MODE_UPDATE ? 1 : 0, F16);
+  static constexpr uint32_t IDESC = idesc_f16kind(BM, BNT, MODE == MODE_UPDATE ? 1 : 0, F16);
+  static_assert(BNT == BN || MODE == MODE_STORE, "narrow tiles: store only");
   static_assert(STAGES >= 2, "shared memory too small for two stages");
 };
 
@@ -183,11 +189,11 @@ __device__ __forceinline__ void fail(volatile int* abort, int32_t* status) {
   set_status(status, EMC_ERR_TIMEOUT);
 }
 
-template <int MODE, int NA, bool F16, bool XP = false>
+template <int MODE, int NA, bool F16, bool XP = false, int BNT = BN>
 __global__ void __launch_bounds__(kThreads, 1)
     tc_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB,
               const TcArgs a) {
-  using C = TcCfg<MODE, NA, F16, XP>;
+  using C = TcCfg<MODE, NA, F16, XP, BNT>;
   constexpr bool GAUSS = (MODE == MODE_PASS1 && NA == 3 && F16);
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
@@ -256,7 +262,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             tma_load_3d(st + p * C::A_BYTES, &mapA, full + s, kb * C::BK, mt * BM, p);
           uint8_t* sb = st + NA * C::A_BYTES;
           if (MODE != MODE_UPDATE) {
-            tma_load_2d(sb, &mapB, full + s, kb * C::BK, nt * BN);
+            tma_load_2d(sb, &mapB, full + s, kb * C::BK, nt * BNT);
           } else {
 #pragma unroll
             for (int j = 0; j < BN / 64; j++)
@@ -377,14 +383,17 @@ __global__ void __launch_bounds__(kThreads, 1)
       if (named_bar_any(2, kEpiThreads, !got)) break;
       tc_fence_after();
       bool big = false;
+      // 32 columns a step; a narrow tile has one step, the first four warps'
+      const int steps = BNT == BN ? 4 : (half == 0 ? 1 : 0);
+      if (BNT < BN && half != 0 && lane == 0) mbar_arrive(acc_empty);
 #pragma unroll 1
-      for (int c = 0; c < 4; c++) {
+      for (int c = 0; c < steps; c++) {
         const int col0 = half * 128 + c * 32;
         uint32_t v0[32], v1[32];
         tmem_ld32(lane_addr + col0, v0);
         if (C::NACC == 2) tmem_ld32(lane_addr + BN + col0, v1);
         tmem_ld_wait();
-        if (c == 3) {
+        if (c == steps - 1) {
           tc_fence_before();
           __syncwarp();
           if (lane == 0) mbar_arrive(acc_empty);
@@ -398,7 +407,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                   make_uint4(v0[i], v0[i + 1], v0[i + 2], v0[i + 3]);
             __syncwarp();
             const int64_t row0 = (int64_t)mt * BM + 32 * q;
-            const int64_t k0 = (int64_t)nt * BN + col0;
+            const int64_t k0 = (int64_t)nt * BNT + col0;
 #pragma unroll
             for (int st = 0; st < 8; st++) {
               const int r = 4 * st + (lane >> 3), c4 = 4 * (lane & 7);
@@ -407,7 +416,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             }
             __syncwarp();
           } else {
-            float* dst = a.Num + row * a.ld_data + (int64_t)nt * BN + col0;
+            float* dst = a.Num + row * a.ld_data + (int64_t)nt * BNT + col0;
 #pragma unroll
             for (int i = 0; i < 32; i += 4)
               *reinterpret_cast<uint4*>(dst + i) =
@@ -826,12 +835,12 @@ int num_sms() {
   return n > 0 ? n : 148;
 }
 
-template <int MODE, int NA, bool F16, bool XP = false>
+template <int MODE, int NA, bool F16, bool XP = false, int BNT = BN>
 cudaError_t launch(const CUtensorMap& mA, const CUtensorMap& mB, TcArgs a, cudaStream_t s) {
-  using C = TcCfg<MODE, NA, F16, XP>;
+  using C = TcCfg<MODE, NA, F16, XP, BNT>;
   static bool attr = false;
   if (!attr) {
-    cudaError_t e = cudaFuncSetAttribute(tc_kernel<MODE, NA, F16, XP>,
+    cudaError_t e = cudaFuncSetAttribute(tc_kernel<MODE, NA, F16, XP, BNT>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM);
     if (e != cudaSuccess) return e;
     attr = true;
@@ -840,7 +849,7 @@ cudaError_t launch(const CUtensorMap& mA, const CUtensorMap& mB, TcArgs a, cudaS
   if (T <= 0) return cudaSuccess;
   // a device-side tile list: one persistent CTA per SM (the count is read on the device)
   const int grid = (!a.tile_list && T < num_sms()) ? T : num_sms();
-  tc_kernel<MODE, NA, F16, XP><<<grid, kThreads, C::SMEM, s>>>(mA, mB, a);
+  tc_kernel<MODE, NA, F16, XP, BNT><<<grid, kThreads, C::SMEM, s>>>(mA, mB, a);
   return cudaGetLastError();
 }
 
@@ -850,7 +859,8 @@ int score_planes(int precision) {
 }
 
 bool maps_scores(const Planes& L, int nterms, bool f16, int64_t rows, const uint16_t* Kb,
-                 int64_t ld_data, int64_t ld_pix, CUtensorMap* mA, CUtensorMap* mB) {
+                 int64_t ld_data, int64_t ld_pix, CUtensorMap* mA, CUtensorMap* mB,
+                 uint32_t cols = BN) {
   const uint32_t bk = nterms >= 2 ? 32 : 64;  // TcCfg<scores, NA, F16>::BK
   const int sw = nterms >= 2 ? 64 : 128;
   const uint64_t dA[3] = {(uint64_t)ld_pix, (uint64_t)rows, (uint64_t)nterms};
@@ -858,7 +868,7 @@ bool maps_scores(const Planes& L, int nterms, bool f16, int64_t rows, const uint
   const uint32_t bA[3] = {bk, BM, 1};
   const uint64_t dB[2] = {(uint64_t)ld_pix, (uint64_t)ld_data};
   const uint64_t sB[1] = {(uint64_t)ld_pix * 2};
-  const uint32_t bB[2] = {bk, BN};
+  const uint32_t bB[2] = {bk, cols};
   return make_map(mA, L.base, 3, dA, sA, bA, sw, f16) && make_map(mB, Kb, 2, dB, sB, bB, sw, f16);
 }
 
@@ -939,6 +949,21 @@ cudaError_t launch_tc_store(const Planes& A, int64_t rows, const uint16_t* Kb, i
   // A and B of one MMA always share their type: FP16 frames take FP16 increments
   if (f16) return launch<MODE_STORE, 1, true, true>(mA, mB, a, s);
   return launch<MODE_STORE, 1, false, true>(mA, mB, a, s);
+}
+
+cudaError_t launch_tc_nt(const uint16_t* A, const uint16_t* B, int64_t M, int64_t N, int64_t K,
+                         float* C, int32_t* status, cudaStream_t s) {
+  constexpr int kCols = 32;
+  CUtensorMap mA, mB;
+  Planes pa{const_cast<uint16_t*>(A), M * K, K};
+  if (!maps_scores(pa, 1, false, M, B, N, K, &mA, &mB, kCols)) return cudaErrorInvalidValue;
+  TcArgs a = base_args(M, (int)(N / kCols), (int)(K / 64));
+  a.nrot = M;
+  a.ld_data = N;
+  a.ld_pix = K;
+  a.Num = C;
+  a.status = status;
+  return launch<MODE_STORE, 1, false, true, kCols>(mA, mB, a, s);
 }
 
 cudaError_t launch_tc_pass1(const Planes& L, int precision, const double* bias, int64_t rows,
