@@ -21,14 +21,21 @@
 // FP32 pairs (numerator, denominator) before one FP64 reduction per touched
 // voxel:
 //  * pixels with the same floor cell share all eight voxels; __match_any_sync
-//    finds them and the lowest lane sums their terms in lane order;
+//    finds them and the lowest lane sums their terms in lane order (shuffles);
 //  * the remaining lanes have distinct floor cells, so for one corner offset c
 //    their voxels are distinct: corner by corner (a __syncwarp between
 //    corners) each lane adds into its slot without atomics;
-//  * the warp then sweeps the box in slot order: each non-zero slot is reduced
-//    once and cleared. Consecutive lanes hold consecutive slots (neighbouring
-//    z of one (x, y) column), so the sweep's loads are conflict-free and its
-//    reductions touch few sectors per instruction.
+//  * the warp then lists the box's non-zero slots in slot order (about 93 of 249) and
+//    reduces the listed ones, 32 to an instruction, clearing them. Neighbouring
+//    lanes hold neighbouring slots, so the reductions touch few sectors per
+//    instruction, and the FP32 -> FP64 conversions (on the FP64 pipe here, at
+//    their full cost however few lanes take part) fall from 16 to 6 a group.
+// Bound by the load/store pipe's wavefronts (88% of their rate in ncu, of them 40% the
+// ordered steps, whose slots fall on the banks like random keys); issue 65%.
+// 10860 rotations x 4999 frames at 64^3: 426 us when the sweep reduced
+// straight from the box (load/store 78%, FP64 74%, issue 71%), 387 us now. Listing slots as the
+// steps first touch them needs no sweep, but its unordered reductions take as
+// much of the pipe as it saves (411 us).
 // The order of every FP32 addition is fixed, so the result does not depend on
 // scheduling beyond the FP64 order of the L2 reductions. A group whose box
 // exceeds kAggCap slots reduces its corners directly.
@@ -41,10 +48,10 @@ namespace emc {
 
 constexpr int kAggWarps = 4;
 constexpr int kAggCap = 576;       // box slots per warp (float2 each), below 1024
-constexpr int kAggStage = 32 * 8;  // merge staging: 8 corner terms per lane
+constexpr int kAggList = 32 * 8;   // touched slots of a group: at most 8 per pixel
 constexpr int kAggThreads = kAggWarps * 32;
 // 26.6 KB per CTA: eight CTAs (32 warps) per SM, at most 64 registers a thread
-constexpr size_t kAggSmem = sizeof(float2) * kAggWarps * (kAggCap + kAggStage);
+constexpr size_t kAggSmem = kAggWarps * (sizeof(float2) * kAggCap + sizeof(int) * kAggList);
 static_assert(kCompressGroup == 32, "one pixel per lane");
 
 __device__ __forceinline__ bool in_grid(int x, int y, int z, int N) {
@@ -76,6 +83,24 @@ __device__ __forceinline__ void reduce_direct(const int* f, const float* t, floa
 __device__ __forceinline__ int warp_min(int v) { return __reduce_min_sync(0xffffffffu, v); }
 __device__ __forceinline__ int warp_max(int v) { return __reduce_max_sync(0xffffffffu, v); }
 
+// two FP32 operations in one instruction
+__device__ __forceinline__ float2 add2(float2 a, float2 b) {
+  unsigned long long r;
+  asm("add.rn.f32x2 %0, %1, %2;"
+      : "=l"(r)
+      : "l"(*reinterpret_cast<unsigned long long*>(&a)),
+        "l"(*reinterpret_cast<unsigned long long*>(&b)));
+  return *reinterpret_cast<float2*>(&r);
+}
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) {
+  unsigned long long r;
+  asm("mul.rn.f32x2 %0, %1, %2;"
+      : "=l"(r)
+      : "l"(*reinterpret_cast<unsigned long long*>(&a)),
+        "l"(*reinterpret_cast<unsigned long long*>(&b)));
+  return *reinterpret_cast<float2*>(&r);
+}
+
 // INTERIOR: all trilinear corners of every pixel lie inside the grid (checked
 // on the host from max |q_i|), so no bounds checks.
 template <bool INTERIOR>
@@ -93,8 +118,9 @@ __global__ void __launch_bounds__(kAggThreads, 8)
   g_num += rep;
   g_den += rep;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  float2* box = agg_smem + warp * (kAggCap + kAggStage);
-  float2* stage = box + kAggCap;
+  float2* box = agg_smem + warp * (kAggCap + kAggList / 2);
+  int* list = reinterpret_cast<int*>(box + kAggCap);
+  const unsigned below = (1u << lane) - 1u;
   // the row's rotation in registers (uniform loads, once per CTA)
   int Rh[9];
   float Rhf[9], Rl[9];
@@ -143,68 +169,68 @@ __global__ void __launch_bounds__(kAggThreads, 8)
     const unsigned m = __match_any_sync(0xffffffffu, key);
     const bool lead = has && (__ffs(m) - 1 == lane);
     float2 acc[8];
+    const float2 vd = make_float2(v, dv);
 #pragma unroll
     for (int c = 0; c < 8; c++) {
       const int cx = (c >> 2) & 1, cy = (c >> 1) & 1, cz = c & 1;
       const float w = (cx ? t[0] : 1.f - t[0]) * (cy ? t[1] : 1.f - t[1]) *
                       (cz ? t[2] : 1.f - t[2]);
-      acc[c] = make_float2(w * v, w * dv);
+      acc[c] = mul2(make_float2(w, w), vd);
     }
     // pixels sharing a floor cell: the lowest lane sums the terms in lane order
-    const bool shared = has && m != (1u << lane);
-    if (__any_sync(0xffffffffu, shared)) {
-      if (shared && !lead)
+    unsigned rest = lead ? m & ~(1u << lane) : 0u;
+    while (__any_sync(0xffffffffu, rest != 0u)) {
+      const int src = rest ? __ffs(rest) - 1 : lane;
 #pragma unroll
-        for (int c = 0; c < 8; c++) stage[lane * 8 + c] = acc[c];
-      __syncwarp();
-      if (shared && lead) {
-        unsigned rest = m & ~(1u << lane);
-        while (rest) {
-          const int l = __ffs(rest) - 1;
-          rest &= rest - 1;
-#pragma unroll
-          for (int c = 0; c < 8; c++) {
-            const float2 o = stage[l * 8 + c];
-            acc[c].x += o.x;
-            acc[c].y += o.y;
-          }
-        }
+      for (int c = 0; c < 8; c++) {
+        const float ox = __shfl_sync(0xffffffffu, acc[c].x, src);
+        const float oy = __shfl_sync(0xffffffffu, acc[c].y, src);
+        if (rest) acc[c] = add2(acc[c], make_float2(ox, oy));
       }
-      __syncwarp();
+      rest &= rest - 1;
     }
     // corner by corner: the leaders' slots for one offset are distinct
 #pragma unroll
     for (int c = 0; c < 8; c++) {
       const int cx = (c >> 2) & 1, cy = (c >> 1) & 1, cz = c & 1;
       if (lead && (INTERIOR || in_grid(f[0] + cx, f[1] + cy, f[2] + cz, N))) {
-        const int s = key + (cx * dim[1] + cy) * dim[2] + cz;
-        float2 b = box[s];
-        b.x += acc[c].x;
-        b.y += acc[c].y;
-        box[s] = b;
+        float2* b = box + key + (cx * dim[1] + cy) * dim[2] + cz;
+        *b = add2(*b, acc[c]);
       }
       __syncwarp();
     }
-    // sweep the box in slot order: one reduction per non-zero slot. Slot
-    // s = (x dim1 + y) dim2 + z; the quotients by multiply and shift with
-    // m = ceil(2^20 / d): floor(s m / 2^20) = floor(s / d) for s < 1024,
-    // since s (m - 2^20 / d) / 2^20 < 2^-10 < 1/d for d <= kAggCap. (Integer
-    // arithmetic: conversions between int and float run on the FP64 pipe here.)
+    // the non-zero slots, listed in slot order
+    int n = 0;
+    for (int s0 = 0; s0 < (int)vol; s0 += 32) {
+      const int s = s0 + lane;
+      bool on = false;
+      if (s < (int)vol) {
+        const float2 b = box[s];
+        on = (__float_as_uint(b.x) | __float_as_uint(b.y)) != 0u;
+      }
+      const unsigned om = __ballot_sync(0xffffffffu, on);
+      if (on) list[n + __popc(om & below)] = s;
+      n += __popc(om);
+    }
+    __syncwarp();
+    // one reduction per listed slot. Slot s = (x dim1 + y) dim2 + z; the
+    // quotients by multiply and shift with m = ceil(2^20 / d): floor(s m / 2^20)
+    // = floor(s / d) for s < 1024, since s (m - 2^20 / d) / 2^20 < 2^-10 < 1/d for
+    // d <= kAggCap. (Integer arithmetic: conversions between int and float run
+    // on the FP64 pipe here.)
     const int d12 = dim[1] * dim[2];
     const unsigned m12 = ((1u << 20) + (unsigned)d12 - 1u) / (unsigned)d12;
     const unsigned m2 = ((1u << 20) + (unsigned)dim[2] - 1u) / (unsigned)dim[2];
-    for (int s = lane; s < (int)vol; s += 32) {
+    for (int e = lane; e < n; e += 32) {
+      const int s = list[e];
       const float2 b = box[s];
-      if (b.x != 0.f || b.y != 0.f) {
-        const int x = (int)(((unsigned)s * m12) >> 20);
-        const int r = s - x * d12;
-        const int y = (int)(((unsigned)r * m2) >> 20);
-        const int z = r - y * dim[2];
-        const int64_t l = (int64_t)(lo[0] + x) * nn + (int64_t)(lo[1] + y) * N + (lo[2] + z);
-        if (b.x != 0.f) atomicAdd(g_num + l, (double)b.x);
-        if (b.y != 0.f) atomicAdd(g_den + l, (double)b.y);
-        box[s] = make_float2(0.f, 0.f);
-      }
+      box[s] = make_float2(0.f, 0.f);
+      const int x = (int)(((unsigned)s * m12) >> 20);
+      const int r = s - x * d12;
+      const int y = (int)(((unsigned)r * m2) >> 20);
+      const int l = ((lo[0] + x) * N + (lo[1] + y)) * N + (lo[2] + r - y * dim[2]);
+      if (b.x != 0.f) atomicAdd(g_num + l, (double)b.x);
+      if (b.y != 0.f) atomicAdd(g_den + l, (double)b.y);
     }
     __syncwarp();  // slots cleared before the next group's steps
   }
