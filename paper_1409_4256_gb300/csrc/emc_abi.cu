@@ -136,9 +136,9 @@ Layout make_layout(const emc_config* c) {
   y.rot = take(sizeof(RotDF) * c->n_rot);
   y.rotfx = take(sizeof(RotFX) * c->n_rot);
   y.epart = take(sizeof(double) * (size_t)expand_tile_slices(y.ld_pix) * y.rows);
-  // the model in the corner-pair layout of the expansions' gathers (16 B a voxel;
-  // grids up to 256^3, 268 MB)
-  y.g4 = c->N <= 256 ? take(sizeof(float4) * (size_t)nvox) : 0;
+  // the model in the cell layout of the expansions' gathers (32 B a voxel;
+  // grids up to 256^3, 537 MB)
+  y.g4 = c->N <= 256 ? take(2 * sizeof(float4) * (size_t)nvox) : 0;
   y.logw = take(sizeof(double) * c->n_rot);
   y.Kb = take(2 * (size_t)y.ld_data * y.ld_pix);
   y.status = take(256);
@@ -692,7 +692,7 @@ int do_expand(emc_ctx* c, const float* grid, int64_t rot0, int64_t nrot, void* L
   const bool g = is_gauss(&c->cfg);
   const Layout& y = c->lay;
   float4* g4 = (y.g4 && c->geom.interior) ? (float4*)(c->ws + y.g4) : nullptr;
-  if (g4) CU(launch_grid_pairs(grid, c->cfg.N, g4, s));
+  if (g4) CU(launch_grid_cells(grid, c->cfg.N, g4, s));
   if (!g && !is_flu(&c->cfg)) {
     CU(launch_expand_tile(c->geom, grid, g4, (const RotFX*)(c->ws + y.rotfx) + rot0, c->logw + rot0,
                           nrot, rows, c->cfg.precision, (float)c->cfg.w_floor, p, bias,
@@ -992,7 +992,7 @@ int emc_iteration(emc_ctx* c, const float* grid_in, float* grid_out, emc_iter_st
                       fused ? bold : nullptr)))
     return st;
   // Gaussian: grid maximum and scales first; Poisson: the row tiles and the bias
-  // sums; the corner-pair layout of the model first where it is used
+  // sums; the cell layout of the model first where it is used
   kernels += (is_gauss(&c->cfg) ? 3 : (is_flu(&c->cfg) ? 1 : 2)) +
              ((y.g4 && c->geom.interior) ? 1 : 0);
   if (stats) CU(cudaEventRecord(c->ev[1], s));

@@ -154,19 +154,34 @@ __device__ __forceinline__ void rotate_fx(const int* Rh, const float* Rhf, const
 }
 
 // Trilinear value (Eq. 2.8, tent weights) at p = f + t from the grid in its
-// corner-pair layout g4[(x N + y) N + z] = (g[x][y][z], g[x][y][z+1],
-// g[x][y+1][z], g[x][y+1][z+1]) (0 beyond the grid): two 16-byte loads per
-// point where the plain layout needs eight scattered 4-byte ones, which is
-// what limits the expansion (its loads are gathers: every lane of a warp reads
-// another cache line). Corners inside the grid only (interior points).
-__device__ __forceinline__ float trilinear_g4(const float4* __restrict__ g4, int N, const int* f,
-                                              const float* t) {
-  const int64_t o = ((int64_t)f[0] * N + f[1]) * N + f[2];
-  const float4 a = __ldg(g4 + o), b = __ldg(g4 + o + (int64_t)N * N);
+// cell layout: the eight corners of voxel l = (x N + y) N + z in g4[2 l] =
+// (g[x][y][z], g[x][y][z+1], g[x][y+1][z], g[x][y+1][z+1]) and, for x + 1, in
+// g4[2 l + 1] (0 beyond the grid). One 32-byte load per point, a whole sector,
+// where the plain layout needs eight scattered 4-byte ones: the loads are
+// gathers (every lane of a warp reads another cache line), and their
+// wavefronts are what the expansion waits for. Corners inside the grid only
+// (interior points), N <= 256.
+struct Cell {
+  float4 a, b;  // corners at x, corners at x + 1
+};
+__device__ __forceinline__ Cell load_cell(const float4* __restrict__ g4, int voxel) {
+  Cell c;
+  asm("ld.global.nc.v8.f32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+      : "=f"(c.a.x), "=f"(c.a.y), "=f"(c.a.z), "=f"(c.a.w), "=f"(c.b.x), "=f"(c.b.y),
+        "=f"(c.b.z), "=f"(c.b.w)
+      : "l"(g4 + 2 * voxel));
+  return c;
+}
+__device__ __forceinline__ float cell_value(const Cell& c, const float* t) {
+  const float4 a = c.a, b = c.b;
   const float tz = t[2], sz = 1.f - tz, ty = t[1], sy = 1.f - ty;
   const float va = sy * fmaf(tz, a.y, sz * a.x) + ty * fmaf(tz, a.w, sz * a.z);
   const float vb = sy * fmaf(tz, b.y, sz * b.x) + ty * fmaf(tz, b.w, sz * b.z);
   return fmaf(t[0], vb, (1.f - t[0]) * va);
+}
+__device__ __forceinline__ float trilinear_g4(const float4* __restrict__ g4, int N, const int* f,
+                                              const float* t) {
+  return cell_value(load_cell(g4, (f[0] * N + f[1]) * N + f[2]), t);
 }
 
 // FP32 -> FP64 with integer operations (the conversion instruction runs on the

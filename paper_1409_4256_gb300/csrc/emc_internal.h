@@ -72,7 +72,7 @@ cudaError_t launch_assign_duplicates(const int32_t* K, int64_t ld_k, int64_t n_d
                                      int32_t* status, cudaStream_t s);
 
 // gsc != NULL: Gaussian model (FP16 three-plane s W, bias log w - sum W^2 / 2 sigma^2)
-// g4 (may be NULL): the grid in the corner-pair layout (launch_grid_pairs)
+// g4 (may be NULL): the grid in the cell layout (launch_grid_cells)
 cudaError_t launch_expand(const Geom& g, const float* grid, const float4* g4, const RotDF* rot,
                           const double* logw, int64_t nrot, int64_t rows, int precision,
                           float w_floor, Planes L, double* bias, const float4* gsc, double sigma,
@@ -84,9 +84,9 @@ cudaError_t launch_expand(const Geom& g, const float* grid, const float4* g4, co
 // increments D ([2 ntp][ld_pix], rounded up to the frames' type), dabs[t] and,
 // from bias_old, bpm (as launch_delta_planes).
 int64_t expand_tile_slices(int64_t ld_pix);
-// g4 (may be NULL): the grid in the corner-pair layout (launch_grid_pairs),
+// g4 (may be NULL): the grid in the cell layout (launch_grid_cells),
 // read where every corner lies inside the grid
-cudaError_t launch_grid_pairs(const float* grid, int N, float4* g4, cudaStream_t s);
+cudaError_t launch_grid_cells(const float* grid, int N, float4* g4, cudaStream_t s);
 cudaError_t launch_expand_tile(const Geom& g, const float* grid, const float4* g4,
                                const RotFX* rot,
                                const double* logw, int64_t nrot, int64_t rows, int precision,

@@ -1,8 +1,9 @@
-// expand_tile.cu -- e-step of EMC (Eq. 2.9) for the Poisson model, one row
-// tile of 128 rotations per CTA (and a slice of 256 pixels: small CTAs, so
-// that the last wave of the grid leaves few SMs idle).
+// expand_tile.cu -- e-step of EMC (Eq. 2.9) for the Poisson model, a quarter or
+// an eighth of a row tile of 128 rotations and a slice of 256 pixels per CTA
+// (small CTAs, so that small blocks of rotations fill the SMs and the last wave
+// leaves few of them idle).
 //
-// Each thread owns two neighbouring pixels and takes the tile's rotations in
+// Each thread owns two neighbouring pixels and takes the CTA's rotations in
 // turn, so the pixels' geometry stays in registers and the rotations come from
 // shared memory. Per (i, j): the grid point p = R_j q_i + N/2, the trilinear
 // value of the model (Eq. 2.8, tent weights), W_ij = max(W, w_floor) and
@@ -19,31 +20,128 @@
 //
 // The grid point is formed in fixed point (rotate_fx): exact 64-bit integer
 // products for the large part, six FP32 FMAs for the rest (error ~1e-10
-// voxel), where expand.cu uses double-float arithmetic.
+// voxel), the FP32 parts of the two pixels in one instruction. The voxel's
+// eight corners come with one 32-byte load, asked for one rotation ahead.
+//
+// Bound by issue (68%; the FMA pipe next) and the load/store pipe (75%: the
+// gathers). 64^3, 10880 rows x 2816 columns, under ncu: 306 us with 128
+// rotations a CTA, scalar FP32 and two 16-byte gathers at the point of use (254
+// instructions per element); 225 us with two-pixel instructions, rounding without
+// the conversion pipe and 32 rotations a CTA (175); 215 us with 32-byte cells; 191 us
+// with the gathers a rotation ahead. 32^3 with 3240 rotations: 223 -> 39 us.
 //
 // With the last iteration's L (DELTA), the CTA also reads the previous planes
 // of its elements and keeps, per pixel, the largest rise and fall of the
 // represented log W over the tile's rows: the rows t and ntp + t of the
 // incremental bound's increments D (prune.cu), rounded up to the operand type
 // of the frames, and their magnitude bound A (the rows 2 ntp + t).
+#include <cooperative_groups.h>
+
 #include "emc_common.cuh"
 #include "emc_internal.h"
+
+namespace cg = cooperative_groups;
 
 namespace emc {
 
 namespace {
 
 constexpr int kTThreads = 128;
-constexpr int kTRows = 128;
+constexpr int kTRows = 128;  // rotations of a row tile
 constexpr int kTPix = 2 * kTThreads;
 
-// one rotation in shared memory: read as seven 16-byte words
+// one rotation in shared memory, read as 16-byte words; the FP32 parts twice,
+// as operands of two-pixel instructions
 struct __align__(16) RowFX {
-  int hi[9];
-  float hf[9];  // hi as FP32 (hi 2^-20, exact)
-  float lo[9];
-  float pad;
+  int hi[12];
+  float2 hf[9];  // hi as FP32 (hi 2^-20, exact)
+  float2 lo[9];
 };
+
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
+  unsigned long long r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;"
+      : "=l"(r)
+      : "l"(*reinterpret_cast<unsigned long long*>(&a)),
+        "l"(*reinterpret_cast<unsigned long long*>(&b)),
+        "l"(*reinterpret_cast<unsigned long long*>(&c)));
+  return *reinterpret_cast<float2*>(&r);
+}
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) {
+  unsigned long long r;
+  asm("mul.rn.f32x2 %0, %1, %2;"
+      : "=l"(r)
+      : "l"(*reinterpret_cast<unsigned long long*>(&a)),
+        "l"(*reinterpret_cast<unsigned long long*>(&b)));
+  return *reinterpret_cast<float2*>(&r);
+}
+__device__ __forceinline__ float2 add2(float2 a, float2 b) {
+  unsigned long long r;
+  asm("add.rn.f32x2 %0, %1, %2;"
+      : "=l"(r)
+      : "l"(*reinterpret_cast<unsigned long long*>(&a)),
+        "l"(*reinterpret_cast<unsigned long long*>(&b)));
+  return *reinterpret_cast<float2*>(&r);
+}
+
+// The grid points of a thread's two pixels: rotate_fx, bit for bit, in two-pixel
+// FP32 instructions. The small part leaves a fraction outside [0, 1) only within
+// 10^-3 of a voxel's face, so all six are looked at once and put right in a
+// branch that few warps take.
+__device__ __forceinline__ void rotate_pair(const RowFX& R, const int4* qi, const float2* qh,
+                                            const float2* ql, long long centre, int (*f)[3],
+                                            float (*t)[3]) {
+  const float2 down = make_float2(0x1p-23f, 0x1p-23f), one = make_float2(-1.f, -1.f);
+#pragma unroll
+  for (int a = 0; a < 3; a++) {
+    const float2 small = fma2(
+        R.hf[3 * a], ql[0],
+        fma2(R.hf[3 * a + 1], ql[1],
+             fma2(R.hf[3 * a + 2], ql[2],
+                  fma2(R.lo[3 * a], qh[0],
+                       fma2(R.lo[3 * a + 1], qh[1], mul2(R.lo[3 * a + 2], qh[2]))))));
+    float hi[2], lo[2];
+#pragma unroll
+    for (int u = 0; u < 2; u++) {
+      long long acc = centre;
+      acc += (long long)R.hi[3 * a] * (long long)qi[u].x;
+      acc += (long long)R.hi[3 * a + 1] * (long long)qi[u].y;
+      acc += (long long)R.hi[3 * a + 2] * (long long)qi[u].z;
+      f[u][a] = (int)(acc >> 32);
+      const unsigned fw = (unsigned)(acc & 0xffffffffLL);
+      hi[u] = __uint_as_float(0x3f800000u | (fw >> 9));
+      lo[u] = __uint_as_float(0x3f800000u | ((fw & 511u) << 14));
+    }
+    const float2 fr = add2(add2(make_float2(hi[0], hi[1]), one),
+                           fma2(add2(make_float2(lo[0], lo[1]), one), down, small));
+    t[0][a] = fr.x;
+    t[1][a] = fr.y;
+  }
+  const float least = fminf(fminf(fminf(t[0][0], t[0][1]), fminf(t[0][2], t[1][0])),
+                            fminf(t[1][1], t[1][2]));
+  const float most = fmaxf(fmaxf(fmaxf(t[0][0], t[0][1]), fmaxf(t[0][2], t[1][0])),
+                           fmaxf(t[1][1], t[1][2]));
+  if (least < 0.f || most >= 1.f) {
+#pragma unroll
+    for (int u = 0; u < 2; u++)
+#pragma unroll
+      for (int a = 0; a < 3; a++) {
+        if (t[u][a] < 0.f) {
+          f[u][a] -= 1;
+          t[u][a] += 1.f;
+        } else if (t[u][a] >= 1.f) {
+          f[u][a] += 1;
+          t[u][a] -= 1.f;
+        }
+      }
+  }
+}
+
+// x to the nearest multiple of 1 / scale (a power of two; ties to even), |x scale|
+// below 2^22: by adding and taking away 1.5 2^23 (rintf is a conversion instruction)
+__device__ __forceinline__ float round_to(float x, float scale) {
+  return ((fmaf(x, scale, 12582912.f)) - 12582912.f) * (1.0f / scale);
+}
 
 template <bool INTERIOR>
 __device__ __forceinline__ float trilinear_fx(const float* __restrict__ grid, int N, const int* f,
@@ -106,7 +204,9 @@ __device__ __forceinline__ uint16_t round_up_operand(float x) {
   return *reinterpret_cast<uint16_t*>(&b);
 }
 
-template <int PREC, bool INTERIOR, bool DELTA>
+// RPC rotations of a tile per CTA; with DELTA the tile's 128 / RPC CTAs are a
+// cluster, whose first one gathers the others' rises and falls.
+template <int PREC, bool INTERIOR, bool DELTA, int RPC>
 __global__ void __launch_bounds__(kTThreads, 6)
     expand_tile_kernel(const int4* __restrict__ qi_g, const float4* __restrict__ qlo_g,
                        int64_t ld_pix, int N, const float* __restrict__ grid,
@@ -114,17 +214,21 @@ __global__ void __launch_bounds__(kTThreads, 6)
                        const RotFX* __restrict__ rot, int64_t nrot, int64_t rows, float w_floor,
                        void* __restrict__ Lbase, int64_t ps, double* __restrict__ partial,
                        const void* __restrict__ Lold, uint16_t* __restrict__ D, int64_t ntp,
-                       int32_t* status) {
-  __shared__ RowFX R[kTRows];
-  __shared__ float2 rsum[kTThreads / 32][kTRows];
+                       unsigned slices, int32_t* status) {
+  __shared__ RowFX R[RPC];
+  __shared__ float2 rsum[kTThreads / 32][RPC];
   // eight rows of every lane's pair, rows padded to 33 so that the transposed
   // reads hit 16 distinct bank pairs per half warp
   __shared__ float2 park[kTThreads / 32][8 * 33];
-  const int64_t t = blockIdx.y;
-  const int64_t r0 = t * kTRows;
-  const int nr = (int)min((int64_t)kTRows, nrot - r0);  // >= 1 for every tile of rows
+  __shared__ float4 rises[DELTA ? kTThreads : 1];
+  // a tile's CTAs are neighbours, then the slices, then the tiles
+  constexpr unsigned kPer = kTRows / RPC;
+  const unsigned slice = blockIdx.x / kPer % slices;
+  const int64_t t = blockIdx.x / kPer / slices;
+  const int64_t r0 = t * kTRows + blockIdx.x % kPer * RPC;
+  const int nr = (int)max((int64_t)0, min((int64_t)RPC, nrot - r0));  // valid rows
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  for (int x = threadIdx.x; x < kTRows * 9; x += kTThreads) {
+  for (int x = threadIdx.x; x < RPC * 9; x += kTThreads) {
     const int r = x / 9, e = x % 9;
     int h = 0;
     float l = 0.f;
@@ -132,48 +236,70 @@ __global__ void __launch_bounds__(kTThreads, 6)
       h = rot[r0 + r].hi[e];
       l = rot[r0 + r].lo[e];
     }
+    const float hf = (float)h * 0x1p-20f;
     R[r].hi[e] = h;
-    R[r].hf[e] = (float)h * 0x1p-20f;
-    R[r].lo[e] = l;
+    R[r].hf[e] = make_float2(hf, hf);
+    R[r].lo[e] = make_float2(l, l);
   }
-  const int64_t i0 = (int64_t)blockIdx.x * kTPix + 2 * threadIdx.x;
+  const int64_t i0 = (int64_t)slice * kTPix + 2 * threadIdx.x;
   const bool inside = i0 < ld_pix;  // ld_pix is even: both pixels or neither
   int4 qi[2];
-  float4 qh[2], ql[2];
+  float2 qh[3], ql[3];
+  {
+    float4 l[2];
 #pragma unroll
-  for (int u = 0; u < 2; u++) {
-    qi[u] = inside ? qi_g[i0 + u] : make_int4(0, 0, 0, 0);
-    ql[u] = inside ? qlo_g[i0 + u] : make_float4(0.f, 0.f, 0.f, 0.f);
-    qh[u] = make_float4((float)qi[u].x * 0x1p-12f, (float)qi[u].y * 0x1p-12f,
-                        (float)qi[u].z * 0x1p-12f, 0.f);
+    for (int u = 0; u < 2; u++) {
+      qi[u] = inside ? qi_g[i0 + u] : make_int4(0, 0, 0, 0);
+      l[u] = inside ? qlo_g[i0 + u] : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    qh[0] = make_float2((float)qi[0].x * 0x1p-12f, (float)qi[1].x * 0x1p-12f);
+    qh[1] = make_float2((float)qi[0].y * 0x1p-12f, (float)qi[1].y * 0x1p-12f);
+    qh[2] = make_float2((float)qi[0].z * 0x1p-12f, (float)qi[1].z * 0x1p-12f);
+    ql[0] = make_float2(l[0].x, l[1].x);
+    ql[1] = make_float2(l[0].y, l[1].y);
+    ql[2] = make_float2(l[0].z, l[1].z);
   }
+  const long long centre = ((long long)(N >> 1) << 32) + ((N & 1) ? (1LL << 31) : 0LL);
   __syncthreads();
   float dp[2] = {-INFINITY, -INFINITY}, dm[2] = {-INFINITY, -INFINITY};
   int bad = 0, nonfinite = 0;
-  for (int r = 0; r < kTRows; r++) {
+  // Row r + 1's grid points are formed and its voxels asked for before row r's
+  // values are used: the gathers' latency is what the loop would wait for.
+  float tt[2][3];
+  Cell cell[2];
+  auto fetch = [&](int r) {
+    int f[2][3];
+    rotate_pair(R[r], qi, qh, ql, centre, f, tt);
+#pragma unroll
+    for (int u = 0; u < 2; u++) {
+      if (INTERIOR && g4)  // padding pixels and rows read the centre
+        cell[u] = load_cell(g4, (f[u][0] * N + f[u][1]) * N + f[u][2]);
+      else
+        cell[u].a.x = r < nr && qi[u].w != 0 ? trilinear_fx<INTERIOR>(grid, N, f[u], tt[u]) : 0.f;
+    }
+  };
+  fetch(0);
+  for (int r = 0; r < RPC; r++) {
     const int64_t row = r0 + r;
     const bool vrow = r < nr;
+    float W2[2];
+#pragma unroll
+    for (int u = 0; u < 2; u++)
+      W2[u] = INTERIOR && g4 ? cell_value(cell[u], tt[u]) : cell[u].a.x;
+    if (r + 1 < RPC) fetch(r + 1);
     float L[2] = {0.f, 0.f};
-    float s = 0.f, se = 0.f;  // row sum of the pair as s + se
-    const RowFX Rr = R[r];
+    float ws[2] = {0.f, 0.f};
 #pragma unroll
     for (int u = 0; u < 2; u++) {
       if (vrow && qi[u].w != 0) {  // w: 1 pixel, 2 duplicate column, 0 padding / ones
-        int f[3];
-        float tt[3];
-        rotate_fx(Rr.hi, Rr.hf, Rr.lo, qi[u], qh[u], ql[u], N, f, tt);
-        float W = (INTERIOR && g4) ? trilinear_g4(g4, N, f, tt)
-                                   : trilinear_fx<INTERIOR>(grid, N, f, tt);
-        nonfinite |= !(fabsf(W) <= 3.4e38f);  // a NaN or infinite voxel of the model
-        W = fmaxf(W, w_floor);
-        if (qi[u].w == 1) {  // duplicate columns repeat a pixel: not summed
-          const f2 a = two_sum(s, W);
-          s = a.h;
-          se += a.l;
-        }
+        nonfinite |= !(fabsf(W2[u]) <= 3.4e38f);  // a NaN or infinite voxel of the model
+        const float W = fmaxf(W2[u], w_floor);
+        if (qi[u].w == 1) ws[u] = W;  // duplicate columns repeat a pixel: not summed
         L[u] = logf(W);
       }
     }
+    const f2 pair = two_sum(ws[0], ws[1]);  // row sum of the pair as s + se
+    const float s = pair.h, se = pair.l;
     if (inside && row < rows) {
       const int64_t o = row * ld_pix + i0;
       // DELTA: the change of the represented value (the planes' sum) of each element
@@ -199,7 +325,7 @@ __global__ void __launch_bounds__(kTThreads, 6)
         float v[2];
 #pragma unroll
         for (int u = 0; u < 2; u++) {
-          float hi = rintf(L[u] * kHi16Scale) * (1.0f / kHi16Scale);
+          float hi = round_to(L[u], kHi16Scale);
           if (vrow && qi[u].w != 0 && (hi < kHiMin || hi > kHi16Max)) bad = 1;
           hi = fminf(fmaxf(hi, kHiMin), kHi16Max);
           h[u] = fp16_bits(hi);
@@ -221,7 +347,7 @@ __global__ void __launch_bounds__(kTThreads, 6)
         float v[2];
 #pragma unroll
         for (int u = 0; u < 2; u++) {
-          float hi = rintf(L[u] * kHiScale) * (1.0f / kHiScale);
+          float hi = round_to(L[u], kHiScale);
           if (vrow && qi[u].w != 0 && (hi < kHiMin || hi > kHiMax)) bad = 1;
           hi = fminf(fmaxf(hi, kHiMin), kHiMax);
           const float r = L[u] - hi;  // exact
@@ -272,7 +398,7 @@ __global__ void __launch_bounds__(kTThreads, 6)
   if (nonfinite) set_status(status, EMC_ERR_NUMERIC);
   if (bad) set_status(status, EMC_ERR_UNSUPPORTED);
   __syncthreads();
-  if (threadIdx.x < kTRows) {
+  if (threadIdx.x < RPC) {
     float s = 0.f, se = 0.f;
     if ((int)threadIdx.x < nr)
       for (int w = 0; w < kTThreads / 32; w++) {
@@ -281,9 +407,20 @@ __global__ void __launch_bounds__(kTThreads, 6)
         s = a.h;
         se += v.y + a.l;
       }
-    partial[(int64_t)blockIdx.x * rows + r0 + threadIdx.x] = f32_to_f64(s) + f32_to_f64(se);
+    partial[(int64_t)slice * rows + r0 + threadIdx.x] = f32_to_f64(s) + f32_to_f64(se);
   }
-  if (DELTA && inside) {
+  if (!DELTA) return;
+  cg::cluster_group cluster = cg::this_cluster();
+  rises[threadIdx.x] = make_float4(dp[0], dp[1], dm[0], dm[1]);
+  cluster.sync();
+  if (cluster.block_rank() == 0 && inside) {
+    for (int q = 1; q < kTRows / RPC; q++) {
+      const float4 o = cluster.map_shared_rank(rises, q)[threadIdx.x];
+      dp[0] = fmaxf(dp[0], o.x);
+      dp[1] = fmaxf(dp[1], o.y);
+      dm[0] = fmaxf(dm[0], o.z);
+      dm[1] = fmaxf(dm[1], o.w);
+    }
     float a[2];
 #pragma unroll
     for (int u = 0; u < 2; u++) {
@@ -301,6 +438,7 @@ __global__ void __launch_bounds__(kTThreads, 6)
     *reinterpret_cast<uint32_t*>(D + (2 * ntp + t) * ld_pix + i0) =
         (uint32_t)a0 | ((uint32_t)a1 << 16);
   }
+  cluster.sync();  // no CTA leaves while its rises may be read
 }
 
 // bias_j = log w_j - (sum of the slices' partial sums, in slice order); with
@@ -335,15 +473,19 @@ __global__ void __launch_bounds__(kTRows)
   }
 }
 
-// the grid in the corner-pair layout of trilinear_g4
-__global__ void grid_pairs_kernel(const float* __restrict__ g, int N, float4* __restrict__ g4) {
+// the grid in the cell layout of load_cell
+__global__ void grid_cells_kernel(const float* __restrict__ g, int N, float4* __restrict__ g4) {
   const int64_t n3 = (int64_t)N * N * N;
   const int64_t l = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (l >= n3) return;
   const int z = (int)(l % N), y = (int)((l / N) % N);
   const bool zi = z + 1 < N, yi = y + 1 < N;
-  g4[l] = make_float4(g[l], zi ? g[l + 1] : 0.f, yi ? g[l + N] : 0.f,
-                      (zi && yi) ? g[l + N + 1] : 0.f);
+  const int64_t m = l + (int64_t)N * N;
+  const bool xi = m < n3;
+  g4[2 * l] = make_float4(g[l], zi ? g[l + 1] : 0.f, yi ? g[l + N] : 0.f,
+                          (zi && yi) ? g[l + N + 1] : 0.f);
+  g4[2 * l + 1] = make_float4(xi ? g[m] : 0.f, xi && zi ? g[m + 1] : 0.f,
+                              xi && yi ? g[m + N] : 0.f, (xi && zi && yi) ? g[m + N + 1] : 0.f);
 }
 
 // fixed-point pixel geometry from the double-float one
@@ -372,9 +514,9 @@ __global__ void fixed_geometry_kernel(const float4* __restrict__ qh, const float
 
 int64_t expand_tile_slices(int64_t ld_pix) { return (ld_pix + kTPix - 1) / kTPix; }
 
-cudaError_t launch_grid_pairs(const float* grid, int N, float4* g4, cudaStream_t s) {
+cudaError_t launch_grid_cells(const float* grid, int N, float4* g4, cudaStream_t s) {
   const int64_t n3 = (int64_t)N * N * N;
-  grid_pairs_kernel<<<(unsigned)((n3 + 255) / 256), 256, 0, s>>>(grid, N, g4);
+  grid_cells_kernel<<<(unsigned)((n3 + 255) / 256), 256, 0, s>>>(grid, N, g4);
   return cudaGetLastError();
 }
 
@@ -395,11 +537,32 @@ cudaError_t launch_expand_tile(const Geom& g, const float* grid, const float4* g
   const int64_t nt = rows / kTRows;
   const int64_t ns = expand_tile_slices(g.ld_pix);
   const bool delta = Lold != nullptr;
-  dim3 grd((unsigned)ns, (unsigned)nt);
-#define EMC_TILE(P, I, DL)                                                                    \
-  expand_tile_kernel<P, I, DL><<<grd, kTThreads, 0, s>>>(                                     \
-      g.qi, g.qlo, g.ld_pix, g.N, grid, g4, rot, nrot, rows, w_floor, L.base, L.plane_stride, \
-      partial, Lold, D, ntp, status)
+  // 32 rotations a CTA (a quarter tile: small CTAs, so that the last wave of the
+  // grid leaves few SMs idle), 16 where those would not give every SM its six
+  int dev = 0, sms = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const int rpc = ns * nt * 4 < 6 * (int64_t)sms ? 16 : 32;
+  cudaLaunchConfig_t lc{};
+  lc.gridDim = dim3((unsigned)(ns * nt * (kTRows / rpc)));
+  lc.blockDim = dim3(kTThreads);
+  lc.stream = s;
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = (unsigned)(kTRows / rpc);
+  at.val.clusterDim.y = at.val.clusterDim.z = 1;
+  lc.attrs = &at;
+  lc.numAttrs = delta ? 1 : 0;
+  cudaError_t e = cudaSuccess;
+#define EMC_TILE_R(P, I, DL, RP)                                                               \
+  e = cudaLaunchKernelEx(&lc, expand_tile_kernel<P, I, DL, RP>, g.qi, g.qlo, g.ld_pix, g.N,    \
+                         grid, g4, rot, nrot, rows, w_floor, L.base, L.plane_stride, partial,  \
+                         Lold, D, ntp, (unsigned)ns, status)
+#define EMC_TILE(P, I, DL)                   \
+  do {                                       \
+    if (rpc == 16) EMC_TILE_R(P, I, DL, 16); \
+    else EMC_TILE_R(P, I, DL, 32);           \
+  } while (0)
 #define EMC_TILE_P(P)                          \
   if (g.interior) {                            \
     if (delta) EMC_TILE(P, true, true);        \
@@ -416,7 +579,7 @@ cudaError_t launch_expand_tile(const Geom& g, const float* grid, const float4* g
   }
 #undef EMC_TILE_P
 #undef EMC_TILE
-  cudaError_t e = cudaGetLastError();
+#undef EMC_TILE_R
   if (e != cudaSuccess) return e;
   expand_bias_kernel<<<(unsigned)nt, kTRows, 0, s>>>(partial, (int)ns, rows, logw, nrot, bias,
                                                      delta ? bias_old : nullptr, bpm, nt);
