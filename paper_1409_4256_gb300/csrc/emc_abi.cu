@@ -831,8 +831,9 @@ int do_update(emc_ctx* c, const void* P, int64_t Prows, int64_t nrot, float* Num
   const Layout& y = c->lay;
   const int64_t rows = round_up(nrot, 128);
   if (c->cfg.precision == EMC_PREC_FP32) {
-    CU(launch_simt_update((const float*)P, y.ld_data, rows, c->Kb, y.ld_pix, c->cfg.n_pix, Num,
-                          den, s));
+    // (pass 1's per-tile sums, consumed by now, hold the bits of the frames to contract)
+    CU(launch_simt_update((const float*)P, y.ld_data, rows, c->Kb, y.ld_pix, c->cfg.n_pix,
+                          (uint32_t*)(c->ws + y.part_s), Num, den, s));
   } else {
     Planes pp{(void*)P, Prows * y.ld_data, y.ld_data};
     if (is_gauss(&c->cfg) || is_flu(&c->cfg)) {

@@ -150,9 +150,10 @@ cudaError_t launch_simt_normalize(const float* L, int64_t ld_pix, const double* 
                                   int64_t nrot, const uint16_t* Kb, int64_t ld_data,
                                   int64_t n_data, const double* lse_m, const double* lse_s,
                                   float* P, cudaStream_t s);
+// nz: scratch of rows / 64 x ld_data / 32 words
 cudaError_t launch_simt_update(const float* P, int64_t ld_data, int64_t rows, const uint16_t* Kb,
-                               int64_t ld_pix, int64_t n_pix, float* Num, float* den,
-                               cudaStream_t s);
+                               int64_t ld_pix, int64_t n_pix, uint32_t* nz, float* Num,
+                               float* den, cudaStream_t s);
 int64_t simt_pass1_tiles(int64_t rows);
 
 // Merge of per-tile (max, sum) pairs into the running per-frame (m, s).
