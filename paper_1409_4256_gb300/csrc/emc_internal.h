@@ -291,12 +291,12 @@ cudaError_t launch_tc_bound(const Planes& L, int precision, const double* bias, 
                             const int32_t* pair_list = nullptr,
                             const int32_t* pair_count = nullptr);
 
-// nrep grid replicas of n_vox each (row j reduces into replica j mod nrep)
+// adds to g_num, g_den
 cudaError_t launch_compress(const Geom& g, const RotFX* rot, int64_t nrot, const float* Num,
-                            const float* den, int mode, double* g_num, double* g_den, int nrep,
+                            const float* den, int mode, double* g_num, double* g_den,
                             cudaStream_t s);
-// grid_out = (sum of nrep numerator replicas) / (sum of denominator replicas)
-cudaError_t launch_finalize(int64_t n_vox, const double* g_num, const double* g_den, int nrep,
+// grid_out = g_num / g_den where g_den > 0, else grid_prev
+cudaError_t launch_finalize(int64_t n_vox, const double* g_num, const double* g_den,
                             const float* grid_prev, float* grid_out, cudaStream_t s);
 
 // ---- learned proposal (learned.cu) ----
