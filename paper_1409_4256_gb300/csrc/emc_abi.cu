@@ -23,7 +23,7 @@ struct Layout {
   size_t qh, ql, quat, rot, logw, Kb, status, L, bias, lse_m, lse_s, lse2, part_m, part_s, S, P,
       Num, den, gnum, gden, scalar, fbin, finv, cand, ccnt, coff, cent, Sc, Pc, lsec, gk, gauss,
       Kb2, skcnt, skoff, skent, dupsrc, duprank, pixmax, fcn, finvn, fB, kbflag, kbcnt, kblist,
-      Kp, perm, perm2, iperm, nsum, nsum_p, cn_p, invn_p, best, lsem_s, lses_s, live, tlist,
+      Kp, perm, perm2, iperm, nsum, nsum_p, cn_p, invn_p, best, lsem_s, lses_s, live, tlist, slot, klist,
       tcount, sortH, sortoff, cgs, cgp, cgqh, cgql, cgqi, cgqlo, cgqf, L2, bias2, Ub, Ub2, Lk, Mk, Mk2, best2,
       osrc, Dd, Cd, bpm, g4, Ua, Ua2, dcand, pflag, plist, flags, qi, qlo, rotfx, epart, total;
   int64_t sort_entries;
@@ -207,6 +207,10 @@ Layout make_layout(const emc_config* c) {
   y.lses_s = pr ? take(sizeof(double) * (size_t)y.ld_data) : 0;
   y.live = pr ? take((size_t)nmt * nnt) : 0;
   y.tlist = pr ? take(sizeof(int32_t) * (size_t)nmt * nnt) : 0;
+  // kept scores of the live tiles (no stored scores): places, and a chunk's kept tiles
+  const bool keep = pr && !(c->flags & EMC_FLAG_STORE_SCORES);
+  y.slot = keep ? take(sizeof(int32_t) * (size_t)nmt * nnt) : 0;
+  y.klist = keep ? take(sizeof(int32_t) * (size_t)(y.chunk_rows / 128) * nnt) : 0;
   y.tcount = pr ? take(256) : 0;
   y.sortH = pr ? take(sizeof(int32_t) * (size_t)y.sort_entries) : 0;
   y.sortoff = pr ? take(sizeof(int64_t) * (size_t)(y.sort_entries + 1)) : 0;
@@ -751,6 +755,11 @@ struct FrameView {
   const uint8_t* tile_live;   // stored scores: the contracted tiles of these rows
   const int32_t* tile_list;   // recomputed scores: the live tiles of these rows
   const int32_t* tile_count;
+  const float* kept;          // scores pass 1 kept: of these rows' tiles with slot < kept_cap,
+  const int32_t* slot;        // listed in kept_list
+  const int32_t* kept_list;
+  const int32_t* kept_count;
+  bool kept_all;              // ... which are all the live tiles
 };
 
 // S, Sref: stored scores of these rows, S frame-major with leading dimension
@@ -781,9 +790,15 @@ int do_normalize(emc_ctx* c, const void* L, int64_t Lrows, int64_t row_off, cons
     } else {
       Planes lp{(void*)((const uint16_t*)L + row_off * y.ld_pix), Lrows * y.ld_pix, y.ld_pix};
       Planes pp{P, Prows * y.ld_data, y.ld_data};
-      CU(launch_tc_normalize(lp, c->cfg.precision, bias, rows, nrot, Kf, y.ld_data,
-                             c->cfg.n_data, y.ld_pix, lse_m, lse_s, lse2, pp, c->status, s,
-                             cn, Bsum, invn, den, kbf, tl, tc, c->tcctl));
+      const bool kept = fv && fv->kept;
+      if (kept)
+        CU(launch_normalize_kept(fv->kept, fv->slot, fv->kept_list, fv->kept_count, lse_m, lse_s,
+                                 lse2, rows, nrot, y.ld_data, c->cfg.n_data, c->cfg.precision, P,
+                                 Prows * y.ld_data, cn, Bsum, invn, den, kbf, s));
+      if (!kept || !fv->kept_all)
+        CU(launch_tc_normalize(lp, c->cfg.precision, bias, rows, nrot, Kf, y.ld_data,
+                               c->cfg.n_data, y.ld_pix, lse_m, lse_s, lse2, pp, c->status, s,
+                               cn, Bsum, invn, den, kbf, tl, tc, c->tcctl, kept));
     }
     return EMC_OK;
   }
@@ -811,9 +826,16 @@ int do_normalize(emc_ctx* c, const void* L, int64_t Lrows, int64_t row_off, cons
   } else {
     Planes lp{(void*)((const uint16_t*)L + row_off * y.ld_pix), Lrows * y.ld_pix, y.ld_pix};
     Planes pp{P, Prows * y.ld_data, y.ld_data};
-    CU(launch_tc_normalize(lp, c->cfg.precision, bias, rows, nrot, Kf, y.ld_data, c->cfg.n_data,
-                           y.ld_pix, lse_m, lse_s, (float2*)(c->ws + y.lse2), pp, c->status, s,
-                           nullptr, nullptr, nullptr, nullptr, kbf, tl, tc, c->tcctl));
+    float2* lse2 = (float2*)(c->ws + y.lse2);
+    const bool kept = fv && fv->kept;
+    if (kept)
+      CU(launch_normalize_kept(fv->kept, fv->slot, fv->kept_list, fv->kept_count, lse_m, lse_s, lse2,
+                               rows, nrot, y.ld_data, c->cfg.n_data, c->cfg.precision, P,
+                               Prows * y.ld_data, nullptr, nullptr, nullptr, nullptr, kbf, s));
+    if (!kept || !fv->kept_all)
+      CU(launch_tc_normalize(lp, c->cfg.precision, bias, rows, nrot, Kf, y.ld_data, c->cfg.n_data,
+                             y.ld_pix, lse_m, lse_s, lse2, pp, c->status, s, nullptr, nullptr,
+                             nullptr, nullptr, kbf, tl, tc, c->tcctl, kept));
   }
   return EMC_OK;
 }
@@ -1000,6 +1022,16 @@ int emc_iteration(emc_ctx* c, const float* grid_in, float* grid_out, emc_iter_st
   double* lm = pr ? (double*)(c->ws + y.lsem_s) : lse_m;  // lse in the internal order
   double* ls = pr ? (double*)(c->ws + y.lses_s) : lse_s;
   const double* cn_p = y.cn_p ? (const double*)(c->ws + y.cn_p) : nullptr;
+  // Where the scores are not stored, a pruned pass 1 keeps those of its live
+  // tiles for pass 2 in the L buffer of the last iteration, whose values are
+  // used up once the increments are formed and which the next expansion writes
+  // over: as many tiles as fit (135 KB each: a fifth of all tiles at the 64^3 and 128^3
+  // workloads, where 8% and 2% are live; every tile at 96^3 with 10007 frames). The rest
+  // is contracted again.
+  float* kept = pruned && !S ? (float*)(c->ws + (lnew ? y.L : y.L2)) : nullptr;
+  const int kept_cap = (int)std::min<int64_t>(
+      (int64_t)(L_bytes(&c->cfg, y.rows, y.ld_pix) / (sizeof(float) * kKeptFloats)), INT32_MAX);
+  int32_t* slot = pr ? (int32_t*)(c->ws + y.slot) : nullptr;
   if (pr && c->order_pending) {
     // the order the previous iteration found: frames, their arrays and the
     // per-frame state of the incremental bound follow it
@@ -1058,12 +1090,13 @@ int emc_iteration(emc_ctx* c, const float* grid_in, float* grid_out, emc_iter_st
                            bound_div(&c->cfg),
                            nmt, y.ld_data, c->cfg.n_data, live, s));
       CU(launch_tile_list(live, (int)nmt, (int)nnt, 8, tlist, tcount, (int32_t*)(c->ws + y.sortH),
-                            s));
+                            s, kept ? slot : nullptr));
       kernels += 10;  // a tile list is three launches
     }
     CU(launch_tc_pass1(p3, c->cfg.precision, bias, y.rows, Kp, y.ld_data, c->cfg.n_data, y.ld_pix,
                        pm, ps, S, S + y.rows * y.ld_data, nullptr, nullptr, c->status, s,
-                       pruned ? tlist : nullptr, pruned ? tcount : nullptr, c->tcctl));
+                       pruned ? tlist : nullptr, pruned ? tcount : nullptr, c->tcctl, kept,
+                       kept_cap));
     // the merge also keeps, for the next iteration's incremental bound, every
     // contracted tile's maximum (plus 1/64) in Ub, the frames' largest maxima and best tiles
     CU(launch_lse_merge(pm, ps, nmt, y.ld_data, c->cfg.n_data, lm, ls, 0, 0, c->status, s, cn_p,
@@ -1098,14 +1131,33 @@ int emc_iteration(emc_ctx* c, const float* grid_in, float* grid_out, emc_iter_st
     // (the chunk's count sits after pass 1's in the same block, which the stats read)
     int32_t* tlist = pr ? (int32_t*)(c->ws + y.tlist) : nullptr;
     int32_t* tcount = pr ? (int32_t*)(c->ws + y.tcount) + 16 : nullptr;
-    if (pruned && !S) {  // recomputed pass 2: the live tiles of this chunk's rows
-      CU(launch_tile_list(live + (r0 / 128) * nnt, (int)(crows / 128), (int)nnt, 8, tlist, tcount,
-                          (int32_t*)(c->ws + y.sortH), s));
-      kernels += 3;
+    FrameView fv{};
+    fv.K = Kp;
+    fv.cn = cn_p;
+    fv.invn = y.invn_p ? (const float*)(c->ws + y.invn_p) : nullptr;
+    if (pruned && S) fv.tile_live = live + (r0 / 128) * nnt;
+    if (kept) {
+      // this chunk's live tiles: the kept ones, and those beyond the kept scores' room, whose
+      // scores are contracted again (both lists have room for every tile)
+      const int64_t t0 = (r0 / 128) * nnt;
+      const bool all = kept_cap >= nmt * nnt;
+      int32_t* klist = (int32_t*)(c->ws + y.klist);
+      CU(launch_tile_list(live + t0, (int)(crows / 128), (int)nnt, 8, klist, tcount,
+                          (int32_t*)(c->ws + y.sortH), s, nullptr,
+                          TilePick{slot + t0, kept_cap, true}));
+      if (!all)
+        CU(launch_tile_list(live + t0, (int)(crows / 128), (int)nnt, 8, tlist, tcount + 8,
+                            (int32_t*)(c->ws + y.sortH), s, nullptr,
+                            TilePick{slot + t0, kept_cap, false}));
+      kernels += all ? 3 : 7;
+      fv.kept = kept;
+      fv.slot = slot + t0;
+      fv.kept_list = klist;
+      fv.kept_count = tcount;
+      fv.kept_all = all;
+      fv.tile_list = tlist;
+      fv.tile_count = tcount + 8;
     }
-    FrameView fv{Kp, cn_p, y.invn_p ? (const float*)(c->ws + y.invn_p) : nullptr,
-                 pruned && S ? live + (r0 / 128) * nnt : nullptr,
-                 pruned && !S ? tlist : nullptr, pruned && !S ? tcount : nullptr};
     if ((st = do_normalize(c, L, y.rows, r0, bias + r0, nr, lm, ls, Sc, y.rows, Sr, P, crows, s,
                            c->flu_B ? c->flu_B + r0 : nullptr, kbf, pr ? &fv : nullptr)))
       return st;

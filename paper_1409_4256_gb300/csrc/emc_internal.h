@@ -223,6 +223,15 @@ cudaError_t launch_normalize_scores(const float* S, int64_t ldS, const float* Sr
                                     int64_t ld_data, int64_t n_data, int precision, void* P,
                                     int64_t P_plane, cudaStream_t s, uint8_t* kb_flag = nullptr,
                                     const uint8_t* tile_live = nullptr);
+// Pass 2 from the kept scores of the listed tiles (codes mt * ld_data / 256 + nt of this
+// chunk's rows, their places in slot), after lse2, kb_flag (zeroed) and, for the
+// Poisson-fluence model (Bsum != NULL), den are set up as the other pass-2 forms set them up.
+cudaError_t launch_normalize_kept(const float* kept, const int32_t* slot, const int32_t* tile_list,
+                                  const int32_t* tile_count, const double* lse_m,
+                                  const double* lse_s, float2* lse2, int64_t rows, int64_t nrot,
+                                  int64_t ld_data, int64_t n_data, int precision, void* P,
+                                  int64_t P_plane, const double* shift, const double* Bsum,
+                                  const float* invn, float* den, uint8_t* kb_flag, cudaStream_t s);
 cudaError_t launch_loglik_sum(const double* lse_m, const double* lse_s, int64_t n_data,
                               double* out, cudaStream_t s);
 
@@ -243,7 +252,12 @@ cudaError_t launch_tc_pass1(const Planes& L, int precision, const double* bias, 
                             double* part_m, float* part_s, float* S, float* Sref,
                             const float4* gk, const float4* gsc, int32_t* status,
                             cudaStream_t s, const int32_t* tile_list = nullptr,
-                            const int32_t* tile_count = nullptr, TcCtl ctl = TcCtl{});
+                            const int32_t* tile_count = nullptr, TcCtl ctl = TcCtl{},
+                            float* kept = nullptr, int kept_cap = 0);
+// Scores a listed pass 1 keeps (kept): tile t of the list, t < kept_cap, at kept + t
+// kKeptFloats: 256 frames x 128 rows relative to the 32-row group maxima, which
+// follow as [4][256].
+constexpr int64_t kKeptFloats = 256 * 128 + 4 * 256;
 // lse2: scratch float2[ld_data] for lse_k split into a 1/8-grid part and a rest.
 // Bsum != NULL: Poisson-fluence model -- shift[ld_data] is added back to lse,
 // the planes receive BF16 hi + lo of P B_j invn[k] and den[rows] = sum_k P_jk
@@ -257,7 +271,9 @@ cudaError_t launch_tc_normalize(const Planes& L, int precision, const double* bi
                                 const double* shift = nullptr, const double* Bsum = nullptr,
                                 const float* invn = nullptr, float* den = nullptr,
                                 uint8_t* kb_flag = nullptr, const int32_t* tile_list = nullptr,
-                                const int32_t* tile_count = nullptr, TcCtl ctl = TcCtl{});
+                                const int32_t* tile_count = nullptr, TcCtl ctl = TcCtl{},
+                                bool prepared = false);  // lse2, kb_flag and den are: see
+                                                         // launch_normalize_kept
 // P planes: hi + lo (BF16 split, FP16 split) or hi only (BF16); FP16 planes
 // carry the scale 2^14. den NULL: not written.
 // kb_cnt, kb_list (optional, from launch_kb_lists): contract only the listed
@@ -375,8 +391,16 @@ cudaError_t launch_lse_values(const double* m, const double* sm, int64_t n, doub
 // the live tiles (flags live[mt][nt]) as codes mt * n_ntiles + nt in raster
 // order (groups of `group` row tiles) into list, their number into *count;
 // scratch: tile_list_scratch_entries int32
+// slot_out (optional): slot_out[mt * n_ntiles + nt] = the tile's position in the list.
+// pick.slot (optional): list only the live tiles with slot < cap (kept), or only the others.
+struct TilePick {
+  const int32_t* slot;
+  int cap;
+  bool kept;
+};
 cudaError_t launch_tile_list(const uint8_t* live, int n_mtiles, int n_ntiles, int group,
-                             int32_t* list, int32_t* count, int32_t* scratch, cudaStream_t s);
+                             int32_t* list, int32_t* count, int32_t* scratch, cudaStream_t s,
+                             int32_t* slot_out = nullptr, TilePick pick = TilePick{});
 int64_t tile_list_scratch_entries(int64_t n_mtiles, int64_t n_ntiles);
 // entries of the histogram scratch H (int32) of launch_sort_frames; off needs one more (int64)
 int64_t sort_scratch_entries(int64_t n_data, int nbins);

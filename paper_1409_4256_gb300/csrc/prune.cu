@@ -57,13 +57,18 @@ __device__ __forceinline__ int raster_code(int t, int n_mtiles, int n_ntiles, in
 }
 
 // live flags of the thread's positions as bits; their number
+// (pick.slot: of the live tiles only those whose kept scores have a place, or
+// only the others)
 __device__ __forceinline__ unsigned list_bits(const uint8_t* __restrict__ live, int n_mtiles,
-                                              int n_ntiles, int group, int T, int t0) {
+                                              int n_ntiles, int group, int T, int t0,
+                                              const TilePick& pick) {
   unsigned bits = 0;
 #pragma unroll
   for (int q = 0; q < kListItems; q++) {
     const int t = t0 + q;
-    if (t < T && live[raster_code(t, n_mtiles, n_ntiles, group)]) bits |= 1u << q;
+    if (t >= T) break;
+    const int code = raster_code(t, n_mtiles, n_ntiles, group);
+    if (live[code] && (!pick.slot || (pick.slot[code] < pick.cap) == pick.kept)) bits |= 1u << q;
   }
   return bits;
 }
@@ -108,10 +113,10 @@ __device__ __forceinline__ int block_exclusive(int v, int* sh) {
 
 __global__ void __launch_bounds__(kListThreads)
     tile_count_kernel(const uint8_t* __restrict__ live, int n_mtiles, int n_ntiles, int group,
-                      int T, int32_t* __restrict__ cnt) {
+                      int T, TilePick pick, int32_t* __restrict__ cnt) {
   __shared__ int sh[32];
   const int t0 = blockIdx.x * kListChunk + threadIdx.x * kListItems;
-  const int n = __popc(list_bits(live, n_mtiles, n_ntiles, group, T, t0));
+  const int n = __popc(list_bits(live, n_mtiles, n_ntiles, group, T, t0, pick));
   const int tot = block_sum(n, sh);
   if (threadIdx.x == 0) cnt[blockIdx.x] = tot;
 }
@@ -134,15 +139,18 @@ __global__ void __launch_bounds__(kListThreads)
 
 __global__ void __launch_bounds__(kListThreads)
     tile_write_kernel(const uint8_t* __restrict__ live, int n_mtiles, int n_ntiles, int group,
-                      int T, const int32_t* __restrict__ off, int32_t* __restrict__ list) {
+                      int T, TilePick pick, const int32_t* __restrict__ off,
+                      int32_t* __restrict__ list, int32_t* __restrict__ slot_out) {
   __shared__ int sh[32];
   const int t0 = blockIdx.x * kListChunk + threadIdx.x * kListItems;
-  unsigned bits = list_bits(live, n_mtiles, n_ntiles, group, T, t0);
+  unsigned bits = list_bits(live, n_mtiles, n_ntiles, group, T, t0, pick);
   int pos = off[blockIdx.x] + block_exclusive(__popc(bits), sh);
   while (bits) {
     const int q = __ffs(bits) - 1;
     bits &= bits - 1;
-    list[pos++] = raster_code(t0 + q, n_mtiles, n_ntiles, group);
+    const int code = raster_code(t0 + q, n_mtiles, n_ntiles, group);
+    if (slot_out) slot_out[code] = pos;
+    list[pos++] = code;
   }
 }
 
@@ -239,12 +247,14 @@ __global__ void unpermute_lse_kernel(const int32_t* __restrict__ perm, int64_t n
 }
 
 cudaError_t launch_tile_list(const uint8_t* live, int n_mtiles, int n_ntiles, int group,
-                             int32_t* list, int32_t* count, int32_t* scratch, cudaStream_t s) {
+                             int32_t* list, int32_t* count, int32_t* scratch, cudaStream_t s,
+                             int32_t* slot_out, TilePick pick) {
   const int T = n_mtiles * n_ntiles;
   const int nb = (T + kListChunk - 1) / kListChunk;
-  tile_count_kernel<<<nb, kListThreads, 0, s>>>(live, n_mtiles, n_ntiles, group, T, scratch);
+  tile_count_kernel<<<nb, kListThreads, 0, s>>>(live, n_mtiles, n_ntiles, group, T, pick, scratch);
   tile_scan_kernel<<<1, kListThreads, 0, s>>>(scratch, nb, count);
-  tile_write_kernel<<<nb, kListThreads, 0, s>>>(live, n_mtiles, n_ntiles, group, T, scratch, list);
+  tile_write_kernel<<<nb, kListThreads, 0, s>>>(live, n_mtiles, n_ntiles, group, T, pick, scratch, list,
+                                               slot_out);
   return cudaGetLastError();
 }
 

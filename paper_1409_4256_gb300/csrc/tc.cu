@@ -115,6 +115,8 @@ struct TcArgs {
   float* part_s;
   float* S;                // pass 1, optional: shifted scores, frame-major [ld_data][rows]
   float* Sref;             // pass 1, optional: 32-row group maxima [rows / 32][ld_data]
+  float* kept;             // pass 1 over a list, optional: the same by tile (kKeptFloats)
+  int kept_cap;            // ... of the list's first tiles
   const float4* gk;        // Gaussian pass 1: per frame (c_k hi, c_k lo, 2 sigma^2 / A_k, 0)
   const float4* gsc;       // Gaussian pass 1: scales (s, 1/s^2, 0, 0)
   uint16_t* P;             // normalize: planes [2][rows][ld_data]
@@ -524,6 +526,12 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
             for (int i = 0; i < 32; i++) Scol[(int64_t)i * a.rows] = xl[i];
             a.Sref[((int64_t)mt * 4 + q) * a.ld_data + k0 + lane] = mcol;
+          } else if (a.kept && t < a.kept_cap) {
+            float* Kt = a.kept + t * kKeptFloats;
+            float* Kcol = Kt + col0 * BM + r_in;
+#pragma unroll
+            for (int i = 0; i < 32; i++) Kcol[i * BM] = xl[i];
+            Kt[BN * BM + q * BN + col0 + lane] = mcol;
           }
           const float scol = warp_transpose_reduce<false>(v, lane);
           scratch[q * BN + col0 + lane] = make_float2(mcol, scol);
@@ -971,7 +979,7 @@ cudaError_t launch_tc_pass1(const Planes& L, int precision, const double* bias, 
                             double* part_m, float* part_s, float* S, float* Sref,
                             const float4* gk, const float4* gsc, int32_t* status,
                             cudaStream_t s, const int32_t* tile_list,
-                            const int32_t* tile_count, TcCtl ctl) {
+                            const int32_t* tile_count, TcCtl ctl, float* kept, int kept_cap) {
   const bool gauss = gk != nullptr;
   const int nterms = gauss ? 3 : score_planes(precision);
   const bool f16 = gauss || precision == EMC_PREC_FP16_SPLIT;
@@ -988,6 +996,8 @@ cudaError_t launch_tc_pass1(const Planes& L, int precision, const double* bias, 
   a.part_s = part_s;
   a.S = S;
   a.Sref = Sref;
+  a.kept = tile_list ? kept : nullptr;
+  a.kept_cap = kept_cap;
   a.gk = gk;
   a.gsc = gsc;
   a.tile_list = tile_list;
@@ -1007,16 +1017,17 @@ cudaError_t launch_tc_normalize(const Planes& L, int precision, const double* bi
                                 float2* lse2, Planes P, int32_t* status, cudaStream_t s,
                                 const double* shift, const double* Bsum, const float* invn,
                                 float* den, uint8_t* kb_flag, const int32_t* tile_list,
-                                const int32_t* tile_count, TcCtl ctl) {
-  cudaError_t e = launch_lse_split(lse_m, lse_s, n_data, ld_data, lse2, s, shift);
+                                const int32_t* tile_count, TcCtl ctl, bool prepared) {
+  cudaError_t e = cudaSuccess;
+  if (!prepared) e = launch_lse_split(lse_m, lse_s, n_data, ld_data, lse2, s, shift);
   if (e != cudaSuccess) return e;
-  if (kb_flag) {
+  if (kb_flag && !prepared) {
     e = cudaMemsetAsync(kb_flag, 0, (size_t)(rows / BM) * (ld_data / 64), s);
     if (e != cudaSuccess) return e;
   }
   if (Bsum) {
     if (!invn || !den || precision == EMC_PREC_FP16_SPLIT) return cudaErrorInvalidValue;
-    e = cudaMemsetAsync(den, 0, sizeof(float) * rows, s);
+    if (!prepared) e = cudaMemsetAsync(den, 0, sizeof(float) * rows, s);
     if (e != cudaSuccess) return e;
   }
   const int nterms = score_planes(precision);
