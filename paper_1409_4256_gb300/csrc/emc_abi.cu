@@ -19,8 +19,8 @@ int64_t round_up(int64_t x, int64_t m) { return (x + m - 1) / m * m; }
 size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 struct Layout {
-  int64_t ld_pix, ld_data, rows, chunk_rows, part_tiles;
-  size_t qh, ql, quat, rot, logw, Kb, status, L, bias, lse_m, lse_s, lse2, part_m, part_s, S, P,
+  int64_t ld_pix, ld_data, rows, chunk_rows, num_rows, part_tiles;
+  size_t qh, ql, logw, Kb, status, L, bias, lse_m, lse_s, lse2, part_m, part_s, S, P,
       Num, den, gnum, gden, scalar, fbin, finv, cand, ccnt, coff, cent, Sc, Pc, lsec, gk, gauss,
       Kb2, skcnt, skoff, skent, dupsrc, duprank, pixmax, fcn, finvn, fB, kbflag, kbcnt, kblist,
       Kp, perm, perm2, iperm, nsum, nsum_p, cn_p, invn_p, best, lsem_s, lses_s, live, tlist, slot, klist,
@@ -131,8 +131,6 @@ Layout make_layout(const emc_config* c) {
   y.cgqf = take(sizeof(float4) * (c->n_pix + 1));
   y.qi = take(sizeof(int4) * y.ld_pix);
   y.qlo = take(sizeof(float4) * y.ld_pix);
-  y.quat = take(sizeof(double) * 4 * c->n_rot);
-  y.rot = take(sizeof(RotDF) * c->n_rot);
   y.rotfx = take(sizeof(RotFX) * c->n_rot);
   y.epart = take(sizeof(double) * (size_t)expand_tile_slices(y.ld_pix) * y.rows);
   // the model in the cell layout of the expansions' gathers (32 B a voxel;
@@ -151,9 +149,9 @@ Layout make_layout(const emc_config* c) {
   y.S = (c->flags & EMC_FLAG_STORE_SCORES) ? take(score_bytes(y.rows, y.ld_data)) : 0;
   y.P = take(P_bytes(c, y.chunk_rows, y.ld_data));
   // the sparse update (n_cand > 0) writes Num and den for every rotation at once
-  const int64_t num_rows = c->n_cand > 0 ? y.rows : y.chunk_rows;
-  y.Num = take(sizeof(float) * (size_t)num_rows * y.ld_pix);
-  y.den = take(sizeof(float) * num_rows);
+  y.num_rows = c->n_cand > 0 ? y.rows : y.chunk_rows;
+  y.Num = take(sizeof(float) * (size_t)y.num_rows * y.ld_pix);
+  y.den = take(sizeof(float) * y.num_rows);
   y.gnum = take(sizeof(double) * nvox);
   y.gden = take(sizeof(double) * nvox);
   y.scalar = take(256);
@@ -257,8 +255,6 @@ struct emc_ctx {
   char* ws;
   size_t ws_bytes;
   Geom geom;
-  double* quat;
-  const RotDF* rot;
   double* logw;
   uint16_t* Kb;
   int32_t* status;
@@ -434,9 +430,7 @@ static int ctx_create(const emc_config* cfg, const double* q, const double* quat
   }
   std::vector<double> lw(cfg->n_rot);
   for (int64_t j = 0; j < cfg->n_rot; j++) lw[j] = log(weight[j]);
-  std::vector<RotDF> rot(cfg->n_rot);
-  for (int64_t j = 0; j < cfg->n_rot; j++) quat_to_rot_df(quat + 4 * j, &rot[j]);
-  // the same matrices in fixed point: hi = round(R 2^20), lo = R - hi 2^-20
+  // the rotation matrices in fixed point: hi = round(R 2^20), lo = R - hi 2^-20
   std::vector<RotFX> rotfx(cfg->n_rot);
   for (int64_t j = 0; j < cfg->n_rot; j++) {
     double R[9];
@@ -505,8 +499,6 @@ static int ctx_create(const emc_config* cfg, const double* q, const double* quat
     }
     c->geom.interior = sqrt(r2max) < 0.5 * cfg->N - 1.0 - 1e-4 ? 1 : 0;
   }
-  c->quat = (double*)(c->ws + y.quat);
-  c->rot = (const RotDF*)(c->ws + y.rot);
   c->logw = (double*)(c->ws + y.logw);
   c->Kb = (uint16_t*)(c->ws + y.Kb);
   c->status = (int32_t*)(c->ws + y.status);
@@ -544,12 +536,8 @@ static int ctx_create(const emc_config* cfg, const double* q, const double* quat
                         cudaMemcpyHostToDevice, s) == cudaSuccess;
   ok &= cudaMemcpyAsync(c->ws + y.cgql, gql.data(), sizeof(float4) * cfg->n_pix,
                         cudaMemcpyHostToDevice, s) == cudaSuccess;
-  ok &= cudaMemcpyAsync(c->quat, quat, sizeof(double) * 4 * cfg->n_rot, cudaMemcpyHostToDevice,
-                        s) == cudaSuccess;
   ok &= cudaMemcpyAsync(c->logw, lw.data(), sizeof(double) * cfg->n_rot, cudaMemcpyHostToDevice,
                         s) == cudaSuccess;
-  ok &= cudaMemcpyAsync(c->ws + y.rot, rot.data(), sizeof(RotDF) * cfg->n_rot,
-                        cudaMemcpyHostToDevice, s) == cudaSuccess;
   ok &= cudaMemcpyAsync(c->ws + y.rotfx, rotfx.data(), sizeof(RotFX) * cfg->n_rot,
                         cudaMemcpyHostToDevice, s) == cudaSuccess;
   ok &= launch_fixed_geometry((const float4*)(c->ws + y.qh), (const float4*)(c->ws + y.ql),
@@ -700,18 +688,20 @@ int do_expand(emc_ctx* c, const float* grid, int64_t rot0, int64_t nrot, void* L
                           Lold ? (float*)(c->ws + y.bpm) : nullptr, c->status, s));
     return EMC_OK;
   }
+  const RotFX* rot = (const RotFX*)(c->ws + y.rotfx) + rot0;
   if (is_flu(&c->cfg)) {
-    CU(launch_expand_flu(c->geom, grid, g4, c->rot + rot0, c->logw + rot0, nrot, rows,
-                         c->cfg.precision, (float)c->cfg.w_floor, c->flu_c, p, bias,
-                         c->flu_B + rot0, c->status, s));
+    // (W takes the slice buffer of the M-step, which runs later)
+    CU(launch_expand_flu(c->geom, grid, g4, rot, c->logw + rot0, nrot, rows,
+                         (float)c->cfg.w_floor, c->flu_c, p, bias, c->flu_B + rot0,
+                         (double*)(c->ws + y.epart), (float*)(c->ws + y.Num), y.num_rows, Lold,
+                         Lold ? (uint16_t*)(c->ws + y.Dd) : nullptr, y.ntp,
+                         Lold ? (float*)(c->ws + y.bpm) : nullptr, c->status, s));
     return EMC_OK;
   }
-  if (g)
-    CU(launch_gauss_scales(grid, (int64_t)c->cfg.N * c->cfg.N * c->cfg.N, c->gmax, c->nmax,
-                           c->gsc, c->status, s));
-  CU(launch_expand(c->geom, grid, g4, c->rot + rot0, c->logw + rot0, nrot, rows,
-                   c->cfg.precision, (float)c->cfg.w_floor, p, bias, g ? c->gsc : nullptr,
-                   c->cfg.sigma, c->status, s));
+  CU(launch_gauss_scales(grid, (int64_t)c->cfg.N * c->cfg.N * c->cfg.N, c->gmax, c->nmax, c->gsc,
+                         c->status, s));
+  CU(launch_expand_gauss(c->geom, grid, g4, rot, c->logw + rot0, nrot, rows, p, bias,
+                         (double*)(c->ws + y.epart), c->gsc, c->cfg.sigma, c->status, s));
   return EMC_OK;
 }
 
@@ -997,21 +987,21 @@ int emc_iteration(emc_ctx* c, const float* grid_in, float* grid_out, emc_iter_st
   bool delta = false;  // the incremental bound ran
 
   // the incremental bound runs when the last iteration left its tile bounds;
-  // for the Poisson model the expansion computes its increments on the way
+  // the expansion forms the increments on the way
   const bool pruned = pr && c->perm_valid;
   delta = pruned && c->ub_valid;
   const void* Lold = delta ? c->ws + (lnew ? y.L : y.L2) : nullptr;
   const double* bold = delta ? (const double*)(c->ws + (lnew ? y.bias : y.bias2)) : nullptr;
-  const bool fused = delta && !is_flu(&c->cfg);
   if (stats) CU(cudaEventRecord(c->ev[0], s));
   c->collected = false;
   if (c->collecting) CU(cudaMemsetAsync(c->col.count, 0, sizeof(unsigned long long), s));
-  if ((st = do_expand(c, grid_in, 0, n_rot, L, bias, s, fused ? Lold : nullptr,
-                      fused ? bold : nullptr)))
-    return st;
-  // Gaussian: grid maximum and scales first; Poisson: the row tiles and the bias
-  // sums; the cell layout of the model first where it is used
-  kernels += (is_gauss(&c->cfg) ? 3 : (is_flu(&c->cfg) ? 1 : 2)) +
+  if ((st = do_expand(c, grid_in, 0, n_rot, L, bias, s, Lold, bold))) return st;
+  // the row tiles and the bias sums (Gaussian: grid maximum and scales first;
+  // Poisson fluence: the split, and all three per block of slice rows); the cell
+  // layout of the model first where it is used
+  kernels += (is_gauss(&c->cfg)
+                  ? 4
+                  : (is_flu(&c->cfg) ? 3 * (int)((y.rows + y.num_rows - 1) / y.num_rows) : 2)) +
              ((y.g4 && c->geom.interior) ? 1 : 0);
   if (stats) CU(cudaEventRecord(c->ev[1], s));
   float* S = (c->cfg.flags & EMC_FLAG_STORE_SCORES) ? (float*)(c->ws + y.S) : nullptr;
@@ -1061,12 +1051,6 @@ int emc_iteration(emc_ctx* c, const float* grid_in, float* grid_out, emc_iter_st
       const float* bpm = (const float*)(c->ws + y.bpm);
       if (delta) {
         const int f16 = c->cfg.precision == EMC_PREC_FP16_SPLIT ? 1 : 0;
-        if (!fused) {  // Poisson-fluence: the increments from both L in a pass of their own
-          CU(launch_delta_planes((const uint16_t*)Lold, (const uint16_t*)L, y.rows * y.ld_pix,
-                                 y.ld_pix, n_rot, bold, bias, y.ntp, (uint16_t*)(c->ws + y.Dd),
-                                 (float*)bpm, f16, s));
-          kernels++;
-        }
         Planes pd{c->ws + y.Dd, 3 * y.ntp * y.ld_pix, y.ld_pix};
         CU(launch_tc_store(pd, 3 * y.ntp, Kp, y.ld_data, y.ld_pix, (float*)Cd, f16, c->status, s,
                            c->tcctl));

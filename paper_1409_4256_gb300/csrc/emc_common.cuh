@@ -47,10 +47,8 @@ __device__ __forceinline__ float2 add2(float2 a, float2 b) {
 }
 
 // ---------------------------------------------------------------------------
-// Double-float ("f2") arithmetic: value = h + l with |l| <= ulp(h)/2.
-// Rotated pixel coordinates need ~1e-8 voxel accuracy (the scores of Eq. 2.3
-// react to log W at the 1e-7 level), which plain FP32 (ulp(64) = 7.6e-6)
-// cannot give; FP64 is rare on this part, so pairs of FP32 are used instead.
+// Double-float ("f2") arithmetic: value = h + l with |l| <= ulp(h)/2, where an
+// FP32 sum is not enough and FP64 is rare on this part.
 // ---------------------------------------------------------------------------
 struct f2 {
   float h, l;
@@ -62,31 +60,6 @@ __device__ __forceinline__ f2 two_sum(float a, float b) {
   float e = (a - (s - bb)) + (b - bb);
   return {s, e};
 }
-__device__ __forceinline__ f2 fast_two_sum(float a, float b) {  // |a| >= |b|
-  float s = a + b;
-  float e = b - (s - a);
-  return {s, e};
-}
-__device__ __forceinline__ f2 two_prod(float a, float b) {
-  float p = a * b;
-  float e = fmaf(a, b, -p);
-  return {p, e};
-}
-__device__ __forceinline__ f2 df_mul(f2 a, f2 b) {
-  f2 p = two_prod(a.h, b.h);
-  p.l = fmaf(a.h, b.l, fmaf(a.l, b.h, p.l));
-  return fast_two_sum(p.h, p.l);
-}
-__device__ __forceinline__ f2 df_add(f2 a, f2 b) {
-  f2 s = two_sum(a.h, b.h);
-  s.l += a.l + b.l;
-  return fast_two_sum(s.h, s.l);
-}
-
-// Rotation R (row-major 3x3) as double-float pairs.
-struct RotDF {
-  f2 r[9];
-};
 
 // Hamilton rotation matrix of a unit quaternion (w, x, y, z), in FP64.
 __host__ __device__ __forceinline__ void quat_to_rot(const double* q, double* R) {
@@ -96,58 +69,14 @@ __host__ __device__ __forceinline__ void quat_to_rot(const double* q, double* R)
   R[6] = 2 * (x * z - w * y);     R[7] = 2 * (y * z + w * x);     R[8] = 1 - 2 * (x * x + y * y);
 }
 
-// The same, split into double-float pairs.
-__host__ __device__ __forceinline__ void quat_to_rot_df(const double* q, RotDF* out) {
-  double R[9];
-  quat_to_rot(q, R);
-  for (int t = 0; t < 9; t++) {
-    float h = (float)R[t];
-    out->r[t].h = h;
-    out->r[t].l = (float)(R[t] - (double)h);
-  }
-}
-
 // Grid coordinate p = R q + N/2 of one pixel, split into the integer corner
-// f (floor) and the fraction t in [0, 1], both accurate to ~1e-9 voxel.
-// Compensated dot product: with R = Rh + Rl and q = qh + ql,
-//   p = N/2 + sum_b Rh_b qh_b + sum_b (Rh_b ql_b + Rl_b qh_b) + O(2^-40),
-// the products Rh_b qh_b are split exactly (FMA), summed onto N/2 with exact
-// two-sums, and every remainder is gathered in one small FP32 term.
-__device__ __forceinline__ void rotate_to_grid(const RotDF& R, float4 qh, float4 ql, float half_n,
-                                               int* f, float* t) {
-  const float qhv[3] = {qh.x, qh.y, qh.z}, qlv[3] = {ql.x, ql.y, ql.z};
-#pragma unroll
-  for (int a = 0; a < 3; a++) {
-    float S = half_n, L = 0.f;
-#pragma unroll
-    for (int b = 0; b < 3; b++) {
-      const f2 r = R.r[3 * a + b];
-      const f2 p = two_prod(r.h, qhv[b]);
-      const f2 s = two_sum(S, p.h);
-      S = s.h;
-      L += s.l + fmaf(r.h, qlv[b], fmaf(r.l, qhv[b], p.l));
-    }
-    float fl = floorf(S);
-    float fr = (S - fl) + L;  // S - fl is exact
-    if (fr < 0.f) {
-      fl -= 1.f;
-      fr += 1.f;
-    } else if (fr >= 1.f) {
-      fl += 1.f;
-      fr -= 1.f;
-    }
-    f[a] = (int)fl;
-    t[a] = fminf(fmaxf(fr, 0.f), 1.f);
-  }
-}
-
-// The same grid point in fixed point. With q = qi 2^-12 + qlo (qi integer,
+// f (floor) and the fraction t in [0, 1], in fixed point. With q = qi 2^-12 + qlo (qi integer,
 // |qlo| <= 2^-13) and R = Rh 2^-20 + Rl (Rh integer, |Rl| <= 2^-21),
 //   p = N/2 + sum_b Rh_b qi_b 2^-32 + sum_b (Rh_b 2^-20 qlo_b + Rl_b qi_b 2^-12)
 // up to |Rl qlo| < 2^-34: the first sum is exact in 64-bit integers (its high
 // word the floor, its low word the fraction to 2^-32), the small terms
 // (|.| < 1e-3) take six FP32 FMAs. Rhf = Rh 2^-20 and qhf = qi 2^-12 as FP32
-// (exact). Same accuracy as rotate_to_grid at a third of its instructions.
+// (exact). Error ~1e-10 voxel.
 __device__ __forceinline__ void rotate_fx(const int* Rh, const float* Rhf, const float* Rl,
                                           int4 qi, float4 qhf, float4 qlo, int N, int* f,
                                           float* t) {

@@ -9,7 +9,6 @@ namespace emc {
 
 // Rotation matrix R_j (row-major 3x3) as double-float pairs (h, l) of FP32,
 // computed once per context on the host in FP64.
-struct RotDF;
 
 // Rotation R_j in fixed point for the e-step: R = hi 2^-20 + lo (hi integer,
 // |lo| <= 2^-21), row-major 3x3.
@@ -71,13 +70,6 @@ cudaError_t launch_assign_duplicates(const int32_t* K, int64_t ld_k, int64_t n_d
                                      int16_t* fbin, int32_t* dup_src, int32_t* dup_rank,
                                      int32_t* status, cudaStream_t s);
 
-// gsc != NULL: Gaussian model (FP16 three-plane s W, bias log w - sum W^2 / 2 sigma^2)
-// g4 (may be NULL): the grid in the cell layout (launch_grid_cells)
-cudaError_t launch_expand(const Geom& g, const float* grid, const float4* g4, const RotDF* rot,
-                          const double* logw, int64_t nrot, int64_t rows, int precision,
-                          float w_floor, Planes L, double* bias, const float4* gsc, double sigma,
-                          int32_t* status, cudaStream_t s);
-
 // Poisson model: the e-step per row tile of 128 rotations (expand_tile.cu).
 // partial: scratch of expand_tile_slices(ld_pix) x rows doubles. With Lold
 // (the last iteration's L, same layout) it also writes the incremental bound's
@@ -97,13 +89,20 @@ cudaError_t launch_expand_tile(const Geom& g, const float* grid, const float4* g
 cudaError_t launch_fixed_geometry(const float4* qh, const float4* ql, int64_t ld_pix, int4* qi,
                                   float4* qlo, float4* qf, cudaStream_t s);
 
-// Poisson-fluence model: L = log(W / B_j) + c as the BF16 three-term split
-// (precision EMC_PREC_BF16_SPLIT only); bias = double[2][rows]: log w_j, then
-// B_j = sum_i W_ij; Bctx[row] = B_j too.
-cudaError_t launch_expand_flu(const Geom& g, const float* grid, const float4* g4, const RotDF* rot,
-                              const double* logw, int64_t nrot, int64_t rows, int precision,
-                              float w_floor, double c, Planes L, double* bias, double* Bctx,
-                              int32_t* status, cudaStream_t s);
+// Gaussian model: s W as three FP16 planes, bias log w - sum W^2 / 2 sigma^2.
+cudaError_t launch_expand_gauss(const Geom& g, const float* grid, const float4* g4,
+                                const RotFX* rot, const double* logw, int64_t nrot, int64_t rows,
+                                Planes L, double* bias, double* partial, const float4* gsc,
+                                double sigma, int32_t* status, cudaStream_t s);
+// Poisson-fluence model: L = log(W / B_j) + c as the BF16 three-term split;
+// bias = double[2][rows]: log w_j, then B_j = sum_i W_ij; Bctx[row] = B_j too.
+// W: scratch of W_rows (a multiple of 128) x ld_pix floats, used for W_rows
+// rotations at a time. Lold, D, ntp, bpm: as launch_expand_tile.
+cudaError_t launch_expand_flu(const Geom& g, const float* grid, const float4* g4, const RotFX* rot,
+                              const double* logw, int64_t nrot, int64_t rows, float w_floor,
+                              double c, Planes L, double* bias, double* Bctx, double* partial,
+                              float* W, int64_t W_rows, const void* Lold, uint16_t* D,
+                              int64_t ntp, float* bpm, int32_t* status, cudaStream_t s);
 // Per frame: cn[k] = c N_k, invn[k] = 1 / N_k (0 for empty and padding frames).
 cudaError_t launch_flu_frames(const int32_t* K, int64_t ld_k, int64_t n_data, int64_t n_pix,
                               int64_t ld_data, double c, double* cn, float* invn,
@@ -171,14 +170,6 @@ cudaError_t launch_lse_merge(const double* part_m, const float* part_s, int64_t 
                              int32_t* best = nullptr, float* Ub = nullptr, double* Mk = nullptr,
                              float* Ua = nullptr);
 // ---- incremental bound between consecutive iterations (prune.cu) ----
-// D ([3 ntp][ld_pix], BF16, or FP16 when f16) rows t and ntp + t: max over the
-// tile's valid rows of L1 - L0 and of L0 - L1 (BF16 split: three planes; f16,
-// the FP16 split's two; plane stride `plane`), rows 2 ntp + t: a bound of both
-// magnitudes; all rounded up; bpm[t], bpm[nt + t] = the same maxima of the
-// bias change (b1 - b0), rounded up.
-cudaError_t launch_delta_planes(const uint16_t* L0, const uint16_t* L1, int64_t plane,
-                                int64_t ld_pix, int64_t nrot, const double* b0, const double* b1,
-                                int64_t ntp, uint16_t* D, float* bpm, int f16, cudaStream_t s);
 // Ub += C+ + b+ + err, Lk from Mk, best and C- (C = D K^T, rows t, ntp + t and
 // 2 ntp + t, the last giving err);
 // cand[t][nt] where Ub >= Lk - 111 and the widening exceeds the hi-plane

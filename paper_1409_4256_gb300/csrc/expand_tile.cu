@@ -1,4 +1,4 @@
-// expand_tile.cu -- e-step of EMC (Eq. 2.9) for the Poisson model, a quarter or
+// expand_tile.cu -- e-step of EMC (Eq. 2.9), a quarter or
 // an eighth of a row tile of 128 rotations and a slice of 256 pixels per CTA
 // (small CTAs, so that small blocks of rotations fill the SMs and the last wave
 // leaves few of them idle).
@@ -7,8 +7,8 @@
 // turn, so the pixels' geometry stays in registers and the rotations come from
 // shared memory. Per (i, j): the grid point p = R_j q_i + N/2, the trilinear
 // value of the model (Eq. 2.8, tent weights), W_ij = max(W, w_floor) and
-// log W_ij in the layout of the chosen precision (as expand.cu), written two
-// pixels at a time. The row sums sum_i W_ij of the bias
+// log W_ij in the layout of the chosen precision, written two pixels at a time
+// (the Gaussian and Poisson-fluence models' own layouts below). The row sums sum_i W_ij of the bias
 //   bias_j = log w_j - sum_i W_ij
 // are kept as double-float pairs of FP32 (exact two-sums: FP64 is rare on
 // this part, and a per-row FP64 reduction kept its pipe 65% busy). A warp
@@ -28,7 +28,8 @@
 // rotations a CTA, scalar FP32 and two 16-byte gathers at the point of use (254
 // instructions per element); 225 us with two-pixel instructions, rounding without
 // the conversion pipe and 32 rotations a CTA (175); 215 us with 32-byte cells; 191 us
-// with the gathers a rotation ahead. 32^3 with 3240 rotations: 223 -> 39 us.
+// with the gathers a rotation ahead. 32^3 with 3240 rotations: 223 -> 39 us. The
+// Gaussian form: 260 us with one CTA per rotation in double-float arithmetic, 171 us here.
 //
 // With the last iteration's L (DELTA), the CTA also reads the previous planes
 // of its elements and keeps, per pixel, the largest rise and fall of the
@@ -36,6 +37,8 @@
 // incremental bound's increments D (prune.cu), rounded up to the operand type
 // of the frames, and their magnitude bound A (the rows 2 ntp + t).
 #include <cooperative_groups.h>
+
+#include <algorithm>
 
 #include "emc_common.cuh"
 #include "emc_internal.h"
@@ -178,6 +181,53 @@ __device__ __forceinline__ uint16_t round_up_operand(float x) {
   return *reinterpret_cast<uint16_t*>(&b);
 }
 
+// What the expansion writes, beside the precisions' layouts of log W:
+//  kOutGauss: s W as three FP16 planes (Gaussian model: no floor and no logarithm,
+//    s = 2^e = gsc->x), hi integral (rint below 2048, else the FP16 rounding, itself
+//    integral there), mid = fp16(s W - hi), lo = fp16(s W - hi - mid), the
+//    representation error below 2^-23 s^-1 W units; the row sums are of W^2;
+//  kOutW: W itself in FP32 (the Poisson-fluence model, whose split needs the row sum first).
+constexpr int kOutGauss = 4, kOutW = 5;
+
+// The rises dp and falls dm of a thread's two pixels over a tile's rows, gathered over the
+// cluster's CTAs by its first one, into rows t, ntp + t and 2 ntp + t of D,
+// rounded up to the operand type. rises: shared, one entry per thread.
+template <int PREC>
+__device__ __forceinline__ void write_increments(float (&dp)[2], float (&dm)[2], float4* rises,
+                                                 bool inside, int64_t t, int64_t i0,
+                                                 int64_t ld_pix, int64_t ntp,
+                                                 uint16_t* __restrict__ D) {
+  cg::cluster_group cluster = cg::this_cluster();
+  rises[threadIdx.x] = make_float4(dp[0], dp[1], dm[0], dm[1]);
+  cluster.sync();
+  if (cluster.block_rank() == 0 && inside) {
+    for (unsigned q = 1; q < cluster.num_blocks(); q++) {
+      const float4 o = cluster.map_shared_rank(rises, q)[threadIdx.x];
+      dp[0] = fmaxf(dp[0], o.x);
+      dp[1] = fmaxf(dp[1], o.y);
+      dm[0] = fmaxf(dm[0], o.z);
+      dm[1] = fmaxf(dm[1], o.w);
+    }
+    float a[2];
+#pragma unroll
+    for (int u = 0; u < 2; u++) {
+      // the sum of the planes rounded at most twice: 2^-23 |d| covers it
+      dp[u] += 2.0f * 1.1920929e-7f * fabsf(dp[u]);
+      dm[u] += 2.0f * 1.1920929e-7f * fabsf(dm[u]);
+      // bound of both rounded magnitudes (BF16 rounding up: at most 2^-7 relative)
+      a[u] = fmaxf(fabsf(dp[u]), fabsf(dm[u])) * 1.0078125f;
+    }
+    const uint16_t p0 = round_up_operand<PREC>(dp[0]), p1 = round_up_operand<PREC>(dp[1]);
+    const uint16_t m0 = round_up_operand<PREC>(dm[0]), m1 = round_up_operand<PREC>(dm[1]);
+    const uint16_t a0 = round_up_operand<PREC>(a[0]), a1 = round_up_operand<PREC>(a[1]);
+    *reinterpret_cast<uint32_t*>(D + t * ld_pix + i0) = (uint32_t)p0 | ((uint32_t)p1 << 16);
+    *reinterpret_cast<uint32_t*>(D + (ntp + t) * ld_pix + i0) = (uint32_t)m0 | ((uint32_t)m1 << 16);
+    *reinterpret_cast<uint32_t*>(D + (2 * ntp + t) * ld_pix + i0) =
+        (uint32_t)a0 | ((uint32_t)a1 << 16);
+  }
+  cluster.sync();  // no CTA leaves while its rises may be read
+}
+
 // RPC rotations of a tile per CTA; with DELTA the tile's 128 / RPC CTAs are a
 // cluster, whose first one gathers the others' rises and falls.
 template <int PREC, bool INTERIOR, bool DELTA, int RPC>
@@ -188,7 +238,7 @@ __global__ void __launch_bounds__(kTThreads, 6)
                        const RotFX* __restrict__ rot, int64_t nrot, int64_t rows, float w_floor,
                        void* __restrict__ Lbase, int64_t ps, double* __restrict__ partial,
                        const void* __restrict__ Lold, uint16_t* __restrict__ D, int64_t ntp,
-                       unsigned slices, int32_t* status) {
+                       unsigned slices, const float4* __restrict__ gsc, int32_t* status) {
   __shared__ RowFX R[RPC];
   __shared__ float2 rsum[kTThreads / 32][RPC];
   // eight rows of every lane's pair, rows padded to 33 so that the transposed
@@ -237,6 +287,7 @@ __global__ void __launch_bounds__(kTThreads, 6)
   __syncthreads();
   float dp[2] = {-INFINITY, -INFINITY}, dm[2] = {-INFINITY, -INFINITY};
   int bad = 0, nonfinite = 0;
+  const float gs = PREC == kOutGauss ? gsc->x : 1.f;
   // Row r + 1's grid points are formed and its voxels asked for before row r's
   // values are used: the gathers' latency is what the loop would wait for.
   float tt[2][3];
@@ -268,8 +319,9 @@ __global__ void __launch_bounds__(kTThreads, 6)
       if (vrow && qi[u].w != 0) {  // w: 1 pixel, 2 duplicate column, 0 padding / ones
         nonfinite |= !(fabsf(W2[u]) <= 3.4e38f);  // a NaN or infinite voxel of the model
         const float W = fmaxf(W2[u], w_floor);
-        if (qi[u].w == 1) ws[u] = W;  // duplicate columns repeat a pixel: not summed
-        L[u] = logf(W);
+        // duplicate columns repeat a pixel: not summed
+        if (qi[u].w == 1) ws[u] = PREC == kOutGauss ? W * W : W;
+        L[u] = PREC == kOutGauss ? W * gs : (PREC == kOutW ? W : logf(W));
       }
     }
     const f2 pair = two_sum(ws[0], ws[1]);  // row sum of the pair as s + se
@@ -277,7 +329,21 @@ __global__ void __launch_bounds__(kTThreads, 6)
     if (inside && row < rows) {
       const int64_t o = row * ld_pix + i0;
       // DELTA: the change of the represented value (the planes' sum) of each element
-      if (PREC == EMC_PREC_FP32) {
+      if (PREC == kOutGauss) {
+        uint16_t h[2], m[2], l[2];
+#pragma unroll
+        for (int u = 0; u < 2; u++) {
+          const float hi = L[u] < 2048.f ? round_to(L[u], 1.f) : fp16_val(fp16_bits(L[u]));
+          const float r = L[u] - hi;  // exact
+          h[u] = fp16_bits(hi);
+          m[u] = fp16_bits(r);
+          l[u] = fp16_bits(r - fp16_val(m[u]));
+        }
+        uint16_t* Lb = (uint16_t*)Lbase + o;
+        *reinterpret_cast<uint32_t*>(Lb) = (uint32_t)h[0] | ((uint32_t)h[1] << 16);
+        *reinterpret_cast<uint32_t*>(Lb + ps) = (uint32_t)m[0] | ((uint32_t)m[1] << 16);
+        *reinterpret_cast<uint32_t*>(Lb + 2 * ps) = (uint32_t)l[0] | ((uint32_t)l[1] << 16);
+      } else if (PREC == EMC_PREC_FP32 || PREC == kOutW) {
         *reinterpret_cast<float2*>((float*)Lbase + o) = make_float2(L[0], L[1]);
         if (DELTA && vrow) {
           const float2 old = read_pair<PREC>(Lold, o, ps);
@@ -383,51 +449,23 @@ __global__ void __launch_bounds__(kTThreads, 6)
       }
     partial[(int64_t)slice * rows + r0 + threadIdx.x] = f32_to_f64(s) + f32_to_f64(se);
   }
-  if (!DELTA) return;
-  cg::cluster_group cluster = cg::this_cluster();
-  rises[threadIdx.x] = make_float4(dp[0], dp[1], dm[0], dm[1]);
-  cluster.sync();
-  if (cluster.block_rank() == 0 && inside) {
-    for (int q = 1; q < kTRows / RPC; q++) {
-      const float4 o = cluster.map_shared_rank(rises, q)[threadIdx.x];
-      dp[0] = fmaxf(dp[0], o.x);
-      dp[1] = fmaxf(dp[1], o.y);
-      dm[0] = fmaxf(dm[0], o.z);
-      dm[1] = fmaxf(dm[1], o.w);
-    }
-    float a[2];
-#pragma unroll
-    for (int u = 0; u < 2; u++) {
-      // the sum of the planes rounded at most twice: 2^-23 |d| covers it
-      dp[u] += 2.0f * 1.1920929e-7f * fabsf(dp[u]);
-      dm[u] += 2.0f * 1.1920929e-7f * fabsf(dm[u]);
-      // bound of both rounded magnitudes (BF16 rounding up: at most 2^-7 relative)
-      a[u] = fmaxf(fabsf(dp[u]), fabsf(dm[u])) * 1.0078125f;
-    }
-    const uint16_t p0 = round_up_operand<PREC>(dp[0]), p1 = round_up_operand<PREC>(dp[1]);
-    const uint16_t m0 = round_up_operand<PREC>(dm[0]), m1 = round_up_operand<PREC>(dm[1]);
-    const uint16_t a0 = round_up_operand<PREC>(a[0]), a1 = round_up_operand<PREC>(a[1]);
-    *reinterpret_cast<uint32_t*>(D + t * ld_pix + i0) = (uint32_t)p0 | ((uint32_t)p1 << 16);
-    *reinterpret_cast<uint32_t*>(D + (ntp + t) * ld_pix + i0) = (uint32_t)m0 | ((uint32_t)m1 << 16);
-    *reinterpret_cast<uint32_t*>(D + (2 * ntp + t) * ld_pix + i0) =
-        (uint32_t)a0 | ((uint32_t)a1 << 16);
-  }
-  cluster.sync();  // no CTA leaves while its rises may be read
+  if constexpr (DELTA)
+    write_increments<PREC>(dp, dm, rises, inside, t, i0, ld_pix, ntp, D);
 }
 
-// bias_j = log w_j - (sum of the slices' partial sums, in slice order); with
+// bias_j = log w_j - scale (sum of the slices' partial sums, in slice order); with
 // the last iteration's bias, the tile's largest rise and fall of it into
 // bpm[t], bpm[nt + t] (rounded up). One CTA of 128 threads per row tile.
 __global__ void __launch_bounds__(kTRows)
     expand_bias_kernel(const double* __restrict__ partial, int n_slices, int64_t rows,
-                       const double* __restrict__ logw, int64_t nrot, double* __restrict__ bias,
-                       const double* __restrict__ bias_old, float* __restrict__ bpm, int64_t nt) {
+                       const double* __restrict__ logw, int64_t nrot, double scale,
+                       double* __restrict__ bias, const double* __restrict__ bias_old, float* __restrict__ bpm, int64_t nt) {
   __shared__ double rp[kTRows], rm[kTRows];
   const int64_t row = (int64_t)blockIdx.x * kTRows + threadIdx.x;
   double s = 0.0;
   for (int c = 0; c < n_slices; c++) s += partial[(int64_t)c * rows + row];
   const bool v = row < nrot;
-  const double b = v ? logw[row] - s : -INFINITY;
+  const double b = v ? logw[row] - s * scale : -INFINITY;
   bias[row] = b;
   if (!bias_old) return;
   const double d = v ? b - bias_old[row] : 0.0;
@@ -445,6 +483,128 @@ __global__ void __launch_bounds__(kTRows)
     bpm[blockIdx.x] = __double2float_ru(rp[0]);
     bpm[nt + blockIdx.x] = __double2float_ru(rm[0]);
   }
+}
+
+// Poisson-fluence model: L_ij = log(W_ij / B_j) + c with B_j = sum_i W_ij,
+// so that sum_i K_ik L_ij = sum_i K_ik log W_ij - N_k log B_j + c N_k, the
+// scores of the maximum-likelihood fluence phi_jk = N_k / B_j up to the
+// per-frame shift c N_k (removed in FP64 by the log-sum-exp merge). B_j is
+// needed before the first L is written, so the expansion writes W in FP32
+// (kOutW) first. a_j = c - log B_j is carried as ah (1/8 grid) + al: x + ah is
+// formed with its exact rounding error e (two-sum), hi is the 1/8-grid rounding
+// of the whole x + ah + e + al, and the rest r = ((x + ah - hi) + e) + al goes
+// to mid + lo. No per-rotation rounding of a_j enters the contraction (it would
+// be multiplied by N_k), and the rest stays centred on zero: were al left in
+// every rest, the mid/lo accumulator would grow to N_k al and round at that
+// size on every K step.
+//
+// Per row: bias = log w_j (-inf on padding rows), B_j (0) into Bsum and Bctx, and
+// (ah, al) over the row's first partial sum.
+__global__ void __launch_bounds__(kTRows)
+    flu_bias_kernel(double* __restrict__ partial, int n_slices, int64_t rows,
+                    const double* __restrict__ logw, int64_t nrot, double c,
+                    double* __restrict__ bias, double* __restrict__ Bsum,
+                    double* __restrict__ Bctx, float* __restrict__ bpm, int64_t nt, int64_t t0) {
+  const int64_t row = (int64_t)blockIdx.x * kTRows + threadIdx.x;
+  double B = 0.0;
+  for (int q = 0; q < n_slices; q++) B += partial[(int64_t)q * rows + row];
+  const bool v = row < nrot;
+  const double aj = v ? c - log(B) : 0.0;
+  const float ah = (float)(rint(aj * kHiScale) / kHiScale);
+  reinterpret_cast<float2*>(partial)[row] = make_float2(ah, (float)(aj - (double)ah));
+  bias[row] = v ? logw[row] : -INFINITY;
+  Bsum[row] = v ? B : 0.0;
+  Bctx[row] = v ? B : 0.0;
+  if (bpm && threadIdx.x == 0) bpm[t0 + blockIdx.x] = bpm[nt + t0 + blockIdx.x] = 0.f;  // log w stays
+}
+
+// W to the three BF16 planes of L, and with DELTA the increments from the last
+// iteration's planes (as expand_tile_kernel; the CTAs of a tile are a cluster).
+// Bound by memory and the latency of its short rows: 4 B of W and 6 B of planes read, 6 B
+// written per element, 3.9 TB/s with eight rows' loads in flight (one by one: 3.3).
+// 96^3, 25728 rows x 7168 columns: W 970 us + split 788 us; one CTA per rotation in
+// double-float arithmetic and a pass of its own for the increments took 1790 + 474 us.
+constexpr int kSplitRows = 32;
+template <bool DELTA>
+__global__ void __launch_bounds__(kTThreads)
+    flu_split_kernel(const float* __restrict__ Wm, const float2* __restrict__ asplit,
+                     const int4* __restrict__ qi_g, int64_t ld_pix, int64_t nrot,
+                     uint16_t* __restrict__ Lbase, int64_t ps, const uint16_t* __restrict__ Lold,
+                     uint16_t* __restrict__ D, int64_t ntp, int64_t t0, unsigned slices,
+                     int32_t* status) {
+  __shared__ float4 rises[DELTA ? kTThreads : 1];
+  constexpr unsigned kPer = kTRows / kSplitRows;
+  const unsigned slice = blockIdx.x / kPer % slices;
+  const int64_t t = blockIdx.x / kPer / slices;
+  const int64_t r0 = t * kTRows + blockIdx.x % kPer * kSplitRows;
+  const int64_t i0 = (int64_t)slice * kTPix + 2 * threadIdx.x;
+  const bool inside = i0 < ld_pix;
+  bool used[2];
+#pragma unroll
+  for (int u = 0; u < 2; u++) used[u] = inside && qi_g[i0 + u].w != 0;
+  float dp[2] = {-INFINITY, -INFINITY}, dm[2] = {-INFINITY, -INFINITY};
+  int bad = 0;
+  if (inside) {
+    constexpr int kAhead = 8;  // rows whose loads are in flight together
+#pragma unroll 1
+    for (int rb = 0; rb < kSplitRows; rb += kAhead) {
+      float2 w[kAhead];
+      uint32_t old[DELTA ? kAhead : 1][3];
+#pragma unroll
+      for (int r = 0; r < kAhead; r++) {
+        const int64_t o = (r0 + rb + r) * ld_pix + i0;
+        w[r] = __ldcs(reinterpret_cast<const float2*>(Wm + o));
+        if (DELTA)
+#pragma unroll
+          for (int q = 0; q < 3; q++)
+            old[r][q] = __ldcs(reinterpret_cast<const uint32_t*>(Lold + o + q * ps));
+      }
+#pragma unroll
+      for (int r = 0; r < kAhead; r++) {
+        const int64_t row = r0 + rb + r, o = row * ld_pix + i0;
+        const bool vrow = row < nrot;
+        const float2 aj = asplit[row];
+        const float ah = aj.x, al = aj.y;
+        uint16_t h[2], m[2], l[2];
+#pragma unroll
+        for (int u = 0; u < 2; u++) {
+          float hi = 0.f, rest = 0.f;
+          if (vrow && used[u]) {
+            const float x = logf(u ? w[r].y : w[r].x);
+            const float s = x + ah;  // two-sum: s + e = x + ah exactly
+            const float bb = s - x;
+            const float e = (x - (s - bb)) + (ah - bb);
+            hi = round_to(s + (e + al), kHiScale);
+            if (hi < kHiMin || hi > kHiMax) bad = 1;
+            hi = fminf(fmaxf(hi, kHiMin), kHiMax);
+            rest = ((s - hi) + e) + al;
+          }
+          h[u] = bf16_bits(hi);
+          m[u] = bf16_bits(rest);
+          l[u] = bf16_bits(rest - bf16_val(m[u]));
+        }
+        uint16_t* Lb = Lbase + o;
+        *reinterpret_cast<uint32_t*>(Lb) = (uint32_t)h[0] | ((uint32_t)h[1] << 16);
+        *reinterpret_cast<uint32_t*>(Lb + ps) = (uint32_t)m[0] | ((uint32_t)m[1] << 16);
+        *reinterpret_cast<uint32_t*>(Lb + 2 * ps) = (uint32_t)l[0] | ((uint32_t)l[1] << 16);
+        if (DELTA && vrow) {
+#pragma unroll
+          for (int u = 0; u < 2; u++) {
+            const int sh = 16 * u;
+            // the difference of each plane is exact in FP32; their sum rounds at most twice
+            float d = bf16_val(h[u]) - bf16_val((uint16_t)(old[r][0] >> sh));
+            d += bf16_val(m[u]) - bf16_val((uint16_t)(old[r][1] >> sh));
+            d += bf16_val(l[u]) - bf16_val((uint16_t)(old[r][2] >> sh));
+            dp[u] = fmaxf(dp[u], d);
+            dm[u] = fmaxf(dm[u], -d);
+          }
+        }
+      }
+    }
+  }
+  if (bad) set_status(status, EMC_ERR_UNSUPPORTED);
+  if constexpr (DELTA)
+    write_increments<EMC_PREC_BF16_SPLIT>(dp, dm, rises, inside, t0 + t, i0, ld_pix, ntp, D);
 }
 
 // the grid in the cell layout of load_cell
@@ -501,13 +661,14 @@ cudaError_t launch_fixed_geometry(const float4* qh, const float4* ql, int64_t ld
   return cudaGetLastError();
 }
 
-cudaError_t launch_expand_tile(const Geom& g, const float* grid, const float4* g4,
-                               const RotFX* rot,
-                               const double* logw, int64_t nrot, int64_t rows, int precision,
-                               float w_floor, Planes L, double* bias, double* partial,
-                               const void* Lold, const double* bias_old, uint16_t* D, int64_t ntp,
-                               float* bpm, int32_t* status, cudaStream_t s) {
-  if (rows <= 0) return cudaSuccess;
+namespace {
+
+// The expansion of rows (a multiple of 128) rotations in the layout `out` (a
+// precision, kOutGauss or kOutW), and the slices' partial row sums.
+cudaError_t launch_tiles(const Geom& g, const float* grid, const float4* g4, const RotFX* rot,
+                         int64_t nrot, int64_t rows, int out, float w_floor, Planes L,
+                         double* partial, const void* Lold, uint16_t* D, int64_t ntp,
+                         const float4* gsc, int32_t* status, cudaStream_t s) {
   const int64_t nt = rows / kTRows;
   const int64_t ns = expand_tile_slices(g.ld_pix);
   const bool delta = Lold != nullptr;
@@ -531,7 +692,7 @@ cudaError_t launch_expand_tile(const Geom& g, const float* grid, const float4* g
 #define EMC_TILE_R(P, I, DL, RP)                                                               \
   e = cudaLaunchKernelEx(&lc, expand_tile_kernel<P, I, DL, RP>, g.qi, g.qlo, g.ld_pix, g.N,    \
                          grid, g4, rot, nrot, rows, w_floor, L.base, L.plane_stride, partial,  \
-                         Lold, D, ntp, (unsigned)ns, status)
+                         Lold, D, ntp, (unsigned)ns, gsc, status)
 #define EMC_TILE(P, I, DL)                   \
   do {                                       \
     if (rpc == 16) EMC_TILE_R(P, I, DL, 16); \
@@ -545,19 +706,96 @@ cudaError_t launch_expand_tile(const Geom& g, const float* grid, const float4* g
     if (delta) EMC_TILE(P, false, true);       \
     else EMC_TILE(P, false, false);            \
   }
-  switch (precision) {
-    case EMC_PREC_FP32: EMC_TILE_P(EMC_PREC_FP32); break;
-    case EMC_PREC_BF16: EMC_TILE_P(EMC_PREC_BF16); break;
+#define EMC_TILE_O(P) /* no increments */      \
+  if (g.interior) EMC_TILE(P, true, false);    \
+  else EMC_TILE(P, false, false);
+  switch (out) {
+    case EMC_PREC_FP32: EMC_TILE_O(EMC_PREC_FP32); break;
+    case EMC_PREC_BF16: EMC_TILE_O(EMC_PREC_BF16); break;
+    case kOutGauss: EMC_TILE_O(kOutGauss); break;
+    case kOutW: EMC_TILE_O(kOutW); break;
     case EMC_PREC_FP16_SPLIT: EMC_TILE_P(EMC_PREC_FP16_SPLIT); break;
     default: EMC_TILE_P(EMC_PREC_BF16_SPLIT); break;
   }
+#undef EMC_TILE_O
 #undef EMC_TILE_P
 #undef EMC_TILE
 #undef EMC_TILE_R
+  return e;
+}
+
+}  // namespace
+
+cudaError_t launch_expand_tile(const Geom& g, const float* grid, const float4* g4,
+                               const RotFX* rot,
+                               const double* logw, int64_t nrot, int64_t rows, int precision,
+                               float w_floor, Planes L, double* bias, double* partial,
+                               const void* Lold, const double* bias_old, uint16_t* D, int64_t ntp,
+                               float* bpm, int32_t* status, cudaStream_t s) {
+  if (rows <= 0) return cudaSuccess;
+  // increments: the split precisions (the contexts that prune)
+  if (Lold && precision != EMC_PREC_BF16_SPLIT && precision != EMC_PREC_FP16_SPLIT)
+    return cudaErrorInvalidValue;
+  cudaError_t e = launch_tiles(g, grid, g4, rot, nrot, rows, precision, w_floor, L, partial, Lold,
+                               D, ntp, nullptr, status, s);
   if (e != cudaSuccess) return e;
-  expand_bias_kernel<<<(unsigned)nt, kTRows, 0, s>>>(partial, (int)ns, rows, logw, nrot, bias,
-                                                     delta ? bias_old : nullptr, bpm, nt);
+  const int64_t nt = rows / kTRows;
+  expand_bias_kernel<<<(unsigned)nt, kTRows, 0, s>>>(
+      partial, (int)expand_tile_slices(g.ld_pix), rows, logw, nrot, 1.0, bias,
+      Lold ? bias_old : nullptr, bpm, nt);
   return cudaGetLastError();
+}
+
+cudaError_t launch_expand_gauss(const Geom& g, const float* grid, const float4* g4,
+                                const RotFX* rot, const double* logw, int64_t nrot, int64_t rows,
+                                Planes L, double* bias, double* partial, const float4* gsc,
+                                double sigma, int32_t* status, cudaStream_t s) {
+  if (rows <= 0) return cudaSuccess;
+  cudaError_t e = launch_tiles(g, grid, g4, rot, nrot, rows, kOutGauss, 0.f, L, partial, nullptr,
+                               nullptr, 0, gsc, status, s);
+  if (e != cudaSuccess) return e;
+  expand_bias_kernel<<<(unsigned)(rows / kTRows), kTRows, 0, s>>>(
+      partial, (int)expand_tile_slices(g.ld_pix), rows, logw, nrot, 1.0 / (2.0 * sigma * sigma),
+      bias, nullptr, nullptr, 0);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_expand_flu(const Geom& g, const float* grid, const float4* g4, const RotFX* rot,
+                              const double* logw, int64_t nrot, int64_t rows, float w_floor,
+                              double c, Planes L, double* bias, double* Bctx, double* partial,
+                              float* W, int64_t W_rows, const void* Lold, uint16_t* D,
+                              int64_t ntp, float* bpm, int32_t* status, cudaStream_t s) {
+  const int64_t ns = expand_tile_slices(g.ld_pix), nt = rows / kTRows;
+  for (int64_t r0 = 0; r0 < rows; r0 += W_rows) {
+    const int64_t nr = std::min(W_rows, rows - r0), valid = std::min(nr, nrot - r0);
+    cudaError_t e = launch_tiles(g, grid, g4, rot + r0, valid, nr, kOutW, w_floor,
+                                 Planes{W, 0, g.ld_pix}, partial, nullptr, nullptr, 0, nullptr,
+                                 status, s);
+    if (e != cudaSuccess) return e;
+    flu_bias_kernel<<<(unsigned)(nr / kTRows), kTRows, 0, s>>>(
+        partial, (int)ns, nr, logw + r0, valid, c, bias + r0, bias + rows + r0, Bctx + r0,
+        Lold ? bpm : nullptr, nt, r0 / kTRows);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    constexpr int kPer = kTRows / kSplitRows;
+    cudaLaunchConfig_t lc{};
+    lc.gridDim = dim3((unsigned)(ns * (nr / kTRows) * kPer));
+    lc.blockDim = dim3(kTThreads);
+    lc.stream = s;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = kPer;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    lc.attrs = &at;
+    lc.numAttrs = Lold ? 1 : 0;
+    const int64_t o = r0 * g.ld_pix;
+    uint16_t* Lb = (uint16_t*)L.base + o;
+    const uint16_t* Lo = Lold ? (const uint16_t*)Lold + o : nullptr;
+    e = cudaLaunchKernelEx(&lc, Lold ? flu_split_kernel<true> : flu_split_kernel<false>,
+                           (const float*)W, (const float2*)partial, g.qi, g.ld_pix, valid, Lb,
+                           L.plane_stride, Lo, D, ntp, r0 / kTRows, (unsigned)ns, status);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
 }
 
 }  // namespace emc

@@ -333,79 +333,6 @@ cudaError_t launch_unpermute_lse(const int32_t* perm, int64_t n_data, const doub
 // contracted with the increments, as a third block of rows.
 // ---------------------------------------------------------------------------
 
-// One plane value of L: BF16 or FP16 bits.
-template <bool F16>
-__device__ __forceinline__ float plane_val(const uint16_t* p, int64_t o) {
-  if (F16) return __half2float(*reinterpret_cast<const __half*>(p + o));
-  return __uint_as_float(((uint32_t)p[o]) << 16);
-}
-// The next BF16 (FP16) value >= x, as bits: the operand type of the frames.
-template <bool F16>
-__device__ __forceinline__ uint16_t round_up_bits(float x) {
-  if (F16) {
-    __half h = __float2half_ru(x);
-    return *reinterpret_cast<uint16_t*>(&h);
-  }
-  __nv_bfloat16 b = __float2bfloat16_ru(x);
-  return *reinterpret_cast<uint16_t*>(&b);
-}
-
-// One CTA per (pixel slice of 256 columns, row tile): each thread a pixel,
-// the tile's valid rows in turn. D = [3 ntp][ld_pix]: rows t (D+), ntp + t
-// (D-) and 2 ntp + t (A = max(|D+|, |D-|)), all rounded up to the frames'
-// operand type; bpm[t], bpm[nt + t] = b+_t, b-_t (rounded up), written by the
-// CTAs of the first slice.
-template <int NP, bool F16>
-__global__ void __launch_bounds__(256)
-    delta_planes_kernel(const uint16_t* __restrict__ L0, const uint16_t* __restrict__ L1,
-                        int64_t plane, int64_t ld_pix, int64_t nrot, const double* __restrict__ b0,
-                        const double* __restrict__ b1, int64_t ntp, uint16_t* __restrict__ D,
-                        float* __restrict__ bpm, int64_t nt) {
-  const int64_t t = blockIdx.y;
-  const int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x;
-  const int64_t r0 = t * 128;
-  const int64_t r1 = min(r0 + 128, nrot);
-  float dp = -INFINITY, dm = -INFINITY;
-  if (i < ld_pix) {
-    for (int64_t j = r0; j < r1; j++) {
-      const int64_t o = j * ld_pix + i;
-      // the difference of each plane is exact in FP32; their sum rounds at most twice
-      float d = plane_val<F16>(L1, o) - plane_val<F16>(L0, o);
-#pragma unroll
-      for (int q = 1; q < NP; q++) d += plane_val<F16>(L1, o + q * plane) - plane_val<F16>(L0, o + q * plane);
-      dp = fmaxf(dp, d);
-      dm = fmaxf(dm, -d);
-    }
-    // those roundings: 2^-23 |d| covers them
-    dp += 2.0f * 1.1920929e-7f * fabsf(dp);
-    dm += 2.0f * 1.1920929e-7f * fabsf(dm);
-    const uint16_t up = round_up_bits<F16>(dp), um = round_up_bits<F16>(dm);
-    D[t * ld_pix + i] = up;
-    D[(ntp + t) * ld_pix + i] = um;
-    // A bounds the magnitude of both rounded values
-    D[(2 * ntp + t) * ld_pix + i] = round_up_bits<F16>(fmaxf(fabsf(dp), fabsf(dm)) * 1.0078125f);
-  }
-  if (blockIdx.x == 0 && threadIdx.x < 128) {
-    __shared__ double rb[2][128];
-    const int64_t j = r0 + threadIdx.x;
-    const double db = j < nrot ? b1[j] - b0[j] : 0.0;
-    rb[0][threadIdx.x] = j < nrot ? db : -INFINITY;
-    rb[1][threadIdx.x] = j < nrot ? -db : -INFINITY;
-    __syncwarp();
-    for (int w = 64; w > 0; w >>= 1) {
-      asm volatile("bar.sync 3, 128;" ::: "memory");
-      if ((int)threadIdx.x < w) {
-        rb[0][threadIdx.x] = fmax(rb[0][threadIdx.x], rb[0][threadIdx.x + w]);
-        rb[1][threadIdx.x] = fmax(rb[1][threadIdx.x], rb[1][threadIdx.x + w]);
-      }
-    }
-    if (threadIdx.x == 0) {
-      bpm[t] = __double2float_ru(rb[0][0]);
-      bpm[nt + t] = __double2float_ru(rb[1][0]);
-    }
-  }
-}
-
 // Per frame (lanes) and row tile (warp strides), with C = [D+; D-; A] K^T of
 // the frames in the current internal order (rows t, ntp + t, 2 ntp + t):
 //   Ub[t][k] += C+[t][k] + b+_t + err_tk        (err = errc (1 + errc) CA[t][k])
@@ -578,20 +505,6 @@ __global__ void __launch_bounds__(256)
     d |= (float)K[k * ld_k + i] != v;
   }
   if (__syncthreads_or(d) && threadIdx.x == 0) *flag = 1;
-}
-
-cudaError_t launch_delta_planes(const uint16_t* L0, const uint16_t* L1, int64_t plane,
-                                int64_t ld_pix, int64_t nrot, const double* b0, const double* b1,
-                                int64_t ntp, uint16_t* D, float* bpm, int f16, cudaStream_t s) {
-  const int64_t nt = (nrot + 127) / 128;
-  dim3 grd((unsigned)((ld_pix + 255) / 256), (unsigned)nt);
-  if (f16)  // FP16 split: hi + rest
-    delta_planes_kernel<2, true><<<grd, 256, 0, s>>>(L0, L1, plane, ld_pix, nrot, b0, b1, ntp, D,
-                                                     bpm, nt);
-  else      // BF16 split: hi + mid + lo
-    delta_planes_kernel<3, false><<<grd, 256, 0, s>>>(L0, L1, plane, ld_pix, nrot, b0, b1, ntp, D,
-                                                      bpm, nt);
-  return cudaGetLastError();
 }
 
 cudaError_t launch_delta_live(const float* C, int64_t ntp, const float* bpm,

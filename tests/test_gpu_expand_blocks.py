@@ -38,3 +38,36 @@ def test_blocks_equal_whole(N, edge, precision):
         assert torch.equal(bb[:nb], bias[r0:r0 + nb])
         assert int(part[:, nb:].count_nonzero()) == 0 and bool(torch.isinf(bb[nb:]).all())
     assert ctx.status() == 0
+
+
+@pytest.mark.parametrize("model,precision", [("poisson_fluence", "bf16_split"),
+                                             ("gaussian", "fp16_split")])
+def test_blocks_equal_whole_other_models(model, precision):
+    """The Poisson-fluence expansion keeps W in a buffer of rot_chunk rotations, so a
+    whole sampling runs in several pieces there; the Gaussian one has its own layout."""
+    import torch
+    from paper_1409_4256_gb300 import emc, synth
+    det = synth.make_detector(32, 32)
+    quat, w = emc.quat_generate(6)
+    n = quat.shape[0]
+    K = torch.ones(8, det.q.shape[0], dtype=torch.int32, device="cuda")
+    g = torch.Generator(device="cuda").manual_seed(7)
+    grid = torch.rand(32, 32, 32, generator=g, device="cuda") + 0.01
+    got = []
+    for chunk, block in ((0, n), (1000, n), (256, 777)):
+        ctx = emc.Context(32, det.q, quat, w, 8, precision=precision, model=model, w_floor=1e-6,
+                          rot_chunk=chunk)
+        ctx.set_frames(K)
+        planes, bias = [], []
+        for r0 in range(0, n, block):
+            nb = min(block, n - r0)
+            L, b = ctx.expand(grid, r0, nb)
+            rows = (nb + 127) // 128 * 128
+            part = L.view(torch.int16).view(3, rows, ctx.ld_pix)
+            assert int(part[:, nb:].count_nonzero()) == 0
+            planes.append(part[:, :nb])
+            bias.append(b.view(-1, rows)[:, :nb])
+        assert ctx.status() == 0
+        got.append((torch.cat(planes, 1), torch.cat(bias, 1)))
+    for planes, bias in got[1:]:
+        assert torch.equal(planes, got[0][0]) and torch.equal(bias, got[0][1])
