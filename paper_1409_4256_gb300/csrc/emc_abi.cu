@@ -1346,7 +1346,8 @@ int emc_sparse_estep(emc_ctx* ctx, const void* L, const double* bias, float* P, 
   CU(launch_sparse_scores(lp, ctx->cfg.precision, y.rows, bias, ctx->Kb, y.ld_pix,
                           (const int64_t*)(ctx->ws + y.coff), (const int2*)(ctx->ws + y.cent), M,
                           csr ? (const int64_t*)(ctx->ws + y.skoff) : nullptr,
-                          csr ? (const uint32_t*)(ctx->ws + y.skent) : nullptr, Sc, s));
+                          csr ? (const uint32_t*)(ctx->ws + y.skent) : nullptr, ctx->cfg.n_data,
+                          P, Sc, s));  // (P holds the choice of pairs until it is written)
   CU(launch_sparse_lse(Sc, ctx->cfg.n_data, y.ld_data, M, P, lse, ctx->status, s, ctx->flu_cn));
   return EMC_OK;
 }

@@ -74,7 +74,7 @@ cudaError_t launch_assign_duplicates(const int32_t* K, int64_t ld_k, int64_t n_d
 // partial: scratch of expand_tile_slices(ld_pix) x rows doubles. With Lold
 // (the last iteration's L, same layout) it also writes the incremental bound's
 // increments D ([2 ntp][ld_pix], rounded up to the frames' type), dabs[t] and,
-// from bias_old, bpm (as launch_delta_planes).
+// from bias_old, bpm: the bias's largest rise (bpm[t]) and fall (bpm[nt + t]) over each tile.
 int64_t expand_tile_slices(int64_t ld_pix);
 // g4 (may be NULL): the grid in the cell layout (launch_grid_cells),
 // read where every corner lies inside the grid
@@ -344,11 +344,13 @@ cudaError_t launch_csr_build(const int32_t* cand, int64_t n_data, int M, int64_t
                              int64_t rows, int32_t* cnt, int64_t* off, int2* ent,
                              int32_t* status, cudaStream_t s);
 // koff/kent (non-NULL): the frames' non-zero pixel lists (EMC_FLAG_SPARSE_K)
-// replace their dense rows in both sparse contractions
+// replace their dense rows in both sparse contractions. need: scratch [n_data][M]; with the
+// lists, pairs that cannot matter (P = 0 in FP32) get the score -infinity.
 cudaError_t launch_sparse_scores(const Planes& L, int precision, int64_t rows, const double* bias,
                                  const uint16_t* Kb, int64_t ld_pix, const int64_t* off,
                                  const int2* ent, int M, const int64_t* koff,
-                                 const uint32_t* kent, double* Sc, cudaStream_t s);
+                                 const uint32_t* kent, int64_t n_data, float* need, double* Sc,
+                                 cudaStream_t s);
 // shift (may be NULL): per-frame constant of the scores, removed from lse_c
 cudaError_t launch_sparse_lse(const double* Sc, int64_t n_data, int64_t ld_data, int M, float* Pc,
                               double* lse_c, int32_t* status, cudaStream_t s,

@@ -605,6 +605,96 @@ __device__ __forceinline__ void unpack2(uint32_t w, float& lo, float& hi) {
   }
 }
 
+// Candidate pairs that can matter, from the hi part of log W alone (frames as
+// lists). With hi on the 1/8 grid (FP16 split: 1/64) and the rest at most half a
+// step, S^hi_jk = sum_i K_ik hi_ij + bias_j is within E_k = N_k / 16 + 1 (N_k / 128
+// + 1) of S_jk, the 1 covering every rounding. A pair whose S^hi lies more than 2 E_k +
+// 111 below the frame's largest scores more than 110 below its best candidate:
+// its P is 0 in FP32 and its share of the log-sum-exp below FP64's rounding.
+// Counts and hi are small integers, so the sums are integer and exact.
+//
+// One CTA per rotation row, a warp per pair. The row is staged in 16 bits: the list's
+// neighbouring entries are near pixels, so a warp's gathers fall on about
+// half as many words as lanes and meet few bank conflicts, where the full split's two FP32
+// gathers cost seven wavefronts. 64^3, 20000 frames x 512 candidates: the
+// scores of every pair took 5.06 ms; this pass 2.86 ms (28 GB of lists through L2), the choice 0.04 ms and the scores of the
+// pairs left 0.41 ms.
+template <int PREC>
+struct HiGrid {  // units of hi
+  static constexpr float scale = PREC == EMC_PREC_FP16_SPLIT ? 64.f : 8.f;
+};
+template <int PREC>
+__global__ void __launch_bounds__(256)
+    sparse_bound_kernel(const void* __restrict__ L, int64_t ld_pix, const double* __restrict__ bias,
+                        const int64_t* __restrict__ off, const int2* __restrict__ ent, int M,
+                        const int64_t* __restrict__ koff, const uint32_t* __restrict__ kent,
+                        float* __restrict__ Sh) {
+  const int64_t j = blockIdx.x;
+  const int64_t e0 = off[j], e1 = off[j + 1];
+  if (e0 == e1) return;
+  extern __shared__ float4 sm4[];
+  int16_t* Lq = reinterpret_cast<int16_t*>(sm4);
+  constexpr float scale = HiGrid<PREC>::scale;
+  for (int64_t i = threadIdx.x; i < ld_pix; i += 256) {
+    float h;
+    if (PREC == EMC_PREC_FP32)
+      h = rintf(reinterpret_cast<const float*>(L)[j * ld_pix + i] * scale);
+    else if (PREC == EMC_PREC_FP16_SPLIT)
+      h = fp16_val(reinterpret_cast<const uint16_t*>(L)[j * ld_pix + i]) * scale;
+    else
+      h = bf16_val(reinterpret_cast<const uint16_t*>(L)[j * ld_pix + i]) * scale;
+    Lq[i] = (int16_t)(int)h;
+  }
+  __syncthreads();
+  const float bj = (float)bias[j];
+  const int lane = threadIdx.x & 31;
+  for (int64_t e = e0 + (threadIdx.x >> 5); e < e1; e += 8) {
+    const int2 km = ent[e];
+    const int64_t f0 = koff[km.x];
+    const int n = (int)(koff[km.x + 1] - f0);
+    const uint32_t* list = kent + f0;
+    int sum = 0;
+    int f = lane;
+    for (; f + 96 < n; f += 128) {
+      uint32_t w[4];
+#pragma unroll
+      for (int u = 0; u < 4; u++) w[u] = list[f + 32 * u];
+#pragma unroll
+      for (int u = 0; u < 4; u++) sum += (int)(w[u] >> 16) * Lq[w[u] & 0xffffu];
+    }
+    for (; f < n; f += 32) {
+      const uint32_t w = list[f];
+      sum += (int)(w >> 16) * Lq[w & 0xffffu];
+    }
+    sum = __reduce_add_sync(0xffffffffu, sum);
+    if (lane == 0) Sh[(int64_t)km.x * M + km.y] = (float)sum * (1.f / scale) + bj;
+  }
+}
+
+// One warp per frame: 1 into Sh where the pair's score is needed, else 0 and a
+// score of -infinity.
+__global__ void __launch_bounds__(256)
+    sparse_choose_kernel(const int64_t* __restrict__ koff, const uint32_t* __restrict__ kent,
+                         int64_t n_data, int M, float step, float* __restrict__ Sh,
+                         double* __restrict__ Sc) {
+  const int64_t k = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const int lane = threadIdx.x & 31;
+  if (k >= n_data) return;
+  int total = 0;  // N_k < 65536
+  for (int64_t f = koff[k] + lane; f < koff[k + 1]; f += 32) total += (int)(kent[f] >> 16);
+  total = __reduce_add_sync(0xffffffffu, total);
+  float* s = Sh + k * M;
+  float mx = -INFINITY;
+  for (int m = lane; m < M; m += 32) mx = fmaxf(mx, s[m]);
+  for (int o = 16; o; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+  const float least = mx - (2.f * ((float)total * step + 1.f) + 111.f);
+  for (int m = lane; m < M; m += 32) {
+    const bool on = !(s[m] < least);  // a NaN stays
+    s[m] = on ? 1.f : 0.f;
+    if (!on) Sc[k * M + m] = -INFINITY;
+  }
+}
+
 // One CTA per rotation row: log W_j split into (hi on the 1/8 grid, rest) in
 // shared memory; each warp takes pairs (frame, slot) of the row's list, two
 // at a time, reading the frames' K rows 8 pixels (16 bytes) per lane.
@@ -612,17 +702,26 @@ __device__ __forceinline__ void unpack2(uint32_t w, float& lo, float& hi) {
 // are read instead of their rows -- 4 bytes per non-zero pixel rather than 2
 // bytes per pixel -- and gathered against the staged row; the count x hi sums
 // stay exact (integral counts, hi on the 1/8 grid, frame totals below 2^16).
+// need (CSR, may be NULL): only the pairs with need[k M + m] != 0.
 template <int PREC, bool CSR>
 __global__ void __launch_bounds__(256)
     sparse_scores_kernel(const void* __restrict__ L, int64_t plane_stride, int64_t ld_pix,
                          const double* __restrict__ bias, const uint16_t* __restrict__ Kb,
                          const int64_t* __restrict__ off, const int2* __restrict__ ent, int M,
                          const int64_t* __restrict__ koff, const uint32_t* __restrict__ kent,
-                         double* __restrict__ Sc) {
+                         const float* __restrict__ need, double* __restrict__ Sc) {
   const int64_t j = blockIdx.x;
   const int64_t e0 = off[j], e1 = off[j + 1];
   if (e0 == e1) return;
   extern __shared__ float4 sm4[];
+  if (CSR && need) {  // a row without a needed pair
+    bool any = false;
+    for (int64_t e = e0 + threadIdx.x; e < e1; e += blockDim.x) {
+      const int2 km = ent[e];
+      any |= need[(int64_t)km.x * M + km.y] != 0.f;
+    }
+    if (!__syncthreads_or(any)) return;
+  }
   float* Lh = reinterpret_cast<float*>(sm4);
   float* Lr = Lh + ld_pix;
   for (int64_t i = threadIdx.x; i < ld_pix; i += blockDim.x) {
@@ -648,22 +747,32 @@ __global__ void __launch_bounds__(256)
   const double bj = bias[j];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
   if (CSR) {
-    for (int64_t e = e0 + wid; e < e1; e += nw) {
-      const int2 km = ent[e];
-      const int64_t f1 = koff[km.x + 1];
-      float ah = 0.f, ar = 0.f;
-      for (int64_t f = koff[km.x] + lane; f < f1; f += 32) {
-        const uint32_t w = kent[f];
-        const int idx = (int)(w & 0xffffu);
-        const float c = (float)(w >> 16);
-        ah = fmaf(c, Lh[idx], ah);
-        ar = fmaf(c, Lr[idx], ar);
+    // a warp looks 32 pairs over at a time (the CTA's warps in turn) and takes the needed ones
+    for (int64_t b = e0 + wid; b < e1; b += 32 * nw) {
+      const int64_t own = b + (int64_t)lane * nw;
+      const int2 mine = own < e1 ? ent[own] : make_int2(0, 0);
+      unsigned todo = __ballot_sync(
+          0xffffffffu, own < e1 && (!need || need[(int64_t)mine.x * M + mine.y] != 0.f));
+      while (todo) {
+        const int src = __ffs(todo) - 1;
+        todo &= todo - 1;
+        const int2 km = make_int2(__shfl_sync(0xffffffffu, mine.x, src),
+                                  __shfl_sync(0xffffffffu, mine.y, src));
+        const int64_t f1 = koff[km.x + 1];
+        float ah = 0.f, ar = 0.f;
+        for (int64_t f = koff[km.x] + lane; f < f1; f += 32) {
+          const uint32_t w = kent[f];
+          const int idx = (int)(w & 0xffffu);
+          const float c = (float)(w >> 16);
+          ah = fmaf(c, Lh[idx], ah);
+          ar = fmaf(c, Lr[idx], ar);
+        }
+        for (int o = 16; o; o >>= 1) {
+          ah += __shfl_xor_sync(0xffffffffu, ah, o);
+          ar += __shfl_xor_sync(0xffffffffu, ar, o);
+        }
+        if (lane == 0) Sc[(int64_t)km.x * M + km.y] = ((double)ah + (double)ar) + bj;
       }
-      for (int o = 16; o; o >>= 1) {
-        ah += __shfl_xor_sync(0xffffffffu, ah, o);
-        ar += __shfl_xor_sync(0xffffffffu, ar, o);
-      }
-      if (lane == 0) Sc[(int64_t)km.x * M + km.y] = ((double)ah + (double)ar) + bj;
     }
     return;
   }
@@ -995,15 +1104,38 @@ cudaError_t launch_lse_values(const double* m, const double* sm, int64_t n, doub
 cudaError_t launch_sparse_scores(const Planes& L, int precision, int64_t rows, const double* bias,
                                  const uint16_t* Kb, int64_t ld_pix, const int64_t* off,
                                  const int2* ent, int M, const int64_t* koff,
-                                 const uint32_t* kent, double* Sc, cudaStream_t s) {
+                                 const uint32_t* kent, int64_t n_data, float* need, double* Sc,
+                                 cudaStream_t s) {
   const size_t smem = 2 * sizeof(float) * (size_t)ld_pix;
   cudaError_t e = cudaSuccess;
+  // (plain BF16 holds one rounded value, not on a grid: every pair is scored)
+  if (!kent || precision == EMC_PREC_BF16) need = nullptr;
+  if (need) {
+    const size_t sb = sizeof(int16_t) * (size_t)ld_pix;
+#define EMC_SPARSE_BOUND(P)                                                                     \
+  e = cudaFuncSetAttribute(sparse_bound_kernel<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
+                           (int)sb);                                                            \
+  if (e != cudaSuccess) return e;                                                               \
+  sparse_bound_kernel<P><<<(unsigned)rows, 256, sb, s>>>(L.base, ld_pix, bias, off, ent, M,     \
+                                                         koff, kent, need)
+    switch (precision) {
+      case EMC_PREC_FP32: EMC_SPARSE_BOUND(EMC_PREC_FP32); break;
+      case EMC_PREC_FP16_SPLIT: EMC_SPARSE_BOUND(EMC_PREC_FP16_SPLIT); break;
+      default: EMC_SPARSE_BOUND(EMC_PREC_BF16_SPLIT); break;
+    }
+#undef EMC_SPARSE_BOUND
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    const float step = precision == EMC_PREC_FP16_SPLIT ? 1.f / 128.f : 1.f / 16.f;
+    sparse_choose_kernel<<<(unsigned)((n_data * 32 + 255) / 256), 256, 0, s>>>(koff, kent, n_data,
+                                                                              M, step, need, Sc);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  }
 #define EMC_SPARSE_SCORES(P, C)                                                              \
   e = cudaFuncSetAttribute(sparse_scores_kernel<P, C>,                                       \
                            cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);         \
   if (e != cudaSuccess) return e;                                                            \
   sparse_scores_kernel<P, C><<<(unsigned)rows, 256, smem, s>>>(                              \
-      L.base, L.plane_stride, ld_pix, bias, Kb, off, ent, M, koff, kent, Sc)
+      L.base, L.plane_stride, ld_pix, bias, Kb, off, ent, M, koff, kent, need, Sc)
 #define EMC_SPARSE_SCORES_P(P)      \
   if (kent) {                       \
     EMC_SPARSE_SCORES(P, true);     \
