@@ -736,8 +736,8 @@ int do_loglik(emc_ctx* c, const void* L, int64_t Lrows, int64_t row_off, const d
   return EMC_OK;
 }
 
-// Frames in emc_iteration's internal order (bound-pruned pass 1): their BF16
-// matrix, the Poisson-fluence arrays, and the contracted tiles of these rows.
+// Frames in emc_iteration's internal order (bound-pruned pass 1), whose split lse
+// is in the workspace's lse2 already: their BF16 matrix, the Poisson-fluence arrays, and the contracted tiles of these rows.
 struct FrameView {
   const uint16_t* K;
   const double* cn;
@@ -773,7 +773,7 @@ int do_normalize(emc_ctx* c, const void* L, int64_t Lrows, int64_t row_off, cons
     const double* cn = fv ? fv->cn : c->flu_cn;
     const float* invn = fv ? fv->invn : c->flu_invn;
     if (S) {
-      CU(launch_lse_split(lse_m, lse_s, c->cfg.n_data, y.ld_data, lse2, s, cn));
+      if (!fv) CU(launch_lse_split(lse_m, lse_s, c->cfg.n_data, y.ld_data, lse2, s, cn));
       CU(launch_normalize_scores_flu(S, ldS, Sref, lse2, Bsum, invn, rows, nrot,
                                      y.ld_data, c->cfg.n_data, (uint16_t*)P, Prows * y.ld_data,
                                      den, s, kbf, tlive));
@@ -782,9 +782,9 @@ int do_normalize(emc_ctx* c, const void* L, int64_t Lrows, int64_t row_off, cons
       Planes pp{P, Prows * y.ld_data, y.ld_data};
       const bool kept = fv && fv->kept;
       if (kept)
-        CU(launch_normalize_kept(fv->kept, fv->slot, fv->kept_list, fv->kept_count, lse_m, lse_s,
-                                 lse2, rows, nrot, y.ld_data, c->cfg.n_data, c->cfg.precision, P,
-                                 Prows * y.ld_data, cn, Bsum, invn, den, kbf, s));
+        CU(launch_normalize_kept(fv->kept, fv->slot, fv->kept_list, fv->kept_count, lse2, rows,
+                                 nrot, y.ld_data, c->cfg.n_data, c->cfg.precision, P,
+                                 Prows * y.ld_data, Bsum, invn, den, kbf, s));
       if (!kept || !fv->kept_all)
         CU(launch_tc_normalize(lp, c->cfg.precision, bias, rows, nrot, Kf, y.ld_data,
                                c->cfg.n_data, y.ld_pix, lse_m, lse_s, lse2, pp, c->status, s,
@@ -804,7 +804,7 @@ int do_normalize(emc_ctx* c, const void* L, int64_t Lrows, int64_t row_off, cons
   }
   if (S) {
     float2* lse2 = (float2*)(c->ws + y.lse2);
-    CU(launch_lse_split(lse_m, lse_s, c->cfg.n_data, y.ld_data, lse2, s));
+    if (!fv) CU(launch_lse_split(lse_m, lse_s, c->cfg.n_data, y.ld_data, lse2, s));
     CU(launch_normalize_scores(S, ldS, Sref, lse2, rows, nrot, y.ld_data, c->cfg.n_data,
                                c->cfg.precision, P, Prows * y.ld_data, s, kbf, tlive));
     return EMC_OK;
@@ -819,9 +819,9 @@ int do_normalize(emc_ctx* c, const void* L, int64_t Lrows, int64_t row_off, cons
     float2* lse2 = (float2*)(c->ws + y.lse2);
     const bool kept = fv && fv->kept;
     if (kept)
-      CU(launch_normalize_kept(fv->kept, fv->slot, fv->kept_list, fv->kept_count, lse_m, lse_s, lse2,
-                               rows, nrot, y.ld_data, c->cfg.n_data, c->cfg.precision, P,
-                               Prows * y.ld_data, nullptr, nullptr, nullptr, nullptr, kbf, s));
+      CU(launch_normalize_kept(fv->kept, fv->slot, fv->kept_list, fv->kept_count, lse2, rows, nrot,
+                               y.ld_data, c->cfg.n_data, c->cfg.precision, P, Prows * y.ld_data,
+                               nullptr, nullptr, nullptr, kbf, s));
     if (!kept || !fv->kept_all)
       CU(launch_tc_normalize(lp, c->cfg.precision, bias, rows, nrot, Kf, y.ld_data, c->cfg.n_data,
                              y.ld_pix, lse_m, lse_s, lse2, pp, c->status, s, nullptr, nullptr,
@@ -1075,7 +1075,7 @@ int emc_iteration(emc_ctx* c, const float* grid_in, float* grid_out, emc_iter_st
                            nmt, y.ld_data, c->cfg.n_data, live, s));
       CU(launch_tile_list(live, (int)nmt, (int)nnt, 8, tlist, tcount, (int32_t*)(c->ws + y.sortH),
                             s, kept ? slot : nullptr));
-      kernels += 10;  // a tile list is three launches
+      kernels += 4 + tile_list_launches((nmt + 1) / 2 * nnt) + tile_list_launches(nmt * nnt);
     }
     CU(launch_tc_pass1(p3, c->cfg.precision, bias, y.rows, Kp, y.ld_data, c->cfg.n_data, y.ld_pix,
                        pm, ps, S, S + y.rows * y.ld_data, nullptr, nullptr, c->status, s,
@@ -1085,19 +1085,17 @@ int emc_iteration(emc_ctx* c, const float* grid_in, float* grid_out, emc_iter_st
     // contracted tile's maximum (plus 1/64) in Ub, the frames' largest maxima and best tiles
     CU(launch_lse_merge(pm, ps, nmt, y.ld_data, c->cfg.n_data, lm, ls, 0, 0, c->status, s, cn_p,
                         pruned ? live : nullptr, c->best, c->Ub, c->Mk, c->Ua));
-    CU(launch_unpermute_lse(c->perm, c->cfg.n_data, lm, ls, lse_m, lse_s, s));
-    // the frames are consumed; a device status recorded by now (a wait that
-    // gave up, a non-finite value) voids the tile bounds for the next iteration
-    CU(cudaMemsetAsync(c->ws + y.flags, 0, sizeof(int32_t), s));
-    CU(cudaMemcpyAsync(c->ws + y.flags + 8, c->status, sizeof(int32_t), cudaMemcpyDeviceToDevice,
-                       s));
-    kernels += 3;  // pass 1, merge, lse order
+    // lse in the frames' order, its split for pass 2 and its sum. The frames are
+    // consumed; a device status recorded by now (a wait that gave up, a non-finite
+    // value) voids the tile bounds for the next iteration
+    CU(launch_lse_finish(c->perm, c->cfg.n_data, y.ld_data, lm, ls, cn_p, lse_m, lse_s,
+                         (float2*)(c->ws + y.lse2), ll, (int32_t*)(c->ws + y.flags), c->status, s));
+    kernels += 3;  // pass 1, merge, finish
   } else {
     if ((st = do_loglik(c, L, y.rows, 0, bias, n_rot, lse_m, lse_s, 0, S, s))) return st;
-    kernels += 2;
+    CU(launch_loglik_sum(lse_m, lse_s, c->cfg.n_data, ll, s));
+    kernels += 3;
   }
-  CU(launch_loglik_sum(lse_m, lse_s, c->cfg.n_data, ll, s));
-  kernels += 1;
   if (stats) CU(cudaEventRecord(c->ev[2], s));
   CU(cudaMemsetAsync(gn, 0, (y.gden - y.gnum) + gb, s));  // both grids, one behind the other
   float t_norm = 0.f, t_upd = 0.f, t_cmp = 0.f;
@@ -1133,7 +1131,8 @@ int emc_iteration(emc_ctx* c, const float* grid_in, float* grid_out, emc_iter_st
         CU(launch_tile_list(live + t0, (int)(crows / 128), (int)nnt, 8, tlist, tcount + 8,
                             (int32_t*)(c->ws + y.sortH), s, nullptr,
                             TilePick{slot + t0, kept_cap, false}));
-      kernels += all ? 3 : 7;
+      const int nl = tile_list_launches(crows / 128 * nnt);
+      kernels += all ? nl : 2 * nl + 1;
       fv.kept = kept;
       fv.slot = slot + t0;
       fv.kept_list = klist;
@@ -1163,8 +1162,10 @@ int emc_iteration(emc_ctx* c, const float* grid_in, float* grid_out, emc_iter_st
     if (stats) CU(cudaEventRecord(c->ev[5], s));
     CU(launch_compress(c->geom, (const RotFX*)(c->ws + y.rotfx) + r0, nr, Num, den, c->cfg.compress_mode, gn, gd, s));
     if (stats) CU(cudaEventRecord(c->ev[6], s));
-    // normalize: lse split + the pass (one SIMT kernel when recomputing in FP32)
-    kernels += (S || c->cfg.precision != EMC_PREC_FP32 ? 2 : 1) + 2 + (kbf ? 1 : 0);
+    // normalize: lse split (but where the finish wrote it) + the pass (one SIMT
+    // kernel when recomputing in FP32)
+    const bool split = pr ? !S && !kept : (S || c->cfg.precision != EMC_PREC_FP32);
+    kernels += (split ? 2 : 1) + 2 + (kbf ? 1 : 0);
     if (stats) {
       // chunk timings need a host wait per chunk; only when stats are asked for
       float a = 0, b = 0, d = 0;

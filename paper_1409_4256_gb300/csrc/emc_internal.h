@@ -215,14 +215,13 @@ cudaError_t launch_normalize_scores(const float* S, int64_t ldS, const float* Sr
                                     int64_t P_plane, cudaStream_t s, uint8_t* kb_flag = nullptr,
                                     const uint8_t* tile_live = nullptr);
 // Pass 2 from the kept scores of the listed tiles (codes mt * ld_data / 256 + nt of this
-// chunk's rows, their places in slot), after lse2, kb_flag (zeroed) and, for the
-// Poisson-fluence model (Bsum != NULL), den are set up as the other pass-2 forms set them up.
+// chunk's rows, their places in slot); zeroes kb_flag and, for the Poisson-fluence model
+// (Bsum != NULL), den first. lse2: as launch_lse_split writes it.
 cudaError_t launch_normalize_kept(const float* kept, const int32_t* slot, const int32_t* tile_list,
-                                  const int32_t* tile_count, const double* lse_m,
-                                  const double* lse_s, float2* lse2, int64_t rows, int64_t nrot,
-                                  int64_t ld_data, int64_t n_data, int precision, void* P,
-                                  int64_t P_plane, const double* shift, const double* Bsum,
-                                  const float* invn, float* den, uint8_t* kb_flag, cudaStream_t s);
+                                  const int32_t* tile_count, const float2* lse2, int64_t rows,
+                                  int64_t nrot, int64_t ld_data, int64_t n_data, int precision,
+                                  void* P, int64_t P_plane, const double* Bsum, const float* invn,
+                                  float* den, uint8_t* kb_flag, cudaStream_t s);
 cudaError_t launch_loglik_sum(const double* lse_m, const double* lse_s, int64_t n_data,
                               double* out, cudaStream_t s);
 
@@ -395,6 +394,7 @@ cudaError_t launch_tile_list(const uint8_t* live, int n_mtiles, int n_ntiles, in
                              int32_t* list, int32_t* count, int32_t* scratch, cudaStream_t s,
                              int32_t* slot_out = nullptr, TilePick pick = TilePick{});
 int64_t tile_list_scratch_entries(int64_t n_mtiles, int64_t n_ntiles);
+int tile_list_launches(int64_t tiles);
 // entries of the histogram scratch H (int32) of launch_sort_frames; off needs one more (int64)
 int64_t sort_scratch_entries(int64_t n_data, int nbins);
 // new_perm[pos] = perm[s] for the frames s stably sorted by key[s] in [0, nbins)
@@ -408,8 +408,10 @@ cudaError_t launch_permute_frames(const int32_t* perm, int64_t ld_data, int64_t 
 cudaError_t launch_frame_totals(const int32_t* K, int64_t ld_k, int64_t n_data, int64_t n_pix,
                                 int64_t ld_data, float* nsum, cudaStream_t s);
 cudaError_t launch_identity(int32_t* p, int64_t n, cudaStream_t s);
-cudaError_t launch_unpermute_lse(const int32_t* perm, int64_t n_data, const double* m_s,
-                                 const double* s_s, double* m, double* s, cudaStream_t st);
+cudaError_t launch_lse_finish(const int32_t* perm, int64_t n_data, int64_t ld_data,
+                              const double* m_s, const double* s_s, const double* shift, double* m,
+                              double* s, float2* lse2, double* total, int32_t* flags,
+                              const int32_t* status, cudaStream_t st);
 
 // exclusive scan of cnt[0, n) into off[0, n] (off[n] = total), one CTA
 cudaError_t launch_scan_counts(const int32_t* cnt, int64_t n, int64_t* off, cudaStream_t s);

@@ -687,15 +687,12 @@ cudaError_t launch_normalize_scores_flu(const float* S, int64_t ldS, const float
 }
 
 cudaError_t launch_normalize_kept(const float* kept, const int32_t* slot, const int32_t* tile_list,
-                                  const int32_t* tile_count, const double* lse_m,
-                                  const double* lse_s, float2* lse2, int64_t rows, int64_t nrot,
-                                  int64_t ld_data, int64_t n_data, int precision, void* P,
-                                  int64_t P_plane, const double* shift, const double* Bsum,
-                                  const float* invn, float* den, uint8_t* kb_flag, cudaStream_t s) {
+                                  const int32_t* tile_count, const float2* lse2, int64_t rows,
+                                  int64_t nrot, int64_t ld_data, int64_t n_data, int precision,
+                                  void* P, int64_t P_plane, const double* Bsum, const float* invn,
+                                  float* den, uint8_t* kb_flag, cudaStream_t s) {
   if (!kb_flag || (Bsum && (!invn || !den))) return cudaErrorInvalidValue;
-  cudaError_t e = launch_lse_split(lse_m, lse_s, n_data, ld_data, lse2, s, shift);
-  if (e != cudaSuccess) return e;
-  e = cudaMemsetAsync(kb_flag, 0, (size_t)(rows / kNormRows) * (ld_data / kNormFrames), s);
+  cudaError_t e = cudaMemsetAsync(kb_flag, 0, (size_t)(rows / kNormRows) * (ld_data / kNormFrames), s);
   if (e != cudaSuccess) return e;
   if (Bsum && (e = cudaMemsetAsync(den, 0, sizeof(float) * rows, s)) != cudaSuccess) return e;
   NormArgs a{kept, 0, nullptr, lse2, nrot, ld_data, n_data, P, P_plane, nullptr, nullptr, den, Bsum,

@@ -154,6 +154,26 @@ __global__ void __launch_bounds__(kListThreads)
   }
 }
 
+// The whole list of at most kListChunk tiles in one launch.
+__global__ void __launch_bounds__(kListThreads)
+    tile_list_kernel(const uint8_t* __restrict__ live, int n_mtiles, int n_ntiles, int group,
+                     int T, TilePick pick, int32_t* __restrict__ list,
+                     int32_t* __restrict__ count, int32_t* __restrict__ slot_out) {
+  __shared__ int sh[32];
+  const int t0 = threadIdx.x * kListItems;
+  unsigned bits = list_bits(live, n_mtiles, n_ntiles, group, T, t0, pick);
+  const int n = __popc(bits);
+  int pos = block_exclusive(n, sh);
+  if (threadIdx.x == kListThreads - 1) *count = pos + n;
+  while (bits) {
+    const int q = __ffs(bits) - 1;
+    bits &= bits - 1;
+    const int code = raster_code(t0 + q, n_mtiles, n_ntiles, group);
+    if (slot_out) slot_out[code] = pos;
+    list[pos++] = code;
+  }
+}
+
 // Counting sort of the frames by key (their best row tile), stable: per chunk
 // of 1024 frames a histogram H[bin * n_chunks + chunk] ...
 __global__ void __launch_bounds__(1024)
@@ -171,22 +191,33 @@ __global__ void __launch_bounds__(1024)
 
 // ... then, after an exclusive scan of H in (bin, chunk) order, every frame's
 // new position is its bin-and-chunk offset plus its rank among the earlier
-// frames of its chunk with the same key. new_perm[pos] = perm[s].
+// frames of its chunk with the same key. new_perm[pos] = perm[s]. The chunk's
+// warps take their turns: equal keys in a warp by a match, those of earlier warps
+// from a count per bin (a thread's own look through the chunk took 14 us, this 5).
 __global__ void __launch_bounds__(1024)
     sort_scatter_kernel(const int32_t* __restrict__ key, const int32_t* __restrict__ perm,
-                        int64_t n_data, int n_chunks, const int64_t* __restrict__ off,
+                        int64_t n_data, int nbins, int n_chunks, const int64_t* __restrict__ off,
                         int32_t* __restrict__ new_perm) {
-  __shared__ int keys[1024];
-  const int chunk = blockIdx.x;
+  extern __shared__ int seen[];
+  const int chunk = blockIdx.x, lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int64_t s = (int64_t)chunk * 1024 + threadIdx.x;
-  const int k = s < n_data ? key[s] : -1;
-  keys[threadIdx.x] = k;
-  __syncthreads();
-  if (s >= n_data) return;
-  int rank = 0;
-  for (int t = 0; t < (int)threadIdx.x; t++) rank += keys[t] == k;
-  const int64_t pos = off[(int64_t)k * n_chunks + chunk] + rank;
-  new_perm[pos] = perm[s];
+  const bool in = s < n_data;
+  const int k = in ? key[s] : -1 - lane;
+  for (int b = threadIdx.x; b < nbins; b += blockDim.x) seen[b] = 0;
+  const unsigned m = __match_any_sync(0xffffffffu, k);
+  const int first = __ffs(m) - 1;
+  int base = 0;
+  for (int w = 0; w < 32; w++) {
+    __syncthreads();
+    if (w == wid && in && lane == first) {
+      base = seen[k];
+      seen[k] = base + __popc(m);
+    }
+  }
+  base = __shfl_sync(0xffffffffu, base, first);
+  if (!in) return;
+  const int rank = base + __popc(m & ((1u << lane) - 1u));
+  new_perm[off[(int64_t)k * n_chunks + chunk] + rank] = perm[s];
 }
 
 // Frames in the new order: rows of the BF16 frame matrix, the frame totals and
@@ -235,15 +266,43 @@ __global__ void identity_kernel(int32_t* __restrict__ p, int64_t n) {
   if (i < n) p[i] = (int32_t)i;
 }
 
-// lse of the sorted frames back to the original order.
-__global__ void unpermute_lse_kernel(const int32_t* __restrict__ perm, int64_t n_data,
-                                     const double* __restrict__ m_s, const double* __restrict__ s_s,
-                                     double* __restrict__ m, double* __restrict__ s) {
-  const int64_t pos = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (pos >= n_data) return;
-  const int64_t k = perm[pos];
-  m[k] = m_s[pos];
-  s[k] = s_s[pos];
+// After the merge in the internal order: lse back to the frames' order, lse_k for
+// pass 2 in the internal one (lse2, as lse_split_kernel writes it; shift: its shift), and
+// sum_k lse_k added to *total. The frames are consumed: flags[0] = 0, and
+// flags[2] = the device status.
+__global__ void __launch_bounds__(256)
+    lse_finish_kernel(const int32_t* __restrict__ perm, int64_t n_data, int64_t ld_data,
+                      const double* __restrict__ m_s, const double* __restrict__ s_s,
+                      const double* __restrict__ shift, double* __restrict__ m,
+                      double* __restrict__ s, float2* __restrict__ lse2, double* total,
+                      int32_t* flags, const int32_t* status) {
+  __shared__ double red[8];
+  const int64_t pos = (int64_t)blockIdx.x * 256 + threadIdx.x;
+  double l = 0.0;
+  if (pos < n_data) {
+    const int64_t k = perm[pos];
+    const double mv = m_s[pos], sv = s_s[pos];
+    m[k] = mv;
+    s[k] = sv;
+    l = mv + log(sv);
+    const double x = l + (shift ? shift[pos] : 0.0);
+    const double h = rint(x * kGridD) / kGridD;
+    lse2[pos] = make_float2((float)h, (float)(x - h));
+  } else if (pos < ld_data) {
+    lse2[pos] = make_float2(0.f, 0.f);
+  }
+  for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = l;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double t = 0.0;
+    for (int w = 0; w < 8; w++) t += red[w];
+    atomicAdd(total, t);
+    if (blockIdx.x == 0) {
+      flags[0] = 0;
+      flags[2] = *status;
+    }
+  }
 }
 
 cudaError_t launch_tile_list(const uint8_t* live, int n_mtiles, int n_ntiles, int group,
@@ -251,12 +310,19 @@ cudaError_t launch_tile_list(const uint8_t* live, int n_mtiles, int n_ntiles, in
                              int32_t* slot_out, TilePick pick) {
   const int T = n_mtiles * n_ntiles;
   const int nb = (T + kListChunk - 1) / kListChunk;
+  if (nb == 1) {
+    tile_list_kernel<<<1, kListThreads, 0, s>>>(live, n_mtiles, n_ntiles, group, T, pick, list,
+                                                count, slot_out);
+    return cudaGetLastError();
+  }
   tile_count_kernel<<<nb, kListThreads, 0, s>>>(live, n_mtiles, n_ntiles, group, T, pick, scratch);
   tile_scan_kernel<<<1, kListThreads, 0, s>>>(scratch, nb, count);
   tile_write_kernel<<<nb, kListThreads, 0, s>>>(live, n_mtiles, n_ntiles, group, T, pick, scratch, list,
                                                slot_out);
   return cudaGetLastError();
 }
+
+int tile_list_launches(int64_t tiles) { return tiles <= kListChunk ? 1 : 3; }
 
 int64_t tile_list_scratch_entries(int64_t n_mtiles, int64_t n_ntiles) {
   return (n_mtiles * n_ntiles + kListChunk - 1) / kListChunk;
@@ -274,6 +340,9 @@ cudaError_t launch_sort_frames(const int32_t* key, const int32_t* perm, int64_t 
   if (sm > 48 * 1024) {
     e = cudaFuncSetAttribute(sort_hist_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)sm);
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(sort_scatter_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               (int)sm);
     if (e != cudaSuccess) return e;
   }
   sort_hist_kernel<<<n_chunks, 1024, sm, s>>>(key, n_data, nbins, n_chunks, H);
@@ -281,7 +350,7 @@ cudaError_t launch_sort_frames(const int32_t* key, const int32_t* perm, int64_t 
   if (e != cudaSuccess) return e;
   e = launch_scan_counts(H, (int64_t)nbins * n_chunks, off, s);
   if (e != cudaSuccess) return e;
-  sort_scatter_kernel<<<n_chunks, 1024, 0, s>>>(key, perm, n_data, n_chunks, off, new_perm);
+  sort_scatter_kernel<<<n_chunks, 1024, sm, s>>>(key, perm, n_data, nbins, n_chunks, off, new_perm);
   return cudaGetLastError();
 }
 
@@ -305,13 +374,17 @@ cudaError_t launch_identity(int32_t* p, int64_t n, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-cudaError_t launch_unpermute_lse(const int32_t* perm, int64_t n_data, const double* m_s,
-                                 const double* s_s, double* m, double* s, cudaStream_t st) {
-  unpermute_lse_kernel<<<(unsigned)((n_data + 255) / 256), 256, 0, st>>>(perm, n_data, m_s, s_s,
-                                                                        m, s);
+cudaError_t launch_lse_finish(const int32_t* perm, int64_t n_data, int64_t ld_data,
+                              const double* m_s, const double* s_s, const double* shift, double* m,
+                              double* s, float2* lse2, double* total, int32_t* flags,
+                              const int32_t* status, cudaStream_t st) {
+  cudaError_t e = cudaMemsetAsync(total, 0, sizeof(double), st);
+  if (e != cudaSuccess) return e;
+  lse_finish_kernel<<<(unsigned)(ld_data / 256), 256, 0, st>>>(perm, n_data, ld_data, m_s, s_s,
+                                                              shift, m, s, lse2, total, flags,
+                                                              status);
   return cudaGetLastError();
 }
-
 
 // ---------------------------------------------------------------------------
 // Incremental bound between consecutive iterations (same frames).

@@ -39,7 +39,7 @@ __device__ __forceinline__ int block_prefix(int flag, int* warp_tot, int* total)
 }
 
 // Top M in one read of the row (M <= kTopHold), one CTA of 512 threads per row.
-//  * A sample of 512 groups of 8 values spread over the row gives a threshold
+//  * A sample of 512 values, or groups of 8, spread over the row gives a threshold
 //    that about 1.2 to 3 M of the row's values exceed (topm_rank). Each warp then reads a
 //    contiguous sixteenth of the row, several loads in flight and no barrier, and
 //    packs the values above the threshold into a list of its own, in index order.
@@ -65,13 +65,17 @@ static_assert(kTopHold + kTopChunk <= kTopCap, "a chunk fits after a selection")
 constexpr size_t kTopSmem = 2 * sizeof(uint32_t) * kTopPad;
 __device__ __forceinline__ int top_at(int e) { return e + (e >> 4); }
 
-// Rank in the sample of 8 * 512 that leaves at least M of n values above it
-// but for a chance of about 1e-4, or 0 where the lists would be too full (or
-// the row too short to gain): four standard deviations of the sample's count more.
+// Values a thread adds to the sample: eight, or one of a short row.
+__host__ __device__ __forceinline__ int topm_share(int64_t n) { return n >= 4 * kTopChunk ? 8 : 1; }
+
+// Rank in the sample that leaves at least M of n values above it but for a
+// chance of about 1e-4 (four standard deviations of the sample's count more), or 0
+// where the lists would be too full, or the row so short that one selection
+// from all of it costs less.
 int topm_rank(int64_t n, int M) {
-  const double mean = (double)M * kTopChunk / (double)n;
+  const double size = (double)topm_share(n) * kTopThreads, mean = (double)M * size / (double)n;
   const int r = (int)(mean + 4.0 * sqrt(mean) + 4.0);
-  return n >= 4 * kTopChunk && (double)r * n <= 2048.0 * kTopChunk ? r : 0;
+  return n > kTopChunk && (double)r * n <= 2048.0 * size ? r : 0;
 }
 
 // block-wide sum; wt: one of two 16-entry buffers used in turn
@@ -259,14 +263,18 @@ __global__ void __launch_bounds__(kTopThreads, 2)
   int par = 0, cnt = 0;
   bool ok = false;
   if (rank > 0) {
-    // the sample: 8 values every n / 512, the start rounded to a multiple of 8
-    const int64_t at = ((int64_t)threadIdx.x * (n - 8) / (kTopThreads - 1)) & ~(int64_t)7;
+    // the sample: a value every n / 512, or 8 from a multiple of 8 on
+    const int share = topm_share(n);
+    const int64_t at = (int64_t)threadIdx.x * (n - share) / (kTopThreads - 1);
     float v[8];
-    top_load8<VEC>(z, at, n, v);
+    if (share == 8)
+      top_load8<VEC>(z, at & ~(int64_t)7, n, v);
+    else
+      v[0] = z[at];
     uint32_t k[8];
 #pragma unroll
-    for (int i = 0; i < 8; i++) k[i] = order_key(v[i]);
-    const uint32_t T0 = top_key(k, 8, rank, 16, wt, par);
+    for (int i = 0; i < 8; i++) k[i] = i < share ? order_key(v[i]) : 0u;
+    const uint32_t T0 = top_key(k, share, rank, 16, wt, par);
     // the warp's sixteenth, 512 values a step (4 x 4 consecutive ones per lane)
     const int64_t seg = ((int64_t)(n + 15) / 16 + 3) & ~(int64_t)3;
     const int64_t b = wid * seg, end = min((int64_t)n, b + seg);
@@ -495,31 +503,47 @@ __global__ void csr_count_kernel(const int32_t* __restrict__ cand, int64_t n_pai
   atomicAdd(&cnt[j], 1);
 }
 
-// exclusive scan of cnt[0, n) into off[0, n] with one CTA of 1024 threads
-__global__ void csr_scan_kernel(const int32_t* __restrict__ cnt, int64_t n,
-                                int64_t* __restrict__ off) {
-  __shared__ int64_t part[1024];
-  const int64_t per = (n + 1023) / 1024;
-  const int64_t b = threadIdx.x * per, e = min(n, b + per);
-  int64_t s = 0;
-  for (int64_t i = b; i < e; i++) s += cnt[i];
-  part[threadIdx.x] = s;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    int64_t acc = 0;
-    for (int t = 0; t < 1024; t++) {
-      const int64_t v = part[t];
-      part[t] = acc;
-      acc += v;
+// exclusive scan of cnt[0, n) into off[0, n] with one CTA of 1024 threads: four
+// counts a thread and a block scan at a time (a thread's run of all its counts and a serial
+// pass over the 1024 sums took 8 us for 26 counts, 14 us for 7840; now 3 and 8 us)
+__global__ void __launch_bounds__(1024)
+    csr_scan_kernel(const int32_t* __restrict__ cnt, int64_t n, int64_t* __restrict__ off) {
+  __shared__ int64_t part[32];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  int64_t carry = 0;
+  for (int64_t b = 0; b < n; b += 4096) {
+    const int64_t i = b + 4 * threadIdx.x;
+    int64_t v[4], own = 0;
+#pragma unroll
+    for (int u = 0; u < 4; u++) {
+      v[u] = i + u < n ? cnt[i + u] : 0;
+      own += v[u];
     }
-    off[n] = acc;
+    int64_t inc = own;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int64_t y = __shfl_up_sync(0xffffffffu, inc, o);
+      if (lane >= o) inc += y;
+    }
+    __syncthreads();  // part is free
+    if (lane == 31) part[wid] = inc;
+    __syncthreads();
+    int64_t w = part[lane];
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int64_t y = __shfl_up_sync(0xffffffffu, w, o);
+      if (lane >= o) w += y;
+    }
+    const int64_t before = __shfl_sync(0xffffffffu, w, wid > 0 ? wid - 1 : 0);
+    int64_t acc = carry + (wid > 0 ? before : 0) + inc - own;
+#pragma unroll
+    for (int u = 0; u < 4; u++) {
+      if (i + u < n) off[i + u] = acc;
+      acc += v[u];
+    }
+    carry += __shfl_sync(0xffffffffu, w, 31);
   }
-  __syncthreads();
-  int64_t acc = part[threadIdx.x];
-  for (int64_t i = b; i < e; i++) {
-    off[i] = acc;
-    acc += cnt[i];
-  }
+  if (threadIdx.x == 0) off[n] = carry;
 }
 
 __global__ void csr_fill_kernel(const int32_t* __restrict__ cand, int64_t n_pairs, int M,
