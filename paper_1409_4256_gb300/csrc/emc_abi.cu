@@ -25,7 +25,8 @@ struct Layout {
       Kb2, skcnt, skoff, skent, dupsrc, duprank, pixmax, fcn, finvn, fB, kbflag, kbcnt, kblist,
       Kp, perm, perm2, iperm, nsum, nsum_p, cn_p, invn_p, best, lsem_s, lses_s, live, tlist, slot, klist,
       tcount, sortH, sortoff, cgs, cgp, cgqh, cgql, cgqi, cgqlo, cgqf, L2, bias2, Ub, Ub2, Lk, Mk, Mk2, best2,
-      osrc, Dd, Cd, bpm, g4, Ua, Ua2, dcand, pflag, plist, flags, qi, qlo, rotfx, epart, total;
+      osrc, Dd, Cd, bpm, g4, Ua, Ua2, dcand, pflag, plist, flags, qi, qlo, rotfx, epart, rpcnt, rpk,
+      rpw, rpp, rptiles, rpcodes, rpn, total;
   int64_t sort_entries;
   int64_t ntp;  // row tiles rounded up to 128: rows of each half of the bound increments
 };
@@ -185,6 +186,15 @@ Layout make_layout(const emc_config* c) {
   y.kbflag = tc ? take((size_t)ctiles * kbs) : 0;
   y.kbcnt = tc ? take(sizeof(int32_t) * (size_t)ctiles) : 0;
   y.kblist = tc ? take(sizeof(int32_t) * (size_t)ctiles * kbs) : 0;
+  // the M-step from the rows' pairs: pairs, the row tiles that are over and their output tiles
+  const bool rp = c->precision == EMC_PREC_BF16_SPLIT || c->precision == EMC_PREC_FP16_SPLIT;
+  y.rpcnt = rp ? take(sizeof(int32_t) * (size_t)y.rows + 5 * (size_t)(y.rows / 128)) : 0;
+  y.rpk = rp ? take(sizeof(int32_t) * kRowPairs * (size_t)y.rows) : 0;
+  y.rpw = rp ? take(sizeof(float) * kRowPairs * (size_t)y.rows) : 0;
+  y.rpp = rp ? take(sizeof(float) * kRowPairs * (size_t)y.rows) : 0;
+  y.rptiles = rp ? take(sizeof(int32_t) * (size_t)(y.rows / 128)) : 0;
+  y.rpcodes = rp ? take(sizeof(int32_t) * (size_t)(y.rows / 128) * ((y.ld_pix + 255) / 256)) : 0;
+  y.rpn = rp ? take(256) : 0;
   // bound-pruned pass 1: frames in their internal order and the tile bookkeeping
   const bool pr = prune_ok(c);
   const int64_t nmt = y.rows / 128, nnt = y.ld_data / 256;
@@ -205,10 +215,10 @@ Layout make_layout(const emc_config* c) {
   y.lses_s = pr ? take(sizeof(double) * (size_t)y.ld_data) : 0;
   y.live = pr ? take((size_t)nmt * nnt) : 0;
   y.tlist = pr ? take(sizeof(int32_t) * (size_t)nmt * nnt) : 0;
-  // kept scores of the live tiles (no stored scores): places, and a chunk's kept tiles
+  // kept scores of the live tiles (no stored scores): places; a chunk's kept or stored tiles
   const bool keep = pr && !(c->flags & EMC_FLAG_STORE_SCORES);
   y.slot = keep ? take(sizeof(int32_t) * (size_t)nmt * nnt) : 0;
-  y.klist = keep ? take(sizeof(int32_t) * (size_t)(y.chunk_rows / 128) * nnt) : 0;
+  y.klist = pr ? take(sizeof(int32_t) * (size_t)(y.chunk_rows / 128) * nnt) : 0;
   y.tcount = pr ? take(256) : 0;
   y.sortH = pr ? take(sizeof(int32_t) * (size_t)y.sort_entries) : 0;
   y.sortoff = pr ? take(sizeof(int64_t) * (size_t)(y.sort_entries + 1)) : 0;
@@ -743,7 +753,7 @@ struct FrameView {
   const double* cn;
   const float* invn;
   const uint8_t* tile_live;   // stored scores: the contracted tiles of these rows
-  const int32_t* tile_list;   // recomputed scores: the live tiles of these rows
+  const int32_t* tile_list;   // the live tiles of these rows: stored scores; to contract again
   const int32_t* tile_count;
   const float* kept;          // scores pass 1 kept: of these rows' tiles with slot < kept_cap,
   const int32_t* slot;        // listed in kept_list
@@ -751,6 +761,62 @@ struct FrameView {
   const int32_t* kept_count;
   bool kept_all;              // ... which are all the live tiles
 };
+
+// Whether the M-step takes the rows' pairs (pairs.cu): in the split precisions, where
+// posteriors are expected to be sharp and the planes of P cost enough. Posteriors sharpen
+// with the pixels that a frame has: at 0.3 photons a pixel nearly every row tile is
+// over up to about 56^2 pixels' detectors (54^3, 6300 x 4000: M-step 675 against 611 us
+// by planes, the search wasted), few from 60^2 on (3240 x 6000: 365 against 501 us;
+// 64^3, 10860 x 4999: 557 against 840). Every frame has its mass in some row: with more
+// than 4 frames a row the tiles fill up (64^3, 3240 x 30000: 3.04 against
+// 2.80 ms an iteration). Planes below 64 MB (half of the L2; 2^24 elements) cost little (48^3,
+// 3240 x 4500: 78 against 66 us at best, all of the iteration 590).
+// (The stall hook stalls a contraction: it keeps one.)
+bool pairs_ok(const emc_ctx* c, int64_t rows) {
+  return c->lay.rpcnt && c->lay.ld_pix >= 2560 && c->cfg.n_data <= 4 * c->cfg.n_rot &&
+         rows * c->lay.ld_data >= (1 << 24) && !c->tcctl.stall;
+}
+
+RowPairs row_pairs(emc_ctx* c, int64_t rows) {
+  const Layout& y = c->lay;
+  int32_t* cnt = (int32_t*)(c->ws + y.rpcnt);
+  return RowPairs{cnt, cnt + rows, (uint8_t*)(cnt + rows + rows / 128), (int32_t*)(c->ws + y.rpk), (float*)(c->ws + y.rpw),
+                  (float*)(c->ws + y.rpp)};
+}
+
+int update_ntiles(const emc_ctx* c) { return (int)((c->lay.ld_pix + 255) / 256); }
+
+// pass 2's output and constants for rows that start at bias, Bsum
+PassTwo pass_two(const emc_ctx* c, const FrameView* fv, const double* bias, const double* Bsum,
+                 int64_t nrot) {
+  const Layout& y = c->lay;
+  const bool f = is_flu(&c->cfg), g = is_gauss(&c->cfg);
+  PassTwo p{};
+  p.out = g ? 4 : (f ? 5 : (c->cfg.precision == EMC_PREC_FP16_SPLIT ? 3 : 2));
+  p.lse2 = (const float2*)(c->ws + y.lse2);
+  p.bias = g ? bias : nullptr;
+  p.gk = c->gk;
+  p.Bsum = f ? Bsum : nullptr;
+  p.invn = fv && f ? fv->invn : c->flu_invn;
+  p.rows = round_up(nrot, 128);
+  p.nrot = nrot;
+  p.ld_data = y.ld_data;
+  p.n_data = c->cfg.n_data;
+  return p;
+}
+
+ScoreSource kept_source(const FrameView* fv) {
+  return ScoreSource{fv->kept, 0, nullptr, fv->slot, fv->kept_list, fv->kept_count};
+}
+
+// flags (and the Poisson-fluence and Gaussian models' den behind P) as the listed forms of pass 2 start from
+int clear_pass_two(emc_ctx* c, void* P, int64_t rows, uint8_t* kbf, cudaStream_t s) {
+  CU(cudaMemsetAsync(kbf, 0, (size_t)(rows / 128) * (c->lay.ld_data / 64), s));
+  if (is_gauss(&c->cfg) || is_flu(&c->cfg))
+    CU(cudaMemsetAsync((char*)P + P_plane_bytes(&c->cfg, rows, c->lay.ld_data), 0,
+                       sizeof(float) * rows, s));
+  return EMC_OK;
+}
 
 // S, Sref: stored scores of these rows, S frame-major with leading dimension
 // ldS (NULL: recompute from L and bias). Bsum: the rows' B_j (Poisson-fluence model).
@@ -781,10 +847,11 @@ int do_normalize(emc_ctx* c, const void* L, int64_t Lrows, int64_t row_off, cons
       Planes lp{(void*)((const uint16_t*)L + row_off * y.ld_pix), Lrows * y.ld_pix, y.ld_pix};
       Planes pp{P, Prows * y.ld_data, y.ld_data};
       const bool kept = fv && fv->kept;
-      if (kept)
-        CU(launch_normalize_kept(fv->kept, fv->slot, fv->kept_list, fv->kept_count, lse2, rows,
-                                 nrot, y.ld_data, c->cfg.n_data, c->cfg.precision, P,
-                                 Prows * y.ld_data, Bsum, invn, den, kbf, s));
+      if (kept) {
+        if (int st = clear_pass_two(c, P, rows, kbf, s)) return st;
+        CU(launch_normalize_over(kept_source(fv), pass_two(c, fv, bias, Bsum, nrot), RowPairs{},
+                                 nullptr, nullptr, P, Prows * y.ld_data, den, kbf, s));
+      }
       if (!kept || !fv->kept_all)
         CU(launch_tc_normalize(lp, c->cfg.precision, bias, rows, nrot, Kf, y.ld_data,
                                c->cfg.n_data, y.ld_pix, lse_m, lse_s, lse2, pp, c->status, s,
@@ -818,10 +885,11 @@ int do_normalize(emc_ctx* c, const void* L, int64_t Lrows, int64_t row_off, cons
     Planes pp{P, Prows * y.ld_data, y.ld_data};
     float2* lse2 = (float2*)(c->ws + y.lse2);
     const bool kept = fv && fv->kept;
-    if (kept)
-      CU(launch_normalize_kept(fv->kept, fv->slot, fv->kept_list, fv->kept_count, lse2, rows, nrot,
-                               y.ld_data, c->cfg.n_data, c->cfg.precision, P, Prows * y.ld_data,
-                               nullptr, nullptr, nullptr, kbf, s));
+    if (kept) {
+      if (int st = clear_pass_two(c, P, rows, kbf, s)) return st;
+      CU(launch_normalize_over(kept_source(fv), pass_two(c, fv, bias, Bsum, nrot), RowPairs{},
+                               nullptr, nullptr, P, Prows * y.ld_data, nullptr, kbf, s));
+    }
     if (!kept || !fv->kept_all)
       CU(launch_tc_normalize(lp, c->cfg.precision, bias, rows, nrot, Kf, y.ld_data, c->cfg.n_data,
                              y.ld_pix, lse_m, lse_s, lse2, pp, c->status, s, nullptr, nullptr,
@@ -830,11 +898,49 @@ int do_normalize(emc_ctx* c, const void* L, int64_t Lrows, int64_t row_off, cons
   return EMC_OK;
 }
 
+// Pass 2 into the rows' pairs, from stored or kept scores (as do_normalize), and
+// into the planes of P for the row tiles that are over, which it lists.
+int do_normalize_pairs(emc_ctx* c, const void* L, int64_t Lrows, int64_t row_off,
+                       const double* bias, int64_t nrot, const double* lse_m, const double* lse_s,
+                       const float* S, int64_t ldS, const float* Sref, void* P, cudaStream_t s,
+                       const double* Bsum, uint8_t* kbf, const FrameView* fv) {
+  const Layout& y = c->lay;
+  const int64_t rows = round_up(nrot, 128);
+  const RowPairs rp = row_pairs(c, rows);
+  const PassTwo p2 = pass_two(c, fv, bias, Bsum, nrot);
+  float2* lse2 = (float2*)(c->ws + y.lse2);
+  const bool again = !S && !fv->kept_all;  // some live tiles are contracted again
+  const ScoreSource src = S ? ScoreSource{S, ldS, Sref, nullptr, fv ? fv->tile_list : nullptr,
+                                          fv ? fv->tile_count : nullptr}
+                            : kept_source(fv);
+  if (!fv) CU(launch_lse_split(lse_m, lse_s, c->cfg.n_data, y.ld_data, lse2, s, c->flu_cn));
+  CU(launch_pairs_reset(rp, rows, s));
+  if (again) CU(launch_mark_over(fv->tile_list, fv->tile_count, y.ld_data / 256, rp, s));
+  CU(launch_normalize_pairs(src, p2, rp, s));
+  int32_t* tiles = (int32_t*)(c->ws + y.rptiles);
+  int32_t* n = (int32_t*)(c->ws + y.rpn);
+  CU(launch_over_lists(rp, rows, update_ntiles(c), tiles, (int32_t*)(c->ws + y.rpcodes), n, s));
+  if (int st = clear_pass_two(c, P, rows, kbf, s)) return st;
+  float* den = (float*)((char*)P + P_plane_bytes(&c->cfg, rows, y.ld_data));  // (those models')
+  CU(launch_normalize_over(src, p2, rp, tiles, n, P, rows * y.ld_data, den, kbf, s));
+  if (again) {
+    Planes lp{(void*)((const uint16_t*)L + row_off * y.ld_pix), Lrows * y.ld_pix, y.ld_pix};
+    Planes pp{P, rows * y.ld_data, y.ld_data};
+    const bool f = is_flu(&c->cfg);
+    CU(launch_tc_normalize(lp, c->cfg.precision, bias, rows, nrot, fv->K, y.ld_data,
+                           c->cfg.n_data, y.ld_pix, lse_m, lse_s, lse2, pp, c->status, s,
+                           f ? fv->cn : nullptr, f ? Bsum : nullptr, f ? fv->invn : nullptr,
+                           f ? den : nullptr, kbf, fv->tile_list, fv->tile_count, c->tcctl, true));
+  }
+  return EMC_OK;
+}
+
 // kbc, kbl (optional): the non-zero 64-frame blocks of each row tile of P;
-// Kf (optional): frames in emc_iteration's internal order
+// Kf (optional): frames in emc_iteration's internal order; tl, tc (optional): the output tiles to form
 int do_update(emc_ctx* c, const void* P, int64_t Prows, int64_t nrot, float* Num, float* den,
               cudaStream_t s, const int32_t* kbc = nullptr, const int32_t* kbl = nullptr,
-              const uint16_t* Kf = nullptr) {
+              const uint16_t* Kf = nullptr, const int32_t* tl = nullptr,
+              const int32_t* tc = nullptr) {
   const Layout& y = c->lay;
   const int64_t rows = round_up(nrot, 128);
   if (c->cfg.precision == EMC_PREC_FP32) {
@@ -851,14 +957,14 @@ int do_update(emc_ctx* c, const void* P, int64_t Prows, int64_t nrot, float* Num
       CU(launch_tc_update(pp, EMC_PREC_BF16_SPLIT, rows,
                           Kf ? Kf : (is_gauss(&c->cfg) ? c->Kb2 : c->Kb), y.ld_data, y.ld_pix,
                           c->cfg.n_pix, Num, nullptr, c->status, s, kbc, kbl, c->tcctl,
-                          kbc != nullptr && !is_gauss(&c->cfg)));
+                          kbc != nullptr && !is_gauss(&c->cfg), tl, tc));
       const char* tail = (const char*)P + P_plane_bytes(&c->cfg, Prows, y.ld_data);
       CU(cudaMemcpyAsync(den, tail, sizeof(float) * rows, cudaMemcpyDeviceToDevice, s));
     } else {
       // over the listed blocks of a sparse P the update is bound by its output
       CU(launch_tc_update(pp, c->cfg.precision, rows, Kf ? Kf : c->Kb, y.ld_data, y.ld_pix,
                           c->cfg.n_pix, Num, den, c->status, s, kbc, kbl, c->tcctl,
-                          kbc != nullptr));
+                          kbc != nullptr, tl, tc));
     }
   }
   return EMC_OK;
@@ -934,7 +1040,22 @@ int emc_update(emc_ctx* ctx, const void* P, int64_t nrot, float* Num, float* den
   if (!ctx || !P || !Num || !den) return EMC_ERR_ARG;
   if (check_rot_range(ctx, 0, nrot)) return EMC_ERR_ARG;
   if (!ctx->frames_loaded) return EMC_ERR_ARG;
-  return do_update(ctx, P, round_up(nrot, 128), nrot, Num, den, (cudaStream_t)stream);
+  cudaStream_t s = (cudaStream_t)stream;
+  const Layout& y = ctx->lay;
+  const int64_t rows = round_up(nrot, 128);
+  if (!pairs_ok(ctx, rows)) return do_update(ctx, P, rows, nrot, Num, den, s);
+  // the rows' pairs from the planes; what is over on the tensor cores
+  const bool tail = is_gauss(&ctx->cfg) || is_flu(&ctx->cfg);  // den lies behind P
+  const int f16 = ctx->cfg.precision == EMC_PREC_FP16_SPLIT && !tail ? 1 : 0;
+  const RowPairs rp = row_pairs(ctx, rows);
+  int32_t* codes = (int32_t*)(ctx->ws + y.rpcodes);
+  int32_t* n = (int32_t*)(ctx->ws + y.rpn);
+  CU(launch_pairs_reset(rp, rows, s));
+  CU(launch_pairs_from_planes((const uint16_t*)P, rows * y.ld_data, rows, y.ld_data, f16, rp, s));
+  CU(launch_over_lists(rp, rows, update_ntiles(ctx), (int32_t*)(ctx->ws + y.rptiles), codes, n, s));
+  CU(launch_update_pairs(rp, rows, is_gauss(&ctx->cfg) ? ctx->Kb2 : ctx->Kb, f16, y.ld_pix, true,
+                         Num, tail ? nullptr : den, s));
+  return do_update(ctx, P, rows, nrot, Num, den, s, nullptr, nullptr, nullptr, codes, n + 1);
 }
 
 int emc_compress(emc_ctx* ctx, int64_t rot0, int64_t nrot, const float* Num, const float* den,
@@ -1117,7 +1238,21 @@ int emc_iteration(emc_ctx* c, const float* grid_in, float* grid_out, emc_iter_st
     fv.K = Kp;
     fv.cn = cn_p;
     fv.invn = y.invn_p ? (const float*)(c->ws + y.invn_p) : nullptr;
-    if (pruned && S) fv.tile_live = live + (r0 / 128) * nnt;
+    // scores that are held go into the rows' pairs (the collected P_jk are read from the planes)
+    const bool pairs = kbf && !c->collecting && (S || kept) && pairs_ok(c, crows);
+    if (pruned && S) {
+      fv.tile_live = live + (r0 / 128) * nnt;
+      fv.tile_list = (const int32_t*)(c->ws + y.tlist);  // (pass 1's, where a chunk has all rows)
+      fv.tile_count = (const int32_t*)(c->ws + y.tcount);
+      if (pairs && crows < y.rows) {
+        int32_t* klist = (int32_t*)(c->ws + y.klist);
+        CU(launch_tile_list(fv.tile_live, (int)(crows / 128), (int)nnt, 8, klist, tcount,
+                            (int32_t*)(c->ws + y.sortH), s));
+        kernels += tile_list_launches(crows / 128 * nnt);
+        fv.tile_list = klist;
+        fv.tile_count = tcount;
+      }
+    }
     if (kept) {
       // this chunk's live tiles: the kept ones, and those beyond the kept scores' room, whose
       // scores are contracted again (both lists have room for every tile)
@@ -1141,9 +1276,12 @@ int emc_iteration(emc_ctx* c, const float* grid_in, float* grid_out, emc_iter_st
       fv.tile_list = tlist;
       fv.tile_count = tcount + 8;
     }
-    if ((st = do_normalize(c, L, y.rows, r0, bias + r0, nr, lm, ls, Sc, y.rows, Sr, P, crows, s,
-                           c->flu_B ? c->flu_B + r0 : nullptr, kbf, pr ? &fv : nullptr)))
-      return st;
+    const double* Bs = c->flu_B ? c->flu_B + r0 : nullptr;
+    st = pairs ? do_normalize_pairs(c, L, y.rows, r0, bias + r0, nr, lm, ls, Sc, y.rows, Sr, P, s,
+                                    Bs, kbf, pr ? &fv : nullptr)
+               : do_normalize(c, L, y.rows, r0, bias + r0, nr, lm, ls, Sc, y.rows, Sr, P, crows, s,
+                              Bs, kbf, pr ? &fv : nullptr);
+    if (st) return st;
     if (kbf)
       CU(launch_kb_lists(kbf, crows / 128, (int)(y.ld_data / 64), (int32_t*)kbc, (int32_t*)kbl,
                          s));
@@ -1158,7 +1296,17 @@ int emc_iteration(emc_ctx* c, const float* grid_in, float* grid_out, emc_iter_st
       kernels++;
     }
     if (stats) CU(cudaEventRecord(c->ev[4], s));
-    if ((st = do_update(c, P, crows, nr, Num, den, s, kbc, kbl, Kp))) return st;
+    if ((st = do_update(c, P, crows, nr, Num, den, s, kbc, kbl, Kp,
+                        pairs ? (const int32_t*)(c->ws + y.rpcodes) : nullptr,
+                        pairs ? (const int32_t*)(c->ws + y.rpn) + 1 : nullptr)))
+      return st;
+    if (pairs) {
+      // (the compression does not read Num of rows without mass)
+      const bool g = is_gauss(&c->cfg);
+      CU(launch_update_pairs(row_pairs(c, crows), crows, pr ? Kp : (g ? c->Kb2 : c->Kb),
+                             c->cfg.precision == EMC_PREC_FP16_SPLIT && !g ? 1 : 0, y.ld_pix,
+                             false, Num, den, s));
+    }
     if (stats) CU(cudaEventRecord(c->ev[5], s));
     CU(launch_compress(c->geom, (const RotFX*)(c->ws + y.rotfx) + r0, nr, Num, den, c->cfg.compress_mode, gn, gd, s));
     if (stats) CU(cudaEventRecord(c->ev[6], s));
@@ -1166,6 +1314,8 @@ int emc_iteration(emc_ctx* c, const float* grid_in, float* grid_out, emc_iter_st
     // kernel when recomputing in FP32)
     const bool split = pr ? !S && !kept : (S || c->cfg.precision != EMC_PREC_FP32);
     kernels += (split ? 2 : 1) + 2 + (kbf ? 1 : 0);
+    // pairs: their search, the over lists, the rows; the row tiles contracted again marked
+    if (pairs) kernels += 3 + (S || fv.kept_all ? 0 : 1);
     if (stats) {
       // chunk timings need a host wait per chunk; only when stats are asked for
       float a = 0, b = 0, d = 0;

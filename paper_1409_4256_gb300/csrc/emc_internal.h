@@ -47,6 +47,24 @@ constexpr int kCompressGroup = 32;
 constexpr double kCompressExtent = 8.0;
 
 // A block of rows of a (possibly multi-plane) row-major matrix.
+// The rows' non-zero pairs (pairs.cu). cnt, then tile_n and over behind it; the arrays of
+// pairs hold kRowPairs a row. A row tile with a row of more, or more than kTilePairs in
+// all, is over: a pair costs its frame's row out of the L2 (2 ld_pix bytes), a 64-frame block of
+// the planes 128 rows of arithmetic and 64 of those; a tile's pairs cluster in
+// few blocks where they are many (neighbouring rotations share frames), and from
+// about eight a row on the tensor cores take less (by their rates, 2880
+// pixels: 1024 pairs 0.6 us of L2, 8 blocks 0.4 us of BF16).
+constexpr int kRowPairs = 64;
+constexpr int kTilePairs = 8 * 128;
+struct RowPairs {
+  int32_t* cnt;   // [rows] pairs found
+  int32_t* tile_n;  // [rows / 128] pairs found of a row tile
+  uint8_t* over;  // [rows / 128] 1: too many pairs, P is in the planes
+  int32_t* k;     // frame (its position where frames are reordered)
+  float* w;       // what the M-step weighs the frame by: P_jk, or with a fluence P_jk / phi_jk
+  float* p;       // P_jk
+};
+
 struct Planes {
   void* base;            // first row of plane 0
   int64_t plane_stride;  // elements between planes
@@ -114,6 +132,45 @@ cudaError_t launch_normalize_scores_flu(const float* S, int64_t ldS, const float
                                         int64_t n_data, uint16_t* P, int64_t P_plane, float* den,
                                         cudaStream_t s, uint8_t* kb_flag = nullptr,
                                         const uint8_t* tile_live = nullptr);
+// The M-step operand as pairs (pairs.cu): zero cnt and over; find the pairs in
+// planes of P; mark the row tiles of listed (row tile, frame tile) codes; decide on
+// and list the tiles that are over (counts[0]) and their output tiles of the update
+// (counts[1], codes mt * n_ntiles + nt); write Num and den (NULL: not) of the other tiles'
+// rows, empty: also the zeros of rows without mass (else their den alone).
+cudaError_t launch_pairs_reset(const RowPairs& rp, int64_t rows, cudaStream_t s);
+cudaError_t launch_pairs_from_planes(const uint16_t* P, int64_t plane, int64_t rows,
+                                     int64_t ld_data, int f16, const RowPairs& rp, cudaStream_t s);
+cudaError_t launch_mark_over(const int32_t* list, const int32_t* count, int64_t nnt,
+                             const RowPairs& rp, cudaStream_t s);
+cudaError_t launch_over_lists(const RowPairs& rp, int64_t rows, int n_ntiles, int32_t* tiles,
+                              int32_t* codes, int32_t* counts, cudaStream_t s);
+cudaError_t launch_update_pairs(const RowPairs& rp, int64_t rows, const uint16_t* Kb, int kf16,
+                                int64_t ld_pix, bool empty, float* Num, float* den,
+                                cudaStream_t s);
+// Pass 2 into pairs (rp reset before), then into the planes of the tiles that are over
+// (listed with their number; a rp without: of all the listed tiles; kb_flag, and den where the model has one here, zeroed before).
+struct ScoreSource {
+  const float* S;             // stored scores of these rows, ldS between frames; or
+  int64_t ldS;
+  const float* Sref;
+  const int32_t* slot;        // ... (given) the scores that pass 1 kept of the listed tiles
+  const int32_t* tile_list;   // the contracted tiles (NULL: all of them)
+  const int32_t* tile_count;
+};
+struct PassTwo {
+  int out;                  // 2 BF16 planes, 3 FP16 planes, 4 Gaussian, 5 Poisson fluence
+  const float2* lse2;
+  const double* bias;       // Gaussian
+  const float4* gk;
+  const double* Bsum;       // Poisson fluence
+  const float* invn;
+  int64_t rows, nrot, ld_data, n_data;
+};
+cudaError_t launch_normalize_pairs(const ScoreSource& src, const PassTwo& p2, const RowPairs& rp,
+                                   cudaStream_t s);
+cudaError_t launch_normalize_over(const ScoreSource& src, const PassTwo& p2, const RowPairs& rp,
+                                  const int32_t* over_tiles, const int32_t* n_over, void* P,
+                                  int64_t P_plane, float* den, uint8_t* kb_flag, cudaStream_t s);
 // Non-zero P blocks (update over those only): the normalisations set
 // flag[mt * kb_ld + kb] (kb_ld = ld_data / 64) for every 128-row x 64-frame
 // block of P with a non-zero entry; this lists them per row tile.
@@ -214,14 +271,6 @@ cudaError_t launch_normalize_scores(const float* S, int64_t ldS, const float* Sr
                                     int64_t ld_data, int64_t n_data, int precision, void* P,
                                     int64_t P_plane, cudaStream_t s, uint8_t* kb_flag = nullptr,
                                     const uint8_t* tile_live = nullptr);
-// Pass 2 from the kept scores of the listed tiles (codes mt * ld_data / 256 + nt of this
-// chunk's rows, their places in slot); zeroes kb_flag and, for the Poisson-fluence model
-// (Bsum != NULL), den first. lse2: as launch_lse_split writes it.
-cudaError_t launch_normalize_kept(const float* kept, const int32_t* slot, const int32_t* tile_list,
-                                  const int32_t* tile_count, const float2* lse2, int64_t rows,
-                                  int64_t nrot, int64_t ld_data, int64_t n_data, int precision,
-                                  void* P, int64_t P_plane, const double* Bsum, const float* invn,
-                                  float* den, uint8_t* kb_flag, cudaStream_t s);
 cudaError_t launch_loglik_sum(const double* lse_m, const double* lse_s, int64_t n_data,
                               double* out, cudaStream_t s);
 
@@ -263,7 +312,7 @@ cudaError_t launch_tc_normalize(const Planes& L, int precision, const double* bi
                                 uint8_t* kb_flag = nullptr, const int32_t* tile_list = nullptr,
                                 const int32_t* tile_count = nullptr, TcCtl ctl = TcCtl{},
                                 bool prepared = false);  // lse2, kb_flag and den are: see
-                                                         // launch_normalize_kept
+                                                         // launch_normalize_over
 // P planes: hi + lo (BF16 split, FP16 split) or hi only (BF16); FP16 planes
 // carry the scale 2^14. den NULL: not written.
 // kb_cnt, kb_list (optional, from launch_kb_lists): contract only the listed
@@ -274,7 +323,8 @@ cudaError_t launch_tc_update(const Planes& P, int precision, int64_t rows, const
                              int64_t ld_data, int64_t ld_pix, int64_t n_pix, float* Num, float* den,
                              int32_t* status, cudaStream_t s, const int32_t* kb_cnt = nullptr,
                              const int32_t* kb_list = nullptr, TcCtl ctl = TcCtl{},
-                             bool staged = false);
+                             bool staged = false, const int32_t* tile_list = nullptr,
+                             const int32_t* tile_count = nullptr);
 int64_t tc_pass1_tiles(int64_t rows);
 // C (float[rows][ld_data]) = A Kb^T over ld_pix columns, A one plane of rows
 // (a multiple of 128) x ld_pix, Kb [ld_data][ld_pix], both BF16 (or both FP16

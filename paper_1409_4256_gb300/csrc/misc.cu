@@ -1,6 +1,9 @@
 // misc.cu -- frame preparation, log-sum-exp merges and the final division.
+#include <type_traits>
+
 #include "emc_common.cuh"
 #include "emc_internal.h"
+#include "row_pairs.cuh"
 
 namespace emc {
 
@@ -431,6 +434,7 @@ struct NormArgs {
   int64_t kb_ld;
   const uint8_t* tile_live;  // optional: [row tile][256-frame tile] of a pruned pass 1;
                              // a block in a tile not contracted has P = 0
+  RowPairs rp;               // pass 2 into pairs
 };
 
 // A 32-row group of stored scores whose maximum r lies more than 110 below
@@ -449,15 +453,19 @@ struct NormShared {
   float sr[kNormRows / 32][kNormFrames];
   float sg[kNormFrames];
 };
+// (two pairs a row of a block's 64 frames, on average)
+using NormPairs = BlockPairs<2 * kNormRows>;
 
 // One block: rows j0 .., frames k0 .. of P. S: frame k0's scores from row j0 on, ldS to the
 // next frame's; ref: the group maxima of frame k0, ldR to the next group's; tile_on: the tile was
 // contracted; flag (optional): set to 1 or 0 as the block's P is non-zero or not (not written when zero).
-template <int OUT>
+// EMIT: the non-zero pairs go to the rows' lists (a.rp, through np) in place of the planes of P.
+template <int OUT, bool EMIT = false>
 __device__ __forceinline__ void normalize_block(const NormArgs& a, NormShared& sh, int64_t j0,
                                                 int64_t k0, const float* __restrict__ S,
                                                 int64_t ldS, const float* __restrict__ ref,
-                                                int64_t ldR, bool tile_on, uint8_t* flag) {
+                                                int64_t ldR, bool tile_on, uint8_t* flag,
+                                                NormPairs* np = nullptr) {
   auto& tile = sh.tile;
   auto& sl = sh.sl;
   auto& sr = sh.sr;
@@ -474,6 +482,7 @@ __device__ __forceinline__ void normalize_block(const NormArgs& a, NormShared& s
     const int gk = tid & 63;
     const bool live = tile_on && (sr[tid >> 6][gk] - sl[gk].x) - sl[gk].y >= kUnderflowArg;
     if (!__syncthreads_or(live)) {
+      if (EMIT) return;
       if (flag) {
         if (tid == 0) *flag = 0;
         return;
@@ -519,6 +528,7 @@ __device__ __forceinline__ void normalize_block(const NormArgs& a, NormShared& s
 #pragma unroll
   for (int u = 0; u < 8; u++) L[u] = sl[kb + u];
   int nz = 0;
+  if (EMIT) block_pairs_clear(*np);
 #pragma unroll 1
   for (int pass = 0; pass < kNormRows / 32; pass++) {
     const int jj = (tid >> 3) + 32 * pass;
@@ -531,13 +541,14 @@ __device__ __forceinline__ void normalize_block(const NormArgs& a, NormShared& s
       bl = (float)(b - (double)bh);
     }
     const float Bj = (OUT == 5 && row_ok) ? (float)a.Bsum[j] : 0.f;
-    float p[8], dsum = 0.f;
+    float p[8], pr8[8], dsum = 0.f;  // (pr8: P, where p is the operand P / phi)
 #pragma unroll
     for (int u = 0; u < 8; u++) {
       const float d = tile[kb + u][jj ^ sw];
       const float r = sr[pass][kb + u];
       const bool ok = row_ok && k + u < a.n_data;
       const float pr = ok ? __expf(d + ((r - L[u].x) - L[u].y)) : 0.f;
+      pr8[u] = pr;
       if (OUT == 4) {
         dsum += pr;
         const float q = fmaxf(d + ((r - bh) - bl), 0.f);
@@ -548,6 +559,50 @@ __device__ __forceinline__ void normalize_block(const NormArgs& a, NormShared& s
       } else {
         p[u] = pr;
       }
+    }
+    if (EMIT) {
+      // (most warps find no pair)
+      int any = 0;
+#pragma unroll
+      for (int u = 0; u < 8; u++) any |= p[u] != 0.f || pr8[u] != 0.f;
+      if (!__any_sync(0xffffffffu, any)) continue;
+      if (OUT >= 4) {
+        // den as the planes' path sums it: one FP32 atomic per row and 64 frames,
+        // which takes a subnormal sum as zero
+        dsum += __shfl_xor_sync(0xffffffffu, dsum, 1);
+        dsum += __shfl_xor_sync(0xffffffffu, dsum, 2);
+        dsum += __shfl_xor_sync(0xffffffffu, dsum, 4);
+        if (!(dsum >= 0x1p-126f)) {
+#pragma unroll
+          for (int u = 0; u < 8; u++) pr8[u] = 0.f;
+        }
+      }
+      // the weight as the planes would hold it; a pair that only adds to den (an
+      // empty frame's, a weight below the planes' range) counts where den is summed here
+      float w[8];
+      unsigned keep = 0;
+#pragma unroll
+      for (int u = 0; u < 8; u++) {
+        if (OUT == 3) {
+          const float s = p[u] * kP16Scale;
+          const uint16_t h = fp16_bits(s);
+          w[u] = (fp16_val(h) + fp16_val(fp16_bits(s - fp16_val(h)))) * (1.0f / kP16Scale);
+        } else {
+          const float h = bf16_val(bf16_bits(p[u]));
+          w[u] = h + bf16_val(bf16_bits(p[u] - h));
+        }
+        if (w[u] != 0.f || (OUT >= 4 && pr8[u] != 0.f)) keep |= 1u << u;
+      }
+      if (keep) {
+        int place, at = block_pairs_take(*np, jj, __popc(keep), &place);
+        if (at >= 0) {
+#pragma unroll
+          for (int u = 0; u < 8; u++)
+            if (keep >> u & 1u)
+              block_pairs_put(*np, at++, jj, place++, kb + u, w[u], OUT >= 4 ? pr8[u] : w[u]);
+        }
+      }
+      continue;
     }
     if (OUT == 0) {
       float4* o = reinterpret_cast<float4*>(reinterpret_cast<float*>(a.P) + j * a.ld_data + k);
@@ -587,6 +642,10 @@ __device__ __forceinline__ void normalize_block(const NormArgs& a, NormShared& s
       if (kq == 0 && row_ok && dsum > 0.f) atomicAdd(a.den + j, dsum);
     }
   }
+  if (EMIT) {
+    block_pairs_flush(*np, a.rp, j0, k0);
+    return;
+  }
   if (flag) {  // uniform: every thread reaches the barrier
     const int any = __syncthreads_or(nz);
     if (tid == 0) *flag = any ? 1 : 0;
@@ -605,28 +664,126 @@ __global__ void __launch_bounds__(256) normalize_scores_kernel(const NormArgs a)
                                  : nullptr);
 }
 
-// The same over listed tiles whose scores pass 1 kept by tile (S: the kept
-// scores): a block's scores are 32 KB in one piece. 96^3, Poisson fluence,
-// 25680 x 10007, 75% of the tiles live: 4.78 ms contracted again, 0.21 ms so.
+constexpr int list_ctas(int out) { return out >= 4 ? 4 : 5; }  // an SM: 64 and 48 registers
+
+// Stored scores of every tile into pairs; row tiles run fastest, so that most
+// blocks of a tile that is over leave at once.
 template <int OUT>
-__global__ void __launch_bounds__(256)
-    normalize_kept_kernel(const NormArgs a, const int32_t* __restrict__ slot,
-                          const int32_t* __restrict__ tile_list,
-                          const int32_t* __restrict__ tile_count) {
+__global__ void __launch_bounds__(256, list_ctas(OUT))
+    normalize_pairs_kernel(const NormArgs a, unsigned nmt) {
   __shared__ NormShared sh;
-  const int n = 4 * *tile_count, nnt = (int)(a.ld_data >> 8);
-  for (int t = blockIdx.x; t < n; t += gridDim.x) {
-    const int code = tile_list[t >> 2], q = t & 3;
-    const int64_t j0 = (int64_t)(code / nnt) * kNormRows;
-    const int64_t k0 = (int64_t)(code % nnt) * 256 + q * kNormFrames;
-    const float* tile = a.S + slot[code] * kKeptFloats;
-    normalize_block<OUT>(a, sh, j0, k0, tile + q * (kNormFrames * kNormRows), kNormRows,
-                         tile + 256 * kNormRows + q * kNormFrames, 256, true,
-                         a.kb_flag + (j0 >> 7) * a.kb_ld + (k0 >> 6));
+  __shared__ NormPairs pairs;
+  const int64_t mt = blockIdx.x % nmt, j0 = mt * kNormRows;
+  const int64_t k0 = (int64_t)(blockIdx.x / nmt) * kNormFrames;
+  // (over changes meanwhile; the block agrees on it at its first barrier)
+  const bool over = *reinterpret_cast<volatile uint8_t*>(a.rp.over + mt);
+  normalize_block<OUT, true>(a, sh, j0, k0, a.S + k0 * a.ldS + j0, a.ldS,
+                             a.Sref + (j0 >> 5) * a.ld_data + k0, a.ld_data, !over, nullptr, &pairs);
+}
+
+// Stored scores of every tile into the planes of the row tiles that are over.
+template <int OUT>
+__global__ void __launch_bounds__(256, list_ctas(OUT))
+    normalize_over_kernel(const NormArgs a, const int32_t* __restrict__ tiles,
+                          const int32_t* __restrict__ n_tiles) {
+  __shared__ NormShared sh;
+  const int nb = (int)a.kb_ld;
+  const int64_t n = (int64_t)*n_tiles * nb;
+  for (int64_t t = blockIdx.x; t < n; t += gridDim.x) {
+    const int64_t mt = tiles[t / nb], b = t % nb, j0 = mt * kNormRows, k0 = b * kNormFrames;
+    normalize_block<OUT>(a, sh, j0, k0, a.S + k0 * a.ldS + j0, a.ldS,
+                         a.Sref + (j0 >> 5) * a.ld_data + k0, a.ld_data, true,
+                         a.kb_flag + mt * a.kb_ld + b);
     __syncthreads();  // the shared block is rewritten
   }
 }
 
+// Both over listed tiles (codes mt * ld_data / 256 + nt), persistent. slot: scores that
+// pass 1 kept by tile, a block's 32 KB in one piece (96^3, Poisson fluence, 25680 x 10007, 75% of
+// the tiles live: 4.78 ms contracted again, 0.18 ms so); else stored ones (64^3,
+// 8% of the tiles live: 266 us by a CTA for every block, 65 us so).
+// a.rp.over given: pairs not for a tile found to be over, planes only for those.
+// Pairs visit the blocks spread over the whole list, so that flat posteriors are
+// found out within the first blocks of each row tile; the rest then goes by in
+// batches whose flags are read at once (64^3 at 0.03 photons a pixel, every tile over:
+// 383 us in list order, 64 us so).
+constexpr int kNormSpread = 1024;
+template <int OUT, bool EMIT = false>
+__global__ void __launch_bounds__(256, list_ctas(OUT))
+    normalize_list_kernel(const NormArgs a, const int32_t* __restrict__ slot,
+                          const int32_t* __restrict__ tile_list,
+                          const int32_t* __restrict__ tile_count,
+                          const int32_t* __restrict__ n_over) {
+  if (n_over && *n_over == 0) return;
+  __shared__ NormShared sh;
+  __shared__ int picked[256], picked_code[256], npick;
+  __shared__ typename std::conditional<EMIT, NormPairs, int>::type pairs;
+  const int n = 4 * *tile_count, nnt = (int)(a.ld_data >> 8);
+  const int step = (n + kNormSpread - 1) / kNormSpread;
+  const int total = EMIT ? kNormSpread * step : n;
+  // the first blocks alone, the rest by batches
+  const int most = min(256, max(1, n / (4 * (int)gridDim.x)));
+  int batch = 1;
+  const volatile uint8_t* over = a.rp.over;
+  auto item = [&](int64_t i) {  // -1: none
+    if (i >= total) return -1;
+    const int x = EMIT ? (int)(i % kNormSpread) * step + (int)(i / kNormSpread) : (int)i;
+    return x < n ? x : -1;
+  };
+  auto code_of = [&](int x) { return tile_list[x >> 2]; };
+  for (int64_t done = 0, next; done < total; done = next) {
+    next = done + (int64_t)gridDim.x * batch;
+    const int64_t base = done + (int64_t)blockIdx.x * batch;  // a CTA's blocks are neighbours
+    int m = batch;
+    const bool pick = over && batch >= 4;
+    if (pick) {
+      if (threadIdx.x == 0) npick = 0;
+      __syncthreads();
+      if (threadIdx.x < batch) {
+        const int x = item(base + threadIdx.x);
+        const int code = x >= 0 ? code_of(x) : 0;
+        if (x >= 0 && (over[code / nnt] != 0) != EMIT) {
+          const int at = atomicAdd(&npick, 1);
+          picked[at] = x;
+          picked_code[at] = code;
+        }
+      }
+      __syncthreads();
+      m = npick;
+    }
+    for (int b = 0; b < m; b++) {
+      const int x = pick ? picked[b] : item(base + b);
+      if (x < 0) continue;
+      const int code = pick ? picked_code[b] : code_of(x), q = x & 3;
+      const int64_t j0 = (int64_t)(code / nnt) * kNormRows;
+      const int64_t k0 = (int64_t)(code % nnt) * 256 + q * kNormFrames;
+      bool on = true;
+      if (over && (EMIT || !pick)) {
+        // (over changes while pairs are found; the block agrees on it at its first barrier)
+        const bool ov = over[code / nnt] != 0;
+        if (EMIT)
+          on = !ov;
+        else if (!ov)
+          continue;
+      }
+      const float *S = a.S + k0 * a.ldS + j0, *ref = a.Sref + (j0 >> 5) * a.ld_data + k0;
+      int64_t ldS = a.ldS, ldR = a.ld_data;
+      if (slot) {
+        const float* tile = a.S + slot[code] * kKeptFloats;
+        S = tile + q * (kNormFrames * kNormRows);
+        ldS = kNormRows;
+        ref = tile + 256 * kNormRows + q * kNormFrames;
+        ldR = 256;
+      }
+      normalize_block<OUT, EMIT>(a, sh, j0, k0, S, ldS, ref, ldR, on,
+                                 EMIT ? nullptr : a.kb_flag + (j0 >> 7) * a.kb_ld + (k0 >> 6),
+                                 EMIT ? reinterpret_cast<NormPairs*>(&pairs) : nullptr);
+      __syncthreads();  // the shared block is rewritten
+    }
+    if (pick) __syncthreads();  // and the picked ones
+    batch = most;
+  }
+}
 
 // rows: multiple of 128 (the stored-score blocks are); ld_data: multiple of 256
 cudaError_t launch_normalize_scores(const float* S, int64_t ldS, const float* Sref,
@@ -686,31 +843,71 @@ cudaError_t launch_normalize_scores_flu(const float* S, int64_t ldS, const float
   return cudaGetLastError();
 }
 
-cudaError_t launch_normalize_kept(const float* kept, const int32_t* slot, const int32_t* tile_list,
-                                  const int32_t* tile_count, const float2* lse2, int64_t rows,
-                                  int64_t nrot, int64_t ld_data, int64_t n_data, int precision,
-                                  void* P, int64_t P_plane, const double* Bsum, const float* invn,
-                                  float* den, uint8_t* kb_flag, cudaStream_t s) {
-  if (!kb_flag || (Bsum && (!invn || !den))) return cudaErrorInvalidValue;
-  cudaError_t e = cudaMemsetAsync(kb_flag, 0, (size_t)(rows / kNormRows) * (ld_data / kNormFrames), s);
-  if (e != cudaSuccess) return e;
-  if (Bsum && (e = cudaMemsetAsync(den, 0, sizeof(float) * rows, s)) != cudaSuccess) return e;
-  NormArgs a{kept, 0, nullptr, lse2, nrot, ld_data, n_data, P, P_plane, nullptr, nullptr, den, Bsum,
-             invn};
-  a.kb_flag = kb_flag;
-  a.kb_ld = ld_data / kNormFrames;
+namespace {
+
+NormArgs pass_two_args(const ScoreSource& src, const PassTwo& p2) {
+  NormArgs a{src.S, src.ldS, src.Sref, p2.lse2, p2.nrot, p2.ld_data, p2.n_data,
+             nullptr, 0, p2.bias, p2.gk, nullptr, p2.Bsum, p2.invn};
+  a.kb_ld = p2.ld_data / kNormFrames;
+  return a;
+}
+
+unsigned norm_grid(int out) {
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  const unsigned grid = 6 * (unsigned)sms;  // CTAs that fit (34 KB each); the count is on the device
-  if (Bsum)
-    normalize_kept_kernel<5><<<grid, 256, 0, s>>>(a, slot, tile_list, tile_count);
-  else if (precision == EMC_PREC_FP16_SPLIT)
-    normalize_kept_kernel<3><<<grid, 256, 0, s>>>(a, slot, tile_list, tile_count);
-  else
-    normalize_kept_kernel<2><<<grid, 256, 0, s>>>(a, slot, tile_list, tile_count);
+  return (unsigned)(list_ctas(out) * sms);
+}
+
+}  // namespace
+
+#define EMC_PASS_TWO(KERNEL, MORE, GRID, ...)                                      \
+  switch (p2.out) {                                                                \
+    case 2: KERNEL<2 MORE><<<GRID, 256, 0, s>>>(a, __VA_ARGS__); break;            \
+    case 3: KERNEL<3 MORE><<<GRID, 256, 0, s>>>(a, __VA_ARGS__); break;            \
+    case 4: KERNEL<4 MORE><<<GRID, 256, 0, s>>>(a, __VA_ARGS__); break;            \
+    case 5: KERNEL<5 MORE><<<GRID, 256, 0, s>>>(a, __VA_ARGS__); break;            \
+    default: return cudaErrorInvalidValue;                                         \
+  }
+#define EMC_EMIT , true
+#define EMC_PLAIN
+
+cudaError_t launch_normalize_pairs(const ScoreSource& src, const PassTwo& p2, const RowPairs& rp,
+                                   cudaStream_t s) {
+  NormArgs a = pass_two_args(src, p2);
+  a.rp = rp;
+  if (src.tile_list) {
+    EMC_PASS_TWO(normalize_list_kernel, EMC_EMIT, norm_grid(p2.out), src.slot, src.tile_list,
+                 src.tile_count, nullptr)
+  } else {
+    const unsigned nmt = (unsigned)(p2.rows / kNormRows);
+    const int64_t grd = (int64_t)nmt * (p2.ld_data / kNormFrames);
+    if (grd > INT32_MAX) return cudaErrorInvalidValue;
+    EMC_PASS_TWO(normalize_pairs_kernel, EMC_PLAIN, (unsigned)grd, nmt)
+  }
   return cudaGetLastError();
 }
+
+cudaError_t launch_normalize_over(const ScoreSource& src, const PassTwo& p2, const RowPairs& rp,
+                                  const int32_t* over_tiles, const int32_t* n_over, void* P,
+                                  int64_t P_plane, float* den, uint8_t* kb_flag, cudaStream_t s) {
+  NormArgs a = pass_two_args(src, p2);
+  a.P = P;
+  a.P_plane = P_plane;
+  a.den = den;
+  a.kb_flag = kb_flag;
+  a.rp = rp;
+  if (src.tile_list) {
+    EMC_PASS_TWO(normalize_list_kernel, EMC_PLAIN, norm_grid(p2.out), src.slot, src.tile_list,
+                 src.tile_count, n_over)
+  } else {
+    EMC_PASS_TWO(normalize_over_kernel, EMC_PLAIN, norm_grid(p2.out), over_tiles, n_over)
+  }
+  return cudaGetLastError();
+}
+#undef EMC_PASS_TWO
+#undef EMC_EMIT
+#undef EMC_PLAIN
 
 // Per row tile mt (one warp each): the indices of the 64-frame blocks whose
 // flag is set, in order, into list[mt * kb_ld ..] and their number into cnt[mt]

@@ -1062,7 +1062,8 @@ cudaError_t launch_tc_normalize(const Planes& L, int precision, const double* bi
 cudaError_t launch_tc_update(const Planes& P, int precision, int64_t rows, const uint16_t* Kb,
                              int64_t ld_data, int64_t ld_pix, int64_t n_pix, float* Num, float* den,
                              int32_t* status, cudaStream_t s, const int32_t* kb_cnt,
-                             const int32_t* kb_list, TcCtl ctl, bool staged) {
+                             const int32_t* kb_list, TcCtl ctl, bool staged,
+                             const int32_t* tile_list, const int32_t* tile_count) {
   const int nterms = precision == EMC_PREC_BF16 ? 1 : 2;
   const bool f16 = precision == EMC_PREC_FP16_SPLIT;
   CUtensorMap mA, mB;
@@ -1084,6 +1085,8 @@ cudaError_t launch_tc_update(const Planes& P, int precision, int64_t rows, const
   a.kb_cnt = kb_cnt;
   a.kb_list = kb_list;
   a.kb_ld = (int)(ld_data / 64);
+  a.tile_list = tile_list;
+  a.tile_count = tile_list ? tile_count : nullptr;
   a.status = status;
   if (ctl.wait_ns) a.wait_ns = ctl.wait_ns;
   a.stall = ctl.stall;
