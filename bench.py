@@ -772,10 +772,10 @@ MEASURED_TRAFFIC_EMC64 = {
     # pass 1 of a steady pruned iteration: the increments' product, the
     # hi-plane bound over the few listed pairs and the exact pass over the
     # live tiles; dense: the single three-plane launch of the first iteration
-    "pass1_pruned": 0.331e9 + 0.0002e9 + 2.02e9,
-    "pass1_dense": 6.650e9 + 4.247e9,
-    "compress": 0.325e9,
-    "expand": 1.668e9,
+    "pass1_pruned": 0.332e9 + 0.00003e9 + 1.957e9,
+    "pass1_dense": 6.713e9 + 4.247e9,
+    "compress": 0.272e9,
+    "expand": 1.673e9,
 }
 
 
@@ -863,9 +863,9 @@ def phase_rooflines(precision, n_pix, ld_pix, n_rot, n_data, phases, pass1_roof)
     out["expand"] = {"bound": "hbm", "unit": "GB/s", "achieved": b / (ms * 1e-3) / 1e9,
                      "peak": hbm, "peak_source": f"{pk_src} copy bandwidth", "ms": ms,
                      "algorithmic_bytes": b, "per_unit": f"{planes * esz} B of L per (i, j)",
-                     "limiter": "instruction issue and gather latency",
-                     "limiter_source": "ncu, 8192-frame case: 64% issue-active, long-scoreboard "
-                                       "stalls first, DRAM at 17%"}
+                     "limiter": "L1 (LSU) wavefronts, instruction issue and gather latency",
+                     "limiter_source": "ncu, 8192-frame case: LSU wavefronts 62%, 63% "
+                                       "issue-active, long-scoreboard stalls first, DRAM at 19%"}
     ms = phases["ms_compress"]
     b = 4 * n_rot * ld_pix  # Num read
     out["compress"] = {"bound": "hbm", "unit": "GB/s", "achieved": b / (ms * 1e-3) / 1e9,
@@ -873,9 +873,9 @@ def phase_rooflines(precision, n_pix, ld_pix, n_rot, n_data, phases, pass1_roof)
                        "algorithmic_bytes": b, "per_unit": "4 B of Num per (i, j)",
                        "limiter": "L1 / shared-memory (LSU) wavefronts of the corner merging "
                                   "and the L2 reductions",
-                       "limiter_frac": 0.86,
+                       "limiter_frac": 0.92,
                        "limiter_source": "ncu l1tex__data_pipe_lsu_wavefronts, 8192-frame case "
-                                         "(DRAM at 2%, FP64 pipe 70% for the conversions)"}
+                                         "(DRAM at 2%, issue 66%, FP64 pipe 37%)"}
     out["pass1"] = dict(pass1_roof, ms=phases["ms_loglik"])
     for k in ("expand", "compress"):
         out[k]["frac"] = out[k]["achieved"] / out[k]["peak"]

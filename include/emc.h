@@ -128,8 +128,9 @@ typedef enum emc_compress_mode {
                                    scores by a contraction of the hi plane alone
                                    (|S - S_hi| <= N_k/16 + 1 for the BF16
                                    split, N_k/128 + 1 for the FP16 split),
-                                   then contracts exactly (in pass 1, and in a
-                                   recomputing pass 2) only the tiles
+                                   then contracts exactly (in pass 1, and in
+                                   pass 2 where its scores are neither stored
+                                   nor kept) only the tiles
                                    that can hold a score within 110 of their
                                    frames' maxima. The others have P = 0 in
                                    FP32 and no weight in lse at FP64 precision,
@@ -419,7 +420,8 @@ int emc_finalize(emc_ctx* ctx, const double* g_num, const double* g_den, const f
  * rotation chunks of cfg.rot_chunk. grid_out may not alias grid_in. With the
  * tensor-core forms the M-step contracts only the 128-rotation x 64-frame
  * blocks of P that the normalisation found non-zero (most underflow to exact
- * zeros); the result is that of the full contraction.
+ * zeros), or, where few of a rotation's P are not zero, sums those pairs'
+ * frames; the result is that of the full contraction.
  * stats (host, may be NULL) is filled after the call synchronises `stream`. */
 int emc_iteration(emc_ctx* ctx, const float* grid_in, float* grid_out, emc_iter_stats* stats,
                   emc_stream stream);
