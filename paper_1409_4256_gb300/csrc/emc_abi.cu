@@ -1,6 +1,7 @@
 // emc_abi.cu -- the C ABI of include/emc.h: context, workspace layout,
 // argument checks and the stream-ordered step calls.
 #include <math.h>
+#include <pthread.h>
 #include <stdlib.h>
 #include <string.h>
 
@@ -26,7 +27,7 @@ struct Layout {
       Kp, perm, perm2, iperm, nsum, nsum_p, cn_p, invn_p, best, lsem_s, lses_s, live, tlist, slot, klist,
       tcount, sortH, sortoff, cgs, cgp, cgqh, cgql, cgqi, cgqlo, cgqf, L2, bias2, Ub, Ub2, Lk, Mk, Mk2, best2,
       osrc, Dd, Cd, bpm, g4, Ua, Ua2, dcand, pflag, plist, flags, qi, qlo, rotfx, epart, rpcnt, rpk,
-      rpw, rpp, rptiles, rpcodes, rpn, total;
+      rpw, rpp, rptiles, rpcodes, rpn, upnz, total;
   int64_t sort_entries;
   int64_t ntp;  // row tiles rounded up to 128: rows of each half of the bound increments
 };
@@ -195,6 +196,8 @@ Layout make_layout(const emc_config* c) {
   y.rptiles = rp ? take(sizeof(int32_t) * (size_t)(y.rows / 128)) : 0;
   y.rpcodes = rp ? take(sizeof(int32_t) * (size_t)(y.rows / 128) * ((y.ld_pix + 255) / 256)) : 0;
   y.rpn = rp ? take(256) : 0;
+  // FP32: the frames that the update contracts, a bit for each 64 rows
+  y.upnz = tc ? 0 : take(sizeof(uint32_t) * (size_t)(y.rows / 64) * (y.ld_data / 32));
   // bound-pruned pass 1: frames in their internal order and the tile bookkeeping
   const bool pr = prune_ok(c);
   const int64_t nmt = y.rows / 128, nnt = y.ld_data / 256;
@@ -303,6 +306,34 @@ struct emc_ctx {
   cudaEvent_t ev[8];
   int kernels;  // launches made by the last emc_iteration
   TcCtl tcctl;  // bounded waits of the tensor-core launches (emc_ctx_set_wait_limit)
+  pthread_mutex_t scratch_mu;  // Scratch
+  cudaEvent_t scratch_done;
+};
+
+// The step calls that take scratch of the context while other calls on it may run (emc_expand,
+// emc_update, and the iterations, which use the same): one at a time, in the order
+// of the calls, whichever streams and threads they come from. A captured call cannot wait
+// for what ran before the capture, so it takes its scratch as the graph is ordered (captured()).
+class Scratch {
+ public:
+  Scratch(emc_ctx* c, cudaStream_t s) : c_(c), s_(s) {
+    pthread_mutex_lock(&c->scratch_mu);
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    captured_ = cudaStreamIsCapturing(s, &st) == cudaSuccess && st != cudaStreamCaptureStatusNone;
+    if (!captured_) cudaStreamWaitEvent(s, c->scratch_done, 0);
+  }
+  ~Scratch() {
+    if (!captured_) cudaEventRecord(c_->scratch_done, s_);
+    pthread_mutex_unlock(&c_->scratch_mu);
+  }
+  Scratch(const Scratch&) = delete;
+  Scratch& operator=(const Scratch&) = delete;
+  bool captured() const { return captured_; }
+
+ private:
+  emc_ctx* c_;
+  cudaStream_t s_;
+  bool captured_;
 };
 
 // The internal frame order the last iteration found (perm2) becomes the
@@ -565,9 +596,12 @@ static int ctx_create(const emc_config* cfg, const double* q, const double* quat
                         s) == cudaSuccess;
   ok &= cudaStreamSynchronize(s) == cudaSuccess;  // host staging buffers go out of scope
   for (int e = 0; e < 8 && ok; e++) ok &= cudaEventCreate(&c->ev[e]) == cudaSuccess;
+  ok = ok && cudaEventCreateWithFlags(&c->scratch_done, cudaEventDisableTiming) == cudaSuccess;
+  ok = ok && pthread_mutex_init(&c->scratch_mu, nullptr) == 0;
   if (!ok) {
     for (int e = 0; e < 8; e++)
       if (c->ev[e]) cudaEventDestroy(c->ev[e]);
+    if (c->scratch_done) cudaEventDestroy(c->scratch_done);
     free(c);
     return EMC_ERR_CUDA;
   }
@@ -579,6 +613,8 @@ int emc_ctx_destroy(emc_ctx* ctx) {
   if (!ctx) return EMC_ERR_ARG;
   for (int e = 0; e < 8; e++)
     if (ctx->ev[e]) cudaEventDestroy(ctx->ev[e]);
+  cudaEventDestroy(ctx->scratch_done);
+  pthread_mutex_destroy(&ctx->scratch_mu);
   free(ctx);
   return EMC_OK;
 }
@@ -944,9 +980,8 @@ int do_update(emc_ctx* c, const void* P, int64_t Prows, int64_t nrot, float* Num
   const Layout& y = c->lay;
   const int64_t rows = round_up(nrot, 128);
   if (c->cfg.precision == EMC_PREC_FP32) {
-    // (pass 1's per-tile sums, consumed by now, hold the bits of the frames to contract)
     CU(launch_simt_update((const float*)P, y.ld_data, rows, c->Kb, y.ld_pix, c->cfg.n_pix,
-                          (uint32_t*)(c->ws + y.part_s), Num, den, s));
+                          (uint32_t*)(c->ws + y.upnz), Num, den, s));
   } else {
     Planes pp{(void*)P, Prows * y.ld_data, y.ld_data};
     if (is_gauss(&c->cfg) || is_flu(&c->cfg)) {
@@ -983,6 +1018,7 @@ int emc_expand(emc_ctx* ctx, const float* grid, int64_t rot0, int64_t nrot, void
                emc_stream stream) {
   if (!ctx || !grid || !L || !bias) return EMC_ERR_ARG;
   if (check_rot_range(ctx, rot0, nrot)) return EMC_ERR_ARG;
+  Scratch scratch(ctx, (cudaStream_t)stream);
   return do_expand(ctx, grid, rot0, nrot, L, bias, (cudaStream_t)stream);
 }
 
@@ -1043,7 +1079,12 @@ int emc_update(emc_ctx* ctx, const void* P, int64_t nrot, float* Num, float* den
   cudaStream_t s = (cudaStream_t)stream;
   const Layout& y = ctx->lay;
   const int64_t rows = round_up(nrot, 128);
-  if (!pairs_ok(ctx, rows)) return do_update(ctx, P, rows, nrot, Num, den, s);
+  // (the dense tensor-core contraction takes no scratch, and needs no order)
+  if (ctx->cfg.precision != EMC_PREC_FP32 && !pairs_ok(ctx, rows))
+    return do_update(ctx, P, rows, nrot, Num, den, s);
+  Scratch scratch(ctx, s);
+  if (!pairs_ok(ctx, rows) || scratch.captured())
+    return do_update(ctx, P, rows, nrot, Num, den, s);
   // the rows' pairs from the planes; what is over on the tensor cores
   const bool tail = is_gauss(&ctx->cfg) || is_flu(&ctx->cfg);  // den lies behind P
   const int f16 = ctx->cfg.precision == EMC_PREC_FP16_SPLIT && !tail ? 1 : 0;
@@ -1086,6 +1127,7 @@ int emc_iteration(emc_ctx* c, const float* grid_in, float* grid_out, emc_iter_st
   if (!c || !grid_in || !grid_out || grid_in == grid_out) return EMC_ERR_ARG;
   if (!c->frames_loaded) return EMC_ERR_ARG;
   cudaStream_t s = (cudaStream_t)stream;
+  Scratch scratch(c, s);
   const Layout& y = c->lay;
   const int64_t n_rot = c->cfg.n_rot;
   // pruned contexts alternate between two L and bias buffers: the last
@@ -1521,6 +1563,7 @@ int emc_sparse_iteration(emc_ctx* c, const float* grid_in, float* grid_out, emc_
   if (!c || !grid_in || !grid_out || grid_in == grid_out) return EMC_ERR_ARG;
   if (!c->frames_loaded || !c->cand_loaded) return EMC_ERR_ARG;
   cudaStream_t s = (cudaStream_t)stream;
+  Scratch scratch(c, s);
   const Layout& y = c->lay;
   // pruned contexts: the buffer the last emc_iteration did not write, so that
   // its L stays for the next one's incremental bound

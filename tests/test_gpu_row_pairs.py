@@ -105,3 +105,41 @@ def test_iteration_equals_planes(model, precision, stored, D, photons, chunk):
     rows = torch.bincount(tidx[tprob > 0].long(), minlength=a.sizes_all.rows).view(-1, 128)
     over = (rows.amax(1) > 64) | (rows.sum(1) > 1024)
     assert bool(over.any()) and bool((~over & (rows.sum(1) > 0)).any())
+
+
+@pytest.mark.parametrize("precision", ["bf16_split", "fp32"])
+def test_updates_on_several_streams(precision):
+    """emc_update takes scratch of the context: calls on two streams at a time give what
+    the same calls give one after the other, bit for bit."""
+    import torch
+    from paper_1409_4256_gb300 import emc, synth
+    det = synth.make_detector(60, 16)
+    quat, w = emc.quat_generate(4)
+    n_rot, n_data = quat.shape[0], 5003
+    ctx = emc.Context(16, det.q, quat, w, n_data, precision=precision)
+    rng = np.random.default_rng(6)
+    K = rng.poisson(0.7, size=(n_data, det.q.shape[0])).astype(np.int32)
+    ctx.set_frames(torch.as_tensor(K, device="cuda"))
+    b = ctx.buffer_sizes(n_rot)
+    planes = []
+    for _ in range(2):
+        P = torch.zeros((b.rows, ctx.ld_data), device="cuda")
+        for _ in range(2):
+            k = torch.as_tensor(rng.integers(0, n_data, n_rot), device="cuda")
+            P[torch.arange(n_rot, device="cuda"), k] = torch.as_tensor(
+                0.1 + rng.random(n_rot).astype(np.float32), device="cuda")
+        if precision != "fp32":
+            P = torch.stack([P.to(torch.bfloat16), torch.zeros_like(P).to(torch.bfloat16)])
+        planes.append(P.contiguous().view(torch.uint8).reshape(-1))
+    want = [ctx.update(P, n_rot) for P in planes]
+    torch.cuda.synchronize()
+    streams = [torch.cuda.Stream(), torch.cuda.Stream()]
+    got = []
+    for i in range(6):
+        with torch.cuda.stream(streams[i % 2]):
+            got.append(ctx.update(planes[i % 2], n_rot, stream=streams[i % 2]))
+    torch.cuda.synchronize()
+    for i, (Num, den) in enumerate(got):
+        assert torch.equal(Num[:n_rot], want[i % 2][0][:n_rot])
+        assert torch.equal(den[:n_rot], want[i % 2][1][:n_rot])
+    assert ctx.status() == 0
