@@ -313,7 +313,8 @@ struct emc_ctx {
 // The step calls that take scratch of the context while other calls on it may run (emc_expand,
 // emc_update, and the iterations, which use the same): one at a time, in the order
 // of the calls, whichever streams and threads they come from. A captured call cannot wait
-// for what ran before the capture, so it takes its scratch as the graph is ordered (captured()).
+// for what ran before the capture, so emc_update then takes none (captured()): the planes of P, or
+// in FP32 every frame (64^3, 3240 x 2000, flat posteriors: 1033 us either way).
 class Scratch {
  public:
   Scratch(emc_ctx* c, cudaStream_t s) : c_(c), s_(s) {
@@ -1083,8 +1084,13 @@ int emc_update(emc_ctx* ctx, const void* P, int64_t nrot, float* Num, float* den
   if (ctx->cfg.precision != EMC_PREC_FP32 && !pairs_ok(ctx, rows))
     return do_update(ctx, P, rows, nrot, Num, den, s);
   Scratch scratch(ctx, s);
-  if (!pairs_ok(ctx, rows) || scratch.captured())
-    return do_update(ctx, P, rows, nrot, Num, den, s);
+  if (ctx->cfg.precision == EMC_PREC_FP32) {  // captured: every frame, without the bits
+    CU(launch_simt_update((const float*)P, y.ld_data, rows, ctx->Kb, y.ld_pix, ctx->cfg.n_pix,
+                          scratch.captured() ? nullptr : (uint32_t*)(ctx->ws + y.upnz), Num, den,
+                          s));
+    return EMC_OK;
+  }
+  if (scratch.captured()) return do_update(ctx, P, rows, nrot, Num, den, s);
   // the rows' pairs from the planes; what is over on the tensor cores
   const bool tail = is_gauss(&ctx->cfg) || is_flu(&ctx->cfg);  // den lies behind P
   const int f16 = ctx->cfg.precision == EMC_PREC_FP16_SPLIT && !tail ? 1 : 0;

@@ -206,7 +206,7 @@ cudaError_t launch_simt_normalize(const float* L, int64_t ld_pix, const double* 
                                   int64_t nrot, const uint16_t* Kb, int64_t ld_data,
                                   int64_t n_data, const double* lse_m, const double* lse_s,
                                   float* P, cudaStream_t s);
-// nz: scratch of rows / 64 x ld_data / 32 words
+// nz: scratch of rows / 64 x ld_data / 32 words (NULL: every frame is contracted)
 cudaError_t launch_simt_update(const float* P, int64_t ld_data, int64_t rows, const uint16_t* Kb,
                                int64_t ld_pix, int64_t n_pix, uint32_t* nz, float* Num,
                                float* den, cudaStream_t s);

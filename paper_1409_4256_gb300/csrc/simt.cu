@@ -247,7 +247,8 @@ __global__ void __launch_bounds__(256)
 
 // Only the frames with a non-zero P in the tile's 64 rows are contracted, in
 // order (most P underflow to exact zeros, which add nothing: 64^3, 3240 rotations x 2000
-// frames, 1315 us over every frame, 107 us over these with their bits). nz: simt_nonzero_kernel's bits.
+// frames, 1315 us over every frame, 107 us over these with their bits). nz: simt_nonzero_kernel's
+// bits, or NULL: every frame.
 constexpr int kNzWords = 128;  // words of nz taken at a time: 4096 frames
 __global__ void __launch_bounds__(S_THREADS)
     simt_update_kernel(const float* __restrict__ P, int64_t ld_data,
@@ -269,10 +270,10 @@ __global__ void __launch_bounds__(S_THREADS)
   const int br = t >> 4, bc = (t & 15) * 8;   // B = K: frame, pixel offset
   const bool bval = c0 + bc < ld_pix;
   const int64_t words = ld_data / 32;
-  nz += blockIdx.y * words;
+  if (nz) nz += blockIdx.y * words;
   for (int64_t w0 = 0; w0 < words; w0 += kNzWords) {
     // the frames of these words (offsets from 32 w0)
-    uint32_t bits = t < kNzWords && w0 + t < words ? nz[w0 + t] : 0u;
+    uint32_t bits = t < kNzWords && w0 + t < words ? (nz ? nz[w0 + t] : ~0u) : 0u;
     int inc = __popc(bits);
     const int own = inc;
 #pragma unroll
@@ -375,10 +376,12 @@ cudaError_t launch_simt_normalize(const float* L, int64_t ld_pix, const double* 
 cudaError_t launch_simt_update(const float* P, int64_t ld_data, int64_t rows, const uint16_t* Kb,
                                int64_t ld_pix, int64_t n_pix, uint32_t* nz, float* Num,
                                float* den, cudaStream_t s) {
-  simt_nonzero_kernel<<<dim3((unsigned)(ld_data / 128), (unsigned)(rows / SB_M)), 256, 0, s>>>(
-      P, ld_data, nz);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
+  if (nz) {
+    simt_nonzero_kernel<<<dim3((unsigned)(ld_data / 128), (unsigned)(rows / SB_M)), 256, 0, s>>>(
+        P, ld_data, nz);
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+  }
   dim3 grd((unsigned)((ld_pix + SB_N - 1) / SB_N), (unsigned)(rows / SB_M));
   simt_update_kernel<<<grd, S_THREADS, 0, s>>>(P, ld_data, Kb, ld_pix, n_pix, nz, Num, den);
   return cudaGetLastError();
