@@ -737,10 +737,8 @@ int do_expand(emc_ctx* c, const float* grid, int64_t rot0, int64_t nrot, void* L
   }
   const RotFX* rot = (const RotFX*)(c->ws + y.rotfx) + rot0;
   if (is_flu(&c->cfg)) {
-    // (W takes the slice buffer of the M-step, which runs later)
     CU(launch_expand_flu(c->geom, grid, g4, rot, c->logw + rot0, nrot, rows,
-                         (float)c->cfg.w_floor, c->flu_c, p, bias, c->flu_B + rot0,
-                         (double*)(c->ws + y.epart), (float*)(c->ws + y.Num), y.num_rows, Lold,
+                         (float)c->cfg.w_floor, c->flu_c, p, bias, c->flu_B + rot0, Lold,
                          Lold ? (uint16_t*)(c->ws + y.Dd) : nullptr, y.ntp,
                          Lold ? (float*)(c->ws + y.bpm) : nullptr, c->status, s));
     return EMC_OK;
@@ -1166,11 +1164,8 @@ int emc_iteration(emc_ctx* c, const float* grid_in, float* grid_out, emc_iter_st
   if (c->collecting) CU(cudaMemsetAsync(c->col.count, 0, sizeof(unsigned long long), s));
   if ((st = do_expand(c, grid_in, 0, n_rot, L, bias, s, Lold, bold))) return st;
   // the row tiles and the bias sums (Gaussian: grid maximum and scales first;
-  // Poisson fluence: the split, and all three per block of slice rows); the cell
-  // layout of the model first where it is used
-  kernels += (is_gauss(&c->cfg)
-                  ? 4
-                  : (is_flu(&c->cfg) ? 3 * (int)((y.rows + y.num_rows - 1) / y.num_rows) : 2)) +
+  // Poisson fluence: the split); the cell layout of the model first where it is used
+  kernels += (is_gauss(&c->cfg) ? 4 : (is_flu(&c->cfg) ? 3 : 2)) +
              ((y.g4 && c->geom.interior) ? 1 : 0);
   if (stats) CU(cudaEventRecord(c->ev[1], s));
   float* S = (c->cfg.flags & EMC_FLAG_STORE_SCORES) ? (float*)(c->ws + y.S) : nullptr;

@@ -114,13 +114,13 @@ cudaError_t launch_expand_gauss(const Geom& g, const float* grid, const float4* 
                                 double sigma, int32_t* status, cudaStream_t s);
 // Poisson-fluence model: L = log(W / B_j) + c as the BF16 three-term split;
 // bias = double[2][rows]: log w_j, then B_j = sum_i W_ij; Bctx[row] = B_j too.
-// W: scratch of W_rows (a multiple of 128) x ld_pix floats, used for W_rows
-// rotations at a time. Lold, D, ntp, bpm: as launch_expand_tile.
+// W and its row sums lie in L's planes on the way: no scratch. Lold, D, ntp, bpm: as
+// launch_expand_tile.
 cudaError_t launch_expand_flu(const Geom& g, const float* grid, const float4* g4, const RotFX* rot,
                               const double* logw, int64_t nrot, int64_t rows, float w_floor,
-                              double c, Planes L, double* bias, double* Bctx, double* partial,
-                              float* W, int64_t W_rows, const void* Lold, uint16_t* D,
-                              int64_t ntp, float* bpm, int32_t* status, cudaStream_t s);
+                              double c, Planes L, double* bias, double* Bctx, const void* Lold,
+                              uint16_t* D, int64_t ntp, float* bpm, int32_t* status,
+                              cudaStream_t s);
 // Per frame: cn[k] = c N_k, invn[k] = 1 / N_k (0 for empty and padding frames).
 cudaError_t launch_flu_frames(const int32_t* K, int64_t ld_k, int64_t n_data, int64_t n_pix,
                               int64_t ld_data, double c, double* cn, float* invn,

@@ -186,7 +186,9 @@ __device__ __forceinline__ uint16_t round_up_operand(float x) {
 //    s = 2^e = gsc->x), hi integral (rint below 2048, else the FP16 rounding, itself
 //    integral there), mid = fp16(s W - hi), lo = fp16(s W - hi - mid), the
 //    representation error below 2^-23 s^-1 W units; the row sums are of W^2;
-//  kOutW: W itself in FP32 (the Poisson-fluence model, whose split needs the row sum first).
+//  kOutW: W itself in FP32 (the Poisson-fluence model, whose split needs the row sum first),
+//    its upper 16 bits in plane 0 and its lower ones in plane 1, and the slices' row sums
+//    in plane 2, each at its row and slice (flu_split_kernel replaces all three in place).
 constexpr int kOutGauss = 4, kOutW = 5;
 
 // The rises dp and falls dm of a thread's two pixels over a tile's rows, gathered over the
@@ -226,6 +228,23 @@ __device__ __forceinline__ void write_increments(float (&dp)[2], float (&dm)[2],
         (uint32_t)a0 | ((uint32_t)a1 << 16);
   }
   cluster.sync();  // no CTA leaves while its rises may be read
+}
+
+// Eight bytes at a place of a 16-bit plane that need not be aligned to them.
+__device__ __forceinline__ void put_bytes8(uint16_t* p, unsigned long long v) {
+  if (((uintptr_t)p & 7) == 0) {
+    *reinterpret_cast<unsigned long long*>(p) = v;
+    return;
+  }
+#pragma unroll
+  for (int k = 0; k < 4; k++) p[k] = (uint16_t)(v >> (16 * k));
+}
+__device__ __forceinline__ unsigned long long get_bytes8(const uint16_t* p) {
+  if (((uintptr_t)p & 7) == 0) return *reinterpret_cast<const unsigned long long*>(p);
+  unsigned long long v = 0;
+#pragma unroll
+  for (int k = 0; k < 4; k++) v |= (unsigned long long)p[k] << (16 * k);
+  return v;
 }
 
 // RPC rotations of a tile per CTA; with DELTA the tile's 128 / RPC CTAs are a
@@ -343,7 +362,12 @@ __global__ void __launch_bounds__(kTThreads, 6)
         *reinterpret_cast<uint32_t*>(Lb) = (uint32_t)h[0] | ((uint32_t)h[1] << 16);
         *reinterpret_cast<uint32_t*>(Lb + ps) = (uint32_t)m[0] | ((uint32_t)m[1] << 16);
         *reinterpret_cast<uint32_t*>(Lb + 2 * ps) = (uint32_t)l[0] | ((uint32_t)l[1] << 16);
-      } else if (PREC == EMC_PREC_FP32 || PREC == kOutW) {
+      } else if (PREC == kOutW) {
+        const uint32_t u0 = __float_as_uint(L[0]), u1 = __float_as_uint(L[1]);
+        uint16_t* Lb = (uint16_t*)Lbase + o;
+        *reinterpret_cast<uint32_t*>(Lb) = __byte_perm(u0, u1, 0x7632);
+        *reinterpret_cast<uint32_t*>(Lb + ps) = __byte_perm(u0, u1, 0x5410);
+      } else if (PREC == EMC_PREC_FP32) {
         *reinterpret_cast<float2*>((float*)Lbase + o) = make_float2(L[0], L[1]);
         if (DELTA && vrow) {
           const float2 old = read_pair<PREC>(Lold, o, ps);
@@ -447,7 +471,12 @@ __global__ void __launch_bounds__(kTThreads, 6)
         s = a.h;
         se += v.y + a.l;
       }
-    partial[(int64_t)slice * rows + r0 + threadIdx.x] = f32_to_f64(s) + f32_to_f64(se);
+    const double sum = f32_to_f64(s) + f32_to_f64(se);
+    if (PREC == kOutW)
+      put_bytes8((uint16_t*)Lbase + 2 * ps + (r0 + threadIdx.x) * ld_pix + (int64_t)slice * kTPix,
+                 (unsigned long long)__double_as_longlong(sum));
+    else
+      partial[(int64_t)slice * rows + r0 + threadIdx.x] = sum;
   }
   if constexpr (DELTA)
     write_increments<PREC>(dp, dm, rises, inside, t, i0, ld_pix, ntp, D);
@@ -499,26 +528,38 @@ __global__ void __launch_bounds__(kTRows)
 // size on every K step.
 //
 // Per row: bias = log w_j (-inf on padding rows), B_j (0) into Bsum and Bctx, and
-// (ah, al) over the row's first partial sum.
+// (ah, al) over the row's partial sums (low: plane 2), one copy for each slice.
 __global__ void __launch_bounds__(kTRows)
-    flu_bias_kernel(double* __restrict__ partial, int n_slices, int64_t rows,
+    flu_bias_kernel(uint16_t* __restrict__ low, int64_t ld_pix, int n_slices,
                     const double* __restrict__ logw, int64_t nrot, double c,
                     double* __restrict__ bias, double* __restrict__ Bsum,
-                    double* __restrict__ Bctx, float* __restrict__ bpm, int64_t nt, int64_t t0) {
+                    double* __restrict__ Bctx, float* __restrict__ bpm, int64_t nt) {
   const int64_t row = (int64_t)blockIdx.x * kTRows + threadIdx.x;
+  uint16_t* own = low + row * ld_pix;
   double B = 0.0;
-  for (int q = 0; q < n_slices; q++) B += partial[(int64_t)q * rows + row];
+  // (a sum's sector is its own: sixteen loads in flight)
+  for (int q0 = 0; q0 < n_slices; q0 += 16) {
+    unsigned long long part[16];
+#pragma unroll
+    for (int u = 0; u < 16; u++)
+      part[u] = q0 + u < n_slices ? get_bytes8(own + (int64_t)(q0 + u) * kTPix) : 0ull;
+#pragma unroll
+    for (int u = 0; u < 16; u++) B += __longlong_as_double((long long)part[u]);
+  }
   const bool v = row < nrot;
   const double aj = v ? c - log(B) : 0.0;
   const float ah = (float)(rint(aj * kHiScale) / kHiScale);
-  reinterpret_cast<float2*>(partial)[row] = make_float2(ah, (float)(aj - (double)ah));
+  const float al = (float)(aj - (double)ah);
+  const unsigned long long a =
+      (unsigned long long)__float_as_uint(al) << 32 | __float_as_uint(ah);
+  for (int q = 0; q < n_slices; q++) put_bytes8(own + (int64_t)q * kTPix, a);
   bias[row] = v ? logw[row] : -INFINITY;
   Bsum[row] = v ? B : 0.0;
   Bctx[row] = v ? B : 0.0;
-  if (bpm && threadIdx.x == 0) bpm[t0 + blockIdx.x] = bpm[nt + t0 + blockIdx.x] = 0.f;  // log w stays
+  if (bpm && threadIdx.x == 0) bpm[blockIdx.x] = bpm[nt + blockIdx.x] = 0.f;  // log w stays
 }
 
-// W to the three BF16 planes of L, and with DELTA the increments from the last
+// W to the three BF16 planes of L in place, and with DELTA the increments from the last
 // iteration's planes (as expand_tile_kernel; the CTAs of a tile are a cluster).
 // Bound by memory and the latency of its short rows: 4 B of W and 6 B of planes read, 6 B
 // written per element, 3.9 TB/s with eight rows' loads in flight (one by one: 3.3).
@@ -527,12 +568,11 @@ __global__ void __launch_bounds__(kTRows)
 constexpr int kSplitRows = 32;
 template <bool DELTA>
 __global__ void __launch_bounds__(kTThreads)
-    flu_split_kernel(const float* __restrict__ Wm, const float2* __restrict__ asplit,
-                     const int4* __restrict__ qi_g, int64_t ld_pix, int64_t nrot,
+    flu_split_kernel(const int4* __restrict__ qi_g, int64_t ld_pix, int64_t nrot,
                      uint16_t* __restrict__ Lbase, int64_t ps, const uint16_t* __restrict__ Lold,
-                     uint16_t* __restrict__ D, int64_t ntp, int64_t t0, unsigned slices,
-                     int32_t* status) {
+                     uint16_t* __restrict__ D, int64_t ntp, unsigned slices, int32_t* status) {
   __shared__ float4 rises[DELTA ? kTThreads : 1];
+  __shared__ float2 asplit[kSplitRows];
   constexpr unsigned kPer = kTRows / kSplitRows;
   const unsigned slice = blockIdx.x / kPer % slices;
   const int64_t t = blockIdx.x / kPer / slices;
@@ -542,35 +582,47 @@ __global__ void __launch_bounds__(kTThreads)
   bool used[2];
 #pragma unroll
   for (int u = 0; u < 2; u++) used[u] = inside && qi_g[i0 + u].w != 0;
+  constexpr int kAhead = 8;  // rows whose loads are in flight together
+  uint32_t wh[kAhead], wl[kAhead];  // W's upper and lower halves
+  uint32_t old[DELTA ? kAhead : 1][3];
+  auto load = [&](int rb) {
+#pragma unroll
+    for (int r = 0; r < kAhead; r++) {
+      const int64_t o = (r0 + rb + r) * ld_pix + i0;
+      wh[r] = __ldcs(reinterpret_cast<const uint32_t*>(Lbase + o));
+      wl[r] = __ldcs(reinterpret_cast<const uint32_t*>(Lbase + o + ps));
+      if (DELTA)
+#pragma unroll
+        for (int q = 0; q < 3; q++)
+          old[r][q] = __ldcs(reinterpret_cast<const uint32_t*>(Lold + o + q * ps));
+    }
+  };
+  unsigned long long a = 0;
+  if (threadIdx.x < kSplitRows)  // this slice's copy, before it is written over
+    a = get_bytes8(Lbase + 2 * ps + (r0 + threadIdx.x) * ld_pix + (int64_t)slice * kTPix);
+  if (inside) load(0);
+  if (threadIdx.x < kSplitRows)
+    asplit[threadIdx.x] =
+        make_float2(__uint_as_float((uint32_t)a), __uint_as_float((uint32_t)(a >> 32)));
+  __syncthreads();
   float dp[2] = {-INFINITY, -INFINITY}, dm[2] = {-INFINITY, -INFINITY};
   int bad = 0;
   if (inside) {
-    constexpr int kAhead = 8;  // rows whose loads are in flight together
 #pragma unroll 1
     for (int rb = 0; rb < kSplitRows; rb += kAhead) {
-      float2 w[kAhead];
-      uint32_t old[DELTA ? kAhead : 1][3];
-#pragma unroll
-      for (int r = 0; r < kAhead; r++) {
-        const int64_t o = (r0 + rb + r) * ld_pix + i0;
-        w[r] = __ldcs(reinterpret_cast<const float2*>(Wm + o));
-        if (DELTA)
-#pragma unroll
-          for (int q = 0; q < 3; q++)
-            old[r][q] = __ldcs(reinterpret_cast<const uint32_t*>(Lold + o + q * ps));
-      }
+      if (rb > 0) load(rb);
 #pragma unroll
       for (int r = 0; r < kAhead; r++) {
         const int64_t row = r0 + rb + r, o = row * ld_pix + i0;
         const bool vrow = row < nrot;
-        const float2 aj = asplit[row];
+        const float2 aj = asplit[rb + r];
         const float ah = aj.x, al = aj.y;
         uint16_t h[2], m[2], l[2];
 #pragma unroll
         for (int u = 0; u < 2; u++) {
           float hi = 0.f, rest = 0.f;
           if (vrow && used[u]) {
-            const float x = logf(u ? w[r].y : w[r].x);
+            const float x = logf(__uint_as_float(__byte_perm(wl[r], wh[r], u ? 0x7632 : 0x5410)));
             const float s = x + ah;  // two-sum: s + e = x + ah exactly
             const float bb = s - x;
             const float e = (x - (s - bb)) + (ah - bb);
@@ -604,7 +656,7 @@ __global__ void __launch_bounds__(kTThreads)
   }
   if (bad) set_status(status, EMC_ERR_UNSUPPORTED);
   if constexpr (DELTA)
-    write_increments<EMC_PREC_BF16_SPLIT>(dp, dm, rises, inside, t0 + t, i0, ld_pix, ntp, D);
+    write_increments<EMC_PREC_BF16_SPLIT>(dp, dm, rises, inside, t, i0, ld_pix, ntp, D);
 }
 
 // the grid in the cell layout of load_cell
@@ -762,40 +814,33 @@ cudaError_t launch_expand_gauss(const Geom& g, const float* grid, const float4* 
 
 cudaError_t launch_expand_flu(const Geom& g, const float* grid, const float4* g4, const RotFX* rot,
                               const double* logw, int64_t nrot, int64_t rows, float w_floor,
-                              double c, Planes L, double* bias, double* Bctx, double* partial,
-                              float* W, int64_t W_rows, const void* Lold, uint16_t* D,
-                              int64_t ntp, float* bpm, int32_t* status, cudaStream_t s) {
+                              double c, Planes L, double* bias, double* Bctx, const void* Lold,
+                              uint16_t* D, int64_t ntp, float* bpm, int32_t* status,
+                              cudaStream_t s) {
+  if (rows <= 0) return cudaSuccess;
   const int64_t ns = expand_tile_slices(g.ld_pix), nt = rows / kTRows;
-  for (int64_t r0 = 0; r0 < rows; r0 += W_rows) {
-    const int64_t nr = std::min(W_rows, rows - r0), valid = std::min(nr, nrot - r0);
-    cudaError_t e = launch_tiles(g, grid, g4, rot + r0, valid, nr, kOutW, w_floor,
-                                 Planes{W, 0, g.ld_pix}, partial, nullptr, nullptr, 0, nullptr,
-                                 status, s);
-    if (e != cudaSuccess) return e;
-    flu_bias_kernel<<<(unsigned)(nr / kTRows), kTRows, 0, s>>>(
-        partial, (int)ns, nr, logw + r0, valid, c, bias + r0, bias + rows + r0, Bctx + r0,
-        Lold ? bpm : nullptr, nt, r0 / kTRows);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    constexpr int kPer = kTRows / kSplitRows;
-    cudaLaunchConfig_t lc{};
-    lc.gridDim = dim3((unsigned)(ns * (nr / kTRows) * kPer));
-    lc.blockDim = dim3(kTThreads);
-    lc.stream = s;
-    cudaLaunchAttribute at{};
-    at.id = cudaLaunchAttributeClusterDimension;
-    at.val.clusterDim.x = kPer;
-    at.val.clusterDim.y = at.val.clusterDim.z = 1;
-    lc.attrs = &at;
-    lc.numAttrs = Lold ? 1 : 0;
-    const int64_t o = r0 * g.ld_pix;
-    uint16_t* Lb = (uint16_t*)L.base + o;
-    const uint16_t* Lo = Lold ? (const uint16_t*)Lold + o : nullptr;
-    e = cudaLaunchKernelEx(&lc, Lold ? flu_split_kernel<true> : flu_split_kernel<false>,
-                           (const float*)W, (const float2*)partial, g.qi, g.ld_pix, valid, Lb,
-                           L.plane_stride, Lo, D, ntp, r0 / kTRows, (unsigned)ns, status);
-    if (e != cudaSuccess) return e;
-  }
-  return cudaSuccess;
+  cudaError_t e = launch_tiles(g, grid, g4, rot, nrot, rows, kOutW, w_floor, L, nullptr, nullptr,
+                               nullptr, 0, nullptr, status, s);
+  if (e != cudaSuccess) return e;
+  uint16_t* Lb = (uint16_t*)L.base;
+  flu_bias_kernel<<<(unsigned)nt, kTRows, 0, s>>>(Lb + 2 * L.plane_stride, g.ld_pix, (int)ns, logw,
+                                                  nrot, c, bias, bias + rows, Bctx,
+                                                  Lold ? bpm : nullptr, nt);
+  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  constexpr int kPer = kTRows / kSplitRows;
+  cudaLaunchConfig_t lc{};
+  lc.gridDim = dim3((unsigned)(ns * nt * kPer));
+  lc.blockDim = dim3(kTThreads);
+  lc.stream = s;
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = kPer;
+  at.val.clusterDim.y = at.val.clusterDim.z = 1;
+  lc.attrs = &at;
+  lc.numAttrs = Lold ? 1 : 0;
+  return cudaLaunchKernelEx(&lc, Lold ? flu_split_kernel<true> : flu_split_kernel<false>, g.qi,
+                            g.ld_pix, nrot, Lb, L.plane_stride, (const uint16_t*)Lold, D, ntp,
+                            (unsigned)ns, status);
 }
 
 }  // namespace emc

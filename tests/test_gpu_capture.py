@@ -1,6 +1,6 @@
 """GPU: calls captured into a CUDA graph. Nothing orders a graph's nodes, or its replays,
-against other calls on the context, so a captured emc_update takes no scratch of it: two on
-parallel branches give the bits of the same calls in turn, and each is one kernel.
+against other calls on the context, so calls that shared nothing with others take no scratch
+of it: two on parallel branches give the bits of the same calls alone.
 """
 import ctypes
 
@@ -126,4 +126,53 @@ def test_captured_updates_share_nothing(rt, precision):
     replay(rt, graph, streams[0])
     for i in (0, 1):
         assert torch.equal(Num[i], want[i][0]) and torch.equal(den[i], want[i][1])
+    assert ctx.status() == 0
+
+
+def test_fluence_expansion_takes_no_scratch(rt):
+    """The Poisson-fluence expansion keeps W and its sums in the caller's L on the way: of the
+    context's workspace a call writes its rotations' B_j alone (pixels at the grid's edge, so
+    without the cell layout of the model), and two captured ones on parallel branches, each
+    with a model and a block of its own, give the bits of the calls alone."""
+    import torch
+    from paper_1409_4256_gb300 import emc, synth
+    det = synth.make_detector(40, 32)
+    q = det.q * (15.99 / 15.0)
+    quat, w = emc.quat_generate(4)
+    n = quat.shape[0]
+    ctx = emc.Context(32, q, quat, w, 300, model="poisson_fluence", w_floor=1e-6)
+    ctx.set_frames(torch.ones(300, q.shape[0], dtype=torch.int32, device="cuda"))
+    g = torch.Generator(device="cuda").manual_seed(3)
+    grids = [torch.rand(32, 32, 32, generator=g, device="cuda") + 0.1 for _ in range(2)]
+    blocks = [(0, 1280), (1280, n - 1280)]
+    out = []
+    for r0, nb in blocks:
+        b = ctx.buffer_sizes(nb)
+        out.append((torch.empty(b.logw_bytes, dtype=torch.uint8, device="cuda"),
+                    torch.empty(b.bias_bytes // 8, dtype=torch.float64, device="cuda")))
+    streams = [torch.cuda.Stream() for _ in range(2)]
+
+    def expand(i):
+        emc._check(emc.lib().emc_expand(ctx.h, grids[i].data_ptr(), *blocks[i],
+                                        out[i][0].data_ptr(), out[i][1].data_ptr(),
+                                        streams[i].cuda_stream), "emc_expand")
+
+    want = []
+    for i in (0, 1):
+        torch.cuda.synchronize()
+        before = ctx.workspace.clone()
+        torch.cuda.synchronize()
+        expand(i)
+        torch.cuda.synchronize()
+        changed = torch.nonzero(ctx.workspace != before)
+        assert int(changed.amax() - changed.amin()) < 8 * ctx.buffer_sizes(blocks[i][1]).rows
+        want.append([x.clone() for x in out[i]])
+    graph, _ = capture(rt, streams[0], lambda: on_two_branches(
+        streams[0], streams[1], lambda: expand(0), lambda: expand(1)))
+    for x in out:
+        x[0].zero_()
+        x[1].zero_()
+    replay(rt, graph, streams[0])
+    for i in (0, 1):
+        assert torch.equal(out[i][0], want[i][0]) and torch.equal(out[i][1], want[i][1])
     assert ctx.status() == 0
