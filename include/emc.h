@@ -17,6 +17,22 @@
  *    stream-ordered; problems found on the device (counts out of range, a
  *    non-finite score, a bounded wait that gave up) are recorded in a device
  *    status word that emc_ctx_status() reads.
+ *  - Streams and threads: a call is ordered on its own stream. emc_expand (and the
+ *    expansion inside emc_iteration and emc_sparse_iteration) and emc_update may
+ *    also be made on one context from several streams and threads at a time: the
+ *    library puts the calls that share scratch in the workspace -- expansions among
+ *    themselves, updates among themselves -- one behind the other on the GPU, in
+ *    the order of the calls. An expansion and an update share nothing. emc_compress,
+ *    emc_finalize, emc_sparse_update and emc_features take no scratch. Every other call
+ *    on a context that may overlap another one on it is ordered by the caller: the
+ *    iterations, emc_loglik, emc_loglik_sparse_k, emc_normalize, emc_sparse_estep,
+ *    emc_missed_mass, emc_responsibilities and emc_collected_targets use the workspace, and
+ *    emc_set_frames and emc_set_candidates change what the others read. An expansion in
+ *    the Gaussian and Poisson-fluence models also leaves the scales and the B_j that
+ *    later calls use (see emc_expand).
+ *    Inside a stream capture the library's order ends at the graph: the caller
+ *    orders replays against other calls on the context, and parallel branches among
+ *    themselves. A captured emc_update takes no scratch and needs no such order.
  *  - Ownership: every array argument is owned by the caller. Device arrays
  *    are plain device pointers; host arrays are marked "host". The library
  *    never allocates device memory: all scratch comes from the workspace the

@@ -19,6 +19,11 @@ namespace {
 int64_t round_up(int64_t x, int64_t m) { return (x + m - 1) / m * m; }
 size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
+// The M-step's lists of pairs: pairs, the row tiles that are over and their output tiles.
+struct PairsAt {
+  size_t cnt, k, w, p, tiles, codes, n;
+};
+
 struct Layout {
   int64_t ld_pix, ld_data, rows, chunk_rows, num_rows, part_tiles;
   size_t qh, ql, logw, Kb, status, L, bias, lse_m, lse_s, lse2, part_m, part_s, S, P,
@@ -26,8 +31,9 @@ struct Layout {
       Kb2, skcnt, skoff, skent, dupsrc, duprank, pixmax, fcn, finvn, fB, kbflag, kbcnt, kblist,
       Kp, perm, perm2, iperm, nsum, nsum_p, cn_p, invn_p, best, lsem_s, lses_s, live, tlist, slot, klist,
       tcount, sortH, sortoff, cgs, cgp, cgqh, cgql, cgqi, cgqlo, cgqf, L2, bias2, Ub, Ub2, Lk, Mk, Mk2, best2,
-      osrc, Dd, Cd, bpm, g4, Ua, Ua2, dcand, pflag, plist, flags, qi, qlo, rotfx, epart, rpcnt, rpk,
-      rpw, rpp, rptiles, rpcodes, rpn, upnz, total;
+      osrc, Dd, Cd, bpm, g4, Ua, Ua2, dcand, pflag, plist, flags, qi, qlo, rotfx, epart, nz, upnz,
+      total;
+  PairsAt rp, uprp;  // emc_iteration's (a chunk of rotations), emc_update's
   int64_t sort_entries;
   int64_t ntp;  // row tiles rounded up to 128: rows of each half of the bound increments
 };
@@ -187,16 +193,24 @@ Layout make_layout(const emc_config* c) {
   y.kbflag = tc ? take((size_t)ctiles * kbs) : 0;
   y.kbcnt = tc ? take(sizeof(int32_t) * (size_t)ctiles) : 0;
   y.kblist = tc ? take(sizeof(int32_t) * (size_t)ctiles * kbs) : 0;
-  // the M-step from the rows' pairs: pairs, the row tiles that are over and their output tiles
+  // The M-step from the rows' pairs (split precisions), or FP32: the frames it contracts, a bit
+  // for each 64 rows. emc_update has its own, so that it shares nothing with an iteration.
   const bool rp = c->precision == EMC_PREC_BF16_SPLIT || c->precision == EMC_PREC_FP16_SPLIT;
-  y.rpcnt = rp ? take(sizeof(int32_t) * (size_t)y.rows + 5 * (size_t)(y.rows / 128)) : 0;
-  y.rpk = rp ? take(sizeof(int32_t) * kRowPairs * (size_t)y.rows) : 0;
-  y.rpw = rp ? take(sizeof(float) * kRowPairs * (size_t)y.rows) : 0;
-  y.rpp = rp ? take(sizeof(float) * kRowPairs * (size_t)y.rows) : 0;
-  y.rptiles = rp ? take(sizeof(int32_t) * (size_t)(y.rows / 128)) : 0;
-  y.rpcodes = rp ? take(sizeof(int32_t) * (size_t)(y.rows / 128) * ((y.ld_pix + 255) / 256)) : 0;
-  y.rpn = rp ? take(256) : 0;
-  // FP32: the frames that the update contracts, a bit for each 64 rows
+  auto take_pairs = [&](int64_t rows) {
+    PairsAt a{};
+    if (!rp) return a;
+    a.cnt = take(sizeof(int32_t) * (size_t)rows + 5 * (size_t)(rows / 128));
+    a.k = take(sizeof(int32_t) * kRowPairs * (size_t)rows);
+    a.w = take(sizeof(float) * kRowPairs * (size_t)rows);
+    a.p = take(sizeof(float) * kRowPairs * (size_t)rows);
+    a.tiles = take(sizeof(int32_t) * (size_t)(rows / 128));
+    a.codes = take(sizeof(int32_t) * (size_t)(rows / 128) * ((y.ld_pix + 255) / 256));
+    a.n = take(256);
+    return a;
+  };
+  y.rp = take_pairs(y.chunk_rows);
+  y.uprp = take_pairs(y.rows);
+  y.nz = tc ? 0 : take(sizeof(uint32_t) * (size_t)(y.chunk_rows / 64) * (y.ld_data / 32));
   y.upnz = tc ? 0 : take(sizeof(uint32_t) * (size_t)(y.rows / 64) * (y.ld_data / 32));
   // bound-pruned pass 1: frames in their internal order and the tile bookkeeping
   const bool pr = prune_ok(c);
@@ -262,6 +276,28 @@ Layout make_layout(const emc_config* c) {
 
 }  // namespace
 
+// The calls on a context that take one set of its scratch, whichever streams and threads they
+// come from, run one at a time in the order of the calls. The sets: what an expansion takes
+// (the cell layout of the model, the slices' sums, the Gaussian scales), by emc_expand and
+// the iterations; what emc_update takes.
+struct Order {
+  pthread_mutex_t mu;
+  cudaEvent_t done;
+  bool made;
+  bool make() {
+    if (cudaEventCreateWithFlags(&done, cudaEventDisableTiming) != cudaSuccess) return false;
+    made = pthread_mutex_init(&mu, nullptr) == 0;
+    if (!made) cudaEventDestroy(done);
+    return made;
+  }
+  void drop() {
+    if (!made) return;
+    cudaEventDestroy(done);
+    pthread_mutex_destroy(&mu);
+    made = false;
+  }
+};
+
 struct emc_ctx {
   emc_config cfg;
   Layout lay;
@@ -306,35 +342,42 @@ struct emc_ctx {
   cudaEvent_t ev[8];
   int kernels;  // launches made by the last emc_iteration
   TcCtl tcctl;  // bounded waits of the tensor-core launches (emc_ctx_set_wait_limit)
-  pthread_mutex_t scratch_mu;  // Scratch
-  cudaEvent_t scratch_done;
+  Order expand_order, update_order;
 };
 
-// The step calls that take scratch of the context while other calls on it may run (emc_expand,
-// emc_update, and the iterations, which use the same): one at a time, in the order
-// of the calls, whichever streams and threads they come from. A captured call cannot wait
-// for what ran before the capture, so emc_update then takes none (captured()): the planes of P, or
-// in FP32 every frame (64^3, 3240 x 2000, flat posteriors: 1033 us either way).
+// A call that takes the scratch of `o` (NULL: it takes none) is put behind the last one that
+// did. A captured call cannot wait for what ran before the capture, nor be waited for:
+// emc_update then takes no scratch (captured(): the planes of P, or in FP32 every frame, 64^3, 3240 x
+// 2000, flat posteriors: 1033 us either way), and the caller orders a captured expansion.
 class Scratch {
  public:
-  Scratch(emc_ctx* c, cudaStream_t s) : c_(c), s_(s) {
-    pthread_mutex_lock(&c->scratch_mu);
+  Scratch(Order* o, cudaStream_t s) : o_(o), s_(s) {
+    if (!o_) return;
+    pthread_mutex_lock(&o_->mu);
     cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
-    captured_ = cudaStreamIsCapturing(s, &st) == cudaSuccess && st != cudaStreamCaptureStatusNone;
-    if (!captured_) cudaStreamWaitEvent(s, c->scratch_done, 0);
+    ok_ = cudaStreamIsCapturing(s, &st) == cudaSuccess;
+    captured_ = st != cudaStreamCaptureStatusNone;
+    if (ok_ && !captured_) ok_ = cudaStreamWaitEvent(s, o_->done, 0) == cudaSuccess;
   }
-  ~Scratch() {
-    if (!captured_) cudaEventRecord(c_->scratch_done, s_);
-    pthread_mutex_unlock(&c_->scratch_mu);
-  }
+  ~Scratch() { release(); }
   Scratch(const Scratch&) = delete;
   Scratch& operator=(const Scratch&) = delete;
+  bool ok() const { return ok_; }  // false: the call must launch nothing
   bool captured() const { return captured_; }
+  // the call's status, once it has launched its work
+  int done(int st) { return release() || st ? st : EMC_ERR_CUDA; }
 
  private:
-  emc_ctx* c_;
+  bool release() {
+    if (!o_) return true;
+    const bool r = !ok_ || captured_ || cudaEventRecord(o_->done, s_) == cudaSuccess;
+    pthread_mutex_unlock(&o_->mu);
+    o_ = nullptr;
+    return r;
+  }
+  Order* o_;
   cudaStream_t s_;
-  bool captured_;
+  bool ok_ = true, captured_ = false;
 };
 
 // The internal frame order the last iteration found (perm2) becomes the
@@ -597,12 +640,12 @@ static int ctx_create(const emc_config* cfg, const double* q, const double* quat
                         s) == cudaSuccess;
   ok &= cudaStreamSynchronize(s) == cudaSuccess;  // host staging buffers go out of scope
   for (int e = 0; e < 8 && ok; e++) ok &= cudaEventCreate(&c->ev[e]) == cudaSuccess;
-  ok = ok && cudaEventCreateWithFlags(&c->scratch_done, cudaEventDisableTiming) == cudaSuccess;
-  ok = ok && pthread_mutex_init(&c->scratch_mu, nullptr) == 0;
+  ok = ok && c->expand_order.make() && c->update_order.make();
   if (!ok) {
     for (int e = 0; e < 8; e++)
       if (c->ev[e]) cudaEventDestroy(c->ev[e]);
-    if (c->scratch_done) cudaEventDestroy(c->scratch_done);
+    c->expand_order.drop();
+    c->update_order.drop();
     free(c);
     return EMC_ERR_CUDA;
   }
@@ -614,8 +657,8 @@ int emc_ctx_destroy(emc_ctx* ctx) {
   if (!ctx) return EMC_ERR_ARG;
   for (int e = 0; e < 8; e++)
     if (ctx->ev[e]) cudaEventDestroy(ctx->ev[e]);
-  cudaEventDestroy(ctx->scratch_done);
-  pthread_mutex_destroy(&ctx->scratch_mu);
+  ctx->expand_order.drop();
+  ctx->update_order.drop();
   free(ctx);
   return EMC_OK;
 }
@@ -808,15 +851,14 @@ struct FrameView {
 // 3240 x 4500: 78 against 66 us at best, all of the iteration 590).
 // (The stall hook stalls a contraction: it keeps one.)
 bool pairs_ok(const emc_ctx* c, int64_t rows) {
-  return c->lay.rpcnt && c->lay.ld_pix >= 2560 && c->cfg.n_data <= 4 * c->cfg.n_rot &&
+  return c->lay.rp.cnt && c->lay.ld_pix >= 2560 && c->cfg.n_data <= 4 * c->cfg.n_rot &&
          rows * c->lay.ld_data >= (1 << 24) && !c->tcctl.stall;
 }
 
-RowPairs row_pairs(emc_ctx* c, int64_t rows) {
-  const Layout& y = c->lay;
-  int32_t* cnt = (int32_t*)(c->ws + y.rpcnt);
-  return RowPairs{cnt, cnt + rows, (uint8_t*)(cnt + rows + rows / 128), (int32_t*)(c->ws + y.rpk), (float*)(c->ws + y.rpw),
-                  (float*)(c->ws + y.rpp)};
+RowPairs row_pairs(emc_ctx* c, const PairsAt& at, int64_t rows) {
+  int32_t* cnt = (int32_t*)(c->ws + at.cnt);
+  return RowPairs{cnt, cnt + rows, (uint8_t*)(cnt + rows + rows / 128), (int32_t*)(c->ws + at.k),
+                  (float*)(c->ws + at.w), (float*)(c->ws + at.p)};
 }
 
 int update_ntiles(const emc_ctx* c) { return (int)((c->lay.ld_pix + 255) / 256); }
@@ -941,7 +983,7 @@ int do_normalize_pairs(emc_ctx* c, const void* L, int64_t Lrows, int64_t row_off
                        const double* Bsum, uint8_t* kbf, const FrameView* fv) {
   const Layout& y = c->lay;
   const int64_t rows = round_up(nrot, 128);
-  const RowPairs rp = row_pairs(c, rows);
+  const RowPairs rp = row_pairs(c, y.rp, rows);
   const PassTwo p2 = pass_two(c, fv, bias, Bsum, nrot);
   float2* lse2 = (float2*)(c->ws + y.lse2);
   const bool again = !S && !fv->kept_all;  // some live tiles are contracted again
@@ -952,9 +994,9 @@ int do_normalize_pairs(emc_ctx* c, const void* L, int64_t Lrows, int64_t row_off
   CU(launch_pairs_reset(rp, rows, s));
   if (again) CU(launch_mark_over(fv->tile_list, fv->tile_count, y.ld_data / 256, rp, s));
   CU(launch_normalize_pairs(src, p2, rp, s));
-  int32_t* tiles = (int32_t*)(c->ws + y.rptiles);
-  int32_t* n = (int32_t*)(c->ws + y.rpn);
-  CU(launch_over_lists(rp, rows, update_ntiles(c), tiles, (int32_t*)(c->ws + y.rpcodes), n, s));
+  int32_t* tiles = (int32_t*)(c->ws + y.rp.tiles);
+  int32_t* n = (int32_t*)(c->ws + y.rp.n);
+  CU(launch_over_lists(rp, rows, update_ntiles(c), tiles, (int32_t*)(c->ws + y.rp.codes), n, s));
   if (int st = clear_pass_two(c, P, rows, kbf, s)) return st;
   float* den = (float*)((char*)P + P_plane_bytes(&c->cfg, rows, y.ld_data));  // (those models')
   CU(launch_normalize_over(src, p2, rp, tiles, n, P, rows * y.ld_data, den, kbf, s));
@@ -980,7 +1022,7 @@ int do_update(emc_ctx* c, const void* P, int64_t Prows, int64_t nrot, float* Num
   const int64_t rows = round_up(nrot, 128);
   if (c->cfg.precision == EMC_PREC_FP32) {
     CU(launch_simt_update((const float*)P, y.ld_data, rows, c->Kb, y.ld_pix, c->cfg.n_pix,
-                          (uint32_t*)(c->ws + y.upnz), Num, den, s));
+                          (uint32_t*)(c->ws + y.nz), Num, den, s));
   } else {
     Planes pp{(void*)P, Prows * y.ld_data, y.ld_data};
     if (is_gauss(&c->cfg) || is_flu(&c->cfg)) {
@@ -1009,6 +1051,36 @@ int check_rot_range(emc_ctx* c, int64_t rot0, int64_t nrot) {
   return EMC_OK;
 }
 
+// the Poisson-fluence expansion keeps what it needs on the way in L
+Order* expand_scratch(emc_ctx* c) {
+  return is_flu(&c->cfg) && !(c->lay.g4 && c->geom.interior) ? nullptr : &c->expand_order;
+}
+
+// emc_update by the scratch that it takes
+int update_pairs(emc_ctx* ctx, const void* P, int64_t nrot, float* Num, float* den,
+                 cudaStream_t s) {
+  const Layout& y = ctx->lay;
+  const int64_t rows = round_up(nrot, 128);
+  if (ctx->cfg.precision == EMC_PREC_FP32) {
+    CU(launch_simt_update((const float*)P, y.ld_data, rows, ctx->Kb, y.ld_pix, ctx->cfg.n_pix,
+                          (uint32_t*)(ctx->ws + y.upnz), Num, den, s));
+    return EMC_OK;
+  }
+  // the rows' pairs from the planes; what is over on the tensor cores
+  const bool tail = is_gauss(&ctx->cfg) || is_flu(&ctx->cfg);  // den lies behind P
+  const int f16 = ctx->cfg.precision == EMC_PREC_FP16_SPLIT && !tail ? 1 : 0;
+  const RowPairs rp = row_pairs(ctx, y.uprp, rows);
+  int32_t* codes = (int32_t*)(ctx->ws + y.uprp.codes);
+  int32_t* n = (int32_t*)(ctx->ws + y.uprp.n);
+  CU(launch_pairs_reset(rp, rows, s));
+  CU(launch_pairs_from_planes((const uint16_t*)P, rows * y.ld_data, rows, y.ld_data, f16, rp, s));
+  CU(launch_over_lists(rp, rows, update_ntiles(ctx), (int32_t*)(ctx->ws + y.uprp.tiles), codes, n,
+                       s));
+  CU(launch_update_pairs(rp, rows, is_gauss(&ctx->cfg) ? ctx->Kb2 : ctx->Kb, f16, y.ld_pix, true,
+                         Num, tail ? nullptr : den, s));
+  return do_update(ctx, P, rows, nrot, Num, den, s, nullptr, nullptr, nullptr, codes, n + 1);
+}
+
 }  // namespace
 
 extern "C" {
@@ -1017,8 +1089,9 @@ int emc_expand(emc_ctx* ctx, const float* grid, int64_t rot0, int64_t nrot, void
                emc_stream stream) {
   if (!ctx || !grid || !L || !bias) return EMC_ERR_ARG;
   if (check_rot_range(ctx, rot0, nrot)) return EMC_ERR_ARG;
-  Scratch scratch(ctx, (cudaStream_t)stream);
-  return do_expand(ctx, grid, rot0, nrot, L, bias, (cudaStream_t)stream);
+  Scratch scratch(expand_scratch(ctx), (cudaStream_t)stream);
+  if (!scratch.ok()) return EMC_ERR_CUDA;
+  return scratch.done(do_expand(ctx, grid, rot0, nrot, L, bias, (cudaStream_t)stream));
 }
 
 int emc_loglik(emc_ctx* ctx, const void* L, const double* bias, int64_t nrot, double* lse_m,
@@ -1076,31 +1149,19 @@ int emc_update(emc_ctx* ctx, const void* P, int64_t nrot, float* Num, float* den
   if (check_rot_range(ctx, 0, nrot)) return EMC_ERR_ARG;
   if (!ctx->frames_loaded) return EMC_ERR_ARG;
   cudaStream_t s = (cudaStream_t)stream;
-  const Layout& y = ctx->lay;
   const int64_t rows = round_up(nrot, 128);
-  // (the dense tensor-core contraction takes no scratch, and needs no order)
-  if (ctx->cfg.precision != EMC_PREC_FP32 && !pairs_ok(ctx, rows))
-    return do_update(ctx, P, rows, nrot, Num, den, s);
-  Scratch scratch(ctx, s);
-  if (ctx->cfg.precision == EMC_PREC_FP32) {  // captured: every frame, without the bits
-    CU(launch_simt_update((const float*)P, y.ld_data, rows, ctx->Kb, y.ld_pix, ctx->cfg.n_pix,
-                          scratch.captured() ? nullptr : (uint32_t*)(ctx->ws + y.upnz), Num, den,
-                          s));
+  const bool fp32 = ctx->cfg.precision == EMC_PREC_FP32;
+  // (the dense contraction takes no scratch, and needs no order)
+  Scratch scratch(fp32 || pairs_ok(ctx, rows) ? &ctx->update_order : nullptr, s);
+  if (!scratch.ok()) return EMC_ERR_CUDA;
+  if (fp32 && scratch.captured()) {
+    CU(launch_simt_update((const float*)P, ctx->lay.ld_data, rows, ctx->Kb, ctx->lay.ld_pix,
+                          ctx->cfg.n_pix, nullptr, Num, den, s));
     return EMC_OK;
   }
-  if (scratch.captured()) return do_update(ctx, P, rows, nrot, Num, den, s);
-  // the rows' pairs from the planes; what is over on the tensor cores
-  const bool tail = is_gauss(&ctx->cfg) || is_flu(&ctx->cfg);  // den lies behind P
-  const int f16 = ctx->cfg.precision == EMC_PREC_FP16_SPLIT && !tail ? 1 : 0;
-  const RowPairs rp = row_pairs(ctx, rows);
-  int32_t* codes = (int32_t*)(ctx->ws + y.rpcodes);
-  int32_t* n = (int32_t*)(ctx->ws + y.rpn);
-  CU(launch_pairs_reset(rp, rows, s));
-  CU(launch_pairs_from_planes((const uint16_t*)P, rows * y.ld_data, rows, y.ld_data, f16, rp, s));
-  CU(launch_over_lists(rp, rows, update_ntiles(ctx), (int32_t*)(ctx->ws + y.rptiles), codes, n, s));
-  CU(launch_update_pairs(rp, rows, is_gauss(&ctx->cfg) ? ctx->Kb2 : ctx->Kb, f16, y.ld_pix, true,
-                         Num, tail ? nullptr : den, s));
-  return do_update(ctx, P, rows, nrot, Num, den, s, nullptr, nullptr, nullptr, codes, n + 1);
+  if (!fp32 && (scratch.captured() || !pairs_ok(ctx, rows)))
+    return do_update(ctx, P, rows, nrot, Num, den, s);
+  return scratch.done(update_pairs(ctx, P, nrot, Num, den, s));
 }
 
 int emc_compress(emc_ctx* ctx, int64_t rot0, int64_t nrot, const float* Num, const float* den,
@@ -1131,7 +1192,6 @@ int emc_iteration(emc_ctx* c, const float* grid_in, float* grid_out, emc_iter_st
   if (!c || !grid_in || !grid_out || grid_in == grid_out) return EMC_ERR_ARG;
   if (!c->frames_loaded) return EMC_ERR_ARG;
   cudaStream_t s = (cudaStream_t)stream;
-  Scratch scratch(c, s);
   const Layout& y = c->lay;
   const int64_t n_rot = c->cfg.n_rot;
   // pruned contexts alternate between two L and bias buffers: the last
@@ -1162,7 +1222,11 @@ int emc_iteration(emc_ctx* c, const float* grid_in, float* grid_out, emc_iter_st
   if (stats) CU(cudaEventRecord(c->ev[0], s));
   c->collected = false;
   if (c->collecting) CU(cudaMemsetAsync(c->col.count, 0, sizeof(unsigned long long), s));
-  if ((st = do_expand(c, grid_in, 0, n_rot, L, bias, s, Lold, bold))) return st;
+  {
+    Scratch scratch(expand_scratch(c), s);
+    if (!scratch.ok()) return EMC_ERR_CUDA;
+    if ((st = scratch.done(do_expand(c, grid_in, 0, n_rot, L, bias, s, Lold, bold)))) return st;
+  }
   // the row tiles and the bias sums (Gaussian: grid maximum and scales first;
   // Poisson fluence: the split); the cell layout of the model first where it is used
   kernels += (is_gauss(&c->cfg) ? 4 : (is_flu(&c->cfg) ? 3 : 2)) +
@@ -1340,13 +1404,13 @@ int emc_iteration(emc_ctx* c, const float* grid_in, float* grid_out, emc_iter_st
     }
     if (stats) CU(cudaEventRecord(c->ev[4], s));
     if ((st = do_update(c, P, crows, nr, Num, den, s, kbc, kbl, Kp,
-                        pairs ? (const int32_t*)(c->ws + y.rpcodes) : nullptr,
-                        pairs ? (const int32_t*)(c->ws + y.rpn) + 1 : nullptr)))
+                        pairs ? (const int32_t*)(c->ws + y.rp.codes) : nullptr,
+                        pairs ? (const int32_t*)(c->ws + y.rp.n) + 1 : nullptr)))
       return st;
     if (pairs) {
       // (the compression does not read Num of rows without mass)
       const bool g = is_gauss(&c->cfg);
-      CU(launch_update_pairs(row_pairs(c, crows), crows, pr ? Kp : (g ? c->Kb2 : c->Kb),
+      CU(launch_update_pairs(row_pairs(c, y.rp, crows), crows, pr ? Kp : (g ? c->Kb2 : c->Kb),
                              c->cfg.precision == EMC_PREC_FP16_SPLIT && !g ? 1 : 0, y.ld_pix,
                              false, Num, den, s));
     }
@@ -1564,7 +1628,6 @@ int emc_sparse_iteration(emc_ctx* c, const float* grid_in, float* grid_out, emc_
   if (!c || !grid_in || !grid_out || grid_in == grid_out) return EMC_ERR_ARG;
   if (!c->frames_loaded || !c->cand_loaded) return EMC_ERR_ARG;
   cudaStream_t s = (cudaStream_t)stream;
-  Scratch scratch(c, s);
   const Layout& y = c->lay;
   // pruned contexts: the buffer the last emc_iteration did not write, so that
   // its L stays for the next one's incremental bound
@@ -1581,7 +1644,11 @@ int emc_sparse_iteration(emc_ctx* c, const float* grid_in, float* grid_out, emc_
   const size_t gb = sizeof(double) * (size_t)c->cfg.N * c->cfg.N * c->cfg.N;
   int st;
   if (stats) CU(cudaEventRecord(c->ev[0], s));
-  if ((st = do_expand(c, grid_in, 0, c->cfg.n_rot, L, bias, s))) return st;
+  {
+    Scratch scratch(expand_scratch(c), s);
+    if (!scratch.ok()) return EMC_ERR_CUDA;
+    if ((st = scratch.done(do_expand(c, grid_in, 0, c->cfg.n_rot, L, bias, s)))) return st;
+  }
   if (stats) CU(cudaEventRecord(c->ev[1], s));
   if ((st = emc_sparse_estep(c, L, bias, Pc, lsec, stream))) return st;
   CU(launch_loglik_sum(lsec, nullptr, c->cfg.n_data, ll, s));  // sum_k lse_k over C_k
