@@ -411,7 +411,7 @@ int emc_loglik_static(const emc_config* cfg, const void* L, const double* bias,
                       int accumulate, int32_t* device_status, emc_stream stream);
 
 /* M-step, Eq. 2.11: Num (device float[rows][ld_pix]) = P K over frames;
- * den (device float[rows]) = sum_k P_jk.
+ * den (device float[rows]) = sum_k P_jk. P and Num must be 16-byte aligned.
  * Gaussian model: Num_ij = sum_k P_jk K_ik / phi_jk (Eq. 2.5 before the
  * division) from the planes emc_normalize wrote; den is copied from the end
  * of the P buffer. Poisson-fluence model: likewise, Num_ij =

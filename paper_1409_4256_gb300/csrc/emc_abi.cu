@@ -1148,6 +1148,8 @@ int emc_update(emc_ctx* ctx, const void* P, int64_t nrot, float* Num, float* den
   if (!ctx || !P || !Num || !den) return EMC_ERR_ARG;
   if (check_rot_range(ctx, 0, nrot)) return EMC_ERR_ARG;
   if (!ctx->frames_loaded) return EMC_ERR_ARG;
+  // (16-byte loads and tensor maps of P, 16-byte stores of Num)
+  if ((((uintptr_t)P | (uintptr_t)Num) & 15) || ((uintptr_t)den & 3)) return EMC_ERR_ARG;
   cudaStream_t s = (cudaStream_t)stream;
   const int64_t rows = round_up(nrot, 128);
   const bool fp32 = ctx->cfg.precision == EMC_PREC_FP32;
