@@ -933,14 +933,14 @@ __device__ __forceinline__ float cta_sum(float v, float* red) {
 // weight of P_jk K_k; den_j = sum of the row's P_jk. Each thread owns 8
 // consecutive pixels (one 16-byte load of a K row per pair), walking the packed
 // pairs four at a time. Rows without pairs are zeroed. Poisson-fluence model
-// (Bsum != NULL): the weights are P_jk B_j / N_k.
+// (Bsum != NULL): the weights are P_jk B_j / N_k. vec: Num is 16-byte aligned.
 template <bool KF16>
 __global__ void __launch_bounds__(256)
     sparse_update_kernel(const uint16_t* __restrict__ Kb, int64_t ld_pix,
                          const int64_t* __restrict__ off, const int2* __restrict__ ent, int M,
                          const float* __restrict__ Pc, float* __restrict__ Num,
                          float* __restrict__ den, const double* __restrict__ Bsum,
-                         const float* __restrict__ invn) {
+                         const float* __restrict__ invn, bool vec) {
   const int64_t j = blockIdx.x;
   const int64_t e0 = off[j], e1 = off[j + 1];
   float* out = Num + j * ld_pix;
@@ -985,10 +985,13 @@ __global__ void __launch_bounds__(256)
       }
       if (!one) __syncthreads();
     }
-    if (g < n8) {
+    if (g < n8 && vec) {
       float4* o4 = reinterpret_cast<float4*>(out + 8 * g);
       o4[0] = make_float4(acc[0], acc[1], acc[2], acc[3]);
       o4[1] = make_float4(acc[4], acc[5], acc[6], acc[7]);
+    } else if (g < n8) {
+#pragma unroll
+      for (int c = 0; c < 8; c++) out[8 * g + c] = acc[c];
     }
   }
   const float d = cta_sum(dsum, red);
@@ -1007,7 +1010,8 @@ __global__ void __launch_bounds__(256)
                              int64_t ld_pix, const int64_t* __restrict__ off,
                              const int2* __restrict__ ent, int M, const float* __restrict__ Pc,
                              float* __restrict__ Num, float* __restrict__ den,
-                             const double* __restrict__ Bsum, const float* __restrict__ invn) {
+                             const double* __restrict__ Bsum, const float* __restrict__ invn,
+                             bool vec) {
   const int64_t j = blockIdx.x;
   const int64_t e0 = off[j], e1 = off[j + 1];
   extern __shared__ float4 sm4u[];
@@ -1040,9 +1044,14 @@ __global__ void __launch_bounds__(256)
       }
     __syncthreads();  // the list is repacked, or the row written, after this
   }
-  float4* out = reinterpret_cast<float4*>(Num + j * ld_pix);
-  for (int64_t i = threadIdx.x; i < n4; i += 256)
-    out[i] = any ? sm4u[i] : make_float4(0.f, 0.f, 0.f, 0.f);
+  float* row = Num + j * ld_pix;
+  if (vec) {
+    float4* out = reinterpret_cast<float4*>(row);
+    for (int64_t i = threadIdx.x; i < n4; i += 256)
+      out[i] = any ? sm4u[i] : make_float4(0.f, 0.f, 0.f, 0.f);
+  } else {
+    for (int64_t i = threadIdx.x; i < ld_pix; i += 256) row[i] = any ? srow[i] : 0.f;
+  }
   const float d = cta_sum(dsum, red);
   if (threadIdx.x == 0) den[j] = d;
 }
@@ -1191,6 +1200,7 @@ cudaError_t launch_sparse_update(const uint16_t* Kb, int kf16, int64_t ld_pix,
                                  float* Num, float* den, cudaStream_t s, const double* Bsum,
                                  const float* invn) {
   if (Bsum && !invn) return cudaErrorInvalidValue;
+  const bool vec = ((uintptr_t)Num & 15) == 0;
   // the row of Num and the list share a CTA's 227 KB; between 56064 and 58048
   // pixels, where only the row fits, the frames' rows are read instead
   const size_t smem = sizeof(float) * (size_t)ld_pix;
@@ -1199,15 +1209,15 @@ cudaError_t launch_sparse_update(const uint16_t* Kb, int kf16, int64_t ld_pix,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     sparse_update_csr_kernel<<<(unsigned)rows, 256, smem, s>>>(koff, kent, ld_pix, off, ent, M, Pc,
-                                                               Num, den, Bsum, invn);
+                                                               Num, den, Bsum, invn, vec);
     return cudaGetLastError();
   }
   if (kf16)
     sparse_update_kernel<true><<<(unsigned)rows, 256, 0, s>>>(Kb, ld_pix, off, ent, M, Pc,
-                                                              Num, den, Bsum, invn);
+                                                              Num, den, Bsum, invn, vec);
   else
     sparse_update_kernel<false><<<(unsigned)rows, 256, 0, s>>>(Kb, ld_pix, off, ent, M, Pc,
-                                                               Num, den, Bsum, invn);
+                                                               Num, den, Bsum, invn, vec);
   return cudaGetLastError();
 }
 
