@@ -230,6 +230,23 @@ __device__ __forceinline__ void write_increments(float (&dp)[2], float (&dm)[2],
   cluster.sync();  // no CTA leaves while its rises may be read
 }
 
+// Two neighbouring elements of a 16-bit plane, in one access where WHOLE (the plane is
+// 4-byte aligned; a caller's L of the Gaussian and Poisson-fluence models need not be. A
+// flag in place of the template costs those 3 and 5%).
+template <bool WHOLE>
+__device__ __forceinline__ void put_pair(uint16_t* p, uint32_t v) {
+  if (WHOLE) {
+    *reinterpret_cast<uint32_t*>(p) = v;
+  } else {
+    p[0] = (uint16_t)v;
+    p[1] = (uint16_t)(v >> 16);
+  }
+}
+template <bool WHOLE>
+__device__ __forceinline__ uint32_t get_pair(const uint16_t* p) {
+  return WHOLE ? __ldcs(reinterpret_cast<const uint32_t*>(p)) : p[0] | (uint32_t)p[1] << 16;
+}
+
 // Eight bytes at a place of a 16-bit plane that need not be aligned to them.
 __device__ __forceinline__ void put_bytes8(uint16_t* p, unsigned long long v) {
   if (((uintptr_t)p & 7) == 0) {
@@ -249,7 +266,7 @@ __device__ __forceinline__ unsigned long long get_bytes8(const uint16_t* p) {
 
 // RPC rotations of a tile per CTA; with DELTA the tile's 128 / RPC CTAs are a
 // cluster, whose first one gathers the others' rises and falls.
-template <int PREC, bool INTERIOR, bool DELTA, int RPC>
+template <int PREC, bool INTERIOR, bool DELTA, int RPC, bool WHOLE = true>
 __global__ void __launch_bounds__(kTThreads, 6)
     expand_tile_kernel(const int4* __restrict__ qi_g, const float4* __restrict__ qlo_g,
                        int64_t ld_pix, int N, const float* __restrict__ grid,
@@ -359,14 +376,14 @@ __global__ void __launch_bounds__(kTThreads, 6)
           l[u] = fp16_bits(r - fp16_val(m[u]));
         }
         uint16_t* Lb = (uint16_t*)Lbase + o;
-        *reinterpret_cast<uint32_t*>(Lb) = (uint32_t)h[0] | ((uint32_t)h[1] << 16);
-        *reinterpret_cast<uint32_t*>(Lb + ps) = (uint32_t)m[0] | ((uint32_t)m[1] << 16);
-        *reinterpret_cast<uint32_t*>(Lb + 2 * ps) = (uint32_t)l[0] | ((uint32_t)l[1] << 16);
+        put_pair<WHOLE>(Lb, (uint32_t)h[0] | ((uint32_t)h[1] << 16));
+        put_pair<WHOLE>(Lb + ps, (uint32_t)m[0] | ((uint32_t)m[1] << 16));
+        put_pair<WHOLE>(Lb + 2 * ps, (uint32_t)l[0] | ((uint32_t)l[1] << 16));
       } else if (PREC == kOutW) {
         const uint32_t u0 = __float_as_uint(L[0]), u1 = __float_as_uint(L[1]);
         uint16_t* Lb = (uint16_t*)Lbase + o;
-        *reinterpret_cast<uint32_t*>(Lb) = __byte_perm(u0, u1, 0x7632);
-        *reinterpret_cast<uint32_t*>(Lb + ps) = __byte_perm(u0, u1, 0x5410);
+        put_pair<WHOLE>(Lb, __byte_perm(u0, u1, 0x7632));
+        put_pair<WHOLE>(Lb + ps, __byte_perm(u0, u1, 0x5410));
       } else if (PREC == EMC_PREC_FP32) {
         *reinterpret_cast<float2*>((float*)Lbase + o) = make_float2(L[0], L[1]);
         if (DELTA && vrow) {
@@ -566,7 +583,7 @@ __global__ void __launch_bounds__(kTRows)
 // 96^3, 25728 rows x 7168 columns: W 970 us + split 788 us; one CTA per rotation in
 // double-float arithmetic and a pass of its own for the increments took 1790 + 474 us.
 constexpr int kSplitRows = 32;
-template <bool DELTA>
+template <bool DELTA, bool WHOLE = true>
 __global__ void __launch_bounds__(kTThreads)
     flu_split_kernel(const int4* __restrict__ qi_g, int64_t ld_pix, int64_t nrot,
                      uint16_t* __restrict__ Lbase, int64_t ps, const uint16_t* __restrict__ Lold,
@@ -589,8 +606,8 @@ __global__ void __launch_bounds__(kTThreads)
 #pragma unroll
     for (int r = 0; r < kAhead; r++) {
       const int64_t o = (r0 + rb + r) * ld_pix + i0;
-      wh[r] = __ldcs(reinterpret_cast<const uint32_t*>(Lbase + o));
-      wl[r] = __ldcs(reinterpret_cast<const uint32_t*>(Lbase + o + ps));
+      wh[r] = get_pair<WHOLE>(Lbase + o);
+      wl[r] = get_pair<WHOLE>(Lbase + o + ps);
       if (DELTA)
 #pragma unroll
         for (int q = 0; q < 3; q++)
@@ -636,9 +653,9 @@ __global__ void __launch_bounds__(kTThreads)
           l[u] = bf16_bits(rest - bf16_val(m[u]));
         }
         uint16_t* Lb = Lbase + o;
-        *reinterpret_cast<uint32_t*>(Lb) = (uint32_t)h[0] | ((uint32_t)h[1] << 16);
-        *reinterpret_cast<uint32_t*>(Lb + ps) = (uint32_t)m[0] | ((uint32_t)m[1] << 16);
-        *reinterpret_cast<uint32_t*>(Lb + 2 * ps) = (uint32_t)l[0] | ((uint32_t)l[1] << 16);
+        put_pair<WHOLE>(Lb, (uint32_t)h[0] | ((uint32_t)h[1] << 16));
+        put_pair<WHOLE>(Lb + ps, (uint32_t)m[0] | ((uint32_t)m[1] << 16));
+        put_pair<WHOLE>(Lb + 2 * ps, (uint32_t)l[0] | ((uint32_t)l[1] << 16));
         if (DELTA && vrow) {
 #pragma unroll
           for (int u = 0; u < 2; u++) {
@@ -729,7 +746,8 @@ cudaError_t launch_tiles(const Geom& g, const float* grid, const float4* g4, con
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  const int rpc = ns * nt * 4 < 6 * (int64_t)sms ? 16 : 32;
+  const bool whole = ((uintptr_t)L.base & 3) == 0 || (out != kOutGauss && out != kOutW);
+  const int rpc = ns * nt * 4 < 6 * (int64_t)sms || !whole ? 16 : 32;
   cudaLaunchConfig_t lc{};
   lc.gridDim = dim3((unsigned)(ns * nt * (kTRows / rpc)));
   lc.blockDim = dim3(kTThreads);
@@ -741,8 +759,8 @@ cudaError_t launch_tiles(const Geom& g, const float* grid, const float4* g4, con
   lc.attrs = &at;
   lc.numAttrs = delta ? 1 : 0;
   cudaError_t e = cudaSuccess;
-#define EMC_TILE_R(P, I, DL, RP)                                                               \
-  e = cudaLaunchKernelEx(&lc, expand_tile_kernel<P, I, DL, RP>, g.qi, g.qlo, g.ld_pix, g.N,    \
+#define EMC_TILE_R(P, I, DL, ...)                                                              \
+  e = cudaLaunchKernelEx(&lc, expand_tile_kernel<P, I, DL, __VA_ARGS__>, g.qi, g.qlo, g.ld_pix, g.N,    \
                          grid, g4, rot, nrot, rows, w_floor, L.base, L.plane_stride, partial,  \
                          Lold, D, ntp, (unsigned)ns, gsc, status)
 #define EMC_TILE(P, I, DL)                   \
@@ -759,16 +777,23 @@ cudaError_t launch_tiles(const Geom& g, const float* grid, const float4* g4, con
     else EMC_TILE(P, false, false);            \
   }
 #define EMC_TILE_O(P) /* no increments */      \
-  if (g.interior) EMC_TILE(P, true, false);    \
-  else EMC_TILE(P, false, false);
+  do {                                         \
+    if (g.interior) EMC_TILE(P, true, false);  \
+    else EMC_TILE(P, false, false);            \
+  } while (0);
+#define EMC_TILE_L(P) /* any address of L */                     \
+  if (whole) EMC_TILE_O(P)                                       \
+  else if (g.interior) EMC_TILE_R(P, true, false, 16, false);    \
+  else EMC_TILE_R(P, false, false, 16, false)
   switch (out) {
     case EMC_PREC_FP32: EMC_TILE_O(EMC_PREC_FP32); break;
     case EMC_PREC_BF16: EMC_TILE_O(EMC_PREC_BF16); break;
-    case kOutGauss: EMC_TILE_O(kOutGauss); break;
-    case kOutW: EMC_TILE_O(kOutW); break;
+    case kOutGauss: EMC_TILE_L(kOutGauss); break;
+    case kOutW: EMC_TILE_L(kOutW); break;
     case EMC_PREC_FP16_SPLIT: EMC_TILE_P(EMC_PREC_FP16_SPLIT); break;
     default: EMC_TILE_P(EMC_PREC_BF16_SPLIT); break;
   }
+#undef EMC_TILE_L
 #undef EMC_TILE_O
 #undef EMC_TILE_P
 #undef EMC_TILE
@@ -838,9 +863,12 @@ cudaError_t launch_expand_flu(const Geom& g, const float* grid, const float4* g4
   at.val.clusterDim.y = at.val.clusterDim.z = 1;
   lc.attrs = &at;
   lc.numAttrs = Lold ? 1 : 0;
-  return cudaLaunchKernelEx(&lc, Lold ? flu_split_kernel<true> : flu_split_kernel<false>, g.qi,
-                            g.ld_pix, nrot, Lb, L.plane_stride, (const uint16_t*)Lold, D, ntp,
-                            (unsigned)ns, status);
+  // (an iteration's L is aligned)
+  auto split = Lold ? flu_split_kernel<true>
+                    : (((uintptr_t)Lb & 3) == 0 ? flu_split_kernel<false>
+                                                : flu_split_kernel<false, false>);
+  return cudaLaunchKernelEx(&lc, split, g.qi, g.ld_pix, nrot, Lb, L.plane_stride,
+                            (const uint16_t*)Lold, D, ntp, (unsigned)ns, status);
 }
 
 }  // namespace emc

@@ -62,3 +62,27 @@ def test_sparse_update_takes_any_float_address(lists):
         assert bool((buf[:off] == -1).all()) and bool((buf[off + want.numel():] == -1).all())
         assert torch.equal(den, wden)
     assert ctx.status() == 0
+
+
+@pytest.mark.parametrize("model,precision", [("poisson_fluence", "bf16_split"),
+                                             ("gaussian", "fp16_split")])
+@pytest.mark.parametrize("D", [14, 40])
+def test_expansion_takes_any_plane_address(model, precision, D):
+    """L of the models whose planes were written one element at a time, at 2, 4 and 6 bytes
+    past an 8-byte boundary: the bits of an aligned one."""
+    import torch
+    from paper_1409_4256_gb300 import emc
+    ctx, n = context(D=D, model=model, precision=precision)
+    g = torch.Generator(device="cuda").manual_seed(2)
+    grid = torch.rand(16, 16, 16, generator=g, device="cuda") + 0.1
+    L, bias = ctx.expand(grid, 0, n)
+    for off in (1, 2, 3):
+        buf = torch.full((L.numel() // 2 + 4,), -1, dtype=torch.int16, device="cuda")
+        got = torch.empty_like(bias)
+        emc._check(emc.lib().emc_expand(ctx.h, grid.data_ptr(), 0, n, buf.data_ptr() + 2 * off,
+                                        got.data_ptr(), 0), "emc_expand")
+        torch.cuda.synchronize()
+        assert torch.equal(buf[off:off + L.numel() // 2], L.view(torch.int16))
+        assert bool((buf[:off] == -1).all()) and bool((buf[off + L.numel() // 2:] == -1).all())
+        assert torch.equal(got, bias)
+    assert ctx.status() == 0
