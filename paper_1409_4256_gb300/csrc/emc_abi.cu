@@ -1230,8 +1230,10 @@ int emc_iteration(emc_ctx* c, const float* grid_in, float* grid_out, emc_iter_st
     if ((st = scratch.done(do_expand(c, grid_in, 0, n_rot, L, bias, s, Lold, bold)))) return st;
   }
   // the row tiles and the bias sums (Gaussian: grid maximum and scales first;
-  // Poisson fluence: the split); the cell layout of the model first where it is used
-  kernels += (is_gauss(&c->cfg) ? 4 : (is_flu(&c->cfg) ? 3 : 2)) +
+  // Poisson fluence: the split, or all in one); the cell layout of the model first where it is used
+  kernels += (is_gauss(&c->cfg) ? 4
+              : is_flu(&c->cfg) ? expand_flu_launches(y.rows, y.ld_pix, Lold != nullptr)
+                                : 2) +
              ((y.g4 && c->geom.interior) ? 1 : 0);
   if (stats) CU(cudaEventRecord(c->ev[1], s));
   float* S = (c->cfg.flags & EMC_FLAG_STORE_SCORES) ? (float*)(c->ws + y.S) : nullptr;

@@ -114,8 +114,9 @@ cudaError_t launch_expand_gauss(const Geom& g, const float* grid, const float4* 
                                 double sigma, int32_t* status, cudaStream_t s);
 // Poisson-fluence model: L = log(W / B_j) + c as the BF16 three-term split;
 // bias = double[2][rows]: log w_j, then B_j = sum_i W_ij; Bctx[row] = B_j too.
-// W and its row sums lie in L's planes on the way: no scratch. Lold, D, ntp, bpm: as
-// launch_expand_tile.
+// W and its row sums lie in L's planes or in shared memory on the way: no scratch. Lold, D,
+// ntp, bpm: as launch_expand_tile. expand_flu_launches: its kernels.
+int expand_flu_launches(int64_t rows, int64_t ld_pix, bool delta);
 cudaError_t launch_expand_flu(const Geom& g, const float* grid, const float4* g4, const RotFX* rot,
                               const double* logw, int64_t nrot, int64_t rows, float w_floor,
                               double c, Planes L, double* bias, double* Bctx, const void* Lold,

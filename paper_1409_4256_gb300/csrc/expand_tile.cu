@@ -544,6 +544,13 @@ __global__ void __launch_bounds__(kTRows)
 // every rest, the mid/lo accumulator would grow to N_k al and round at that
 // size on every K step.
 //
+// c - log B as ah (1/8 grid) + al
+__device__ __forceinline__ float2 flu_shift_split(double c, double B, bool valid) {
+  const double aj = valid ? c - log(B) : 0.0;
+  const float ah = (float)(rint(aj * kHiScale) / kHiScale);
+  return make_float2(ah, (float)(aj - (double)ah));
+}
+
 // Per row: bias = log w_j (-inf on padding rows), B_j (0) into Bsum and Bctx, and
 // (ah, al) over the row's partial sums (low: plane 2), one copy for each slice.
 __global__ void __launch_bounds__(kTRows)
@@ -564,16 +571,38 @@ __global__ void __launch_bounds__(kTRows)
     for (int u = 0; u < 16; u++) B += __longlong_as_double((long long)part[u]);
   }
   const bool v = row < nrot;
-  const double aj = v ? c - log(B) : 0.0;
-  const float ah = (float)(rint(aj * kHiScale) / kHiScale);
-  const float al = (float)(aj - (double)ah);
+  const float2 as = flu_shift_split(c, B, v);
   const unsigned long long a =
-      (unsigned long long)__float_as_uint(al) << 32 | __float_as_uint(ah);
+      (unsigned long long)__float_as_uint(as.y) << 32 | __float_as_uint(as.x);
   for (int q = 0; q < n_slices; q++) put_bytes8(own + (int64_t)q * kTPix, a);
   bias[row] = v ? logw[row] : -INFINITY;
   Bsum[row] = v ? B : 0.0;
   Bctx[row] = v ? B : 0.0;
   if (bpm && threadIdx.x == 0) bpm[blockIdx.x] = bpm[nt + blockIdx.x] = 0.f;  // log w stays
+}
+
+struct FluSplit {
+  uint16_t h, m, l;
+  bool bad;
+};
+__device__ __forceinline__ FluSplit flu_split(float W, bool used, float ah, float al) {
+  FluSplit o;
+  float hi = 0.f, rest = 0.f;
+  o.bad = false;
+  if (used) {
+    const float x = logf(W);
+    const float s = x + ah;  // two-sum: s + e = x + ah exactly
+    const float bb = s - x;
+    const float e = (x - (s - bb)) + (ah - bb);
+    hi = round_to(s + (e + al), kHiScale);
+    o.bad = hi < kHiMin || hi > kHiMax;
+    hi = fminf(fmaxf(hi, kHiMin), kHiMax);
+    rest = ((s - hi) + e) + al;
+  }
+  o.h = bf16_bits(hi);
+  o.m = bf16_bits(rest);
+  o.l = bf16_bits(rest - bf16_val(o.m));
+  return o;
 }
 
 // W to the three BF16 planes of L in place, and with DELTA the increments from the last
@@ -637,20 +666,13 @@ __global__ void __launch_bounds__(kTThreads)
         uint16_t h[2], m[2], l[2];
 #pragma unroll
         for (int u = 0; u < 2; u++) {
-          float hi = 0.f, rest = 0.f;
-          if (vrow && used[u]) {
-            const float x = logf(__uint_as_float(__byte_perm(wl[r], wh[r], u ? 0x7632 : 0x5410)));
-            const float s = x + ah;  // two-sum: s + e = x + ah exactly
-            const float bb = s - x;
-            const float e = (x - (s - bb)) + (ah - bb);
-            hi = round_to(s + (e + al), kHiScale);
-            if (hi < kHiMin || hi > kHiMax) bad = 1;
-            hi = fminf(fmaxf(hi, kHiMin), kHiMax);
-            rest = ((s - hi) + e) + al;
-          }
-          h[u] = bf16_bits(hi);
-          m[u] = bf16_bits(rest);
-          l[u] = bf16_bits(rest - bf16_val(m[u]));
+          const FluSplit f =
+              flu_split(__uint_as_float(__byte_perm(wl[r], wh[r], u ? 0x7632 : 0x5410)),
+                        vrow && used[u], ah, al);
+          h[u] = f.h;
+          m[u] = f.m;
+          l[u] = f.l;
+          bad |= f.bad;
         }
         uint16_t* Lb = Lbase + o;
         put_pair<WHOLE>(Lb, (uint32_t)h[0] | ((uint32_t)h[1] << 16));
@@ -674,6 +696,135 @@ __global__ void __launch_bounds__(kTThreads)
   if (bad) set_status(status, EMC_ERR_UNSUPPORTED);
   if constexpr (DELTA)
     write_increments<EMC_PREC_BF16_SPLIT>(dp, dm, rises, inside, t, i0, ld_pix, ntp, D);
+}
+
+// The whole Poisson-fluence expansion of small problems in one launch, a CTA of TH threads per
+// rotation with W in shared memory: the three launches above leave most SMs idle there and
+// each waits for the one before. TH / 128 slices of 256 pixels at a time; the sums in
+// the order of the other form, so the bits are the same whichever runs. Bound by the
+// latency of a slice's chain of loads: 384 threads where the SMs hold all rows' CTAs at
+// once, 128 (ten CTAs an SM) where they do not (flu_row_threads).
+constexpr int kFluSlices = 40;  // 40 KB of W
+template <int TH>
+constexpr int flu_ctas() {  // an SM
+  return TH == 128 ? 10 : 3;
+}
+template <int TH, bool INTERIOR, bool WHOLE>
+__global__ void __launch_bounds__(TH, flu_ctas<TH>())
+    expand_flu_row_kernel(const int4* __restrict__ qi_g, const float4* __restrict__ qlo_g,
+                          int64_t ld_pix, int N, const float* __restrict__ grid,
+                          const float4* __restrict__ g4, const RotFX* __restrict__ rot,
+                          const double* __restrict__ logw, int64_t nrot, float w_floor, double c,
+                          int slices, uint16_t* __restrict__ Lbase, int64_t ps,
+                          double* __restrict__ bias, double* __restrict__ Bsum,
+                          double* __restrict__ Bctx, int32_t* status) {
+  extern __shared__ float2 wrow[];  // W of the row, a pixel pair an entry
+  __shared__ RowFX R;
+  __shared__ float2 rs[kFluSlices][kTThreads / 32];
+  __shared__ double part[kFluSlices];
+  __shared__ float2 as;
+  const int64_t row = blockIdx.x;
+  const bool valid = row < nrot;
+  const int lane = threadIdx.x & 31, tt = threadIdx.x & (kTThreads - 1);
+  if (threadIdx.x < 9) {
+    const int e = threadIdx.x;
+    const int h = valid ? rot[row].hi[e] : 0;
+    const float l = valid ? rot[row].lo[e] : 0.f;
+    const float hf = (float)h * 0x1p-20f;
+    R.hi[e] = h;
+    R.hf[e] = make_float2(hf, hf);
+    R.lo[e] = make_float2(l, l);
+  }
+  const long long centre = ((long long)(N >> 1) << 32) + ((N & 1) ? (1LL << 31) : 0LL);
+  __syncthreads();
+  int nonfinite = 0;
+  for (int sl = threadIdx.x / kTThreads; valid && sl < slices; sl += TH / kTThreads) {
+    const int64_t i0 = (int64_t)sl * kTPix + 2 * tt;
+    const bool inside = i0 < ld_pix;
+    int4 qi[2];
+    float4 q[2];
+#pragma unroll
+    for (int u = 0; u < 2; u++) {
+      qi[u] = inside ? qi_g[i0 + u] : make_int4(0, 0, 0, 0);
+      q[u] = inside ? qlo_g[i0 + u] : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    const float2 qh[3] = {make_float2((float)qi[0].x * 0x1p-12f, (float)qi[1].x * 0x1p-12f),
+                          make_float2((float)qi[0].y * 0x1p-12f, (float)qi[1].y * 0x1p-12f),
+                          make_float2((float)qi[0].z * 0x1p-12f, (float)qi[1].z * 0x1p-12f)};
+    const float2 ql[3] = {make_float2(q[0].x, q[1].x), make_float2(q[0].y, q[1].y),
+                          make_float2(q[0].z, q[1].z)};
+    int f[2][3];
+    float t[2][3], L[2], ws[2];
+    rotate_pair(R, qi, qh, ql, centre, f, t);
+#pragma unroll
+    for (int u = 0; u < 2; u++) {
+      const bool used = qi[u].w != 0;
+      float W = 0.f;
+      if (INTERIOR && g4)
+        W = cell_value(load_cell(g4, (f[u][0] * N + f[u][1]) * N + f[u][2]), t[u]);
+      else if (used)
+        W = trilinear_fx<INTERIOR>(grid, N, f[u], t[u]);
+      nonfinite |= used && !(fabsf(W) <= 3.4e38f);
+      W = fmaxf(W, w_floor);
+      ws[u] = used && qi[u].w == 1 ? W : 0.f;
+      L[u] = used ? W : 0.f;
+    }
+    if (inside) wrow[i0 / 2] = make_float2(L[0], L[1]);
+    const f2 pair = two_sum(ws[0], ws[1]);
+    float a = 0.f, ae = 0.f;
+#pragma unroll
+    for (int m = 0; m < 8; m++) {  // eight lanes' pairs, then the four sums of them
+      const float x = __shfl_sync(0xffffffffu, pair.h, (lane & 24) + m);
+      const float y = __shfl_sync(0xffffffffu, pair.l, (lane & 24) + m);
+      const f2 z = two_sum(a, x);
+      a = z.h;
+      ae += y + z.l;
+    }
+#pragma unroll
+    for (int off = 8; off <= 16; off <<= 1) {
+      const float ao = __shfl_xor_sync(0xffffffffu, a, off);
+      const float eo = __shfl_xor_sync(0xffffffffu, ae, off);
+      const f2 z = two_sum(a, ao);
+      a = z.h;
+      ae += eo + z.l;
+    }
+    if (lane == 0) rs[sl][tt >> 5] = make_float2(a, ae);
+  }
+  __syncthreads();
+  if ((int)threadIdx.x < slices) {
+    float s = 0.f, se = 0.f;
+    for (int w = 0; valid && w < kTThreads / 32; w++) {
+      const float2 v = rs[threadIdx.x][w];
+      const f2 a = two_sum(s, v.x);
+      s = a.h;
+      se += v.y + a.l;
+    }
+    part[threadIdx.x] = f32_to_f64(s) + f32_to_f64(se);
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double B = 0.0;
+    for (int q = 0; q < slices; q++) B += part[q];
+    as = flu_shift_split(c, B, valid);
+    bias[row] = valid ? logw[row] : -INFINITY;
+    Bsum[row] = valid ? B : 0.0;
+    Bctx[row] = valid ? B : 0.0;
+  }
+  __syncthreads();
+  const float ah = as.x, al = as.y;
+  int bad = 0;
+  for (int64_t i0 = 2 * threadIdx.x; i0 < ld_pix; i0 += 2 * TH) {
+    const float2 W = valid ? wrow[i0 / 2] : make_float2(0.f, 0.f);
+    const FluSplit x = flu_split(W.x, valid && qi_g[i0].w != 0, ah, al);
+    const FluSplit y = flu_split(W.y, valid && qi_g[i0 + 1].w != 0, ah, al);
+    bad |= x.bad || y.bad;
+    uint16_t* Lb = Lbase + row * ld_pix + i0;
+    put_pair<WHOLE>(Lb, (uint32_t)x.h | ((uint32_t)y.h << 16));
+    put_pair<WHOLE>(Lb + ps, (uint32_t)x.m | ((uint32_t)y.m << 16));
+    put_pair<WHOLE>(Lb + 2 * ps, (uint32_t)x.l | ((uint32_t)y.l << 16));
+  }
+  if (nonfinite) set_status(status, EMC_ERR_NUMERIC);
+  if (bad) set_status(status, EMC_ERR_UNSUPPORTED);
 }
 
 // the grid in the cell layout of load_cell
@@ -837,6 +988,27 @@ cudaError_t launch_expand_gauss(const Geom& g, const float* grid, const float4* 
   return cudaGetLastError();
 }
 
+namespace {
+
+// Threads a rotation of the one-launch form, or 0 for the tile kernels. us of a call by the
+// tile kernels, 384 and 128 threads a rotation (rows x columns):
+//   512 x 832 39, 19, 21    512 x 3264 48, 31, 42     512 x 7296 73, 56, 89
+//   1408 x 832 45, 38, 27   1408 x 3264 68, 74, 67    1408 x 7296 120, 138, 181
+//   3328 x 832 56, 66, 48   3328 x 1856 81, 93, 82    10880 x 128 48, -, about 57
+// (one CTA of 256 threads a rotation and a double-float grid point, before the tile kernels:
+// 19, 36 and 66; 31, 66 and 132; 54 and 81)
+int flu_row_threads(int64_t rows, int64_t ns) {
+  if (ns > kFluSlices) return 0;
+  if (rows <= 512) return 384;
+  return rows <= 4096 && rows * ns <= 16384 ? 128 : 0;
+}
+
+}  // namespace
+
+int expand_flu_launches(int64_t rows, int64_t ld_pix, bool delta) {
+  return !delta && flu_row_threads(rows, expand_tile_slices(ld_pix)) ? 1 : 3;
+}
+
 cudaError_t launch_expand_flu(const Geom& g, const float* grid, const float4* g4, const RotFX* rot,
                               const double* logw, int64_t nrot, int64_t rows, float w_floor,
                               double c, Planes L, double* bias, double* Bctx, const void* Lold,
@@ -844,10 +1016,25 @@ cudaError_t launch_expand_flu(const Geom& g, const float* grid, const float4* g4
                               cudaStream_t s) {
   if (rows <= 0) return cudaSuccess;
   const int64_t ns = expand_tile_slices(g.ld_pix), nt = rows / kTRows;
+  uint16_t* Lb = (uint16_t*)L.base;
+  const int th = Lold ? 0 : flu_row_threads(rows, ns);
+  if (th) {
+    const bool whole = ((uintptr_t)Lb & 3) == 0;
+    const int threads = whole ? th : 128;
+    auto kern = threads == 384 ? (g.interior ? expand_flu_row_kernel<384, true, true>
+                                             : expand_flu_row_kernel<384, false, true>)
+                : whole        ? (g.interior ? expand_flu_row_kernel<128, true, true>
+                                             : expand_flu_row_kernel<128, false, true>)
+                               : (g.interior ? expand_flu_row_kernel<128, true, false>
+                                             : expand_flu_row_kernel<128, false, false>);
+    kern<<<(unsigned)rows, threads, sizeof(float) * (size_t)g.ld_pix, s>>>(
+        g.qi, g.qlo, g.ld_pix, g.N, grid, g4, rot, logw, nrot, w_floor, c, (int)ns, Lb,
+        L.plane_stride, bias, bias + rows, Bctx, status);
+    return cudaGetLastError();
+  }
   cudaError_t e = launch_tiles(g, grid, g4, rot, nrot, rows, kOutW, w_floor, L, nullptr, nullptr,
                                nullptr, 0, nullptr, status, s);
   if (e != cudaSuccess) return e;
-  uint16_t* Lb = (uint16_t*)L.base;
   flu_bias_kernel<<<(unsigned)nt, kTRows, 0, s>>>(Lb + 2 * L.plane_stride, g.ld_pix, (int)ns, logw,
                                                   nrot, c, bias, bias + rows, Bctx,
                                                   Lold ? bpm : nullptr, nt);
