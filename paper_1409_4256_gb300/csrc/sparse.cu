@@ -9,6 +9,8 @@
 // frames' rows of K, which are 3x smaller than a split log W row and stay in L2
 // at the 64^3 size. Scores use the same exact split as the dense forms (hi on
 // the 1/8 grid accumulated exactly, a small residual).
+#include <limits.h>
+
 #include "emc_common.cuh"
 #include "emc_internal.h"
 
@@ -635,7 +637,10 @@ __device__ __forceinline__ void unpack2(uint32_t w, float& lo, float& hi) {
 // + 1) of S_jk, the 1 covering every rounding. A pair whose S^hi lies more than 2 E_k +
 // 111 below the frame's largest scores more than 110 below its best candidate:
 // its P is 0 in FP32 and its share of the log-sum-exp below FP64's rounding.
-// Counts and hi are small integers, so the sums are integer and exact.
+// Counts and hi are small integers, so the sums are integer and exact; with the bias in
+// 1/1024 of hi's unit (for a |bias| below 2^48; beyond, rows go by that limit) S^hi is a
+// 64-bit integer and no rounding enters the comparison, however large bias and scores.
+// A row whose bias is not finite keeps its pairs.
 //
 // One CTA per rotation row, a warp per pair. The row is staged in 16 bits: the list's
 // neighbouring entries are near pixels, so a warp's gathers fall on about
@@ -647,12 +652,20 @@ template <int PREC>
 struct HiGrid {  // units of hi
   static constexpr float scale = PREC == EMC_PREC_FP16_SPLIT ? 64.f : 8.f;
 };
+constexpr long long kBoundKeep = LLONG_MAX;
+// the bias in units of 2^-10 / scale
+__device__ __forceinline__ long long bound_bias(double b, float scale) {
+  const double x = b * (double)(1024.f * scale);
+  if (!isfinite(x)) return kBoundKeep;
+  return __double2ll_rn(fmin(fmax(x, -0x1p61), 0x1p61));
+}
+
 template <int PREC>
 __global__ void __launch_bounds__(256)
     sparse_bound_kernel(const void* __restrict__ L, int64_t ld_pix, const double* __restrict__ bias,
                         const int64_t* __restrict__ off, const int2* __restrict__ ent, int M,
                         const int64_t* __restrict__ koff, const uint32_t* __restrict__ kent,
-                        float* __restrict__ Sh) {
+                        long long* __restrict__ Sh) {
   const int64_t j = blockIdx.x;
   const int64_t e0 = off[j], e1 = off[j + 1];
   if (e0 == e1) return;
@@ -669,8 +682,10 @@ __global__ void __launch_bounds__(256)
       h = bf16_val(reinterpret_cast<const uint16_t*>(L)[j * ld_pix + i]) * scale;
     Lq[i] = (int16_t)(int)h;
   }
+  __shared__ long long row_bias;
+  if (threadIdx.x == 0) row_bias = bound_bias(bias[j], scale);
   __syncthreads();
-  const float bj = (float)bias[j];
+  const long long bj = row_bias;
   const int lane = threadIdx.x & 31;
   for (int64_t e = e0 + (threadIdx.x >> 5); e < e1; e += 8) {
     const int2 km = ent[e];
@@ -691,15 +706,16 @@ __global__ void __launch_bounds__(256)
       sum += (int)(w >> 16) * Lq[w & 0xffffu];
     }
     sum = __reduce_add_sync(0xffffffffu, sum);
-    if (lane == 0) Sh[(int64_t)km.x * M + km.y] = (float)sum * (1.f / scale) + bj;
+    if (lane == 0)
+      Sh[(int64_t)km.x * M + km.y] = bj == kBoundKeep ? bj : bj + ((long long)sum << 10);
   }
 }
 
-// One warp per frame: 1 into Sh where the pair's score is needed, else 0 and a
-// score of -infinity.
+// One warp per frame: 1 into need where the pair's score is needed, else 0 and a
+// score of -infinity over its S^hi. units: of S^hi in one.
 __global__ void __launch_bounds__(256)
     sparse_choose_kernel(const int64_t* __restrict__ koff, const uint32_t* __restrict__ kent,
-                         int64_t n_data, int M, float step, float* __restrict__ Sh,
+                         int64_t n_data, int M, long long units, float* __restrict__ need,
                          double* __restrict__ Sc) {
   const int64_t k = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
@@ -707,15 +723,21 @@ __global__ void __launch_bounds__(256)
   int total = 0;  // N_k < 65536
   for (int64_t f = koff[k] + lane; f < koff[k + 1]; f += 32) total += (int)(kent[f] >> 16);
   total = __reduce_add_sync(0xffffffffu, total);
-  float* s = Sh + k * M;
-  float mx = -INFINITY;
-  for (int m = lane; m < M; m += 32) mx = fmaxf(mx, s[m]);
-  for (int o = 16; o; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-  const float least = mx - (2.f * ((float)total * step + 1.f) + 111.f);
+  double* score = Sc + k * M;
+  const long long* s = reinterpret_cast<const long long*>(score);
+  long long mx = LLONG_MIN;
   for (int m = lane; m < M; m += 32) {
-    const bool on = !(s[m] < least);  // a NaN stays
-    s[m] = on ? 1.f : 0.f;
-    if (!on) Sc[k * M + m] = -INFINITY;
+    const long long x = s[m];
+    if (x != kBoundKeep) mx = max(mx, x);
+  }
+  for (int o = 16; o; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+  // 2 E_k + 111, where E_k = N_k step / 2 + 1 and 1024 units are one step
+  const long long gap = 1024ll * total + 113 * units;
+  const long long least = mx == LLONG_MIN ? mx : mx - gap;
+  for (int m = lane; m < M; m += 32) {
+    const bool on = s[m] >= least;
+    need[k * M + m] = on ? 1.f : 0.f;
+    if (!on) score[m] = -INFINITY;
   }
 }
 
@@ -1150,7 +1172,7 @@ cudaError_t launch_sparse_scores(const Planes& L, int precision, int64_t rows, c
                            (int)sb);                                                            \
   if (e != cudaSuccess) return e;                                                               \
   sparse_bound_kernel<P><<<(unsigned)rows, 256, sb, s>>>(L.base, ld_pix, bias, off, ent, M,     \
-                                                         koff, kent, need)
+                                                         koff, kent, (long long*)Sc)
     switch (precision) {
       case EMC_PREC_FP32: EMC_SPARSE_BOUND(EMC_PREC_FP32); break;
       case EMC_PREC_FP16_SPLIT: EMC_SPARSE_BOUND(EMC_PREC_FP16_SPLIT); break;
@@ -1158,9 +1180,9 @@ cudaError_t launch_sparse_scores(const Planes& L, int precision, int64_t rows, c
     }
 #undef EMC_SPARSE_BOUND
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    const float step = precision == EMC_PREC_FP16_SPLIT ? 1.f / 128.f : 1.f / 16.f;
+    const long long units = 1024 * (precision == EMC_PREC_FP16_SPLIT ? 64 : 8);
     sparse_choose_kernel<<<(unsigned)((n_data * 32 + 255) / 256), 256, 0, s>>>(koff, kent, n_data,
-                                                                              M, step, need, Sc);
+                                                                              M, units, need, Sc);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
 #define EMC_SPARSE_SCORES(P, C)                                                              \
