@@ -27,7 +27,7 @@ struct PairsAt {
 struct Layout {
   int64_t ld_pix, ld_data, rows, chunk_rows, num_rows, part_tiles;
   size_t qh, ql, logw, Kb, status, L, bias, lse_m, lse_s, lse2, part_m, part_s, S, P,
-      Num, den, gnum, gden, scalar, fbin, finv, cand, ccnt, coff, cent, Sc, Pc, lsec, gk, gauss,
+      Num, den, gnum, gden, scalar, fbin, finv, cand, ccnt, coff, cent, Sc, subias, Pc, lsec, gk, gauss,
       Kb2, skcnt, skoff, skent, dupsrc, duprank, pixmax, fcn, finvn, fB, kbflag, kbcnt, kblist,
       Kp, perm, perm2, iperm, nsum, nsum_p, cn_p, invn_p, best, lsem_s, lses_s, live, tlist, slot, klist,
       tcount, sortH, sortoff, cgs, cgp, cgqh, cgql, cgqi, cgqlo, cgqf, L2, bias2, Ub, Ub2, Lk, Mk, Mk2, best2,
@@ -171,6 +171,7 @@ Layout make_layout(const emc_config* c) {
   y.coff = M ? take(sizeof(int64_t) * (size_t)(y.rows + 1)) : 0;
   y.cent = M ? take(sizeof(int2) * (size_t)c->n_data * M) : 0;
   y.Sc = M ? take(sizeof(double) * (size_t)y.ld_data * M) : 0;
+  y.subias = M ? take(sizeof(int64_t) * (size_t)y.rows) : 0;
   y.Pc = M ? take(sizeof(float) * (size_t)y.ld_data * M) : 0;
   y.lsec = M ? take(sizeof(double) * (size_t)y.ld_data) : 0;
   y.gk = is_gauss(c) ? take(sizeof(float4) * (size_t)y.ld_data) : 0;
@@ -1609,7 +1610,9 @@ int emc_sparse_estep(emc_ctx* ctx, const void* L, const double* bias, float* P, 
                           (const int64_t*)(ctx->ws + y.coff), (const int2*)(ctx->ws + y.cent), M,
                           csr ? (const int64_t*)(ctx->ws + y.skoff) : nullptr,
                           csr ? (const uint32_t*)(ctx->ws + y.skent) : nullptr, ctx->cfg.n_data,
-                          P, Sc, s));  // (P holds the choice of pairs until it is written)
+                          (const int32_t*)(ctx->ws + y.cand), ctx->cfg.n_rot,
+                          (long long*)(ctx->ws + y.subias), (int*)P, Sc,
+                          s));  // (P holds sums of the pairs until it is written)
   CU(launch_sparse_lse(Sc, ctx->cfg.n_data, y.ld_data, M, P, lse, ctx->status, s, ctx->flu_cn));
   return EMC_OK;
 }

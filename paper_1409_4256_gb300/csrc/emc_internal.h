@@ -394,12 +394,14 @@ cudaError_t launch_csr_build(const int32_t* cand, int64_t n_data, int M, int64_t
                              int64_t rows, int32_t* cnt, int64_t* off, int2* ent,
                              int32_t* status, cudaStream_t s);
 // koff/kent (non-NULL): the frames' non-zero pixel lists (EMC_FLAG_SPARSE_K)
-// replace their dense rows in both sparse contractions. need: scratch [n_data][M]; with the
-// lists, pairs that cannot matter (P = 0 in FP32) get the score -infinity.
+// replace their dense rows in both sparse contractions; pairs that cannot matter (P = 0 in
+// FP32) may then get the score -infinity. upper: scratch [n_data][M];
+// ubias: [rows].
 cudaError_t launch_sparse_scores(const Planes& L, int precision, int64_t rows, const double* bias,
                                  const uint16_t* Kb, int64_t ld_pix, const int64_t* off,
                                  const int2* ent, int M, const int64_t* koff,
-                                 const uint32_t* kent, int64_t n_data, float* need, double* Sc,
+                                 const uint32_t* kent, int64_t n_data, const int32_t* cand,
+                                 int64_t n_rot, long long* ubias, int* upper, double* Sc,
                                  cudaStream_t s);
 // shift (may be NULL): per-frame constant of the scores, removed from lse_c
 cudaError_t launch_sparse_lse(const double* Sc, int64_t n_data, int64_t ld_data, int M, float* Pc,

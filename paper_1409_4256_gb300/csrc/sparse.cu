@@ -11,6 +11,8 @@
 // the 1/8 grid accumulated exactly, a small residual).
 #include <limits.h>
 
+#include <algorithm>
+
 #include "emc_common.cuh"
 #include "emc_internal.h"
 
@@ -631,197 +633,372 @@ __device__ __forceinline__ void unpack2(uint32_t w, float& lo, float& hi) {
   }
 }
 
-// Candidate pairs that can matter, from the hi part of log W alone (frames as
-// lists). With hi on the 1/8 grid (FP16 split: 1/64) and the rest at most half a
-// step, S^hi_jk = sum_i K_ik hi_ij + bias_j is within E_k = N_k / 16 + 1 (N_k / 128
-// + 1) of S_jk, the 1 covering every rounding. A pair whose S^hi lies more than 2 E_k +
-// 111 below the frame's largest scores more than 110 below its best candidate:
-// its P is 0 in FP32 and its share of the log-sum-exp below FP64's rounding.
-// Counts and hi are small integers, so the sums are integer and exact; with the bias in
-// 1/1024 of hi's unit (for a |bias| below 2^48; beyond, rows go by that limit) S^hi is a
-// 64-bit integer and no rounding enters the comparison, however large bias and scores.
-// A row whose bias is not finite keeps its pairs.
-//
-// One CTA per rotation row, a warp per pair. The row is staged in 16 bits: the list's
-// neighbouring entries are near pixels, so a warp's gathers fall on about
-// half as many words as lanes and meet few bank conflicts, where the full split's two FP32
-// gathers cost seven wavefronts. 64^3, 20000 frames x 512 candidates: the
-// scores of every pair took 5.06 ms; this pass 2.86 ms (28 GB of lists through L2), the choice 0.04 ms and the scores of the
-// pairs left 0.41 ms.
+// log W_ij as the contraction sees it, hi + rest with hi on the precision's grid (1/8; FP16
+// split: 1/64).
 template <int PREC>
-struct HiGrid {  // units of hi
-  static constexpr float scale = PREC == EMC_PREC_FP16_SPLIT ? 64.f : 8.f;
-};
-constexpr long long kBoundKeep = LLONG_MAX;
-// the bias in units of 2^-10 / scale
-__device__ __forceinline__ long long bound_bias(double b, float scale) {
-  const double x = b * (double)(1024.f * scale);
-  if (!isfinite(x)) return kBoundKeep;
-  return __double2ll_rn(fmin(fmax(x, -0x1p61), 0x1p61));
+__device__ __forceinline__ void row_parts(const void* __restrict__ L, int64_t plane_stride,
+                                          int64_t o, float& h, float& r) {
+  if (PREC == EMC_PREC_FP32) {
+    const float x = reinterpret_cast<const float*>(L)[o];
+    h = rintf(x * 8.f) * 0.125f;
+    r = x - h;
+  } else if (PREC == EMC_PREC_FP16_SPLIT) {
+    const uint16_t* Lb = reinterpret_cast<const uint16_t*>(L) + o;
+    h = fp16_val(Lb[0]);
+    r = fp16_val(Lb[plane_stride]);
+  } else {
+    const uint16_t* Lb = reinterpret_cast<const uint16_t*>(L) + o;
+    h = bf16_val(Lb[0]);
+    if (PREC == EMC_PREC_BF16_SPLIT) {
+      r = bf16_val(Lb[plane_stride]) + bf16_val(Lb[2 * plane_stride]);
+    } else {
+      r = h;
+      h = rintf(h * 8.f) * 0.125f;
+      r -= h;
+    }
+  }
+}
+
+// Scores from the frames' non-zero lists (a pixel and its count in 32 bits an entry). One CTA
+// per rotation row, a warp per pair. log W_j is staged as integers in units of 2^-24 (hi
+// exactly, the rest to 2^-25, below the split's own rounding), so the sums are integer and
+// exact: nothing depends on their order or on the size of scores and bias.
+//  * Lists of few entries on average: one gather an entry, of the 32-bit integer. A lane
+//    finishes the pairs that the warp summed for it, 32 at a time: an FP64 instruction
+//    takes a warp 16 cycles of its pipe however few lanes need it, and five a pair took as long
+//    as a short list's gathers.
+//  * Longer ones (lists_long): first the upper 16 bits alone, whose gathers meet half the bank
+//    conflicts (neighbouring entries are near pixels), bound S_jk to N_k / 256. Only pairs that
+//    may lie within 111 of their frame's best are then given the lower 16 bits' sum; the
+//    others' P is 0 in FP32 and their share of the log-sum-exp below FP64's rounding.
+// 64^3, 20000 frames of 710 entries x 512 candidates: two FP32 gathers an entry (seven shared-memory
+// wavefronts) 5.25 ms, one integer gather 4.19, two stages 3.56; 32^3, 8000 x 512, 92 entries 1.08 ms,
+// 0.49, 1.24.
+// A row with a value beyond +-127.8 or not finite (no model's log W is, but FP32's of a
+// zero floor) sums its parts in FP32 from memory, as such values always were.
+constexpr float kFixUnits = 16777216.f;
+constexpr size_t kSparseRowMax = 232448;  // a row of hi and rest in a CTA's shared memory
+
+// hi + rest in units of 2^-24 (to integers by adding 1.5 2^23: the conversion runs on the
+// FP64 pipe); beyond is set where they do not fit.
+__device__ __forceinline__ int fixed_value(float h, float r, bool& beyond) {
+  beyond |= !(fabsf(h) < 127.8f && fabsf(r) < 0.1f);
+  const int hq = __float_as_int(fmaf(h, 64.f, 12582912.f)) - 0x4b400000;
+  const int rq = __float_as_int(fmaf(r, kFixUnits, 12582912.f)) - 0x4b400000;
+  return hq * (1 << 18) + rq;
+}
+
+// A row of L as integers, two pixels at a time: put(i / 2, values). By the CTA's 256 threads;
+// returns, behind a barrier, whether a value lies beyond.
+template <int PREC, class Put>
+__device__ __forceinline__ bool stage_row(const void* __restrict__ L, int64_t plane_stride,
+                                          int64_t row, int64_t ld_pix, Put put) {
+  bool beyond = false;
+  if (PREC == EMC_PREC_FP32 || ((uintptr_t)L & 3)) {
+    for (int64_t i = 2 * threadIdx.x; i < ld_pix; i += 512) {
+      float h[2], r[2];
+#pragma unroll
+      for (int u = 0; u < 2; u++) row_parts<PREC>(L, plane_stride, row + i + u, h[u], r[u]);
+      put(i / 2, make_int2(fixed_value(h[0], r[0], beyond), fixed_value(h[1], r[1], beyond)));
+    }
+  } else {
+    const uint32_t* p = reinterpret_cast<const uint32_t*>(reinterpret_cast<const uint16_t*>(L) + row);
+    const int64_t next = plane_stride / 2;  // planes are whole rows of 64
+    for (int64_t i = threadIdx.x; i < ld_pix / 2; i += 256) {
+      const uint32_t a = p[i];
+      const uint32_t b = PREC == EMC_PREC_BF16 ? 0u : p[i + next];
+      const uint32_t c = PREC == EMC_PREC_BF16_SPLIT ? p[i + 2 * next] : 0u;
+      int q[2];
+#pragma unroll
+      for (int u = 0; u < 2; u++) {
+        const uint16_t x = (uint16_t)(a >> (16 * u)), y = (uint16_t)(b >> (16 * u));
+        float h, r;
+        if (PREC == EMC_PREC_FP16_SPLIT) {
+          h = fp16_val(x);
+          r = fp16_val(y);
+        } else if (PREC == EMC_PREC_BF16_SPLIT) {
+          h = bf16_val(x);
+          r = bf16_val(y) + bf16_val((uint16_t)(c >> (16 * u)));
+        } else {
+          h = rintf(bf16_val(x) * 8.f) * 0.125f;
+          r = bf16_val(x) - h;
+        }
+        q[u] = fixed_value(h, r, beyond);
+      }
+      put(i, make_int2(q[0], q[1]));
+    }
+  }
+  return __syncthreads_or(beyond);
 }
 
 template <int PREC>
-__global__ void __launch_bounds__(256)
-    sparse_bound_kernel(const void* __restrict__ L, int64_t ld_pix, const double* __restrict__ bias,
-                        const int64_t* __restrict__ off, const int2* __restrict__ ent, int M,
-                        const int64_t* __restrict__ koff, const uint32_t* __restrict__ kent,
-                        long long* __restrict__ Sh) {
-  const int64_t j = blockIdx.x;
-  const int64_t e0 = off[j], e1 = off[j + 1];
-  if (e0 == e1) return;
-  extern __shared__ float4 sm4[];
-  int16_t* Lq = reinterpret_cast<int16_t*>(sm4);
-  constexpr float scale = HiGrid<PREC>::scale;
-  for (int64_t i = threadIdx.x; i < ld_pix; i += 256) {
-    float h;
-    if (PREC == EMC_PREC_FP32)
-      h = rintf(reinterpret_cast<const float*>(L)[j * ld_pix + i] * scale);
-    else if (PREC == EMC_PREC_FP16_SPLIT)
-      h = fp16_val(reinterpret_cast<const uint16_t*>(L)[j * ld_pix + i]) * scale;
-    else
-      h = bf16_val(reinterpret_cast<const uint16_t*>(L)[j * ld_pix + i]) * scale;
-    Lq[i] = (int16_t)(int)h;
+__device__ __forceinline__ double sum_parts(const void* __restrict__ L, int64_t plane_stride,
+                                            int64_t row, const int64_t* __restrict__ koff,
+                                            const uint32_t* __restrict__ kent) {
+  float ah = 0.f, ar = 0.f;
+  for (int64_t f = koff[0] + (threadIdx.x & 31); f < koff[1]; f += 32) {
+    float h, r;
+    row_parts<PREC>(L, plane_stride, row + (kent[f] & 0xffffu), h, r);
+    ah = fmaf((float)(kent[f] >> 16), h, ah);
+    ar = fmaf((float)(kent[f] >> 16), r, ar);
   }
-  __shared__ long long row_bias;
-  if (threadIdx.x == 0) row_bias = bound_bias(bias[j], scale);
-  __syncthreads();
-  const long long bj = row_bias;
+  for (int o = 16; o; o >>= 1) {
+    ah += __shfl_xor_sync(0xffffffffu, ah, o);
+    ar += __shfl_xor_sync(0xffffffffu, ar, o);
+  }
+  return (double)ah + (double)ar;
+}
+
+// Whether the frames' lists take the two stages: the mean number of entries, from
+// `least` on (0: never).
+__device__ __forceinline__ bool lists_long(const int64_t* __restrict__ koff, int64_t n_data,
+                                           int least) {
+  return least > 0 && koff[n_data] >= least * n_data;
+}
+
+template <int PREC>
+__device__ __forceinline__ void score_row(const void* __restrict__ L, int64_t plane_stride,
+                                          int64_t ld_pix, const double* __restrict__ bias,
+                                          int64_t j, int64_t e0, int64_t e1,
+                                          const int2* __restrict__ ent, int M,
+                                          const int64_t* __restrict__ koff,
+                                          const uint32_t* __restrict__ kent, int2* Lq2,
+                                          double* __restrict__ Sc) {
+  const int* Lq = reinterpret_cast<const int*>(Lq2);
+  const int lane = threadIdx.x & 31;
+  const bool beyond = stage_row<PREC>(L, plane_stride, j * ld_pix, ld_pix,
+                                      [&](int64_t i2, int2 q) { Lq2[i2] = q; });
+  const double bj = bias[j];
+  for (int64_t b = e0 + (threadIdx.x >> 5); b < e1; b += 256) {
+    const bool on = b + 8 * lane < e1;  // the CTA's warps take the list's pairs in turn
+    const int2 mine = on ? ent[b + 8 * lane] : make_int2(0, 0);
+    const int pairs = (int)min((int64_t)32, (e1 - b + 7) / 8);
+    double own = 0.0;
+    if (!beyond) {
+      long long sum = 0;
+      for (int src = 0; src < pairs; src++) {
+        const int k = __shfl_sync(0xffffffffu, mine.x, src);
+        const int64_t f0 = koff[k];
+        const int n = (int)(koff[k + 1] - f0);
+        const uint32_t* list = kent + f0;
+        long long acc = 0;
+        for (int f = lane; f < n; f += 128) {
+          uint32_t w[4];
+#pragma unroll
+          for (int u = 0; u < 4; u++) w[u] = f + 32 * u < n ? list[f + 32 * u] : 0u;
+#pragma unroll
+          for (int u = 0; u < 4; u++) acc += (long long)(int)(w[u] >> 16) * Lq[w[u] & 0xffffu];
+        }
+        // |acc| < 2^47 (N_k < 2^16): 24 bits and the rest, each summed in one instruction
+        const unsigned low = __reduce_add_sync(0xffffffffu, (unsigned)(acc & 0xffffff));
+        const int high = __reduce_add_sync(0xffffffffu, (int)(acc >> 24));
+        if (lane == src) sum = ((long long)high << 24) + low;
+      }
+      own = (double)sum * (1.0 / kFixUnits);
+    } else {
+      for (int src = 0; src < pairs; src++) {
+        const int k = __shfl_sync(0xffffffffu, mine.x, src);
+        const double sum = sum_parts<PREC>(L, plane_stride, j * ld_pix, koff + k, kent);
+        if (lane == src) own = sum;
+      }
+    }
+    if (on) Sc[(int64_t)mine.x * M + mine.y] = own + bj;
+  }
+}
+
+// Stage one: the sum of the upper 16 bits (units of 2^-8) into the place of the pair's P. With
+// the bias, S_jk is within [0, N_k / 256) above it (S^u_jk). The choice compares these in
+// units of 2^-18 as 64-bit integers (FP64 took 100 us of 3.6 ms), with the biases in
+// `ubias` (|bias| by at most 2^43: beyond, rows go by that limit; one that is not finite
+// keeps its pairs).
+constexpr int kPairBeyond = INT_MIN, kPairLeft = INT_MIN + 1;  // to be scored; not to be
+constexpr long long kBoundKeep = LLONG_MAX;
+__device__ __forceinline__ long long bound_bias(double b) {
+  const double x = b * 0x1p18;
+  if (!isfinite(x)) return kBoundKeep;
+  return __double2ll_rn(fmin(fmax(x, -0x1p61), 0x1p61));
+}
+template <int PREC>
+__device__ __forceinline__ void bound_row(const void* __restrict__ L, int64_t plane_stride,
+                                          int64_t ld_pix, const double* __restrict__ bias,
+                                          int64_t j, int64_t e0, int64_t e1,
+                                          const int2* __restrict__ ent, int M,
+                                          const int64_t* __restrict__ koff,
+                                          const uint32_t* __restrict__ kent, int2* Lq2,
+                                          long long* __restrict__ ubias,
+                                          int* __restrict__ upper) {
+  const int16_t* Lu = reinterpret_cast<const int16_t*>(Lq2);
+  if (threadIdx.x == 0) ubias[j] = bound_bias(bias[j]);
+  const bool beyond =
+      stage_row<PREC>(L, plane_stride, j * ld_pix, ld_pix, [&](int64_t i2, int2 q) {
+        reinterpret_cast<unsigned*>(Lq2)[i2] = __byte_perm(q.x, q.y, 0x7632);
+      });
   const int lane = threadIdx.x & 31;
   for (int64_t e = e0 + (threadIdx.x >> 5); e < e1; e += 8) {
     const int2 km = ent[e];
     const int64_t f0 = koff[km.x];
     const int n = (int)(koff[km.x + 1] - f0);
     const uint32_t* list = kent + f0;
-    int sum = 0;
+    int sum = 0;  // below 65535 x 32743 < 2^31
     int f = lane;
     for (; f + 96 < n; f += 128) {
       uint32_t w[4];
 #pragma unroll
       for (int u = 0; u < 4; u++) w[u] = list[f + 32 * u];
 #pragma unroll
-      for (int u = 0; u < 4; u++) sum += (int)(w[u] >> 16) * Lq[w[u] & 0xffffu];
+      for (int u = 0; u < 4; u++) sum += (int)(w[u] >> 16) * Lu[w[u] & 0xffffu];
     }
     for (; f < n; f += 32) {
       const uint32_t w = list[f];
-      sum += (int)(w >> 16) * Lq[w & 0xffffu];
+      sum += (int)(w >> 16) * Lu[w & 0xffffu];
     }
     sum = __reduce_add_sync(0xffffffffu, sum);
-    if (lane == 0)
-      Sh[(int64_t)km.x * M + km.y] = bj == kBoundKeep ? bj : bj + ((long long)sum << 10);
+    if (lane == 0) upper[(int64_t)km.x * M + km.y] = beyond ? kPairBeyond : sum;
   }
 }
 
-// One warp per frame: 1 into need where the pair's score is needed, else 0 and a
-// score of -infinity over its S^hi. units: of S^hi in one.
+// A CTA per rotation row, in the form that the lists' length asks for. FORM: both in one launch,
+// or one of them alone (a launch of 50100 CTAs that find nothing to do takes 33 us), where
+// eight CTAs' 32-bit rows exceed an SM's shared memory and the 16-bit ones want less.
+enum { kFormBoth = 0, kFormScore = 1, kFormBound = 2 };
+template <int PREC, int FORM>
+__global__ void __launch_bounds__(256, 8)
+    sparse_rows_kernel(const void* __restrict__ L, int64_t plane_stride, int64_t ld_pix,
+                       const double* __restrict__ bias, const int64_t* __restrict__ off,
+                       const int2* __restrict__ ent, int M, const int64_t* __restrict__ koff,
+                       const uint32_t* __restrict__ kent, int64_t n_data, int least,
+                       long long* __restrict__ ubias, int* __restrict__ upper,
+                       double* __restrict__ Sc) {
+  const int64_t j = blockIdx.x;
+  const int64_t e0 = off[j], e1 = off[j + 1];
+  if (e0 == e1) return;
+  extern __shared__ int2 Lq2[];
+  const bool two = lists_long(koff, n_data, least);
+  if (FORM != kFormScore && two)
+    bound_row<PREC>(L, plane_stride, ld_pix, bias, j, e0, e1, ent, M, koff, kent, Lq2, ubias, upper);
+  if (FORM != kFormBound && !two)
+    score_row<PREC>(L, plane_stride, ld_pix, bias, j, e0, e1, ent, M, koff, kent, Lq2, Sc);
+}
+
+// One warp per frame: the pairs whose score is not needed are marked and get -infinity.
 __global__ void __launch_bounds__(256)
     sparse_choose_kernel(const int64_t* __restrict__ koff, const uint32_t* __restrict__ kent,
-                         int64_t n_data, int M, long long units, float* __restrict__ need,
+                         int64_t n_data, int least, int M, const int32_t* __restrict__ cand,
+                         int64_t n_rot, const long long* __restrict__ ubias, int* __restrict__ upper,
                          double* __restrict__ Sc) {
   const int64_t k = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
-  if (k >= n_data) return;
+  if (k >= n_data || !lists_long(koff, n_data, least)) return;
   int total = 0;  // N_k < 65536
   for (int64_t f = koff[k] + lane; f < koff[k + 1]; f += 32) total += (int)(kent[f] >> 16);
   total = __reduce_add_sync(0xffffffffu, total);
-  double* score = Sc + k * M;
-  const long long* s = reinterpret_cast<const long long*>(score);
+  int* u = upper + k * M;
+  const int32_t* c = cand + k * M;
+  auto bound = [&](int m) {  // S^u of pair m, or kBoundKeep; LLONG_MIN: no rotation of the sampling
+    if ((unsigned)c[m] >= (unsigned)n_rot) return LLONG_MIN;
+    const int x = u[m];
+    const long long b = ubias[c[m]];
+    return x == kPairBeyond || b == kBoundKeep ? kBoundKeep : b + ((long long)x << 10);
+  };
   long long mx = LLONG_MIN;
+#pragma unroll 4
   for (int m = lane; m < M; m += 32) {
-    const long long x = s[m];
+    const long long x = bound(m);
     if (x != kBoundKeep) mx = max(mx, x);
   }
   for (int o = 16; o; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-  // 2 E_k + 111, where E_k = N_k step / 2 + 1 and 1024 units are one step
-  const long long gap = 1024ll * total + 113 * units;
-  const long long least = mx == LLONG_MIN ? mx : mx - gap;
-  for (int m = lane; m < M; m += 32) {
-    const bool on = s[m] >= least;
-    need[k * M + m] = on ? 1.f : 0.f;
-    if (!on) score[m] = -INFINITY;
+  // N_k / 256 + 112, where 111 and the bias's rounding are enough
+  const long long gap = 1024ll * total + (112ll << 18);
+  const long long bottom = mx == LLONG_MIN ? mx + 1 : mx - gap;
+#pragma unroll 4
+  for (int m = lane; m < M; m += 32)
+    if (bound(m) < bottom) {
+      u[m] = kPairLeft;
+      Sc[k * M + m] = -INFINITY;
+    }
+}
+
+// Stage two: the lower 16 bits' sums of the needed pairs on top. The CTAs take rows in turn (a
+// grid of the SMs' own number: where lists are short nothing is left to do).
+template <int PREC>
+__global__ void __launch_bounds__(256, 8)
+    sparse_lower_kernel(const void* __restrict__ L, int64_t plane_stride, int64_t ld_pix,
+                        int64_t rows, const double* __restrict__ bias,
+                        const int64_t* __restrict__ off, const int2* __restrict__ ent, int M,
+                        const int64_t* __restrict__ koff, const uint32_t* __restrict__ kent,
+                        int64_t n_data, int least, const int* __restrict__ upper,
+                        double* __restrict__ Sc) {
+  if (!lists_long(koff, n_data, least)) return;
+  extern __shared__ int2 Lq2[];
+  const uint16_t* Ll = reinterpret_cast<const uint16_t*>(Lq2);
+  const int lane = threadIdx.x & 31;
+  for (int64_t j = blockIdx.x; j < rows; j += gridDim.x) {
+    const int64_t e0 = off[j], e1 = off[j + 1];
+    bool any = false;  // a row without a needed pair is passed over
+    for (int64_t e = e0 + threadIdx.x; e < e1; e += 256) {
+      const int2 km = ent[e];
+      any |= upper[(int64_t)km.x * M + km.y] != kPairLeft;
+    }
+    if (!__syncthreads_or(any)) continue;
+    const bool beyond =
+        stage_row<PREC>(L, plane_stride, j * ld_pix, ld_pix, [&](int64_t i2, int2 q) {
+          reinterpret_cast<unsigned*>(Lq2)[i2] = __byte_perm(q.x, q.y, 0x5410);
+        });
+    const double bj = bias[j];
+    for (int64_t b = e0 + (threadIdx.x >> 5); b < e1; b += 256) {
+      const int64_t e = b + 8 * lane;
+      const int2 mine = e < e1 ? ent[e] : make_int2(0, 0);
+      const int64_t at = (int64_t)mine.x * M + mine.y;
+      const int up = e < e1 ? upper[at] : kPairLeft;
+      const bool on = up != kPairLeft;
+      unsigned todo = __ballot_sync(0xffffffffu, on);
+      double parts = 0.0;
+      unsigned low = 0;
+      while (todo) {
+        const int src = __ffs(todo) - 1;
+        todo &= todo - 1;
+        const int k = __shfl_sync(0xffffffffu, mine.x, src);
+        if (beyond) {
+          const double x = sum_parts<PREC>(L, plane_stride, j * ld_pix, koff + k, kent);
+          if (lane == src) parts = x;
+          continue;
+        }
+        const int64_t f1 = koff[k + 1];
+        unsigned sum = 0;  // below 65535 x 65535 < 2^32
+        for (int64_t f = koff[k] + lane; f < f1; f += 32) {
+          const uint32_t w = kent[f];
+          sum += (w >> 16) * Ll[w & 0xffffu];
+        }
+        sum = __reduce_add_sync(0xffffffffu, sum);
+        if (lane == src) low = sum;
+      }
+      if (on)
+        Sc[at] = (beyond ? parts : (double)(((long long)up << 16) + low) * (1.0 / kFixUnits)) + bj;
+    }
+    __syncthreads();  // the row is staged anew
   }
 }
 
 // One CTA per rotation row: log W_j split into (hi on the 1/8 grid, rest) in
 // shared memory; each warp takes pairs (frame, slot) of the row's list, two
 // at a time, reading the frames' K rows 8 pixels (16 bytes) per lane.
-// CSR: the frames' non-zero pixel lists (pixel | count << 16, EMC_FLAG_SPARSE_K)
-// are read instead of their rows -- 4 bytes per non-zero pixel rather than 2
-// bytes per pixel -- and gathered against the staged row; the count x hi sums
-// stay exact (integral counts, hi on the 1/8 grid, frame totals below 2^16).
-// need (CSR, may be NULL): only the pairs with need[k M + m] != 0.
-template <int PREC, bool CSR>
+template <int PREC>
 __global__ void __launch_bounds__(256)
     sparse_scores_kernel(const void* __restrict__ L, int64_t plane_stride, int64_t ld_pix,
                          const double* __restrict__ bias, const uint16_t* __restrict__ Kb,
                          const int64_t* __restrict__ off, const int2* __restrict__ ent, int M,
-                         const int64_t* __restrict__ koff, const uint32_t* __restrict__ kent,
-                         const float* __restrict__ need, double* __restrict__ Sc) {
+                         double* __restrict__ Sc) {
   const int64_t j = blockIdx.x;
   const int64_t e0 = off[j], e1 = off[j + 1];
   if (e0 == e1) return;
   extern __shared__ float4 sm4[];
-  if (CSR && need) {  // a row without a needed pair
-    bool any = false;
-    for (int64_t e = e0 + threadIdx.x; e < e1; e += blockDim.x) {
-      const int2 km = ent[e];
-      any |= need[(int64_t)km.x * M + km.y] != 0.f;
-    }
-    if (!__syncthreads_or(any)) return;
-  }
   float* Lh = reinterpret_cast<float*>(sm4);
   float* Lr = Lh + ld_pix;
-  for (int64_t i = threadIdx.x; i < ld_pix; i += blockDim.x) {
-    float h, r;
-    if (PREC == EMC_PREC_FP32) {
-      const float x = reinterpret_cast<const float*>(L)[j * ld_pix + i];
-      h = rintf(x * 8.f) * 0.125f;
-      r = x - h;
-    } else if (PREC == EMC_PREC_FP16_SPLIT) {
-      const uint16_t* Lb = reinterpret_cast<const uint16_t*>(L) + j * ld_pix + i;
-      h = fp16_val(Lb[0]);
-      r = fp16_val(Lb[plane_stride]);
-    } else {
-      const uint16_t* Lb = reinterpret_cast<const uint16_t*>(L) + j * ld_pix + i;
-      h = bf16_val(Lb[0]);
-      r = PREC == EMC_PREC_BF16_SPLIT ? bf16_val(Lb[plane_stride]) + bf16_val(Lb[2 * plane_stride])
-                                      : 0.f;
-    }
-    Lh[i] = h;
-    Lr[i] = r;
-  }
+  for (int64_t i = threadIdx.x; i < ld_pix; i += blockDim.x)
+    row_parts<PREC>(L, plane_stride, j * ld_pix + i, Lh[i], Lr[i]);
   __syncthreads();
   const double bj = bias[j];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  if (CSR) {
-    // a warp looks 32 pairs over at a time (the CTA's warps in turn) and takes the needed ones
-    for (int64_t b = e0 + wid; b < e1; b += 32 * nw) {
-      const int64_t own = b + (int64_t)lane * nw;
-      const int2 mine = own < e1 ? ent[own] : make_int2(0, 0);
-      unsigned todo = __ballot_sync(
-          0xffffffffu, own < e1 && (!need || need[(int64_t)mine.x * M + mine.y] != 0.f));
-      while (todo) {
-        const int src = __ffs(todo) - 1;
-        todo &= todo - 1;
-        const int2 km = make_int2(__shfl_sync(0xffffffffu, mine.x, src),
-                                  __shfl_sync(0xffffffffu, mine.y, src));
-        const int64_t f1 = koff[km.x + 1];
-        float ah = 0.f, ar = 0.f;
-        for (int64_t f = koff[km.x] + lane; f < f1; f += 32) {
-          const uint32_t w = kent[f];
-          const int idx = (int)(w & 0xffffu);
-          const float c = (float)(w >> 16);
-          ah = fmaf(c, Lh[idx], ah);
-          ar = fmaf(c, Lr[idx], ar);
-        }
-        for (int o = 16; o; o >>= 1) {
-          ah += __shfl_xor_sync(0xffffffffu, ah, o);
-          ar += __shfl_xor_sync(0xffffffffu, ar, o);
-        }
-        if (lane == 0) Sc[(int64_t)km.x * M + km.y] = ((double)ah + (double)ar) + bj;
-      }
-    }
-    return;
-  }
   const int64_t n8 = ld_pix / 8;
   for (int64_t e = e0 + 2 * wid; e < e1; e += 2 * nw) {
     const bool two = e + 1 < e1;
@@ -1156,56 +1333,81 @@ cudaError_t launch_lse_values(const double* m, const double* sm, int64_t n, doub
   return cudaGetLastError();
 }
 
+namespace {
+
+// Mean entries of a list from which the two stages run (lists_long), or 0: never. us of a
+// call by one gather an entry, and by two stages:
+//   pairs a row, entries  204, 710     377, 397     158, 710   159, 266  158, 403  80, 403   80, 199
+//                         4194, 3562   1164, 1018   246, 237   924, 897  178, 212  651, 685  428, 736
+// Where a row has few pairs, the second launches gain nothing: 20, 710 310, 398; 35, 1527 392, 414.
+int two_stages_from(int64_t n_data, int M, int64_t n_rot) {
+  return n_data * M >= 64 * n_rot ? 384 : 0;
+}
+
+template <int PREC>
+cudaError_t sparse_scores(const Planes& L, int64_t rows, const double* bias, const uint16_t* Kb,
+                          int64_t ld_pix, const int64_t* off, const int2* ent, int M,
+                          const int64_t* koff, const uint32_t* kent, int64_t n_data,
+                          const int32_t* cand, int64_t n_rot, long long* ubias, int* upper,
+                          double* Sc, cudaStream_t s) {
+  const size_t row = sizeof(float) * (size_t)ld_pix;
+  const auto attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
+  cudaError_t e;
+  if (!kent) {
+    e = cudaFuncSetAttribute(sparse_scores_kernel<PREC>, attr, (int)(2 * row));
+    if (e != cudaSuccess) return e;
+    sparse_scores_kernel<PREC><<<(unsigned)rows, 256, 2 * row, s>>>(
+        L.base, L.plane_stride, ld_pix, bias, Kb, off, ent, M, Sc);
+    return cudaGetLastError();
+  }
+  const int least = two_stages_from(n_data, M, n_rot);
+  auto rows_kernel = [&](auto kern, size_t smem) {
+    cudaError_t r = cudaFuncSetAttribute(kern, attr, (int)smem);
+    if (r != cudaSuccess) return r;
+    kern<<<(unsigned)rows, 256, smem, s>>>(L.base, L.plane_stride, ld_pix, bias, off, ent, M, koff,
+                                           kent, n_data, least, ubias, upper, Sc);
+    return cudaGetLastError();
+  };
+  if (least == 0) return rows_kernel(sparse_rows_kernel<PREC, kFormScore>, row);
+  if ((e = cudaFuncSetAttribute(sparse_lower_kernel<PREC>, attr, (int)(row / 2))) != cudaSuccess)
+    return e;
+  if (8 * (row + 1024) <= 233472) {
+    e = rows_kernel(sparse_rows_kernel<PREC, kFormBoth>, row);
+  } else {
+    e = rows_kernel(sparse_rows_kernel<PREC, kFormScore>, row);
+    if (e == cudaSuccess) e = rows_kernel(sparse_rows_kernel<PREC, kFormBound>, row / 2);
+  }
+  if (e != cudaSuccess) return e;
+  int dev = 0, sms = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  sparse_choose_kernel<<<(unsigned)((n_data * 32 + 255) / 256), 256, 0, s>>>(
+      koff, kent, n_data, least, M, cand, n_rot, ubias, upper, Sc);
+  sparse_lower_kernel<PREC><<<(unsigned)std::min<int64_t>(rows, 8 * sms), 256, row / 2, s>>>(
+      L.base, L.plane_stride, ld_pix, rows, bias, off, ent, M, koff, kent, n_data, least, upper,
+      Sc);
+  return cudaGetLastError();
+}
+
+}  // namespace
+
 cudaError_t launch_sparse_scores(const Planes& L, int precision, int64_t rows, const double* bias,
                                  const uint16_t* Kb, int64_t ld_pix, const int64_t* off,
                                  const int2* ent, int M, const int64_t* koff,
-                                 const uint32_t* kent, int64_t n_data, float* need, double* Sc,
+                                 const uint32_t* kent, int64_t n_data, const int32_t* cand,
+                                 int64_t n_rot, long long* ubias, int* upper, double* Sc,
                                  cudaStream_t s) {
-  const size_t smem = 2 * sizeof(float) * (size_t)ld_pix;
-  cudaError_t e = cudaSuccess;
-  // (plain BF16 holds one rounded value, not on a grid: every pair is scored)
-  if (!kent || precision == EMC_PREC_BF16) need = nullptr;
-  if (need) {
-    const size_t sb = sizeof(int16_t) * (size_t)ld_pix;
-#define EMC_SPARSE_BOUND(P)                                                                     \
-  e = cudaFuncSetAttribute(sparse_bound_kernel<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
-                           (int)sb);                                                            \
-  if (e != cudaSuccess) return e;                                                               \
-  sparse_bound_kernel<P><<<(unsigned)rows, 256, sb, s>>>(L.base, ld_pix, bias, off, ent, M,     \
-                                                         koff, kent, (long long*)Sc)
-    switch (precision) {
-      case EMC_PREC_FP32: EMC_SPARSE_BOUND(EMC_PREC_FP32); break;
-      case EMC_PREC_FP16_SPLIT: EMC_SPARSE_BOUND(EMC_PREC_FP16_SPLIT); break;
-      default: EMC_SPARSE_BOUND(EMC_PREC_BF16_SPLIT); break;
-    }
-#undef EMC_SPARSE_BOUND
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    const long long units = 1024 * (precision == EMC_PREC_FP16_SPLIT ? 64 : 8);
-    sparse_choose_kernel<<<(unsigned)((n_data * 32 + 255) / 256), 256, 0, s>>>(koff, kent, n_data,
-                                                                              M, units, need, Sc);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  }
-#define EMC_SPARSE_SCORES(P, C)                                                              \
-  e = cudaFuncSetAttribute(sparse_scores_kernel<P, C>,                                       \
-                           cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);         \
-  if (e != cudaSuccess) return e;                                                            \
-  sparse_scores_kernel<P, C><<<(unsigned)rows, 256, smem, s>>>(                              \
-      L.base, L.plane_stride, ld_pix, bias, Kb, off, ent, M, koff, kent, need, Sc)
-#define EMC_SPARSE_SCORES_P(P)      \
-  if (kent) {                       \
-    EMC_SPARSE_SCORES(P, true);     \
-  } else {                          \
-    EMC_SPARSE_SCORES(P, false);    \
-  }
+  if (2 * sizeof(float) * (size_t)ld_pix > kSparseRowMax) return cudaErrorInvalidValue;
+#define EMC_SPARSE_SCORES(P)                                                                    \
+  return sparse_scores<P>(L, rows, bias, Kb, ld_pix, off, ent, M, koff, kent, n_data, cand, n_rot, \
+                             ubias, upper, Sc, s)
   switch (precision) {
-    case EMC_PREC_FP32: EMC_SPARSE_SCORES_P(EMC_PREC_FP32); break;
-    case EMC_PREC_BF16: EMC_SPARSE_SCORES_P(EMC_PREC_BF16); break;
-    case EMC_PREC_FP16_SPLIT: EMC_SPARSE_SCORES_P(EMC_PREC_FP16_SPLIT); break;
-    default: EMC_SPARSE_SCORES_P(EMC_PREC_BF16_SPLIT); break;
+    case EMC_PREC_FP32: EMC_SPARSE_SCORES(EMC_PREC_FP32);
+    case EMC_PREC_BF16: EMC_SPARSE_SCORES(EMC_PREC_BF16);
+    case EMC_PREC_FP16_SPLIT: EMC_SPARSE_SCORES(EMC_PREC_FP16_SPLIT);
+    default: EMC_SPARSE_SCORES(EMC_PREC_BF16_SPLIT);
   }
-#undef EMC_SPARSE_SCORES_P
 #undef EMC_SPARSE_SCORES
-  return cudaGetLastError();
 }
 
 cudaError_t launch_sparse_lse(const double* Sc, int64_t n_data, int64_t ld_data, int M, float* Pc,
