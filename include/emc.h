@@ -527,7 +527,7 @@ int emc_merge_candidates(const int32_t* first, int R, const int32_t* rest, int M
 
 /* Load candidate sets cand (device int32[n_data][n_cand], rotation indices)
  * and build the per-rotation pair lists the sparse calls use. An index outside
- * [0, n_rot) sets EMC_ERR_ARG in the device status. */
+ * [0, n_rot) sets EMC_ERR_ARG in the device status; the pair then has P = 0. */
 int emc_set_candidates(emc_ctx* ctx, const int32_t* cand, emc_stream stream);
 
 /* Eq. 2.4 over the candidate sets, from L and bias of emc_expand over all

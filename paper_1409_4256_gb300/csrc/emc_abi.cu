@@ -1591,7 +1591,7 @@ int emc_set_candidates(emc_ctx* ctx, const int32_t* cand, emc_stream stream) {
                      cudaMemcpyDeviceToDevice, s));
   CU(launch_csr_build(dc, ctx->cfg.n_data, M, ctx->cfg.n_rot, y.rows,
                       (int32_t*)(ctx->ws + y.ccnt), (int64_t*)(ctx->ws + y.coff),
-                      (int2*)(ctx->ws + y.cent), ctx->status, s));
+                      (int2*)(ctx->ws + y.cent), (double*)(ctx->ws + y.Sc), ctx->status, s));
   ctx->cand_loaded = true;
   return EMC_OK;
 }

@@ -390,9 +390,9 @@ cudaError_t launch_topr_columns(const float* S, int64_t ldS, const float* Sref, 
                                 const uint8_t* live = nullptr);
 cudaError_t launch_merge_candidates(const int32_t* first, int R, const int32_t* rest, int M_rest,
                                     int64_t n, int M, int32_t* out, cudaStream_t s);
-cudaError_t launch_csr_build(const int32_t* cand, int64_t n_data, int M, int64_t n_rot,
-                             int64_t rows, int32_t* cnt, int64_t* off, int2* ent,
-                             int32_t* status, cudaStream_t s);
+cudaError_t launch_csr_build(int32_t* cand, int64_t n_data, int M, int64_t n_rot, int64_t rows,
+                             int32_t* cnt, int64_t* off, int2* ent, double* Sc, int32_t* status,
+                             cudaStream_t s);
 // koff/kent (non-NULL): the frames' non-zero pixel lists (EMC_FLAG_SPARSE_K)
 // replace their dense rows in both sparse contractions; pairs that cannot matter (P = 0 in
 // FP32) may then get the score -infinity. upper: scratch [n_data][M];

@@ -495,13 +495,15 @@ cudaError_t launch_topr_columns(const float* S, int64_t ldS, const float* Sref, 
 }
 
 // --------------------------------------------------------- CSR by rotation --
-__global__ void csr_count_kernel(const int32_t* __restrict__ cand, int64_t n_pairs,
-                                 int64_t n_rot, int32_t* __restrict__ cnt, int32_t* status) {
+// An index outside the sampling becomes -1: it is in no list, and its score stays -infinity.
+__global__ void csr_count_kernel(int32_t* __restrict__ cand, int64_t n_pairs, int64_t n_rot,
+                                 int32_t* __restrict__ cnt, int32_t* status) {
   const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= n_pairs) return;
   const int32_t j = cand[e];
   if (j < 0 || j >= n_rot) {
     set_status(status, EMC_ERR_ARG);
+    cand[e] = -1;
     return;
   }
   atomicAdd(&cnt[j], 1);
@@ -552,10 +554,14 @@ __global__ void __launch_bounds__(1024)
 
 __global__ void csr_fill_kernel(const int32_t* __restrict__ cand, int64_t n_pairs, int M,
                                 const int64_t* __restrict__ off, int32_t* __restrict__ cur,
-                                int2* __restrict__ ent) {
+                                int2* __restrict__ ent, double* __restrict__ Sc) {
   const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= n_pairs) return;
   const int32_t j = cand[e];
+  if (j < 0) {
+    Sc[e] = -INFINITY;
+    return;
+  }
   const int64_t pos = off[j] + atomicAdd(&cur[j], 1);
   ent[pos] = make_int2((int)(e / M), (int)(e % M));
 }
@@ -606,9 +612,9 @@ cudaError_t launch_scan_counts(const int32_t* cnt, int64_t n, int64_t* off, cuda
   return cudaGetLastError();
 }
 
-cudaError_t launch_csr_build(const int32_t* cand, int64_t n_data, int M, int64_t n_rot,
-                             int64_t rows, int32_t* cnt, int64_t* off, int2* ent,
-                             int32_t* status, cudaStream_t s) {
+cudaError_t launch_csr_build(int32_t* cand, int64_t n_data, int M, int64_t n_rot, int64_t rows,
+                             int32_t* cnt, int64_t* off, int2* ent, double* Sc, int32_t* status,
+                             cudaStream_t s) {
   const int64_t n_pairs = n_data * M;
   cudaError_t e = cudaMemsetAsync(cnt, 0, sizeof(int32_t) * rows, s);
   if (e != cudaSuccess) return e;
@@ -616,7 +622,7 @@ cudaError_t launch_csr_build(const int32_t* cand, int64_t n_data, int M, int64_t
   csr_count_kernel<<<blocks, 256, 0, s>>>(cand, n_pairs, n_rot, cnt, status);
   csr_scan_kernel<<<1, 1024, 0, s>>>(cnt, rows, off);
   if ((e = cudaMemsetAsync(cnt, 0, sizeof(int32_t) * rows, s)) != cudaSuccess) return e;
-  csr_fill_kernel<<<blocks, 256, 0, s>>>(cand, n_pairs, M, off, cnt, ent);
+  csr_fill_kernel<<<blocks, 256, 0, s>>>(cand, n_pairs, M, off, cnt, ent, Sc);
   return cudaGetLastError();
 }
 
@@ -884,7 +890,7 @@ __global__ void __launch_bounds__(256, 8)
 __global__ void __launch_bounds__(256)
     sparse_choose_kernel(const int64_t* __restrict__ koff, const uint32_t* __restrict__ kent,
                          int64_t n_data, int least, int M, const int32_t* __restrict__ cand,
-                         int64_t n_rot, const long long* __restrict__ ubias, int* __restrict__ upper,
+                         const long long* __restrict__ ubias, int* __restrict__ upper,
                          double* __restrict__ Sc) {
   const int64_t k = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
@@ -894,8 +900,8 @@ __global__ void __launch_bounds__(256)
   total = __reduce_add_sync(0xffffffffu, total);
   int* u = upper + k * M;
   const int32_t* c = cand + k * M;
-  auto bound = [&](int m) {  // S^u of pair m, or kBoundKeep; LLONG_MIN: no rotation of the sampling
-    if ((unsigned)c[m] >= (unsigned)n_rot) return LLONG_MIN;
+  auto bound = [&](int m) {  // S^u of pair m, or kBoundKeep; LLONG_MIN: no rotation
+    if (c[m] < 0) return LLONG_MIN;
     const int x = u[m];
     const long long b = ubias[c[m]];
     return x == kPairBeyond || b == kBoundKeep ? kBoundKeep : b + ((long long)x << 10);
@@ -1272,6 +1278,7 @@ __global__ void missed_mass_kernel(const float* __restrict__ S, int64_t ldS,
   double sum = 0.0;
   for (int m = 0; m < M; m++) {
     const int64_t j = cand[k * M + m];
+    if (j < 0) continue;
     if (lv && !lv[(j >> 7) * nnt]) continue;
     const float e = S[c * ldS + j] + ((Sref[(j >> 5) * ld_data + c] - L.x) - L.y);
     sum += (double)__expf(e);
@@ -1382,7 +1389,7 @@ cudaError_t sparse_scores(const Planes& L, int64_t rows, const double* bias, con
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   sparse_choose_kernel<<<(unsigned)((n_data * 32 + 255) / 256), 256, 0, s>>>(
-      koff, kent, n_data, least, M, cand, n_rot, ubias, upper, Sc);
+      koff, kent, n_data, least, M, cand, ubias, upper, Sc);
   sparse_lower_kernel<PREC><<<(unsigned)std::min<int64_t>(rows, 8 * sms), 256, row / 2, s>>>(
       L.base, L.plane_stride, ld_pix, rows, bias, off, ent, M, koff, kent, n_data, least, upper,
       Sc);

@@ -148,3 +148,51 @@ def test_rows_beyond_the_integers(entries):
     L[7, 0] = np.inf
     ctx.sparse_estep(dev(L), dev(bias))
     assert ctx.status() == (-6 if K[:, 0].any() else 0)
+
+
+@pytest.mark.parametrize("lists,entries", [(False, 90), (True, 90), (True, 500)])
+def test_candidates_outside_the_sampling(lists, entries):
+    """An index outside [0, n_rot) is reported and left out: the other pairs' P and lse are
+    those of the frame without it, and so are the M-step and the missed mass."""
+    import torch
+    from paper_1409_4256_gb300 import emc, synth
+    det = synth.make_detector(30, 32)
+    quat, w = emc.quat_generate(2)
+    n_pix, n_rot, n_data, M = det.q.shape[0], quat.shape[0], 150, 200
+    rng = np.random.default_rng(entries)
+    ctx = emc.Context(32, det.q, quat, w, n_data, n_cand=M, sparse_k=lists, store_scores=True,
+                      w_floor=1e-6)
+    K = np.zeros((n_data, n_pix), dtype=np.int32)
+    for k in range(n_data):
+        K[k, rng.permutation(n_pix)[:entries]] = 1
+    ctx.set_frames(torch.as_tensor(K, device="cuda"))
+    cand = np.argsort(rng.random((n_data, n_rot)), axis=1)[:, :M].astype(np.int32)
+    g = torch.Generator(device="cuda").manual_seed(1)
+    grid = torch.exp(0.1 * torch.randn(32, 32, 32, generator=g, device="cuda"))
+    L, bias = ctx.expand(grid, 0, n_rot)
+    ctx.set_candidates(torch.as_tensor(cand, device="cuda"))
+    P, lse = ctx.sparse_estep(L, bias)
+    assert ctx.status() == 0
+    bad = cand.copy()
+    out = rng.random(cand.shape) < 0.1
+    bad[out] = rng.choice([-1, -(2 ** 31), n_rot, 2 ** 31 - 1], size=int(out.sum()))
+    ctx.set_candidates(torch.as_tensor(bad, device="cuda"))
+    assert ctx.status() == -1
+    Pb, lseb = ctx.sparse_estep(L, bias)
+    Num, den = ctx.sparse_update(Pb)
+    assert ctx.status() == 0
+    off = torch.as_tensor(out, device="cuda")
+    S = torch.log(P[:n_data].double()) + lse[:n_data, None]
+    want = torch.logsumexp(torch.where(off, -torch.inf, S), 1)
+    assert float((lseb[:n_data] - want).abs().max()) <= 1e-5
+    assert bool((Pb[:n_data][off] == 0).all())
+    assert float((Pb[:n_data].double().sum(1) - 1).abs().max()) <= 1e-5
+    assert abs(float(den[:n_rot].double().sum()) - n_data) <= 1e-5 * n_data
+    ctx.iteration(grid)
+    missed = ctx.missed_mass()
+    fr = torch.arange(n_data, dtype=torch.int32, device="cuda")
+    dense = ctx.responsibilities(fr).double()
+    held = torch.gather(dense, 1, torch.as_tensor(cand, device="cuda").long())
+    left = 1 - torch.where(off, 0.0, held).sum(1)
+    assert float((missed.double() - left).abs().max()) <= 1e-6
+    assert ctx.status() == 0
