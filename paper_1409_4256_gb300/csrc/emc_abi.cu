@@ -1074,7 +1074,8 @@ int update_pairs(emc_ctx* ctx, const void* P, int64_t nrot, float* Num, float* d
   int32_t* codes = (int32_t*)(ctx->ws + y.uprp.codes);
   int32_t* n = (int32_t*)(ctx->ws + y.uprp.n);
   CU(launch_pairs_reset(rp, rows, s));
-  CU(launch_pairs_from_planes((const uint16_t*)P, rows * y.ld_data, rows, y.ld_data, f16, rp, s));
+  CU(launch_pairs_from_planes((const uint16_t*)P, rows * y.ld_data, rows, y.ld_data,
+                              ctx->cfg.n_data, f16, rp, s));
   CU(launch_over_lists(rp, rows, update_ntiles(ctx), (int32_t*)(ctx->ws + y.uprp.tiles), codes, n,
                        s));
   CU(launch_update_pairs(rp, rows, is_gauss(&ctx->cfg) ? ctx->Kb2 : ctx->Kb, f16, y.ld_pix, true,

@@ -140,7 +140,8 @@ cudaError_t launch_normalize_scores_flu(const float* S, int64_t ldS, const float
 // rows, empty: also the zeros of rows without mass (else their den alone).
 cudaError_t launch_pairs_reset(const RowPairs& rp, int64_t rows, cudaStream_t s);
 cudaError_t launch_pairs_from_planes(const uint16_t* P, int64_t plane, int64_t rows,
-                                     int64_t ld_data, int f16, const RowPairs& rp, cudaStream_t s);
+                                     int64_t ld_data, int64_t n_data, int f16, const RowPairs& rp,
+                                     cudaStream_t s);
 cudaError_t launch_mark_over(const int32_t* list, const int32_t* count, int64_t nnt,
                              const RowPairs& rp, cudaStream_t s);
 cudaError_t launch_over_lists(const RowPairs& rp, int64_t rows, int n_ntiles, int32_t* tiles,

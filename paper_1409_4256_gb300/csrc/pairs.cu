@@ -33,16 +33,19 @@ namespace {
 // the one read (217 MB: 38 us, 5.7 TB/s). A warp
 // reads 256 frames of a row (16 bytes per lane and plane), a CTA 128 rows x 256
 // frames; row tiles run fastest, so that the CTAs of a tile already found to be
-// over leave at once, and a block with more than 512 pairs is given up.
+// over leave at once, and a block with more than 512 pairs is given up. Padding frames
+// (from n_data on) carry no counts: what a caller's P holds there adds nothing, to den neither.
 template <bool F16>
 __global__ void __launch_bounds__(256)
     pairs_from_planes_kernel(const uint16_t* __restrict__ P, int64_t plane, int64_t ld_data,
-                             unsigned nmt, RowPairs rp) {
+                             int64_t n_data, unsigned nmt, RowPairs rp) {
   const int64_t mt = blockIdx.x % nmt;
   if (__syncthreads_or(*reinterpret_cast<volatile uint8_t*>(rp.over + mt))) return;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int64_t c0 = (int64_t)(blockIdx.x / nmt) * 256, k0 = c0 + 8 * lane;
   const uint16_t* base = P + (mt * 128 + warp) * ld_data + k0;
+  const int used = (int)max((int64_t)0, min((int64_t)8, n_data - k0));
+  const unsigned take = (1u << used) - 1u;  // the lane's frames that are no padding
   __shared__ BlockPairs<512> bp;
   block_pairs_clear(bp);
 #pragma unroll 1
@@ -62,7 +65,8 @@ __global__ void __launch_bounds__(256)
       // (a negative zero is listed with weight 0)
       int n = 0;
 #pragma unroll
-      for (int i = 0; i < 8; i++) n += ((hv[i >> 1] | lv[i >> 1]) >> (16 * (i & 1)) & 0xffffu) != 0u;
+      for (int i = 0; i < 8; i++)
+        n += (take >> i & 1u) != 0u && ((hv[i >> 1] | lv[i >> 1]) >> (16 * (i & 1)) & 0xffffu) != 0u;
       if (n == 0) continue;
       const int jj = warp + 8 * (b + u);
       int place, at = block_pairs_take(bp, jj, n, &place);
@@ -71,7 +75,7 @@ __global__ void __launch_bounds__(256)
       for (int i = 0; i < 8; i++) {
         const uint16_t hb = (uint16_t)(hv[i >> 1] >> (16 * (i & 1)));
         const uint16_t lb = (uint16_t)(lv[i >> 1] >> (16 * (i & 1)));
-        if ((hb | lb) == 0) continue;
+        if ((hb | lb) == 0 || !(take >> i & 1u)) continue;
         const float w = F16 ? (fp16_val(hb) + fp16_val(lb)) * (1.0f / kP16Scale)
                             : bf16_val(hb) + bf16_val(lb);
         block_pairs_put(bp, at++, jj, place++, 8 * lane + i, w, w);
@@ -192,14 +196,15 @@ cudaError_t launch_pairs_reset(const RowPairs& rp, int64_t rows, cudaStream_t s)
 }
 
 cudaError_t launch_pairs_from_planes(const uint16_t* P, int64_t plane, int64_t rows,
-                                     int64_t ld_data, int f16, const RowPairs& rp, cudaStream_t s) {
+                                     int64_t ld_data, int64_t n_data, int f16, const RowPairs& rp,
+                                     cudaStream_t s) {
   const unsigned nmt = (unsigned)(rows / 128);
   const int64_t grd = (int64_t)nmt * (ld_data / 256);
   if (grd > INT32_MAX) return cudaErrorInvalidValue;
   if (f16)
-    pairs_from_planes_kernel<true><<<(unsigned)grd, 256, 0, s>>>(P, plane, ld_data, nmt, rp);
+    pairs_from_planes_kernel<true><<<(unsigned)grd, 256, 0, s>>>(P, plane, ld_data, n_data, nmt, rp);
   else
-    pairs_from_planes_kernel<false><<<(unsigned)grd, 256, 0, s>>>(P, plane, ld_data, nmt, rp);
+    pairs_from_planes_kernel<false><<<(unsigned)grd, 256, 0, s>>>(P, plane, ld_data, n_data, nmt, rp);
   return cudaGetLastError();
 }
 
