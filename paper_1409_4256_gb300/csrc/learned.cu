@@ -65,6 +65,7 @@ cudaError_t launch_features(const uint16_t* Kb, int kf16, int64_t ld_pix, int64_
 // A 512 x 512 x 512 layer is 32 x 64 tiles on 128 CTAs, one per SM, the next K
 // block's loads in flight while this one is summed: 38 -> 22 us (64 x 64 tiles on
 // 64 CTAs waited out every block's load latency). Every element still sums its products in order of k.
+// (Rows of tiles go on in grid z: y holds 65535, 2.1 million rows of a batch.)
 constexpr int G_BM = 32, G_BN = 64, G_BK = 32, G_THREADS = 256;
 
 __device__ __forceinline__ float bf16_round(float x) { return bf16_val(bf16_bits(x)); }
@@ -96,8 +97,9 @@ __global__ void __launch_bounds__(G_THREADS)
   constexpr int NA = G_BM * G_BK / G_THREADS, NB = G_BN * G_BK / G_THREADS;
   __shared__ float Bw[EPI == 0 ? G_BK : 1][G_BN];
   const int t = threadIdx.x, tx = t & 15, ty = t >> 4;
-  const int m0 = blockIdx.y * G_BM, n0 = blockIdx.x * G_BN;
-  const bool sums = EPI == 0 && ep.bsum && blockIdx.y == 0;
+  const int m0 = (int)(blockIdx.z * gridDim.y + blockIdx.y) * G_BM, n0 = blockIdx.x * G_BN;
+  if (m0 >= M) return;
+  const bool sums = EPI == 0 && ep.bsum && m0 == 0;
   float bs = 0.f;
   float ra[NA], rb[NB];
   auto load = [&](int k0) {
@@ -171,10 +173,16 @@ __global__ void __launch_bounds__(G_THREADS)
   }
 }
 
+// across x down blocks, the rows of blocks beyond 65535 in z
+dim3 rows_grid(int64_t across, int64_t down) {
+  const int64_t y = std::min<int64_t>(down, 65535);
+  return dim3((unsigned)across, (unsigned)y, (unsigned)((down + y - 1) / y));
+}
+
 template <bool TA, bool TB, int EPI>
 cudaError_t gemm(int M, int N, int K, const float* A, int64_t lda, const float* B, int64_t ldb,
                  float* C, int64_t ldc, const GemmEpi& ep, cudaStream_t s) {
-  dim3 grid((unsigned)((N + G_BN - 1) / G_BN), (unsigned)((M + G_BM - 1) / G_BM));
+  const dim3 grid = rows_grid(((int64_t)N + G_BN - 1) / G_BN, ((int64_t)M + G_BM - 1) / G_BM);
   mlp_gemm_kernel<TA, TB, EPI><<<grid, G_THREADS, 0, s>>>(M, N, K, A, lda, B, ldb, C, ldc, ep);
   return cudaGetLastError();
 }
@@ -196,10 +204,10 @@ __global__ void to_bf16_kernel(const float* __restrict__ src, int64_t n, uint16_
 
 __global__ void add_bias_kernel(float* __restrict__ Z, int64_t ld, int64_t rows, int64_t cols,
                                 const float* __restrict__ b) {
-  const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const int64_t c = (int64_t)blockIdx.x * 256 + threadIdx.x;
   if (c >= cols) return;
   const float v = b[c];
-  const int64_t r0 = (int64_t)blockIdx.y * 8;
+  const int64_t r0 = ((int64_t)blockIdx.z * gridDim.y + blockIdx.y) * 8;
 #pragma unroll
   for (int r = 0; r < 8; r++)
     if (r0 + r < rows) Z[(r0 + r) * ld + c] += v;
@@ -487,7 +495,7 @@ cudaError_t mlp_forward(const MlpLayout& y, const float* params, const float* X,
                         float* work, float* logits, cudaStream_t s) {
   cudaError_t e = forward(y, params, X, B, work, logits, s);
   if (e != cudaSuccess || !tc_batch(B)) return e;
-  add_bias_kernel<<<dim3((unsigned)((y.n_out + 255) / 256), (unsigned)((B + 7) / 8)), 256, 0, s>>>(
+  add_bias_kernel<<<rows_grid((y.n_out + 255) / 256, ((int64_t)B + 7) / 8), 256, 0, s>>>(
       logits, y.ld_out, B, y.n_out, params + y.b[3]);
   return cudaGetLastError();
 }
