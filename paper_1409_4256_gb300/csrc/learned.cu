@@ -62,11 +62,13 @@ cudaError_t launch_features(const uint16_t* Kb, int kf16, int64_t ld_pix, int64_
 // 2 bias + GELU (the pre-activation goes to `pre`, GELU of it to C, and where
 // given its BF16 copies to hb [M][ldc] and transposed to ht [N][M]),
 // 3 times GELU'(pre) (the backward pass through the activation).
-// A 512 x 512 x 512 layer is 32 x 64 tiles on 128 CTAs, one per SM, the next K
+// BM rows a tile. A 512 x 512 x 512 layer is 32 x 64 tiles on 128 CTAs, one per SM, the next K
 // block's loads in flight while this one is summed: 38 -> 22 us (64 x 64 tiles on
-// 64 CTAs waited out every block's load latency). Every element still sums its products in order of k.
+// 64 CTAs waited out every block's load latency). Batches that fill the SMs with 64 x 64 tiles
+// twice over read less by those (16384 rows, forward: 1.19 ms by 32-row tiles, 0.87 so). Every
+// element sums its products in order of k either way.
 // (Rows of tiles go on in grid z: y holds 65535, 2.1 million rows of a batch.)
-constexpr int G_BM = 32, G_BN = 64, G_BK = 32, G_THREADS = 256;
+constexpr int G_BN = 64, G_THREADS = 256;
 
 __device__ __forceinline__ float bf16_round(float x) { return bf16_val(bf16_bits(x)); }
 
@@ -87,11 +89,12 @@ struct GemmEpi {
   float* bsum;  // column sums of op(B) in order of k, unrounded (EPI 0; bias gradients)
 };
 
-template <bool TA, bool TB, int EPI>
+template <int G_BM, bool TA, bool TB, int EPI>
 __global__ void __launch_bounds__(G_THREADS)
     mlp_gemm_kernel(int M, int N, int K, const float* __restrict__ A, int64_t lda,
                     const float* __restrict__ B, int64_t ldb, float* __restrict__ C, int64_t ldc,
                     const GemmEpi ep) {
+  constexpr int G_BK = G_BM == 64 ? 16 : 32, TM = G_BM / 16;  // TM rows a thread
   __shared__ __align__(16) float As[G_BK][G_BM + 4];
   __shared__ __align__(16) float Bs[G_BK][G_BN + 4];
   constexpr int NA = G_BM * G_BK / G_THREADS, NB = G_BN * G_BK / G_THREADS;
@@ -116,7 +119,7 @@ __global__ void __launch_bounds__(G_THREADS)
       rb[u] = gn < N && gk < K ? (TB ? B[(int64_t)gn * ldb + gk] : B[(int64_t)gk * ldb + gn]) : 0.f;
     }
   };
-  float acc[2][4] = {};
+  float acc[TM][4] = {};
   load(0);
   for (int k0 = 0; k0 < K; k0 += G_BK) {
 #pragma unroll
@@ -137,11 +140,22 @@ __global__ void __launch_bounds__(G_THREADS)
       for (int kk = 0; kk < G_BK; kk++) bs += Bw[kk][t];
 #pragma unroll
     for (int kk = 0; kk < G_BK; kk++) {
-      const float2 a2 = *reinterpret_cast<const float2*>(&As[kk][ty * 2]);
+      float a[TM];
+      if (TM == 4) {
+        const float4 a4 = *reinterpret_cast<const float4*>(&As[kk][ty * TM]);
+        a[0] = a4.x;
+        a[1] = a4.y;
+        a[TM - 2] = a4.z;
+        a[TM - 1] = a4.w;
+      } else {
+        const float2 a2 = *reinterpret_cast<const float2*>(&As[kk][ty * TM]);
+        a[0] = a2.x;
+        a[1] = a2.y;
+      }
       const float4 b4 = *reinterpret_cast<const float4*>(&Bs[kk][tx * 4]);
-      const float a[2] = {a2.x, a2.y}, b[4] = {b4.x, b4.y, b4.z, b4.w};
+      const float b[4] = {b4.x, b4.y, b4.z, b4.w};
 #pragma unroll
-      for (int i = 0; i < 2; i++)
+      for (int i = 0; i < TM; i++)
 #pragma unroll
         for (int j = 0; j < 4; j++) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
     }
@@ -149,8 +163,8 @@ __global__ void __launch_bounds__(G_THREADS)
   }
   if (sums && t < G_BN && n0 + t < N) ep.bsum[n0 + t] = bs;
 #pragma unroll
-  for (int i = 0; i < 2; i++) {
-    const int gm = m0 + ty * 2 + i;
+  for (int i = 0; i < TM; i++) {
+    const int gm = m0 + ty * TM + i;
     if (gm >= M) continue;
 #pragma unroll
     for (int j = 0; j < 4; j++) {
@@ -164,13 +178,20 @@ __global__ void __launch_bounds__(G_THREADS)
         if (ep.hb) {
           const uint16_t h = bf16_bits(v);
           ep.hb[(int64_t)gm * ldc + gn] = h;
-          ep.ht[(int64_t)gn * M + gm] = h;
+          if (ep.ht) ep.ht[(int64_t)gn * M + gm] = h;
         }
       }
       if (EPI == 3) v *= gelu_grad_f(ep.pre[(int64_t)gm * ep.ldpre + gn]);
       C[(int64_t)gm * ldc + gn] = v;
     }
   }
+}
+
+int num_sms() {
+  int dev = 0, n = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
+  return n;
 }
 
 // across x down blocks, the rows of blocks beyond 65535 in z
@@ -182,8 +203,13 @@ dim3 rows_grid(int64_t across, int64_t down) {
 template <bool TA, bool TB, int EPI>
 cudaError_t gemm(int M, int N, int K, const float* A, int64_t lda, const float* B, int64_t ldb,
                  float* C, int64_t ldc, const GemmEpi& ep, cudaStream_t s) {
-  const dim3 grid = rows_grid(((int64_t)N + G_BN - 1) / G_BN, ((int64_t)M + G_BM - 1) / G_BM);
-  mlp_gemm_kernel<TA, TB, EPI><<<grid, G_THREADS, 0, s>>>(M, N, K, A, lda, B, ldb, C, ldc, ep);
+  const int64_t across = ((int64_t)N + G_BN - 1) / G_BN;
+  if (across * (((int64_t)M + 63) / 64) >= 2 * num_sms())
+    mlp_gemm_kernel<64, TA, TB, EPI><<<rows_grid(across, ((int64_t)M + 63) / 64), G_THREADS, 0, s>>>(
+        M, N, K, A, lda, B, ldb, C, ldc, ep);
+  else
+    mlp_gemm_kernel<32, TA, TB, EPI><<<rows_grid(across, ((int64_t)M + 31) / 32), G_THREADS, 0, s>>>(
+        M, N, K, A, lda, B, ldb, C, ldc, ep);
   return cudaGetLastError();
 }
 
@@ -290,12 +316,17 @@ __global__ void __launch_bounds__(512)
 // (dzb), or in FP32 over z itself (dzb NULL), and its column sums in row order
 // (the bias gradient). A warp walks 32 columns of every row, 16 rows' loads in
 // flight; the CTA first marks the rows that have a target among its 128 columns, and
-// only those look their targets up.
+// only those look their targets up. chunk: rows a CTA (grid y); several chunks leave their
+// sums in db[chunk][ld], in row order each, for sum_chunks_kernel (3240 columns are 26 CTAs:
+// 4096 rows with 64 targets took 2.85 ms in one chunk with the targets a row at a time, 0.30 ms
+// so; 50100 columns 1.37 and 0.69 ms).
+// MANY: rows' targets fall on a CTA's columns often. SPLIT: several chunks.
+template <bool MANY, bool SPLIT>
 __global__ void __launch_bounds__(128)
     softmax_grad_kernel(float* __restrict__ z, int64_t ld, int n_out,
                         const float* __restrict__ zb, const int32_t* __restrict__ tidx,
                         const float* __restrict__ tprob, int R, int B,
-                        const float* __restrict__ lse, const float* __restrict__ mass,
+                        const float* __restrict__ lse, const float* __restrict__ mass, int chunk,
                         uint16_t* __restrict__ dzb, float* __restrict__ db) {
   constexpr int kRows = 16, kBatch = 512;
   __shared__ unsigned hits[kBatch / 32];
@@ -305,8 +336,9 @@ __global__ void __launch_bounds__(128)
   const float bias = zb && in ? zb[c] : 0.f;
   const float invB = 1.f / (float)B;
   float sum = 0.f;
-  for (int b0 = 0; b0 < B; b0 += kBatch) {
-    const int b1 = min(B, b0 + kBatch);
+  const int first = SPLIT ? blockIdx.y * chunk : 0, last = SPLIT ? min(B, first + chunk) : B;
+  for (int b0 = first; b0 < last; b0 += kBatch) {
+    const int b1 = min(last, b0 + kBatch);
     __syncthreads();
     if (threadIdx.x < kBatch / 32) hits[threadIdx.x] = 0u;
     __syncthreads();
@@ -335,7 +367,24 @@ __global__ void __launch_bounds__(128)
       }
       if (r0 + kRows < b1) load(r0 + kRows);
       const unsigned h16 = hits[(r0 - b0) >> 5] >> ((r0 - b0) & 31) & 0xffffu;
-      if (h16) {
+      if (MANY && h16) {
+        for (int t0 = 0; t0 < R; t0 += 32) {
+          int q[kRows];  // the rows' targets together: one wait for 16 rows
+#pragma unroll
+          for (int u = 0; u < kRows; u++)
+            q[u] = (h16 >> u & 1u) && t0 + lane < R ? tidx[(int64_t)(r0 + u) * R + t0 + lane] : -1;
+#pragma unroll
+          for (int u = 0; u < kRows; u++) {
+            unsigned hit = __ballot_sync(0xffffffffu, q[u] >= c0 && q[u] < c0 + 32);
+            while (hit) {
+              const int w = __ffs(hit) - 1;
+              hit &= hit - 1;
+              if (__shfl_sync(0xffffffffu, q[u], w) == c)
+                v[u] -= tprob[(int64_t)(r0 + u) * R + t0 + w] * invB;
+            }
+          }
+        }
+      } else if (h16) {
 #pragma unroll
         for (int u = 0; u < kRows; u++) {
           if (!(h16 >> u & 1u)) continue;
@@ -360,7 +409,17 @@ __global__ void __launch_bounds__(128)
       }
     }
   }
-  if (in) db[c] = sum;
+  if (in) db[(SPLIT ? (int64_t)blockIdx.y * ld : 0) + c] = sum;
+}
+
+// out[c] = the chunks' sums, in their order
+__global__ void sum_chunks_kernel(const float* __restrict__ part, int64_t ld, int n, int chunks,
+                                  float* __restrict__ out) {
+  const int c = blockIdx.x * blockDim.x + threadIdx.x;
+  if (c >= n) return;
+  float s = 0.f;
+  for (int k = 0; k < chunks; k++) s += part[k * ld + c];
+  out[c] = s;
 }
 
 // d = g * GELU'(a), elementwise
@@ -465,10 +524,10 @@ Work carve(const MlpLayout& y, float* w) {
 bool tc_batch(int B) { return B >= 128 && B % 128 == 0; }
 }  // namespace
 
-// Forward into logits. train: with a tensor-core batch the output layer's bias is
-// left to the loss kernels, and H3^T is kept for the weight gradient.
+// Forward into logits, without the output layer's bias where a batch goes by tensor cores.
+// train: H3^T is then kept for the weight gradient.
 static cudaError_t forward(const MlpLayout& y, const float* params, const float* X, int B,
-                           float* work, float* logits, cudaStream_t s) {
+                           float* work, float* logits, bool train, cudaStream_t s) {
   Work w = carve(y, work);
   const int H = kFeat;
   const bool tc = tc_batch(B);
@@ -478,7 +537,7 @@ static cudaError_t forward(const MlpLayout& y, const float* params, const float*
     const bool last = tc && l == 2;
     e = gemm<false, false, 2>(B, H, H, in, H, params + y.W[l], H, w.h[l], H,
                               GemmEpi{params + y.b[l], w.a[l], H, last ? w.h3b : nullptr,
-                                      last ? w.h3t : nullptr},
+                                      last && train ? w.h3t : nullptr},
                               s);
     if (e != cudaSuccess) return e;
     in = w.h[l];
@@ -493,7 +552,7 @@ static cudaError_t forward(const MlpLayout& y, const float* params, const float*
 
 cudaError_t mlp_forward(const MlpLayout& y, const float* params, const float* X, int B,
                         float* work, float* logits, cudaStream_t s) {
-  cudaError_t e = forward(y, params, X, B, work, logits, s);
+  cudaError_t e = forward(y, params, X, B, work, logits, false, s);
   if (e != cudaSuccess || !tc_batch(B)) return e;
   add_bias_kernel<<<rows_grid((y.n_out + 255) / 256, ((int64_t)B + 7) / 8), 256, 0, s>>>(
       logits, y.ld_out, B, y.n_out, params + y.b[3]);
@@ -508,24 +567,39 @@ cudaError_t mlp_train_step(const MlpLayout& y, float* params, float* grads, floa
   const int H = kFeat;
   const bool tc = tc_batch(B);
   const int64_t BH = (int64_t)B * H;
-  cudaError_t e = forward(y, params, X, B, work, w.z, s);
+  cudaError_t e = forward(y, params, X, B, work, w.z, true, s);
   if (e != cudaSuccess) return e;
   float *lse = w.dh, *mass = w.dh + B;  // dh is written after the loss
   const float* zb = tc ? params + y.b[3] : nullptr;
   softmax_lse_kernel<<<B, 512, 0, s>>>(w.z, y.ld_out, (int)y.n_out, zb, tidx, tprob, R, B, lse,
                                        mass, loss);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  softmax_grad_kernel<<<(unsigned)((y.ld_out + 127) / 128), 128, 0, s>>>(
-      w.z, y.ld_out, (int)y.n_out, zb, tidx, tprob, R, B, lse, mass, tc ? w.dzb : nullptr,
-      grads + y.b[3]);
+  // chunks of 512 rows where the columns leave SMs idle (their sums fit da, which is written later)
+  const int64_t cols = (y.ld_out + 127) / 128;
+  const int chunk = cols >= 4 * num_sms() || y.ld_out > 512 * H ? B : std::min(B, 512);
+  const int chunks = (B + chunk - 1) / chunk;
+  auto grad = (int64_t)R * 256 >= y.n_out ? softmax_grad_kernel<true, true>
+              : chunks > 1                ? softmax_grad_kernel<false, true>
+                                          : softmax_grad_kernel<false, false>;
+  grad<<<dim3((unsigned)cols, (unsigned)chunks), 128, 0, s>>>(
+      w.z, y.ld_out, (int)y.n_out, zb, tidx, tprob, R, B, lse, mass, chunk, tc ? w.dzb : nullptr,
+      chunks > 1 ? w.da : grads + y.b[3]);
+  if (chunks > 1)
+    sum_chunks_kernel<<<(unsigned)((y.n_out + 255) / 256), 256, 0, s>>>(
+        w.da, y.ld_out, (int)y.n_out, chunks, grads + y.b[3]);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   // output layer: dW4 = h3^T dz, da3 = (dz W4^T) GELU'(a3)
   if (tc) {
     // on the tensor cores (the whole padded width: dZ is 0 beyond n_out)
     if ((e = tc_gemm(w.h3t, H, B, w.dzb, y.ld_out, grads + y.W[3], nullptr, s)) != cudaSuccess)
       return e;
-    if ((e = launch_tc_nt(w.dzb, w.w4b, B, H, y.ld_out, w.dh, nullptr, s)) != cudaSuccess)
-      return e;
+    // narrow tiles while they fit the SMs at once, else 256 columns a tile (a tile's sum runs on one
+    // SM, 225 and 270 us over 50112; B = 4096: 889 us narrow, 334 us so)
+    const Planes dz{w.dzb, (int64_t)B * y.ld_out, y.ld_out};
+    e = (B / 128) * (H / 32) <= num_sms()
+            ? launch_tc_nt(w.dzb, w.w4b, B, H, y.ld_out, w.dh, nullptr, s)
+            : launch_tc_store(dz, B, w.w4b, H, y.ld_out, w.dh, 0, nullptr, s);
+    if (e != cudaSuccess) return e;
     gelu_backward_kernel<<<(unsigned)((BH + 255) / 256), 256, 0, s>>>(w.dh, w.a[2], w.da, BH);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   } else {
