@@ -261,8 +261,9 @@ cudaError_t tc_gemm(const uint16_t* A, int64_t M, int64_t K, const uint16_t* B, 
 // ------------------------------------------------- loss and its gradient --
 // Row b of z (n_out logits, stride ld; zb (may be NULL): a bias still to be added):
 // lse[b] = log sum_j exp(z_j), mass[b] = sum_r p_r and loss
-// += -sum_r p_r (z_{idx_r} - lse) / B. The sum is kept per thread as a
-// double-float pair (FP64 additions and conversions are rare on this part), merged in FP64.
+// += -sum_r p_r (z_{idx_r} - lse) / B. The sum is kept per thread as three FP32 words, each
+// taking the exact rounding errors of the one before (what the third rounds is below 2^-64 of
+// the sum; FP64 additions and conversions are rare on this part), merged in FP64.
 __global__ void __launch_bounds__(512)
     softmax_lse_kernel(const float* __restrict__ z, int64_t ld, int n_out,
                        const float* __restrict__ zb, const int32_t* __restrict__ tidx,
@@ -281,14 +282,16 @@ __global__ void __launch_bounds__(512)
   __syncthreads();
   M = red[0];
   for (int w = 1; w < 16; w++) M = fmaxf(M, red[w]);
-  float s = 0.f, se = 0.f;
+  float s = 0.f, se = 0.f, st = 0.f;
 #pragma unroll 8
   for (int j = threadIdx.x; j < n_out; j += 512) {
     const f2 a = two_sum(s, __expf((row[j] + (zb ? zb[j] : 0.f)) - M));
+    const f2 b = two_sum(se, a.l);
     s = a.h;
-    se += a.l;
+    se = b.h;
+    st += b.l;
   }
-  double d = (double)s + (double)se;
+  double d = (double)s + ((double)se + (double)st);
   for (int o = 16; o; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
   if (lane == 0) dred[wid] = d;
   __syncthreads();
