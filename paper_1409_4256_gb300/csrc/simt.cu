@@ -248,8 +248,9 @@ __global__ void __launch_bounds__(256)
 // Only the frames with a non-zero P in the tile's 64 rows are contracted, in
 // order (most P underflow to exact zeros, which add nothing: 64^3, 3240 rotations x 2000
 // frames, 1315 us over every frame, 107 us over these with their bits). nz: simt_nonzero_kernel's
-// bits, or NULL: every frame.
+// bits; ALL: every frame.
 constexpr int kNzWords = 128;  // words of nz taken at a time: 4096 frames
+template <bool ALL>
 __global__ void __launch_bounds__(S_THREADS)
     simt_update_kernel(const float* __restrict__ P, int64_t ld_data,
                        const uint16_t* __restrict__ Kb, int64_t ld_pix, int64_t n_pix,
@@ -270,10 +271,10 @@ __global__ void __launch_bounds__(S_THREADS)
   const int br = t >> 4, bc = (t & 15) * 8;   // B = K: frame, pixel offset
   const bool bval = c0 + bc < ld_pix;
   const int64_t words = ld_data / 32;
-  if (nz) nz += blockIdx.y * words;
+  if (!ALL) nz += blockIdx.y * words;
   for (int64_t w0 = 0; w0 < words; w0 += kNzWords) {
     // the frames of these words (offsets from 32 w0)
-    uint32_t bits = t < kNzWords && w0 + t < words ? (nz ? nz[w0 + t] : ~0u) : 0u;
+    uint32_t bits = t < kNzWords && w0 + t < words ? (ALL ? ~0u : nz[w0 + t]) : 0u;
     int inc = __popc(bits);
     const int own = inc;
 #pragma unroll
@@ -383,7 +384,8 @@ cudaError_t launch_simt_update(const float* P, int64_t ld_data, int64_t rows, co
     if (e != cudaSuccess) return e;
   }
   dim3 grd((unsigned)((ld_pix + SB_N - 1) / SB_N), (unsigned)(rows / SB_M));
-  simt_update_kernel<<<grd, S_THREADS, 0, s>>>(P, ld_data, Kb, ld_pix, n_pix, nz, Num, den);
+  auto kern = nz ? simt_update_kernel<false> : simt_update_kernel<true>;
+  kern<<<grd, S_THREADS, 0, s>>>(P, ld_data, Kb, ld_pix, n_pix, nz, Num, den);
   return cudaGetLastError();
 }
 
