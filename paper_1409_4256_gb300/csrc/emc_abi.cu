@@ -1073,7 +1073,7 @@ int update_pairs(emc_ctx* ctx, const void* P, int64_t nrot, float* Num, float* d
   const RowPairs rp = row_pairs(ctx, y.uprp, rows);
   int32_t* codes = (int32_t*)(ctx->ws + y.uprp.codes);
   int32_t* n = (int32_t*)(ctx->ws + y.uprp.n);
-  CU(launch_pairs_reset(rp, rows, s));
+  CU(launch_pairs_begin((const uint16_t*)P, rows * y.ld_data, rows, y.ld_data, rp, s));
   CU(launch_pairs_from_planes((const uint16_t*)P, rows * y.ld_data, rows, y.ld_data,
                               ctx->cfg.n_data, f16, rp, s));
   CU(launch_over_lists(rp, rows, update_ntiles(ctx), (int32_t*)(ctx->ws + y.uprp.tiles), codes, n,

@@ -133,12 +133,14 @@ cudaError_t launch_normalize_scores_flu(const float* S, int64_t ldS, const float
                                         int64_t n_data, uint16_t* P, int64_t P_plane, float* den,
                                         cudaStream_t s, uint8_t* kb_flag = nullptr,
                                         const uint8_t* tile_live = nullptr);
-// The M-step operand as pairs (pairs.cu): zero cnt and over; find the pairs in
-// planes of P; mark the row tiles of listed (row tile, frame tile) codes; decide on
+// The M-step operand as pairs (pairs.cu): zero cnt and over (begin: and mark the tiles whose
+// planes of P look flat); find the pairs in planes of P; mark the row tiles of listed (row tile, frame tile) codes; decide on
 // and list the tiles that are over (counts[0]) and their output tiles of the update
 // (counts[1], codes mt * n_ntiles + nt); write Num and den (NULL: not) of the other tiles'
 // rows, empty: also the zeros of rows without mass (else their den alone).
 cudaError_t launch_pairs_reset(const RowPairs& rp, int64_t rows, cudaStream_t s);
+cudaError_t launch_pairs_begin(const uint16_t* P, int64_t plane, int64_t rows, int64_t ld_data,
+                               const RowPairs& rp, cudaStream_t s);
 cudaError_t launch_pairs_from_planes(const uint16_t* P, int64_t plane, int64_t rows,
                                      int64_t ld_data, int64_t n_data, int f16, const RowPairs& rp,
                                      cudaStream_t s);

@@ -85,6 +85,35 @@ __global__ void __launch_bounds__(256)
   block_pairs_flush(bp, rp, mt * 128, c0);
 }
 
+// A CTA per row tile: its counters cleared, and a look at eight of its rows in 256 frames. Where
+// an eighth of those is not zero, the posterior is flat and the tile over, so that the search
+// need not find it out block by block (64^3, 10860 x 4999 at 0.1 photons a pixel: 490 us with the search,
+// 446 so, 423 contracted straight away; the clearing takes a launch in any case).
+__global__ void __launch_bounds__(256)
+    pairs_begin_kernel(const uint16_t* __restrict__ P, int64_t plane, int64_t ld_data,
+                       RowPairs rp) {
+  const int64_t mt = blockIdx.x;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int64_t k0 = ld_data / 512 * 256 + 8 * lane;
+  const uint16_t* p = P + (mt * 128 + 16 * warp) * ld_data + k0;
+  const uint4 h = *reinterpret_cast<const uint4*>(p);
+  const uint4 l = *reinterpret_cast<const uint4*>(p + plane);
+  if (threadIdx.x < 128) rp.cnt[mt * 128 + threadIdx.x] = 0;
+  const uint32_t v[4] = {h.x | l.x, h.y | l.y, h.z | l.z, h.w | l.w};
+  int n = 0;
+#pragma unroll
+  for (int i = 0; i < 8; i++) n += (v[i >> 1] >> (16 * (i & 1)) & 0xffffu) != 0u;
+  __shared__ int sum[8];
+  n = __reduce_add_sync(0xffffffffu, n);
+  if (lane == 0) sum[warp] = n;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < 8; w++) n += sum[w];
+    rp.tile_n[mt] = 0;
+    rp.over[mt] = n > 256 ? 1 : 0;
+  }
+}
+
 // Row tiles that are over: their list, and their tiles of the update's output (codes
 // mt * n_ntiles + nt).
 __global__ void __launch_bounds__(1024)
@@ -193,6 +222,12 @@ __global__ void __launch_bounds__(128)
 cudaError_t launch_pairs_reset(const RowPairs& rp, int64_t rows, cudaStream_t s) {
   // cnt, tile_n and over lie one behind the other
   return cudaMemsetAsync(rp.cnt, 0, sizeof(int32_t) * rows + 5 * (rows / 128), s);
+}
+
+cudaError_t launch_pairs_begin(const uint16_t* P, int64_t plane, int64_t rows, int64_t ld_data,
+                               const RowPairs& rp, cudaStream_t s) {
+  pairs_begin_kernel<<<(unsigned)(rows / 128), 256, 0, s>>>(P, plane, ld_data, rp);
+  return cudaGetLastError();
 }
 
 cudaError_t launch_pairs_from_planes(const uint16_t* P, int64_t plane, int64_t rows,

@@ -153,8 +153,10 @@ __device__ __forceinline__ int tile_kblock(const TcArgs& a, int mt, int x) {
   return a.kb_cnt ? a.kb_list[(int64_t)mt * a.kb_ld + x] : x;
 }
 
-__device__ __forceinline__ void tile_coords(int t, const TcArgs& a, int* mt, int* nt) {
-  if (a.tile_list) {
+// all: the list holds every tile, in the order of no list
+__device__ __forceinline__ void tile_coords(int t, const TcArgs& a, int* mt, int* nt,
+                                            bool all = false) {
+  if (a.tile_list && !all) {
     const int code = a.tile_list[t];
     *mt = code / a.n_ntiles;
     *nt = code % a.n_ntiles;
@@ -238,6 +240,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
   const int T = a.tile_count ? *a.tile_count : a.n_mtiles * a.n_ntiles;
+  const bool all = MODE == MODE_UPDATE && T == a.n_mtiles * a.n_ntiles;
 
   if (warp == 0) {
     // ------------------------------------------------------------ producer --
@@ -246,7 +249,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       bool ok = true;
       for (int t = blockIdx.x; t < T && ok; t += gridDim.x) {
         int mt, nt;
-        tile_coords(t, a, &mt, &nt);
+        tile_coords(t, a, &mt, &nt, all);
         const int nkb = tile_kblocks(a, mt);
         for (int x = 0; x < nkb; x++, it++) {
           const int kb = tile_kblock(a, mt, x);
@@ -292,7 +295,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
         tc_fence_after();
         int mt_, nt_;
-        tile_coords(t, a, &mt_, &nt_);
+        tile_coords(t, a, &mt_, &nt_, all);
         const int nkb = tile_kblocks(a, mt_);
         for (int kb = 0; kb < nkb; kb++, it++) {
           const int s = it % C::STAGES;
@@ -348,7 +351,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     int tcount = 0;
     for (int t = blockIdx.x; t < T; t += gridDim.x, tcount++) {
       int mt, nt;
-      tile_coords(t, a, &mt, &nt);
+      tile_coords(t, a, &mt, &nt, all);
       const int64_t row = (int64_t)mt * BM + r_in;
       float bh = 0.f, bl = 0.f;
       bool valid = row < a.nrot;
