@@ -349,19 +349,22 @@ __global__ void __launch_bounds__(kTThreads, 6)
       W2[u] = INTERIOR && g4 ? cell_value(cell[u], tt[u]) : cell[u].a.x;
     if (r + 1 < RPC) fetch(r + 1);
     float L[2] = {0.f, 0.f};
-    float ws[2] = {0.f, 0.f};
+    float ws[2] = {0.f, 0.f}, we[2] = {0.f, 0.f};  // (kOutGauss: W^2 as ws + we)
 #pragma unroll
     for (int u = 0; u < 2; u++) {
       if (vrow && qi[u].w != 0) {  // w: 1 pixel, 2 duplicate column, 0 padding / ones
         nonfinite |= !(fabsf(W2[u]) <= 3.4e38f);  // a NaN or infinite voxel of the model
         const float W = fmaxf(W2[u], w_floor);
         // duplicate columns repeat a pixel: not summed
-        if (qi[u].w == 1) ws[u] = PREC == kOutGauss ? W * W : W;
+        if (qi[u].w == 1) {
+          ws[u] = PREC == kOutGauss ? W * W : W;
+          if (PREC == kOutGauss) we[u] = fmaf(W, W, -ws[u]);
+        }
         L[u] = PREC == kOutGauss ? W * gs : (PREC == kOutW ? W : logf(W));
       }
     }
     const f2 pair = two_sum(ws[0], ws[1]);  // row sum of the pair as s + se
-    const float s = pair.h, se = pair.l;
+    const float s = pair.h, se = PREC == kOutGauss ? pair.l + (we[0] + we[1]) : pair.l;
     if (inside && row < rows) {
       const int64_t o = row * ld_pix + i0;
       // DELTA: the change of the represented value (the planes' sum) of each element
