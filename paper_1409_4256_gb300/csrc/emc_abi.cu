@@ -1233,7 +1233,7 @@ int emc_iteration(emc_ctx* c, const float* grid_in, float* grid_out, emc_iter_st
   }
   // the row tiles and the bias sums (Gaussian: grid maximum and scales first;
   // Poisson fluence: the split, or all in one); the cell layout of the model first where it is used
-  kernels += (is_gauss(&c->cfg) ? 4
+  kernels += (is_gauss(&c->cfg) ? 2 + expand_gauss_launches(y.rows, y.ld_pix)
               : is_flu(&c->cfg) ? expand_flu_launches(y.rows, y.ld_pix, Lold != nullptr)
                                 : 2) +
              ((y.g4 && c->geom.interior) ? 1 : 0);

@@ -107,7 +107,9 @@ cudaError_t launch_expand_tile(const Geom& g, const float* grid, const float4* g
 cudaError_t launch_fixed_geometry(const float4* qh, const float4* ql, int64_t ld_pix, int4* qi,
                                   float4* qlo, float4* qf, cudaStream_t s);
 
-// Gaussian model: s W as three FP16 planes, bias log w - sum W^2 / 2 sigma^2.
+// Gaussian model: s W as three FP16 planes, bias log w - sum W^2 / 2 sigma^2;
+// expand_gauss_launches: its kernels.
+int expand_gauss_launches(int64_t rows, int64_t ld_pix);
 cudaError_t launch_expand_gauss(const Geom& g, const float* grid, const float4* g4,
                                 const RotFX* rot, const double* logw, int64_t nrot, int64_t rows,
                                 Planes L, double* bias, double* partial, const float4* gsc,

@@ -264,6 +264,20 @@ __device__ __forceinline__ unsigned long long get_bytes8(const uint16_t* p) {
   return v;
 }
 
+// s W as three FP16 planes (kOutGauss)
+struct GaussSplit {
+  uint16_t h, m, l;
+};
+__device__ __forceinline__ GaussSplit gauss_split(float x) {
+  GaussSplit o;
+  const float hi = x < 2048.f ? round_to(x, 1.f) : fp16_val(fp16_bits(x));
+  const float r = x - hi;  // exact
+  o.h = fp16_bits(hi);
+  o.m = fp16_bits(r);
+  o.l = fp16_bits(r - fp16_val(o.m));
+  return o;
+}
+
 // RPC rotations of a tile per CTA; with DELTA the tile's 128 / RPC CTAs are a
 // cluster, whose first one gathers the others' rises and falls.
 template <int PREC, bool INTERIOR, bool DELTA, int RPC, bool WHOLE = true>
@@ -372,11 +386,10 @@ __global__ void __launch_bounds__(kTThreads, 6)
         uint16_t h[2], m[2], l[2];
 #pragma unroll
         for (int u = 0; u < 2; u++) {
-          const float hi = L[u] < 2048.f ? round_to(L[u], 1.f) : fp16_val(fp16_bits(L[u]));
-          const float r = L[u] - hi;  // exact
-          h[u] = fp16_bits(hi);
-          m[u] = fp16_bits(r);
-          l[u] = fp16_bits(r - fp16_val(m[u]));
+          const GaussSplit g = gauss_split(L[u]);
+          h[u] = g.h;
+          m[u] = g.m;
+          l[u] = g.l;
         }
         uint16_t* Lb = (uint16_t*)Lbase + o;
         put_pair<WHOLE>(Lb, (uint32_t)h[0] | ((uint32_t)h[1] << 16));
@@ -701,30 +714,30 @@ __global__ void __launch_bounds__(kTThreads)
     write_increments<EMC_PREC_BF16_SPLIT>(dp, dm, rises, inside, t, i0, ld_pix, ntp, D);
 }
 
-// The whole Poisson-fluence expansion of small problems in one launch, a CTA of TH threads per
-// rotation with W in shared memory: the three launches above leave most SMs idle there and
-// each waits for the one before. TH / 128 slices of 256 pixels at a time; the sums in
+// The whole Poisson-fluence expansion of small problems in one launch, and the Gaussian one
+// (OUT: kOutW, kOutGauss), a CTA of TH threads per rotation, with W in shared memory: the
+// tile kernels' launches leave most SMs idle there and each waits for the one before. TH / 128 slices of 256 pixels at a time; the sums in
 // the order of the other form, so the bits are the same whichever runs. Bound by the
 // latency of a slice's chain of loads: 384 threads where the SMs hold all rows' CTAs at
-// once, 128 (ten CTAs an SM) where they do not (flu_row_threads).
-constexpr int kFluSlices = 40;  // 40 KB of W
+// once, 128 (ten CTAs an SM) where they do not (row_threads).
+constexpr int kRowSlices = 40;  // 40 KB of W
 template <int TH>
-constexpr int flu_ctas() {  // an SM
+constexpr int row_ctas() {  // an SM
   return TH == 128 ? 10 : 3;
 }
-template <int TH, bool INTERIOR, bool WHOLE>
-__global__ void __launch_bounds__(TH, flu_ctas<TH>())
-    expand_flu_row_kernel(const int4* __restrict__ qi_g, const float4* __restrict__ qlo_g,
-                          int64_t ld_pix, int N, const float* __restrict__ grid,
-                          const float4* __restrict__ g4, const RotFX* __restrict__ rot,
-                          const double* __restrict__ logw, int64_t nrot, float w_floor, double c,
-                          int slices, uint16_t* __restrict__ Lbase, int64_t ps,
-                          double* __restrict__ bias, double* __restrict__ Bsum,
-                          double* __restrict__ Bctx, int32_t* status) {
+template <int OUT, int TH, bool INTERIOR, bool WHOLE>
+__global__ void __launch_bounds__(TH, row_ctas<TH>())
+    expand_row_kernel(const int4* __restrict__ qi_g, const float4* __restrict__ qlo_g,
+                      int64_t ld_pix, int N, const float* __restrict__ grid,
+                      const float4* __restrict__ g4, const RotFX* __restrict__ rot,
+                      const double* __restrict__ logw, int64_t nrot, float w_floor, double c,
+                      const float4* __restrict__ gsc, int slices, uint16_t* __restrict__ Lbase,
+                      int64_t ps, double* __restrict__ bias, double* __restrict__ Bsum,
+                      double* __restrict__ Bctx, int32_t* status) {
   extern __shared__ float2 wrow[];  // W of the row, a pixel pair an entry
   __shared__ RowFX R;
-  __shared__ float2 rs[kFluSlices][kTThreads / 32];
-  __shared__ double part[kFluSlices];
+  __shared__ float2 rs[kRowSlices][kTThreads / 32];
+  __shared__ double part[kRowSlices];
   __shared__ float2 as;
   const int64_t row = blockIdx.x;
   const bool valid = row < nrot;
@@ -740,6 +753,8 @@ __global__ void __launch_bounds__(TH, flu_ctas<TH>())
   }
   const long long centre = ((long long)(N >> 1) << 32) + ((N & 1) ? (1LL << 31) : 0LL);
   __syncthreads();
+  const float gs = OUT == kOutGauss ? gsc->x : 1.f;
+  uint16_t* Lrow = Lbase + row * ld_pix;
   int nonfinite = 0;
   for (int sl = threadIdx.x / kTThreads; valid && sl < slices; sl += TH / kTThreads) {
     const int64_t i0 = (int64_t)sl * kTPix + 2 * tt;
@@ -757,7 +772,7 @@ __global__ void __launch_bounds__(TH, flu_ctas<TH>())
     const float2 ql[3] = {make_float2(q[0].x, q[1].x), make_float2(q[0].y, q[1].y),
                           make_float2(q[0].z, q[1].z)};
     int f[2][3];
-    float t[2][3], L[2], ws[2];
+    float t[2][3], L[2], ws[2], we[2] = {0.f, 0.f};
     rotate_pair(R, qi, qh, ql, centre, f, t);
 #pragma unroll
     for (int u = 0; u < 2; u++) {
@@ -769,11 +784,19 @@ __global__ void __launch_bounds__(TH, flu_ctas<TH>())
         W = trilinear_fx<INTERIOR>(grid, N, f[u], t[u]);
       nonfinite |= used && !(fabsf(W) <= 3.4e38f);
       W = fmaxf(W, w_floor);
-      ws[u] = used && qi[u].w == 1 ? W : 0.f;
-      L[u] = used ? W : 0.f;
+      ws[u] = used && qi[u].w == 1 ? (OUT == kOutGauss ? W * W : W) : 0.f;
+      if (OUT == kOutGauss && used && qi[u].w == 1) we[u] = fmaf(W, W, -ws[u]);
+      L[u] = used ? W * gs : 0.f;
     }
-    if (inside) wrow[i0 / 2] = make_float2(L[0], L[1]);
-    const f2 pair = two_sum(ws[0], ws[1]);
+    if (OUT == kOutW && inside) wrow[i0 / 2] = make_float2(L[0], L[1]);
+    if (OUT == kOutGauss && inside) {
+      const GaussSplit x = gauss_split(L[0]), y = gauss_split(L[1]);
+      put_pair<WHOLE>(Lrow + i0, (uint32_t)x.h | ((uint32_t)y.h << 16));
+      put_pair<WHOLE>(Lrow + i0 + ps, (uint32_t)x.m | ((uint32_t)y.m << 16));
+      put_pair<WHOLE>(Lrow + i0 + 2 * ps, (uint32_t)x.l | ((uint32_t)y.l << 16));
+    }
+    f2 pair = two_sum(ws[0], ws[1]);
+    if (OUT == kOutGauss) pair.l += we[0] + we[1];
     float a = 0.f, ae = 0.f;
 #pragma unroll
     for (int m = 0; m < 8; m++) {  // eight lanes' pairs, then the four sums of them
@@ -808,10 +831,21 @@ __global__ void __launch_bounds__(TH, flu_ctas<TH>())
   if (threadIdx.x == 0) {
     double B = 0.0;
     for (int q = 0; q < slices; q++) B += part[q];
-    as = flu_shift_split(c, B, valid);
-    bias[row] = valid ? logw[row] : -INFINITY;
-    Bsum[row] = valid ? B : 0.0;
-    Bctx[row] = valid ? B : 0.0;
+    if (OUT == kOutGauss) {  // c: 1 / 2 sigma^2
+      bias[row] = valid ? logw[row] - B * c : -INFINITY;
+    } else {
+      as = flu_shift_split(c, B, valid);
+      bias[row] = valid ? logw[row] : -INFINITY;
+      Bsum[row] = valid ? B : 0.0;
+      Bctx[row] = valid ? B : 0.0;
+    }
+  }
+  if (OUT == kOutGauss) {
+    if (!valid)  // (a padding row: the loop above left it)
+      for (int64_t i0 = 2 * threadIdx.x; i0 < ld_pix; i0 += 2 * TH)
+        for (int q = 0; q < 3; q++) put_pair<WHOLE>(Lrow + i0 + q * ps, 0u);
+    if (nonfinite) set_status(status, EMC_ERR_NUMERIC);
+    return;
   }
   __syncthreads();
   const float ah = as.x, al = as.y;
@@ -821,7 +855,7 @@ __global__ void __launch_bounds__(TH, flu_ctas<TH>())
     const FluSplit x = flu_split(W.x, valid && qi_g[i0].w != 0, ah, al);
     const FluSplit y = flu_split(W.y, valid && qi_g[i0 + 1].w != 0, ah, al);
     bad |= x.bad || y.bad;
-    uint16_t* Lb = Lbase + row * ld_pix + i0;
+    uint16_t* Lb = Lrow + i0;
     put_pair<WHOLE>(Lb, (uint32_t)x.h | ((uint32_t)y.h << 16));
     put_pair<WHOLE>(Lb + ps, (uint32_t)x.m | ((uint32_t)y.m << 16));
     put_pair<WHOLE>(Lb + 2 * ps, (uint32_t)x.l | ((uint32_t)y.l << 16));
@@ -977,20 +1011,6 @@ cudaError_t launch_expand_tile(const Geom& g, const float* grid, const float4* g
   return cudaGetLastError();
 }
 
-cudaError_t launch_expand_gauss(const Geom& g, const float* grid, const float4* g4,
-                                const RotFX* rot, const double* logw, int64_t nrot, int64_t rows,
-                                Planes L, double* bias, double* partial, const float4* gsc,
-                                double sigma, int32_t* status, cudaStream_t s) {
-  if (rows <= 0) return cudaSuccess;
-  cudaError_t e = launch_tiles(g, grid, g4, rot, nrot, rows, kOutGauss, 0.f, L, partial, nullptr,
-                               nullptr, 0, gsc, status, s);
-  if (e != cudaSuccess) return e;
-  expand_bias_kernel<<<(unsigned)(rows / kTRows), kTRows, 0, s>>>(
-      partial, (int)expand_tile_slices(g.ld_pix), rows, logw, nrot, 1.0 / (2.0 * sigma * sigma),
-      bias, nullptr, nullptr, 0);
-  return cudaGetLastError();
-}
-
 namespace {
 
 // Threads a rotation of the one-launch form, or 0 for the tile kernels. us of a call by the
@@ -1000,16 +1020,69 @@ namespace {
 //   3328 x 832 56, 66, 48   3328 x 1856 81, 93, 82    10880 x 128 48, -, about 57
 // (one CTA of 256 threads a rotation and a double-float grid point, before the tile kernels:
 // 19, 36 and 66; 31, 66 and 132; 54 and 81)
-int flu_row_threads(int64_t rows, int64_t ns) {
-  if (ns > kFluSlices) return 0;
+int row_threads(int64_t rows, int64_t ns) {
+  if (ns > kRowSlices) return 0;
   if (rows <= 512) return 384;
   return rows <= 4096 && rows * ns <= 16384 ? 128 : 0;
 }
 
+// The Gaussian model has one launch less to save (the scales come first in any form):
+//   512 x 128 31, 21, 21   512 x 3264 44, 44, 49   128 x 9536 55, 60, 96
+//   1408 x 832 36, 38, 33  3328 x 128 33, 40, 28   3328 x 832 46, 58, 48
+// (before the tile kernels 21, 46 and 82; 34, 36 and 48)
+int gauss_row_threads(int64_t rows, int64_t ns) {
+  if (rows <= 512) return ns <= 16 ? 384 : 0;
+  return rows <= 4096 && rows * ns <= 6144 ? 128 : 0;
+}
+
+template <int OUT>
+cudaError_t launch_rows(int threads, const Geom& g, const float* grid, const float4* g4,
+                        const RotFX* rot, const double* logw, int64_t nrot, int64_t rows,
+                        float w_floor, double c, const float4* gsc, Planes L, double* bias,
+                        double* Bsum, double* Bctx, int32_t* status, cudaStream_t s) {
+  const bool whole = ((uintptr_t)L.base & 3) == 0;
+  if (!whole) threads = 128;
+  auto kern = threads == 384 ? (g.interior ? expand_row_kernel<OUT, 384, true, true>
+                                           : expand_row_kernel<OUT, 384, false, true>)
+              : whole        ? (g.interior ? expand_row_kernel<OUT, 128, true, true>
+                                           : expand_row_kernel<OUT, 128, false, true>)
+                             : (g.interior ? expand_row_kernel<OUT, 128, true, false>
+                                           : expand_row_kernel<OUT, 128, false, false>);
+  const size_t smem = OUT == kOutW ? sizeof(float) * (size_t)g.ld_pix : 0;
+  kern<<<(unsigned)rows, threads, smem, s>>>(
+      g.qi, g.qlo, g.ld_pix, g.N, grid, g4, rot, logw, nrot, w_floor, c, gsc,
+      (int)expand_tile_slices(g.ld_pix), (uint16_t*)L.base, L.plane_stride, bias, Bsum, Bctx,
+      status);
+  return cudaGetLastError();
+}
+
 }  // namespace
 
+cudaError_t launch_expand_gauss(const Geom& g, const float* grid, const float4* g4,
+                                const RotFX* rot, const double* logw, int64_t nrot, int64_t rows,
+                                Planes L, double* bias, double* partial, const float4* gsc,
+                                double sigma, int32_t* status, cudaStream_t s) {
+  if (rows <= 0) return cudaSuccess;
+  const double inv = 1.0 / (2.0 * sigma * sigma);
+  const int th = gauss_row_threads(rows, expand_tile_slices(g.ld_pix));
+  if (th)
+    return launch_rows<kOutGauss>(th, g, grid, g4, rot, logw, nrot, rows, 0.f, inv, gsc, L, bias,
+                                  nullptr, nullptr, status, s);
+  cudaError_t e = launch_tiles(g, grid, g4, rot, nrot, rows, kOutGauss, 0.f, L, partial, nullptr,
+                               nullptr, 0, gsc, status, s);
+  if (e != cudaSuccess) return e;
+  expand_bias_kernel<<<(unsigned)(rows / kTRows), kTRows, 0, s>>>(
+      partial, (int)expand_tile_slices(g.ld_pix), rows, logw, nrot, inv,
+      bias, nullptr, nullptr, 0);
+  return cudaGetLastError();
+}
+
+int expand_gauss_launches(int64_t rows, int64_t ld_pix) {
+  return gauss_row_threads(rows, expand_tile_slices(ld_pix)) ? 1 : 2;
+}
+
 int expand_flu_launches(int64_t rows, int64_t ld_pix, bool delta) {
-  return !delta && flu_row_threads(rows, expand_tile_slices(ld_pix)) ? 1 : 3;
+  return !delta && row_threads(rows, expand_tile_slices(ld_pix)) ? 1 : 3;
 }
 
 cudaError_t launch_expand_flu(const Geom& g, const float* grid, const float4* g4, const RotFX* rot,
@@ -1020,21 +1093,10 @@ cudaError_t launch_expand_flu(const Geom& g, const float* grid, const float4* g4
   if (rows <= 0) return cudaSuccess;
   const int64_t ns = expand_tile_slices(g.ld_pix), nt = rows / kTRows;
   uint16_t* Lb = (uint16_t*)L.base;
-  const int th = Lold ? 0 : flu_row_threads(rows, ns);
-  if (th) {
-    const bool whole = ((uintptr_t)Lb & 3) == 0;
-    const int threads = whole ? th : 128;
-    auto kern = threads == 384 ? (g.interior ? expand_flu_row_kernel<384, true, true>
-                                             : expand_flu_row_kernel<384, false, true>)
-                : whole        ? (g.interior ? expand_flu_row_kernel<128, true, true>
-                                             : expand_flu_row_kernel<128, false, true>)
-                               : (g.interior ? expand_flu_row_kernel<128, true, false>
-                                             : expand_flu_row_kernel<128, false, false>);
-    kern<<<(unsigned)rows, threads, sizeof(float) * (size_t)g.ld_pix, s>>>(
-        g.qi, g.qlo, g.ld_pix, g.N, grid, g4, rot, logw, nrot, w_floor, c, (int)ns, Lb,
-        L.plane_stride, bias, bias + rows, Bctx, status);
-    return cudaGetLastError();
-  }
+  const int th = Lold ? 0 : row_threads(rows, ns);
+  if (th)
+    return launch_rows<kOutW>(th, g, grid, g4, rot, logw, nrot, rows, w_floor, c, nullptr, L, bias,
+                              bias + rows, Bctx, status, s);
   cudaError_t e = launch_tiles(g, grid, g4, rot, nrot, rows, kOutW, w_floor, L, nullptr, nullptr,
                                nullptr, 0, nullptr, status, s);
   if (e != cudaSuccess) return e;
