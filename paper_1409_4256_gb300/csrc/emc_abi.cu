@@ -1052,6 +1052,17 @@ int check_rot_range(emc_ctx* c, int64_t rot0, int64_t nrot) {
   return EMC_OK;
 }
 
+// Kernels of an expansion of every rotation: the row tiles and the bias sums (Gaussian: grid maximum
+// and scales first; Poisson fluence: the split; small ones all in one); the cell layout of the
+// model first where it is used.
+int expand_launches(const emc_ctx* c, bool delta) {
+  const Layout& y = c->lay;
+  return (is_gauss(&c->cfg)  ? 2 + expand_gauss_launches(y.rows, y.ld_pix)
+          : is_flu(&c->cfg) ? expand_flu_launches(y.rows, y.ld_pix, delta)
+                            : 2) +
+         ((y.g4 && c->geom.interior) ? 1 : 0);
+}
+
 // the Poisson-fluence expansion keeps what it needs on the way in L
 Order* expand_scratch(emc_ctx* c) {
   return is_flu(&c->cfg) && !(c->lay.g4 && c->geom.interior) ? nullptr : &c->expand_order;
@@ -1231,12 +1242,7 @@ int emc_iteration(emc_ctx* c, const float* grid_in, float* grid_out, emc_iter_st
     if (!scratch.ok()) return EMC_ERR_CUDA;
     if ((st = scratch.done(do_expand(c, grid_in, 0, n_rot, L, bias, s, Lold, bold)))) return st;
   }
-  // the row tiles and the bias sums (Gaussian: grid maximum and scales first;
-  // Poisson fluence: the split, or all in one); the cell layout of the model first where it is used
-  kernels += (is_gauss(&c->cfg) ? 2 + expand_gauss_launches(y.rows, y.ld_pix)
-              : is_flu(&c->cfg) ? expand_flu_launches(y.rows, y.ld_pix, Lold != nullptr)
-                                : 2) +
-             ((y.g4 && c->geom.interior) ? 1 : 0);
+  kernels += expand_launches(c, Lold != nullptr);
   if (stats) CU(cudaEventRecord(c->ev[1], s));
   float* S = (c->cfg.flags & EMC_FLAG_STORE_SCORES) ? (float*)(c->ws + y.S) : nullptr;
   // bound-pruned pass 1 over the frames in their internal order
@@ -1427,6 +1433,7 @@ int emc_iteration(emc_ctx* c, const float* grid_in, float* grid_out, emc_iter_st
     // kernel when recomputing in FP32)
     const bool split = pr ? !S && !kept : (S || c->cfg.precision != EMC_PREC_FP32);
     kernels += (split ? 2 : 1) + 2 + (kbf ? 1 : 0);
+    if (c->cfg.precision == EMC_PREC_FP32) kernels++;  // the update's non-zero frames
     // pairs: their search, the over lists, the rows; the row tiles contracted again marked
     if (pairs) kernels += 3 + (S || fv.kept_all ? 0 : 1);
     if (stats) {
@@ -1687,7 +1694,10 @@ int emc_sparse_iteration(emc_ctx* c, const float* grid_in, float* grid_out, emc_
     int32_t dst = 0;
     CU(cudaMemcpy(&dst, c->status, sizeof(int32_t), cudaMemcpyDeviceToHost));
     stats->device_status = dst;
-    stats->kernels = 9;
+    // expansion, scores, lse and its sum, update, compression, division
+    stats->kernels = expand_launches(c, false) + 5 +
+                     sparse_score_launches(c->cfg.n_data, c->cfg.n_cand, c->cfg.n_rot, y.ld_pix,
+                                           (c->cfg.flags & EMC_FLAG_SPARSE_K) != 0);
   }
   return EMC_OK;
 }

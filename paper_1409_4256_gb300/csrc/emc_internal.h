@@ -408,6 +408,7 @@ cudaError_t launch_sparse_scores(const Planes& L, int precision, int64_t rows, c
                                  const uint32_t* kent, int64_t n_data, const int32_t* cand,
                                  int64_t n_rot, long long* ubias, int* upper, double* Sc,
                                  cudaStream_t s);
+int sparse_score_launches(int64_t n_data, int M, int64_t n_rot, int64_t ld_pix, bool lists);
 // shift (may be NULL): per-frame constant of the scores, removed from lse_c
 cudaError_t launch_sparse_lse(const double* Sc, int64_t n_data, int64_t ld_data, int M, float* Pc,
                               double* lse_c, int32_t* status, cudaStream_t s,

@@ -1361,6 +1361,9 @@ int two_stages_from(int64_t n_data, int M, int64_t n_rot) {
   return n_data * M >= 64 * n_rot ? 384 : 0;
 }
 
+// the first stage of both forms in one launch: eight CTAs' 32-bit rows fit an SM
+bool both_forms(size_t row) { return 8 * (row + 1024) <= 233472; }
+
 template <int PREC>
 cudaError_t sparse_scores(const Planes& L, int64_t rows, const double* bias, const uint16_t* Kb,
                           int64_t ld_pix, const int64_t* off, const int2* ent, int M,
@@ -1388,7 +1391,7 @@ cudaError_t sparse_scores(const Planes& L, int64_t rows, const double* bias, con
   if (least == 0) return rows_kernel(sparse_rows_kernel<PREC, kFormScore>, row);
   if ((e = cudaFuncSetAttribute(sparse_lower_kernel<PREC>, attr, (int)(row / 2))) != cudaSuccess)
     return e;
-  if (8 * (row + 1024) <= 233472) {
+  if (both_forms(row)) {
     e = rows_kernel(sparse_rows_kernel<PREC, kFormBoth>, row);
   } else {
     e = rows_kernel(sparse_rows_kernel<PREC, kFormScore>, row);
@@ -1425,6 +1428,11 @@ cudaError_t launch_sparse_scores(const Planes& L, int precision, int64_t rows, c
     default: EMC_SPARSE_SCORES(EMC_PREC_BF16_SPLIT);
   }
 #undef EMC_SPARSE_SCORES
+}
+
+int sparse_score_launches(int64_t n_data, int M, int64_t n_rot, int64_t ld_pix, bool lists) {
+  if (!lists || two_stages_from(n_data, M, n_rot) == 0) return 1;
+  return both_forms(sizeof(float) * (size_t)ld_pix) ? 3 : 4;
 }
 
 cudaError_t launch_sparse_lse(const double* Sc, int64_t n_data, int64_t ld_data, int M, float* Pc,
