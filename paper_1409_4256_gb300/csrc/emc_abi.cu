@@ -568,8 +568,6 @@ static int ctx_create(const emc_config* cfg, const double* q, const double* quat
   c->geom.ngroups = (int)gstart.size() - 1;
   c->geom.gstart = (const int32_t*)(c->ws + y.cgs);
   c->geom.gpix = (const int32_t*)(c->ws + y.cgp);
-  c->geom.gqh = (const float4*)(c->ws + y.cgqh);
-  c->geom.gql = (const float4*)(c->ws + y.cgql);
   c->geom.gqi = (const int4*)(c->ws + y.cgqi);
   c->geom.gqlo = (const float4*)(c->ws + y.cgqlo);
   c->geom.gqf = (const float4*)(c->ws + y.cgqf);

@@ -137,10 +137,6 @@ __device__ __forceinline__ float cell_value(const Cell& c, const float* t) {
   const float vb = sy * fmaf(tz, b.y, sz * b.x) + ty * fmaf(tz, b.w, sz * b.z);
   return fmaf(t[0], vb, (1.f - t[0]) * va);
 }
-__device__ __forceinline__ float trilinear_g4(const float4* __restrict__ g4, int N, const int* f,
-                                              const float* t) {
-  return cell_value(load_cell(g4, (f[0] * N + f[1]) * N + f[2]), t);
-}
 
 // FP32 -> FP64 with integer operations (the conversion instruction runs on the
 // FP64 pipe, at 1/64 of the FP32 rate on this part): sign, exponent rebiased by

@@ -7,11 +7,8 @@
 
 namespace emc {
 
-// Rotation matrix R_j (row-major 3x3) as double-float pairs (h, l) of FP32,
-// computed once per context on the host in FP64.
-
-// Rotation R_j in fixed point for the e-step: R = hi 2^-20 + lo (hi integer,
-// |lo| <= 2^-21), row-major 3x3.
+// Rotation R_j (row-major 3x3) in fixed point, computed once per context on the
+// host in FP64: R = hi 2^-20 + lo (hi integer, |lo| <= 2^-21).
 struct RotFX {
   int32_t hi[9];
   float lo[9];
@@ -32,21 +29,18 @@ struct Geom {
   // compression groups: the used pixels split by (q_x, q_y) into groups of at
   // most kCompressGroup pixels spanning at most kCompressExtent voxels along
   // q_x and q_y (pixel_groups.h); group g holds the positions
-  // gstart[g] .. gstart[g + 1] of gpix (pixel columns) and of gqh/gql (their
+  // gstart[g] .. gstart[g + 1] of gpix (pixel columns) and of gqi/gqlo/gqf (their
   // geometry in that order)
   int ngroups;
   const int32_t* gstart;
   const int32_t* gpix;
-  const float4* gqh;
-  const float4* gql;
-  const int4* gqi;    // the same in fixed point
+  const int4* gqi;    // position q of each, fixed point 2^-12 (gqlo: the rest)
   const float4* gqlo;
   const float4* gqf;  // gqi 2^-12 as FP32
 };
 constexpr int kCompressGroup = 32;
 constexpr double kCompressExtent = 8.0;
 
-// A block of rows of a (possibly multi-plane) row-major matrix.
 // The rows' non-zero pairs (pairs.cu). cnt, then tile_n and over behind it; the arrays of
 // pairs hold kRowPairs a row. A row tile with a row of more, or more than kTilePairs in
 // all, is over: a pair costs its frame's row out of the L2 (2 ld_pix bytes), a 64-frame block of
@@ -65,6 +59,7 @@ struct RowPairs {
   float* p;       // P_jk
 };
 
+// A block of rows of a (possibly multi-plane) row-major matrix.
 struct Planes {
   void* base;            // first row of plane 0
   int64_t plane_stride;  // elements between planes

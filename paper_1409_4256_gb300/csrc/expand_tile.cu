@@ -150,10 +150,9 @@ __device__ __forceinline__ float trilinear_fx(const float* __restrict__ grid, in
   return W;
 }
 
-// value of one element of L in the precision's layout (old planes, DELTA)
+// values of two elements of a split L (old planes, DELTA)
 template <int PREC>
 __device__ __forceinline__ float2 read_pair(const void* L, int64_t o, int64_t ps) {
-  if (PREC == EMC_PREC_FP32) return *reinterpret_cast<const float2*>((const float*)L + o);
   const uint16_t* b = (const uint16_t*)L;
   auto val = [&](int64_t oo) -> float2 {
     const uint32_t u = *reinterpret_cast<const uint32_t*>(b + oo);
@@ -162,7 +161,7 @@ __device__ __forceinline__ float2 read_pair(const void* L, int64_t o, int64_t ps
     return make_float2(bf16_val((uint16_t)(u & 0xffffu)), bf16_val((uint16_t)(u >> 16)));
   };
   float2 v = val(o);
-  const int np = PREC == EMC_PREC_BF16_SPLIT ? 3 : (PREC == EMC_PREC_FP16_SPLIT ? 2 : 1);
+  const int np = PREC == EMC_PREC_BF16_SPLIT ? 3 : 2;
   for (int q = 1; q < np; q++) {
     const float2 w = val(o + q * ps);
     v.x += w.x;  // planes of one element: their sum rounds at most twice
@@ -289,6 +288,8 @@ __global__ void __launch_bounds__(kTThreads, 6)
                        void* __restrict__ Lbase, int64_t ps, double* __restrict__ partial,
                        const void* __restrict__ Lold, uint16_t* __restrict__ D, int64_t ntp,
                        unsigned slices, const float4* __restrict__ gsc, int32_t* status) {
+  static_assert(!DELTA || PREC == EMC_PREC_BF16_SPLIT || PREC == EMC_PREC_FP16_SPLIT,
+                "increments: the contexts that prune");
   __shared__ RowFX R[RPC];
   __shared__ float2 rsum[kTThreads / 32][RPC];
   // eight rows of every lane's pair, rows padded to 33 so that the transposed
@@ -402,21 +403,9 @@ __global__ void __launch_bounds__(kTThreads, 6)
         put_pair<WHOLE>(Lb + ps, __byte_perm(u0, u1, 0x5410));
       } else if (PREC == EMC_PREC_FP32) {
         *reinterpret_cast<float2*>((float*)Lbase + o) = make_float2(L[0], L[1]);
-        if (DELTA && vrow) {
-          const float2 old = read_pair<PREC>(Lold, o, ps);
-          const float d0 = L[0] - old.x, d1 = L[1] - old.y;
-          dp[0] = fmaxf(dp[0], d0); dm[0] = fmaxf(dm[0], -d0);
-          dp[1] = fmaxf(dp[1], d1); dm[1] = fmaxf(dm[1], -d1);
-        }
       } else if (PREC == EMC_PREC_BF16) {
         const uint16_t b0 = bf16_bits(L[0]), b1 = bf16_bits(L[1]);
         *reinterpret_cast<uint32_t*>((uint16_t*)Lbase + o) = (uint32_t)b0 | ((uint32_t)b1 << 16);
-        if (DELTA && vrow) {
-          const float2 old = read_pair<PREC>(Lold, o, ps);
-          const float d0 = bf16_val(b0) - old.x, d1 = bf16_val(b1) - old.y;
-          dp[0] = fmaxf(dp[0], d0); dm[0] = fmaxf(dm[0], -d0);
-          dp[1] = fmaxf(dp[1], d1); dm[1] = fmaxf(dm[1], -d1);
-        }
       } else if (PREC == EMC_PREC_FP16_SPLIT) {
         uint16_t h[2], rr[2];
         float v[2];

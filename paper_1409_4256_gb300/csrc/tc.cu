@@ -77,7 +77,7 @@ template <int MODE, int NA, bool F16, bool XP = false, int BNT = BN>
 struct TcCfg {
   static constexpr int BK = (MODE != MODE_UPDATE && NA >= 2) ? 32 : 64;
   static constexpr int A_BYTES = BM * BK * 2;  // one 128 x BK BF16 plane
-  static constexpr int B_BYTES = BNT * BK * 2;  // 256 x BK BF16
+  static constexpr int B_BYTES = BNT * BK * 2;  // BNT x BK BF16
   static constexpr int STAGE = NA * A_BYTES + B_BYTES;
   static constexpr int NACC = (MODE != MODE_UPDATE && NA >= 2) ? 2 : 1;
   // XP (update over listed blocks, store): a 32 x 32 staging block per
