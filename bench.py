@@ -764,32 +764,36 @@ def adaptive_form(torch, args, cfg, ds, grid, K_dev, stream, ctx, fixed_ms):
             "fixed_d_loglik_per_iteration": fixed_ll}
 
 
-# DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) per launch of the
-# steady iterations, from the one-pass ncu launch-list capture of this exact
-# configuration (emc64, BF16 split, 20000 frames, stored scores; the full-size
-# workload; its summary is kept with the other profiles)
+# DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) of a launch, from ncu
+# captures of this configuration with fewer frames (emc64, BF16 split, 50100
+# rotations, stored scores; the summaries are kept with the other profiles), and
+# those frames. The expansion's do not depend on them; the compression's grow with
+# the rows that have mass, pass 1's with the frames.
 MEASURED_TRAFFIC_EMC64 = {
-    # pass 1 of a steady pruned iteration: the increments' product, the
-    # hi-plane bound over the few listed pairs and the exact pass over the
-    # live tiles; dense: the single three-plane launch of the first iteration
-    "pass1_pruned": 0.332e9 + 0.00003e9 + 1.957e9,
-    "pass1_dense": 6.713e9 + 4.247e9,
-    "compress": 0.272e9,
-    "expand": 1.673e9,
+    # the first pruned iteration's hi-plane bound over every pair and its exact
+    # pass over the live tiles; dense: the single three-plane launch
+    "pass1_pruned": (0.303e9 + 1.013e9, 2048),
+    "pass1_dense": (1.223e9 + 0.409e9, 2048),
+    "compress": (0.134e9 + 0.004e9, 8192),
+    "expand": (0.857e9 + 0.820e9, 8192),
 }
 
 
 def traffic_for(workload, precision, n_rot, n_data, recompute, phases, kernel="pass1"):
-    """DRAM bytes per launch (pass 1: per iteration) of one phase's kernels from
-    the ncu capture of this exact configuration; None where no capture of the
-    configuration exists."""
+    """(DRAM bytes of one phase's kernels, frames of the capture they come from);
+    (None, None) where no capture of the configuration exists."""
     if not (workload == "emc64" and precision == "bf16_split" and n_data == 20000
             and n_rot == 50100 and not recompute):
-        return None
+        return None, None
     if kernel == "pass1":
-        pruned = bool(phases.get("pass1_bound_pruned_steps"))
-        return MEASURED_TRAFFIC_EMC64["pass1_pruned" if pruned else "pass1_dense"]
-    return MEASURED_TRAFFIC_EMC64.get(kernel)
+        kernel = "pass1_pruned" if phases.get("pass1_bound_pruned_steps") else "pass1_dense"
+    return MEASURED_TRAFFIC_EMC64[kernel]
+
+
+def traffic_source(frames):
+    return ("unmeasured for this configuration" if frames is None else
+            "ncu dram__bytes_read.sum + dram__bytes_write.sum, the same rotations with "
+            f"{frames} frames")
 
 
 def pass1_roofline(precision, n_pix, n_rot, n_data, phases, traffic):
@@ -830,11 +834,10 @@ def pass1_roofline(precision, n_pix, n_rot, n_data, phases, traffic):
                  "frac": (done if pruned else achieved) / peak,
                  "dense_equivalent_achieved": achieved,
                  "dense_equivalent_frac": achieved / peak,
-                 "traffic": traffic,
-                 "traffic_unit": ("bytes per iteration's pass 1 (increments, bound and exact "
-                                  "launches)" if pruned else "bytes per launch"),
-                 "traffic_source": ("ncu capture of this configuration" if traffic is not None
-                                    else "unmeasured for this configuration"),
+                 "traffic": traffic[0],
+                 "traffic_unit": ("bytes of the first pruned iteration's bound and exact "
+                                  "launches" if pruned else "bytes per launch"),
+                 "traffic_source": traffic_source(traffic[1]),
                  "algorithmic_flops_per_launch": flops, "executed_flops_per_launch": executed,
                  "executed_frac": executed / (dom_ms * 1e-3) / 1e12 / peak,
                  "exact_tile_fraction": exact,
@@ -993,17 +996,15 @@ def run_ours(args):
                                           ctx.buffer_sizes(n_rot).ld_pix, n_rot, n_data,
                                           phases, roof1)
     # the roofline line is the dominant phase's; the others follow in "rooflines"
-    traffic_src = ("ncu dram__bytes_read.sum + dram__bytes_write.sum of one full-size launch "
-                   "(one-pass launch-list capture of this configuration)")
     for k, name in (("compress", "compress_kernel (c-step, Eq. 2.12): trilinear scatter of the "
                                  "slices into the grid, corner terms merged in shared memory, "
                                  "FP64 reductions in L2"),
                     ("expand", "expand_tile_kernel (e-step, Eq. 2.9): trilinear gather of the "
                                "slices, log W split into planes, increments of the bound")):
-        tr = traffic_for(args.workload, args.precision, n_rot, n_data, args.recompute, phases, k)
+        tr, tr_frames = traffic_for(args.workload, args.precision, n_rot, n_data,
+                                    args.recompute, phases, k)
         rooflines[k].update({"kernel": name, "traffic": tr,
-                             "traffic_source": traffic_src if tr is not None
-                             else "unmeasured for this configuration"})
+                             "traffic_source": traffic_source(tr_frames)})
     roof = dict(rooflines[dominant], phase=dominant)
 
     # ---- other precision forms, briefly --------------------------------------

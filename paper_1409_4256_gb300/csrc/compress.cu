@@ -50,7 +50,7 @@ constexpr int kAggWarps = 4;
 constexpr int kAggCap = 576;       // box slots per warp (float2 each), below 1024
 constexpr int kAggList = 32 * 8;   // touched slots of a group: at most 8 per pixel
 constexpr int kAggThreads = kAggWarps * 32;
-// 22 KB per CTA: eight CTAs (32 warps) per SM, at most 64 registers a thread
+// 22.5 KB per CTA: eight CTAs (32 warps) per SM, at most 64 registers a thread
 constexpr size_t kAggSmem = kAggWarps * (sizeof(float2) * kAggCap + sizeof(int) * kAggList);
 static_assert(kCompressGroup == 32, "one pixel per lane");
 

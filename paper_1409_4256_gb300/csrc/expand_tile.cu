@@ -703,9 +703,10 @@ __global__ void __launch_bounds__(kTThreads)
     write_increments<EMC_PREC_BF16_SPLIT>(dp, dm, rises, inside, t, i0, ld_pix, ntp, D);
 }
 
-// The whole Poisson-fluence expansion of small problems in one launch, and the Gaussian one
-// (OUT: kOutW, kOutGauss), a CTA of TH threads per rotation, with W in shared memory: the
-// tile kernels' launches leave most SMs idle there and each waits for the one before. TH / 128 slices of 256 pixels at a time; the sums in
+// The whole Poisson-fluence expansion of small problems in one launch, and the
+// Gaussian one (OUT: kOutW, kOutGauss), a CTA of TH threads per rotation, with W
+// in shared memory: the tile kernels' launches leave most SMs idle there and each
+// waits for the one before. TH / 128 slices of 256 pixels at a time; the sums in
 // the order of the other form, so the bits are the same whichever runs. Bound by the
 // latency of a slice's chain of loads: 384 threads where the SMs hold all rows' CTAs at
 // once, 128 (ten CTAs an SM) where they do not (row_threads).

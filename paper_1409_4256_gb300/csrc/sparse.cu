@@ -7,8 +7,9 @@
 // The pairs are transposed once into a CSR list per rotation, so that both
 // contractions read one log W row (staged in shared memory) and gather the
 // frames' rows of K, which are 3x smaller than a split log W row and stay in L2
-// at the 64^3 size. Scores use the same exact split as the dense forms (hi on
-// the 1/8 grid accumulated exactly, a small residual).
+// at the 64^3 size. Scores use the dense forms' split of log W, its sums exact:
+// as integers from a frame's non-zero list (sparse_rows_kernel), or hi on the 1/8
+// grid and a small residual from its row (sparse_scores_kernel).
 #include <limits.h>
 
 #include <algorithm>
