@@ -577,9 +577,11 @@ cudaError_t mlp_train_step(const MlpLayout& y, float* params, float* grads, floa
   softmax_lse_kernel<<<B, 512, 0, s>>>(w.z, y.ld_out, (int)y.n_out, zb, tidx, tprob, R, B, lse,
                                        mass, loss);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  // chunks of 512 rows where the columns leave SMs idle (their sums fit da, which is written later)
+  // chunks of 512 rows where the columns leave SMs idle; their sums are kept in da, which is
+  // written later: ceil(B / 512) ld_out values in B H, which fit from 256 H columns down (two chunks
+  // of 513 rows are the tightest)
   const int64_t cols = (y.ld_out + 127) / 128;
-  const int chunk = cols >= 4 * num_sms() || y.ld_out > 512 * H ? B : std::min(B, 512);
+  const int chunk = cols >= 4 * num_sms() || y.ld_out > 256 * H ? B : std::min(B, 512);
   const int chunks = (B + chunk - 1) / chunk;
   auto grad = (int64_t)R * 256 >= y.n_out ? softmax_grad_kernel<true, true>
               : chunks > 1                ? softmax_grad_kernel<false, true>

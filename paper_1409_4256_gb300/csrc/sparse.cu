@@ -360,9 +360,9 @@ __global__ void __launch_bounds__(kTopThreads, 2)
   top_select<true>(keys, idx, cnt, M, wt, par, &s_min, cand + (int64_t)blockIdx.x * M);
 }
 
-// Longer lists, and many short rows. One CTA (256 threads) per row: radix selection of the M-th largest key over
-// four 8-bit digits, then the keys above it in index order followed by the
-// first equal keys in index order (ties towards the lower index).
+// Longer lists, and many short rows. One CTA (256 threads) per row: radix selection
+// of the M-th largest key over four 8-bit digits, then the keys above it in index order
+// followed by the first equal keys in index order (ties towards the lower index).
 __global__ void __launch_bounds__(256)
     topm_kernel(const float* __restrict__ logits, int64_t ld, int n, int M,
                 int32_t* __restrict__ cand) {
@@ -421,10 +421,10 @@ cudaError_t launch_topm(const float* logits, int64_t B, int64_t n, int64_t ld, i
                         int32_t* cand, cudaStream_t s) {
   if (B <= 0) return cudaSuccess;
   // Rows of up to four chunks that are streamed (no sample) are bound by the selection, two
-  // CTAs an SM at a time; with more of them than five an SM the histograms' eight CTAs of 256 threads
-  // finish earlier (2048 x 1380, M = 64: 59 and 46 us; 2048 x 9000, M = 4096: 195 and 134; 800 x 1380, M = 64:
-  // 29 and 27; but 100 x 1380, M = 512: 11 and 25; 2048 x 100, M = 100: 35 and 44; 2048 x 20000, M = 4096,
-  // ties: 240 and 292).
+  // CTAs an SM at a time; with more of them than five an SM the histograms' eight CTAs of
+  // 256 threads finish earlier (2048 x 1380, M = 64: 59 and 46 us; 2048 x 9000, M = 4096:
+  // 195 and 134; 800 x 1380, M = 64: 29 and 27; but 100 x 1380, M = 512: 11 and 25;
+  // 2048 x 100, M = 100: 35 and 44; 2048 x 20000, M = 4096, ties: 240 and 292).
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
